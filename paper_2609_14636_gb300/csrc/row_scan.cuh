@@ -1,6 +1,8 @@
-// row_scan.cuh -- the per-row tail of the batch scoring kernels: the row's
-// log-probs and outputs, its element of the decoupled-lookback segmented
-// scan, turn statistics, the stop test and the carried state.
+// row_scan.cuh -- the per-row tail of the batch kernel that takes one CTA per
+// row: the row's log-probs and outputs, its element of the decoupled-lookback
+// segmented scan, turn statistics, the stop test and the carried state.  The
+// lookback itself also serves the tiled scans (warp_tile_scan.cuh, and the
+// scan on log-probs in vocab_parallel.cu), whose tiles are many rows.
 //
 // The running stop sum is a plain prefix sum over rows of a per-row term:
 //   TOKEN_SUM (Sec. 5.5):   term = log pi_T(y_t)
@@ -219,9 +221,7 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
 // The part of a row's tail that waits on nobody: outputs, the row's scan
 // element, the within-turn profile, and the element's publication (an
 // AGGREGATE, or, for a tile that starts a trajectory or the window, the
-// INCLUSIVE prefix seeded from the carried state).  Lane 0 only.  `prof`
-// (30 doubles, or NULL) receives the profile: with atomics when it is the
-// caller's global array, plainly when it is one writer's shared copy.
+// INCLUSIVE prefix seeded from the carried state).  Lane 0 only.
 struct RowCarry {
   ScanElem e;
   ScanElem incl;      // valid for seeded tiles
@@ -232,8 +232,7 @@ struct RowCarry {
 
 __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t tile, int64_t r,
                                                  const RowMeta& meta, bool token_ok, float xs, float xt,
-                                                 float lse_s, float lse_t, double* prof,
-                                                 bool prof_atomic) {
+                                                 float lse_s, float lse_t) {
   RowCarry rc;
   const int64_t n_k = meta.turn_end - meta.turn_start;
   const float nan = __int_as_float(0x7fc00000);
@@ -260,17 +259,11 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
   e.sd = (double)dd;
   e.sl = (double)lps * (double)dd;  // -log pi_S * r_t (Eq. 2)
   e.fturn = (r == meta.turn_start) ? 1 : 0;
-  if (prof && !meta.bad) {
+  if (p.profile && !meta.bad) {
     const int j = (int)((10 * (r - meta.turn_start)) / n_k);  // Observation 1 decile
-    if (prof_atomic) {
-      atomicAdd(prof + 3 * j + 0, e.sd);
-      atomicAdd(prof + 3 * j + 1, e.st);
-      atomicAdd(prof + 3 * j + 2, 1.0);
-    } else {
-      prof[3 * j + 0] += e.sd;
-      prof[3 * j + 1] += e.st;
-      prof[3 * j + 2] += 1.0;
-    }
+    atomicAdd(p.profile + 3 * j + 0, e.sd);
+    atomicAdd(p.profile + 3 * j + 1, e.st);
+    atomicAdd(p.profile + 3 * j + 2, 1.0);
   }
   rc.e = e;
   rc.seeded = (tile == 0) || (r == meta.traj_start) || meta.bad;
@@ -397,7 +390,7 @@ __device__ __forceinline__ void finish_row(const BatchParams& p, int64_t tile, i
                                            const RowMeta& meta, int32_t y, float xs, float xt,
                                            float lse_s, float lse_t, int lane) {
   RowCarry rc;
-  if (lane == 0) rc = row_finalize(p, tile, r, meta, y >= 0 && y < p.V, xs, xt, lse_s, lse_t, p.profile, true);
+  if (lane == 0) rc = row_finalize(p, tile, r, meta, y >= 0 && y < p.V, xs, xt, lse_s, lse_t);
   row_resolve(p, tile, r, meta, rc, lane);
 }
 

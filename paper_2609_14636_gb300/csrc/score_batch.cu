@@ -455,16 +455,16 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
     q.ticket = p.ticket + 1;
     return launch_scan_logprobs(q, p.ws_logp_s, p.ws_logp_t, stream, true);
   }
-  {
-    const cudaError_t e = launch_clear_workspace(p.ticket, clear_bytes, sms, stream);
-    if (e != cudaSuccess) return e;
-  }
   const int per_vec = dtype == STRIDE_DTYPE_BF16 ? 8 : 4;
   // (the persistent kernel counts a row's bytes in 32 bits: rows of up to
   // 2 GB, far beyond any vocabulary, take it)
   const int64_t row_bytes = (int64_t)p.V * (dtype == STRIDE_DTYPE_BF16 ? 2 : 4);
-  if (vec && p.V >= per_vec && row_bytes <= ((int64_t)1 << 31) && !f_rows)
-    return launch_score_batch_stream(p, dtype, stream);
+  const bool persistent = vec && p.V >= per_vec && row_bytes <= ((int64_t)1 << 31) && !f_rows;
+  // the persistent kernel scans 32-row tiles: one flag line per tile
+  const size_t clear = persistent ? stream_clear_bytes(p.n_rows) : clear_bytes;
+  const cudaError_t ce = launch_clear_workspace(p.ticket, clear, sms, stream);
+  if (ce != cudaSuccess) return ce;
+  if (persistent) return launch_score_batch_stream(p, dtype, stream);
   const dim3 grid((unsigned)p.n_rows), block(kBatchThreads);
   if (dtype == STRIDE_DTYPE_BF16) {
     if (vec)

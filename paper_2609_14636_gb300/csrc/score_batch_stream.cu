@@ -13,25 +13,29 @@
 //                      without spending registers on them.
 //   warps 6..21,       read each stage from shared memory into single-pass
 //   consumers          online log-sum-exp pairs (stride_device.cuh), release
-//                      the stage, and at a row's last chunk merge their pairs
-//                      for the row warp.
-//   warp 1, row warp   per row, while the row streams: trajectory/turn lookup,
-//                      token, gathered logits, the ragged tail (V mod 8
-//                      logits); once the row's pairs land: log-probs, outputs,
-//                      and the row's scan element published at once
-//                      (row_finalize).  It never waits on another CTA, so
-//                      every row's AGGREGATE appears as soon as the row is
-//                      scored, which keeps every lookback short.
-//   warps 2..5, scan   rows taken round-robin (row n by scan warp n mod 4):
-//                      the decoupled lookback, the INCLUSIVE publication,
-//                      turn statistics, stop test and carried state
-//                      (row_resolve).  Four lookbacks can be in flight per
-//                      SM, and the scan warps may lag the row warp by up to
-//                      kSlots rows without stalling the stream.
+//                      the stage, and at a row's last chunk post their pairs
+//                      for the row's row warp.
+//   warps 1..4, row    rows taken round-robin (row n by row warp n mod 4).
+//   warps              While the row streams: token, gathered logits, the
+//                      ragged tail (V mod 8 logits).  Once the consumers'
+//                      pairs land: their merge, log-probs and outputs, then
+//                      the row is counted in at its 32-row tile; the warp
+//                      that counts a tile's last row publishes the tile
+//                      (warp_tile_scan.cuh) and queues it for the scan warp.
+//   warp 5, scan warp  completes the queued tiles: lookback, turn
+//                      statistics, stop test, carried state.
+//
+// Rows of any length should be bound by HBM.  With one row warp, which also
+// searched the row's turn and formed its scan element, a row cost about 4.7
+// us of dependent latency, more than its bytes take below about 100,000 bf16
+// logits.  GB300, before -> now: 30,011 rows of 32,000 bf16 logits 919 -> 544
+// us (4,180 -> 7,060 GB/s); 3,001 rows of 151,936 267.5 -> 263.5 us; 20,000
+// rows of 151,936 in two windows 1,654 -> 1,645 us (7,390 GB/s): with long
+// rows what was left is the shorter tail of a window's scan.
 //
 // Hand-offs inside the CTA use mbarriers only (no named barriers): full/empty
 // per stage, and per row slot (kSlots rows in flight) start / red_done /
-// lse_ready / agg_ready / slot_free.  Every wait is bounded by a
+// slot_free.  Every wait is bounded by a
 // %globaltimer budget; on expiry the CTA sets STRIDE_DEV_TIMEOUT, stops
 // issuing, waits (bounded) for the copies it has in flight, and returns.
 #include <math.h>
@@ -43,6 +47,7 @@
 #include "stride.h"
 #include "stride_device.cuh"
 #include "stride_internal.h"
+#include "warp_tile_scan.cuh"
 
 // Ring shape: 3 stages of 32 KB per tensor (192 KB in flight per SM).  A
 // sweep on GB300 over stages x chunk bytes at up to 218 KB of ring (the
@@ -66,31 +71,33 @@ constexpr int kChunk = STRIDE_BULK_CHUNK;     // bytes per tensor per stage
 constexpr int kSlots = 8;                     // rows in flight per CTA
 constexpr int kConsumerWarps = 16;
 constexpr int kConsumers = kConsumerWarps * 32;
-constexpr int kScanWarps = 4;
-constexpr int kFirstConsumerWarp = 2 + kScanWarps;
+constexpr int kRowWarps = 4;
+constexpr int kScanWarp = 1 + kRowWarps;
+constexpr int kFirstConsumerWarp = 2 + kRowWarps;
 constexpr int kStreamThreads = 32 * kFirstConsumerWarp + kConsumers;
 constexpr int kInfoEnd = -1;
 constexpr int kInfoLast = 1 << 16;
 static_assert(kChunk % 16 == 0, "bulk copies move multiples of 16 bytes");
+constexpr int kQueue = 8;  // published tiles waiting for the scan warp
+static_assert(kSlots % kRowWarps == 0, "a row warp keeps its own slots");
 
 struct alignas(128) StreamShared {
   uint64_t full[kStages];
   uint64_t empty[kStages];
   uint64_t start[kSlots];
-  uint64_t lse_ready[kSlots];
-  uint64_t slot_free[kSlots];
   uint64_t red_done[kSlots];
-  uint64_t agg_ready[kSlots];
+  uint64_t slot_free[kSlots];
   int32_t stage_info[kStages];
   uint32_t stage_bytes[kStages];
-  int64_t slot_tile[kSlots];
-  float slot_pair[kSlots][4];
-  float red[kSlots][kConsumerWarps][4];
-  RowMeta slot_meta[kSlots];
-  RowCarry slot_carry[kSlots];
-  double prof[3 * STRIDE_PROFILE_BINS];  // this CTA's within-turn profile (row warp only)
-  int64_t end_seq;  // first row sequence number without a row (set by the row warp)
+  int64_t slot_tile[kSlots];  // window row, -1 past the last
+  float4 red[kSlots][kConsumerWarps];  // the consumer warps' (mS, sS, mT, sT)
+  uint64_t queue_full[kQueue];
+  uint32_t queue_head;          // entries claimed by the row warps
+  uint32_t queue_tail;          // entries completed by the scan warp
+  uint32_t rows_done[kRowWarps];
   int32_t abort;
+  TileCarry queue[kQueue];      // tile -1: a row warp has finished
+  TileCarry own[kRowWarps];     // a row warp's tile that found the queue full
 };
 
 constexpr size_t kStreamHeader = (sizeof(StreamShared) + 127) & ~size_t(127);
@@ -100,6 +107,19 @@ static_assert(kStreamSmem <= 227 * 1024, "ring and header exceed the shared memo
 __device__ __forceinline__ void raise_abort(StreamShared& sh, const BatchParams& p) {
   *reinterpret_cast<volatile int32_t*>(&sh.abort) = 1;
   set_status(p.dev_status, STRIDE_DEV_TIMEOUT);
+}
+
+// Claims the next entry of the queue to the scan warp, -1 if it is full.
+__device__ __forceinline__ int queue_claim(StreamShared& sh) {
+  uint32_t n = *reinterpret_cast<volatile uint32_t*>(&sh.queue_head);
+  while (true) {
+    if (n - *reinterpret_cast<volatile uint32_t*>(&sh.queue_tail) >= (uint32_t)kQueue) return -1;
+    const uint32_t was = atomicCAS(&sh.queue_head, n, n + 1);
+    if (was == n) break;
+    n = was;
+  }
+  __threadfence_block();  // the entry's last reader has left it (it moved queue_tail after its last read)
+  return (int)(n % kQueue);
 }
 
 template <typename LT>
@@ -117,6 +137,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
   const int v_body = p.V / P;  // 16-byte vectors per row streamed by bulk copies
   const uint32_t row_bytes = (uint32_t)v_body * 16u;
   const int n_chunks = (int)((row_bytes + kChunk - 1) / kChunk);
+  // chunks of equal size, so that a row's last stage is as full as the others
+  const uint32_t chunk = ((row_bytes / 16u + n_chunks - 1) / n_chunks) * 16u;
   const uint64_t tmo = p.timeout_ns;
 
   if (tid == 0) {
@@ -126,14 +148,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     }
     for (int q = 0; q < kSlots; ++q) {
       mbar_init(&sh.start[q], 1);
-      mbar_init(&sh.lse_ready[q], 1);
-      mbar_init(&sh.slot_free[q], 1);
       mbar_init(&sh.red_done[q], kConsumerWarps);
-      mbar_init(&sh.agg_ready[q], 1);
+      mbar_init(&sh.slot_free[q], 1);
     }
+    for (int i = 0; i < kQueue; ++i) mbar_init(&sh.queue_full[i], 1);
+    for (int i = 0; i < kRowWarps; ++i) sh.rows_done[i] = 0;
+    sh.queue_head = sh.queue_tail = 0;
     sh.abort = 0;
-    sh.end_seq = INT64_MAX;
-    for (int i = 0; i < 3 * STRIDE_PROFILE_BINS; ++i) sh.prof[i] = 0.0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -156,29 +177,29 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       uint32_t it = 0;  // stages issued
       int64_t seq = 0;  // rows started by this CTA
       bool ok = true;
-      while (ok) {
+      uint32_t t = atomicAdd(p.ticket, 1u);
+      while ((int64_t)t < p.n_rows) {
         const int q = (int)(seq % kSlots);
         const uint32_t use = (uint32_t)(seq / kSlots);
         if (use > 0 && !mbar_wait(&sh.slot_free[q], (use - 1) & 1u, tmo, abort)) {
           ok = false;
           break;
         }
-        const uint32_t t = atomicAdd(p.ticket, 1u);
-        const bool done = (int64_t)t >= p.n_rows;
-        sh.slot_tile[q] = done ? -1 : (int64_t)t;
+        sh.slot_tile[q] = (int64_t)t;
         mbar_arrive(&sh.start[q]);
-        if (done) break;
         const unsigned char* srow = reinterpret_cast<const unsigned char*>(p.S) + (int64_t)t * p.ld * sizeof(LT);
         const unsigned char* trow = reinterpret_cast<const unsigned char*>(teacher_row<LT>(p, (int64_t)t));
         for (int c = 0; c < n_chunks; ++c) {
+          // the next row's ticket arrives while the last chunk waits for its stage
+          if (c == n_chunks - 1) t = atomicAdd(p.ticket, 1u);
           const int s = (int)(it % kStages);
           const uint32_t k = it / kStages;
           if (k > 0 && !mbar_wait(&sh.empty[s], (k - 1) & 1u, tmo, abort)) {
             ok = false;
             break;
           }
-          const uint32_t off = (uint32_t)c * kChunk;
-          const uint32_t bytes = min((uint32_t)kChunk, row_bytes - off);
+          const uint32_t off = (uint32_t)c * chunk;
+          const uint32_t bytes = min(chunk, row_bytes - off);
           sh.stage_info[s] = q | (c == n_chunks - 1 ? kInfoLast : 0);
           sh.stage_bytes[s] = bytes;
           mbar_arrive_expect_tx(&sh.full[s], 2u * bytes);
@@ -186,10 +207,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
           bulk_g2s(bufT + (size_t)s * kChunk, trow + off, bytes, &sh.full[s], policy);
           ++it;
         }
+        if (!ok) break;
         ++seq;
       }
       if (ok) {
-        // end marker for the consumers in the next stage
+        // end markers: for the consumers in the next stage, for the row
+        // warps in their next slots
         const int s = (int)(it % kStages);
         const uint32_t k = it / kStages;
         if (k == 0 || mbar_wait(&sh.empty[s], (k - 1) & 1u, tmo, abort)) {
@@ -198,6 +221,16 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
           mbar_arrive(&sh.full[s]);
         } else {
           ok = false;
+        }
+        for (int i = 0; ok && i < kRowWarps; ++i, ++seq) {
+          const int q = (int)(seq % kSlots);
+          const uint32_t use = (uint32_t)(seq / kSlots);
+          if (use > 0 && !mbar_wait(&sh.slot_free[q], (use - 1) & 1u, tmo, abort)) {
+            ok = false;
+            break;
+          }
+          sh.slot_tile[q] = -1;
+          mbar_arrive(&sh.start[q]);
         }
       }
       if (!ok) {
@@ -221,7 +254,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     const int cw = warp - kFirstConsumerWarp;
     const int ct = tid - 32 * kFirstConsumerWarp;
     uint32_t it = 0;
-    int64_t seq = 0;  // rows finished, in the producer's order
     float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
     while (true) {
       const int s = (int)(it % kStages);
@@ -252,38 +284,15 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       if (lane == 0) mbar_arrive(&sh.empty[s]);
       ++it;
       if (info & kInfoLast) {
-        // Row end: each warp posts its pair under the row's slot; warp 0
-        // merges them once all 16 have arrived.  red[q] is reused only after
-        // the scan warp has released slot q, which follows warp 0's read.
+        // Row end: each warp posts its pair under the row's slot; the row
+        // warp merges them once all 16 have arrived.  red[q] is reused only
+        // after that warp has read it (slot_free).
         const int q = info & 0xffff;
-        const uint32_t use = (uint32_t)(seq / kSlots);
         warp_merge2(mS, sS, mT, sT);
         if (lane == 0) {
-          sh.red[q][cw][0] = mS;
-          sh.red[q][cw][1] = sS;
-          sh.red[q][cw][2] = mT;
-          sh.red[q][cw][3] = sT;
+          sh.red[q][cw] = make_float4(mS, sS, mT, sT);
           mbar_arrive(&sh.red_done[q]);
         }
-        if (cw == 0) {
-          if (!mbar_wait_warp(&sh.red_done[q], use & 1u, tmo, abort)) {
-            raise_abort(sh, p);
-            break;
-          }
-          mS = lane < kConsumerWarps ? sh.red[q][lane][0] : kMaxStart;
-          sS = lane < kConsumerWarps ? sh.red[q][lane][1] : 0.f;
-          mT = lane < kConsumerWarps ? sh.red[q][lane][2] : kMaxStart;
-          sT = lane < kConsumerWarps ? sh.red[q][lane][3] : 0.f;
-          warp_merge2(mS, sS, mT, sT);
-          if (lane == 0) {
-            sh.slot_pair[q][0] = mS;
-            sh.slot_pair[q][1] = sS;
-            sh.slot_pair[q][2] = mT;
-            sh.slot_pair[q][3] = sT;
-            mbar_arrive(&sh.lse_ready[q]);
-          }
-        }
-        ++seq;
         mS = kMaxStart;
         sS = 0.f;
         mT = kMaxStart;
@@ -293,109 +302,130 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     return;
   }
 
-  if (warp == 1) {
-    // ------------------------------------------------------------ row warp
-    int64_t seq = 0;
-    const float nan = __int_as_float(0x7fc00000);
-    while (true) {
-      const int q = (int)(seq % kSlots);
-      const uint32_t use = (uint32_t)(seq / kSlots);
-      if (!mbar_wait_warp(&sh.start[q], use & 1u, tmo, abort)) {
+  if (warp == kScanWarp) {
+    // ----------------------------------------------------------- scan warp
+    int running = kRowWarps;
+    uint32_t seen = 0;
+    for (uint32_t n = 0; running > 0;) {
+      const int i = (int)(n % kQueue);
+      if (!mbar_wait_warp(&sh.queue_full[i], (n / kQueue) & 1u, tmo, abort)) {
+        // a long wait is an error only if no row was finished meanwhile
+        uint32_t done = 0;
+        for (int k = 0; k < kRowWarps; ++k) done += *reinterpret_cast<volatile uint32_t*>(&sh.rows_done[k]);
+        done = __shfl_sync(0xffffffffu, done, 0);
+        if (done != seen && !__any_sync(0xffffffffu, *abort)) {
+          seen = done;
+          continue;
+        }
         if (lane == 0) raise_abort(sh, p);
         break;
       }
-      const int64_t tile = sh.slot_tile[q];
-      if (tile < 0) {
-        __syncwarp();
-        if (lane == 0) {
-          *reinterpret_cast<volatile int64_t*>(&sh.end_seq) = seq;  // every scan warp stops here
-          mbar_arrive(&sh.agg_ready[q]);
-        }
-        break;
-      }
-      const int64_t r = p.row_begin + tile;
-      const LT* srow = reinterpret_cast<const LT*>(p.S) + tile * p.ld;
-      const LT* trow = teacher_row<LT>(p, tile);
-      int32_t y = 0;
-      float xs = nan, xt = nan;
-      if (lane == 0) {
-        y = __ldg(p.tokens + tile);
-        if (y >= 0 && y < p.V) {
-          xs = to_f32(srow[y]);
-          xt = to_f32(trow[y]);
-        }
-        validate_layout(p, tile);
-      }
-      const RowMeta meta = find_row_meta(p, r, lane);
-      // ragged tail: the logits past the last whole 16-byte vector
-      float tmS = kMaxStart, tsS = 0.f, tmT = kMaxStart, tsT = 0.f;
-      for (int j = v_body * P + lane; j < p.V; j += 32) {
-        lse_one(to_f32(srow[j]), tmS, tsS);
-        lse_one(to_f32(trow[j]), tmT, tsT);
-      }
-      warp_merge2(tmS, tsS, tmT, tsT);
-      if (!mbar_wait_warp(&sh.lse_ready[q], use & 1u, tmo, abort)) {
-        if (lane == 0) raise_abort(sh, p);
-        break;
-      }
-      float mS = sh.slot_pair[q][0], sS = sh.slot_pair[q][1];
-      float mT = sh.slot_pair[q][2], sT = sh.slot_pair[q][3];
-      lse_merge(mS, sS, tmS, tsS);
-      lse_merge(mT, sT, tmT, tsT);
-      if (lane == 0) {
-        sh.slot_carry[q] = row_finalize(p, tile, r, meta, y >= 0 && y < p.V, xs, xt, lse_finish(mS, sS),
-                                        lse_finish(mT, sT), p.profile ? sh.prof : nullptr, false);
-        sh.slot_meta[q] = meta;
-        mbar_arrive(&sh.agg_ready[q]);
-      }
+      if (sh.queue[i].tile < 0)
+        --running;
+      else
+        complete_tile(p, sh.queue[i], lane);
+      ++n;
       __syncwarp();
-      ++seq;
-    }
-    if (lane == 0 && p.profile) {
-      for (int i = 0; i < 3 * STRIDE_PROFILE_BINS; ++i)
-        if (sh.prof[i] != 0.0) atomicAdd(p.profile + i, sh.prof[i]);
+      __threadfence_block();
+      if (lane == 0) *reinterpret_cast<volatile uint32_t*>(&sh.queue_tail) = n;
     }
     return;
   }
 
-  // --------------------------------------------------------------- scan warps
-  volatile int64_t* end_seq = &sh.end_seq;
-  for (int64_t seq = warp - 2;; seq += kScanWarps) {
+  // ---------------------------------------------------------------- row warps
+  const float nan = __int_as_float(0x7fc00000);
+  for (int64_t seq = warp - 1;; seq += kRowWarps) {
     const int q = (int)(seq % kSlots);
     const uint32_t use = (uint32_t)(seq / kSlots);
-    // Wait for row `seq`, unless the rows ran out before it.  The slots
-    // past the last row never fill, so the wait polls (test_wait and a short
-    // sleep) and looks at the end marker in between: a blocking try_wait
-    // kept each scan warp suspended about 7.5 us after the row warp had
-    // marked the end (probe timeline of 16,384-row windows: every CTA left
-    // 7.4-7.7 us after its scan warps began their last wait).
-    if (*end_seq <= seq) break;
-    bool ready = mbar_test_wait(&sh.agg_ready[q], use & 1u);
-    if (!ready) {
-      const uint64_t t0 = globaltimer_ns();
-      while (!(ready = mbar_test_wait(&sh.agg_ready[q], use & 1u))) {
-        __nanosleep(100);
-        if (*end_seq <= seq || *abort) break;
-        if (globaltimer_ns() - t0 > tmo) {
-          if (lane == 0) raise_abort(sh, p);
-          break;
-        }
-      }
+    if (!mbar_wait_warp(&sh.start[q], use & 1u, tmo, abort)) {
+      if (lane == 0) raise_abort(sh, p);
+      break;
     }
-    // the warp leaves together (lanes whose waits ended differently agree)
-    ready = __all_sync(0xffffffffu, ready);
-    if (!ready) break;
-    const int64_t tile = sh.slot_tile[q];
-    if (tile < 0) break;
-    const RowMeta meta = sh.slot_meta[q];
-    const RowCarry rc = sh.slot_carry[q];
-    row_resolve(p, tile, p.row_begin + tile, meta, rc, lane);
+    const int64_t w = sh.slot_tile[q];  // window row
+    if (w < 0) break;
+    const LT* srow = reinterpret_cast<const LT*>(p.S) + w * p.ld;
+    const LT* trow = teacher_row<LT>(p, w);
+    const int32_t y = __ldg(p.tokens + w);
+    const bool y_ok = y >= 0 && y < p.V;
+    float xs = nan, xt = nan;
+    if (y_ok) {
+      xs = to_f32(srow[y]);
+      xt = to_f32(trow[y]);
+    }
+    // ragged tail: the logits past the last whole 16-byte vector
+    const int j = v_body * P + lane;
+    const bool in_tail = j < p.V;
+    const float es = in_tail ? to_f32(srow[j]) : 0.f, et = in_tail ? to_f32(trow[j]) : 0.f;
+    if (!mbar_wait_warp(&sh.red_done[q], use & 1u, tmo, abort)) {
+      if (lane == 0) raise_abort(sh, p);
+      break;
+    }
+    float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
+    if (lane < kConsumerWarps) {
+      const float4 v = sh.red[q][lane];
+      mS = v.x;
+      sS = v.y;
+      mT = v.z;
+      sT = v.w;
+    }
     __syncwarp();
-    if (lane == 0) mbar_arrive(&sh.slot_free[q]);
+    if (lane == 0) mbar_arrive(&sh.slot_free[q]);  // the slot has been read
+    if (in_tail) {
+      lse_one(es, mS, sS);
+      lse_one(et, mT, sT);
+    }
+    warp_merge2(mS, sS, mT, sT);
+    uint32_t counted = 0;
+    const int64_t t = w / kTileRows;
+    if (lane == 0) {
+      const float lse_s = lse_finish(mS, sS), lse_t = lse_finish(mT, sT);
+      const float lps = xs - lse_s, lpt = xt - lse_t;
+      if (!y_ok) set_status(p.dev_status, STRIDE_DEV_TOKEN_RANGE);
+      const stride_row_outputs& o = p.out;
+      if (o.logp_s) o.logp_s[w] = lps;
+      if (o.logp_t) o.logp_t[w] = lpt;
+      if (o.opd) o.opd[w] = lps - lpt;
+      if (o.lse_s) o.lse_s[w] = lse_s;
+      if (o.lse_t) o.lse_t[w] = lse_t;
+      if (o.x_s) o.x_s[w] = xs;
+      if (o.x_t) o.x_t[w] = xt;
+      p.ws_logp_s[w] = lps;
+      p.ws_logp_t[w] = lpt;
+      counted = count_in(p.flags + t * kFlagStride + kCounterWord) + 1;
+    }
+    counted = __shfl_sync(0xffffffffu, counted, 0);
+    if ((int64_t)counted == min((int64_t)kTileRows, p.n_rows - t * kTileRows)) {
+      int i = lane == 0 ? queue_claim(sh) : 0;
+      i = __shfl_sync(0xffffffffu, i, 0);
+      TileCarry& tc = i < 0 ? sh.own[warp - 1] : sh.queue[i];
+      publish_tile(p, t, lane, tc);
+      __syncwarp();
+      if (i < 0)
+        complete_tile(p, tc, lane);
+      else if (lane == 0)
+        mbar_arrive(&sh.queue_full[i]);
+      __syncwarp();
+    }
+    if (lane == 0) *reinterpret_cast<volatile uint32_t*>(&sh.rows_done[warp - 1]) = (uint32_t)(seq / kRowWarps) + 1;
+  }
+  // nothing more from this row warp (its rows are done: it may wait here)
+  if (lane == 0) {
+    int i;
+    const uint64_t t0 = globaltimer_ns();
+    while ((i = queue_claim(sh)) < 0 && !*abort) {
+      __nanosleep(200);
+      if (globaltimer_ns() - t0 > tmo) raise_abort(sh, p);
+    }
+    if (i >= 0) {
+      sh.queue[i].tile = -1;
+      mbar_arrive(&sh.queue_full[i]);
+    }
   }
 }
 
-size_t stream_smem_bytes() { return kStreamSmem; }
+size_t stream_clear_bytes(int64_t n_rows) {
+  return 256 + (size_t)((n_rows + kTileRows - 1) / kTileRows) * kFlagStride * sizeof(uint32_t);
+}
 
 cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, cudaStream_t stream) {
   // The dynamic shared-memory limit is a per-device function attribute: set

@@ -1,0 +1,64 @@
+"""GPU parity of the persistent kernel's 32-row scan tiles at the sizes where
+they can go wrong: windows that end inside, at and just past a tile, turns of
+one row (a tile full of turns), runs of more empty trajectories than a tile
+stages, and very short rows (tiles complete faster than the scan warp takes
+them, so its queue fills)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_helpers import compare_rows, compare_scan, oracle_batch, run_batch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def stride():
+    import paper_2609_14636_gb300 as s
+
+    return s
+
+
+def _layout(rng, rows):
+    """Turns of one row (half of them) or 2-70 rows, 1-4 per trajectory,
+    and now and then 40 trajectories without turns in a row."""
+    lens, left = [], rows
+    while left > 0:
+        turns = []
+        for _ in range(int(rng.integers(1, 5))):
+            n = min(left, 1 if rng.random() < 0.5 else int(rng.integers(2, 71)))
+            if n:
+                turns.append(n)
+            left -= n
+        lens.append(turns)
+        if rng.random() < 0.1:
+            lens.extend([[]] * 40)
+    return synth.layout_from_turn_lengths(lens)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("rows, V", [(1, 64), (31, 64), (32, 64), (33, 64), (95, 264), (1024, 264), (1057, 64),
+                                     (20_000, 16)])
+def test_warp_tiles(stride, rows, V, mode):
+    rng = np.random.default_rng(rows * 2 + mode)
+    lay = _layout(rng, rows)
+    # Unit logits: compare_scan bounds a running sum's error by 1e-5 of the sum, and a single log-prob's rounding is
+    # about 2 ulp of its log-sum-exp (<= 5e-7 below 8), so |log-prob| has to stay above 0.05.  With N(0, 1) logits and
+    # 16 entries it does; N(0, 3^2) rows have entries of probability 0.999 (log-prob -1e-3: 5e-4 relative).
+    S = synth.bf16_bits_from_f32(rng.standard_normal((rows, V), dtype=np.float32))
+    T = synth.bf16_bits_from_f32(synth.f32_from_bf16_bits(S) + rng.standard_normal((rows, V), dtype=np.float32) * np.float32(0.3))
+    tok = rng.integers(0, V, rows).astype(np.int32)
+    lam = rng.uniform(-60.0, -3.0, lay.n_traj).astype(np.float32)
+    o = oracle_batch(S, T, tok, lay, mode, lam)
+    assert o["logp_t"].max() < -0.05
+    stride.stride_force_batch_kernel("stream")
+    try:
+        for windows in (None, [w for w in ((0, rows // 3), (rows // 3, rows)) if w[0] < w[1]]):
+            g = run_batch(stride, S, T, tok, lay, mode, lam, windows=windows)
+            assert g["status"] == 0
+            compare_rows(g, o)
+            compare_scan(g, o, lay, mode, lam)
+    finally:
+        stride.stride_force_batch_kernel("auto")
