@@ -54,8 +54,8 @@
  * - The batch calls choose among three kernels with the same results: for
  *   windows of at most 8 rows per SM, a kernel that splits each row over a
  *   thread-block cluster of 1, 2, 4 or 8 CTAs (the window is one wave); a
- *   persistent bulk-copy kernel for 16-byte-aligned rows; and one CTA per
- *   row otherwise.  The decode-step calls split each row over a cluster of
+ *   persistent bulk-copy kernel for the others; and one CTA per row where a
+ *   row is larger than 2 GB.  The decode-step calls split each row over a cluster of
  *   1 to 16 CTAs of 128 or 512 threads, chosen from the step's row count so
  *   that all rows run in one wave.  stride_force_batch_kernel and
  *   stride_force_step_shape (below) fix these choices for tests and
@@ -413,8 +413,7 @@ STRIDE_API int stride_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32
  * stride_force_batch_kernel: NULL, "" or "auto" = automatic choice; "split"
  * (automatic cluster size), "split1", "split2", "split4", "split8" (the
  * small-window kernel with that cluster size), "stream" (the persistent
- * kernel; rows that are not 16-byte aligned still take the per-row kernel)
- * or "rows" (one CTA per row).  Its initial value is the environment variable
+ * kernel; rows larger than 2 GB still take the per-row kernel) or "rows" (one CTA per row).  Its initial value is the environment variable
  * STRIDE_BATCH_KERNEL (same names), read once, at the first batch call.
  * stride_force_step_shape: the decode-step calls' CTA size (128 or 512
  * threads; 0 = 128 when a cluster size is given) and CTAs per row (1..16;

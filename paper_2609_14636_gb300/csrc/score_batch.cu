@@ -422,10 +422,13 @@ cudaError_t launch_clear_workspace(void* ws, size_t bytes, int sms, cudaStream_t
 }
 
 cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t clear_bytes, cudaStream_t stream) {
-  // Small windows split each row over a cluster (split_cluster); 16-byte-
-  // aligned rows with at least one whole vector otherwise take the
-  // persistent bulk-copy kernel (score_batch_stream.cu); the rest take one
-  // CTA per row.
+  // Small windows split each row over a cluster (split_cluster); the others
+  // take the persistent bulk-copy kernel (score_batch_stream.cu), aligned
+  // rows or not, and only rows past its 32-bit byte count one CTA per row.
+  // (6,000 packed rows of 151,933 bf16 logits, GB300: 504 us, 7,230 GB/s,
+  // against 631 us with one CTA per row; when S and T also differ in their
+  // misalignment, which the latter reads logit by logit, 286 against 470 us
+  // on one such workload.)
   int dev = 0;
   cudaError_t qe = cudaSuccess;
   const int sms = current_device_sms(&dev, &qe);
@@ -455,16 +458,15 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
     q.ticket = p.ticket + 1;
     return launch_scan_logprobs(q, p.ws_logp_s, p.ws_logp_t, stream, true);
   }
-  const int per_vec = dtype == STRIDE_DTYPE_BF16 ? 8 : 4;
   // (the persistent kernel counts a row's bytes in 32 bits: rows of up to
   // 2 GB, far beyond any vocabulary, take it)
   const int64_t row_bytes = (int64_t)p.V * (dtype == STRIDE_DTYPE_BF16 ? 2 : 4);
-  const bool persistent = vec && p.V >= per_vec && row_bytes <= ((int64_t)1 << 31) && !f_rows;
+  const bool persistent = row_bytes <= ((int64_t)1 << 31) && !f_rows;
   // the persistent kernel scans 32-row tiles: one flag line per tile
   const size_t clear = persistent ? stream_clear_bytes(p.n_rows) : clear_bytes;
   const cudaError_t ce = launch_clear_workspace(p.ticket, clear, sms, stream);
   if (ce != cudaSuccess) return ce;
-  if (persistent) return launch_score_batch_stream(p, dtype, stream);
+  if (persistent) return launch_score_batch_stream(p, dtype, vec, stream);
   const dim3 grid((unsigned)p.n_rows), block(kBatchThreads);
   if (dtype == STRIDE_DTYPE_BF16) {
     if (vec)

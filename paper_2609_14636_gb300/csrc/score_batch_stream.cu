@@ -1,5 +1,5 @@
 // score_batch_stream.cu -- persistent, warp-specialised batch scoring kernel
-// for 16-byte-aligned rows (sm_103a).
+// (sm_103a).
 //
 // One CTA per SM runs until the window's rows are exhausted.  Its warps have
 // fixed roles:
@@ -17,7 +17,8 @@
 //                      for the row's row warp.
 //   warps 1..4, row    rows taken round-robin (row n by row warp n mod 4).
 //   warps              While the row streams: token, gathered logits, the
-//                      ragged tail (V mod 8 logits).  Once the consumers'
+//                      row's ragged ends (the logits before its first
+//                      16-byte boundary and after its last whole vector).  Once the consumers'
 //                      pairs land: their merge, log-probs and outputs, then
 //                      the row is counted in at its 32-row tile; the warp
 //                      that counts a tile's last row publishes the tile
@@ -88,7 +89,7 @@ struct alignas(128) StreamShared {
   uint64_t red_done[kSlots];
   uint64_t slot_free[kSlots];
   int32_t stage_info[kStages];
-  uint32_t stage_bytes[kStages];
+  uint2 stage_vecs[kStages];  // 16-byte vectors of S and of T
   int64_t slot_tile[kSlots];  // window row, -1 past the last
   float4 red[kSlots][kConsumerWarps];  // the consumer warps' (mS, sS, mT, sT)
   uint64_t queue_full[kQueue];
@@ -122,7 +123,35 @@ __device__ __forceinline__ int queue_claim(StreamShared& sh) {
   return (int)(n % kQueue);
 }
 
-template <typename LT>
+// The logits of a row that bulk copies move: whole 16-byte vectors from the
+// row's first 16-byte boundary on.  The up to P - 1 logits before (`head`)
+// and after them are the row warp's.  EDGE = false: every row starts on a
+// boundary.
+template <typename LT, bool EDGE>
+struct RowBody {
+  int head;       // logits before the first vector
+  uint32_t vecs;  // 16-byte vectors
+  __device__ __forceinline__ RowBody(const LT* row, int V) : head(0) {
+    constexpr int P = LogitTraits<LT>::kPerVec;
+    if (EDGE) head = min((int)(((16u - (unsigned)(reinterpret_cast<uintptr_t>(row) & 15u)) & 15u) / sizeof(LT)), V);
+    vecs = (uint32_t)((V - head) / P);
+  }
+  // Vectors of chunk c (every chunk but the last has `chunk` of them).
+  __device__ __forceinline__ uint32_t chunk_vecs(uint32_t c, uint32_t chunk) const {
+    const uint32_t off = c * chunk;
+    return off < vecs ? min(chunk, vecs - off) : 0u;
+  }
+  // The row's logits outside its body, one per lane; false past the last.
+  __device__ __forceinline__ bool edge(const LT* row, int V, int lane, float& x) const {
+    constexpr int P = LogitTraits<LT>::kPerVec;
+    const int j = (lane < head ? 0 : (int)vecs * P) + lane;
+    const bool in = j < V;
+    x = in ? to_f32(row[j]) : 0.f;
+    return in;
+  }
+};
+
+template <typename LT, bool EDGE>
 __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(const BatchParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamShared& sh = *reinterpret_cast<StreamShared*>(smem_raw);
@@ -134,11 +163,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
   const int tid = threadIdx.x;
   const int lane = tid & 31;
   const int warp = tid >> 5;
-  const int v_body = p.V / P;  // 16-byte vectors per row streamed by bulk copies
-  const uint32_t row_bytes = (uint32_t)v_body * 16u;
-  const int n_chunks = (int)((row_bytes + kChunk - 1) / kChunk);
-  // chunks of equal size, so that a row's last stage is as full as the others
-  const uint32_t chunk = ((row_bytes / 16u + n_chunks - 1) / n_chunks) * 16u;
+  // A row's chunks: as few as fit the stages, of equal size, so that its last
+  // stage is as full as the others.  (V / P vectors is the most a row's body
+  // can have; a row of less than a vector still passes one empty stage.)
+  const uint32_t max_vecs = (uint32_t)(p.V / P);
+  const uint32_t n_chunks = max((max_vecs * 16u + kChunk - 1) / kChunk, 1u);
+  const uint32_t chunk = (max_vecs + n_chunks - 1) / n_chunks;  // vectors
   const uint64_t tmo = p.timeout_ns;
 
   if (tid == 0) {
@@ -187,9 +217,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
         }
         sh.slot_tile[q] = (int64_t)t;
         mbar_arrive(&sh.start[q]);
-        const unsigned char* srow = reinterpret_cast<const unsigned char*>(p.S) + (int64_t)t * p.ld * sizeof(LT);
-        const unsigned char* trow = reinterpret_cast<const unsigned char*>(teacher_row<LT>(p, (int64_t)t));
-        for (int c = 0; c < n_chunks; ++c) {
+        const LT* srow = reinterpret_cast<const LT*>(p.S) + (int64_t)t * p.ld;
+        const LT* trow = teacher_row<LT>(p, (int64_t)t);
+        const RowBody<LT, EDGE> body_s(srow, p.V), body_t(trow, p.V);
+        const unsigned char* src_s = reinterpret_cast<const unsigned char*>(srow + body_s.head);
+        const unsigned char* src_t = reinterpret_cast<const unsigned char*>(trow + body_t.head);
+        for (uint32_t c = 0; c < n_chunks; ++c) {
           // the next row's ticket arrives while the last chunk waits for its stage
           if (c == n_chunks - 1) t = atomicAdd(p.ticket, 1u);
           const int s = (int)(it % kStages);
@@ -198,13 +231,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
             ok = false;
             break;
           }
-          const uint32_t off = (uint32_t)c * chunk;
-          const uint32_t bytes = min(chunk, row_bytes - off);
+          const uint32_t n_s = body_s.chunk_vecs(c, chunk), n_t = body_t.chunk_vecs(c, chunk);
+          const size_t off = (size_t)c * chunk * 16;
           sh.stage_info[s] = q | (c == n_chunks - 1 ? kInfoLast : 0);
-          sh.stage_bytes[s] = bytes;
-          mbar_arrive_expect_tx(&sh.full[s], 2u * bytes);
-          bulk_g2s(bufS + (size_t)s * kChunk, srow + off, bytes, &sh.full[s], policy);
-          bulk_g2s(bufT + (size_t)s * kChunk, trow + off, bytes, &sh.full[s], policy);
+          sh.stage_vecs[s] = make_uint2(n_s, n_t);
+          mbar_arrive_expect_tx(&sh.full[s], (n_s + n_t) * 16u);
+          if (n_s) bulk_g2s(bufS + (size_t)s * kChunk, src_s + off, n_s * 16u, &sh.full[s], policy);
+          if (n_t) bulk_g2s(bufT + (size_t)s * kChunk, src_t + off, n_t * 16u, &sh.full[s], policy);
           ++it;
         }
         if (!ok) break;
@@ -217,7 +250,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
         const uint32_t k = it / kStages;
         if (k == 0 || mbar_wait(&sh.empty[s], (k - 1) & 1u, tmo, abort)) {
           sh.stage_info[s] = kInfoEnd;
-          sh.stage_bytes[s] = 0;
           mbar_arrive(&sh.full[s]);
         } else {
           ok = false;
@@ -264,21 +296,26 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       }
       const int info = sh.stage_info[s];
       if (info == kInfoEnd) break;
-      const int nvec = (int)(sh.stage_bytes[s] >> 4);
+      const uint2 nv = sh.stage_vecs[s];
+      const int n_s = (int)nv.x, n_t = EDGE ? (int)nv.y : n_s;  // (they differ by one vector at most, in the last chunk)
       const uint4* vs = reinterpret_cast<const uint4*>(bufS + (size_t)s * kChunk);
       const uint4* vt = reinterpret_cast<const uint4*>(bufT + (size_t)s * kChunk);
       int v = ct;
-      for (; v + kConsumers < nvec; v += 2 * kConsumers) {
+      for (; v + kConsumers < (EDGE ? min(n_s, n_t) : n_s); v += 2 * kConsumers) {
         const uint4 a[2] = {vs[v], vs[v + kConsumers]};
         const uint4 b[2] = {vt[v], vt[v + kConsumers]};
         LogitTraits<LT>::template chunk<2>(a, mS, sS);
         LogitTraits<LT>::template chunk<2>(b, mT, sT);
       }
-      for (; v < nvec; v += kConsumers) {
-        const uint4 a[1] = {vs[v]};
-        const uint4 b[1] = {vt[v]};
-        LogitTraits<LT>::template chunk<1>(a, mS, sS);
-        LogitTraits<LT>::template chunk<1>(b, mT, sT);
+      for (; v < (EDGE ? max(n_s, n_t) : n_s); v += kConsumers) {
+        if (!EDGE || v < n_s) {
+          const uint4 a[1] = {vs[v]};
+          LogitTraits<LT>::template chunk<1>(a, mS, sS);
+        }
+        if (!EDGE || v < n_t) {
+          const uint4 b[1] = {vt[v]};
+          LogitTraits<LT>::template chunk<1>(b, mT, sT);
+        }
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.empty[s]);
@@ -352,10 +389,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       xs = to_f32(srow[y]);
       xt = to_f32(trow[y]);
     }
-    // ragged tail: the logits past the last whole 16-byte vector
-    const int j = v_body * P + lane;
-    const bool in_tail = j < p.V;
-    const float es = in_tail ? to_f32(srow[j]) : 0.f, et = in_tail ? to_f32(trow[j]) : 0.f;
+    // the row's ragged ends: the logits before and after its whole vectors
+    float es, et;
+    const bool in_s = RowBody<LT, EDGE>(srow, p.V).edge(srow, p.V, lane, es);
+    const bool in_t = RowBody<LT, EDGE>(trow, p.V).edge(trow, p.V, lane, et);
     if (!mbar_wait_warp(&sh.red_done[q], use & 1u, tmo, abort)) {
       if (lane == 0) raise_abort(sh, p);
       break;
@@ -370,10 +407,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.slot_free[q]);  // the slot has been read
-    if (in_tail) {
-      lse_one(es, mS, sS);
-      lse_one(et, mT, sT);
-    }
+    if (in_s) lse_one(es, mS, sS);
+    if (in_t) lse_one(et, mT, sT);
     warp_merge2(mS, sS, mT, sT);
     uint32_t counted = 0;
     const int64_t t = w / kTileRows;
@@ -427,24 +462,23 @@ size_t stream_clear_bytes(int64_t n_rows) {
   return 256 + (size_t)((n_rows + kTileRows - 1) / kTileRows) * kFlagStride * sizeof(uint32_t);
 }
 
-cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, cudaStream_t stream) {
+cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, bool aligned, cudaStream_t stream) {
   // The dynamic shared-memory limit is a per-device function attribute: set
-  // once per device and dtype (setting it again is harmless, so two threads
+  // once per device and kernel (setting it again is harmless, so two threads
   // racing here both succeed).
-  static std::atomic<bool> attr_done[64][2];
+  static std::atomic<bool> attr_done[64][4];
   int dev = 0;
   cudaError_t e = cudaSuccess;
   const int sms = current_device_sms(&dev, &e);
   if (sms <= 0) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
-  const int di = dtype == STRIDE_DTYPE_BF16 ? 0 : 1;
-  if (!attr_done[dev][di].load(std::memory_order_acquire)) {
-    e = dtype == STRIDE_DTYPE_BF16
-            ? cudaFuncSetAttribute(score_batch_stream_kernel<__nv_bfloat16>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem)
-            : cudaFuncSetAttribute(score_batch_stream_kernel<float>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem);
+  const bool bf16 = dtype == STRIDE_DTYPE_BF16;
+  auto kern = bf16 ? (aligned ? score_batch_stream_kernel<__nv_bfloat16, false> : score_batch_stream_kernel<__nv_bfloat16, true>)
+                   : (aligned ? score_batch_stream_kernel<float, false> : score_batch_stream_kernel<float, true>);
+  std::atomic<bool>& done = attr_done[dev][(bf16 ? 0 : 2) + (aligned ? 0 : 1)];
+  if (!done.load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem);
     if (e != cudaSuccess) return e;
-    attr_done[dev][di].store(true, std::memory_order_release);
+    done.store(true, std::memory_order_release);
   }
   const int64_t grid = p.n_rows < sms ? p.n_rows : sms;
   cudaLaunchConfig_t cfg = {};
@@ -457,8 +491,7 @@ cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, cudaStrea
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = dtype == STRIDE_DTYPE_BF16 ? cudaLaunchKernelEx(&cfg, score_batch_stream_kernel<__nv_bfloat16>, p)
-                                 : cudaLaunchKernelEx(&cfg, score_batch_stream_kernel<float>, p);
+  e = cudaLaunchKernelEx(&cfg, kern, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

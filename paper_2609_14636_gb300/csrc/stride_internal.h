@@ -140,7 +140,7 @@ int current_device_sms(int* dev_out, cudaError_t* err);
 // start: the clearing kernel, or on the small-window path the split kernel
 // itself) and launches the batch scoring kernels.
 cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t clear_bytes, cudaStream_t stream);
-cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, cudaStream_t stream);
+cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, bool aligned, cudaStream_t stream);
 // What the persistent kernel needs at zero from the workspace's start: the
 // header (ticket) and one flag line per 32-row tile.
 size_t stream_clear_bytes(int64_t n_rows);

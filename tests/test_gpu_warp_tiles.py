@@ -2,7 +2,12 @@
 they can go wrong: windows that end inside, at and just past a tile, turns of
 one row (a tile full of turns), runs of more empty trajectories than a tile
 stages, and very short rows (tiles complete faster than the scan warp takes
-them, so its queue fills)."""
+them, so its queue fills).
+
+And rows at every alignment through the same kernel: S and T starting on
+different element offsets from a 16-byte boundary, strides that move the
+offset from row to row, vocabularies of less than a vector, around one and
+two vectors, and around one full stage (16,384 bf16 or 8,192 fp32 logits)."""
 from __future__ import annotations
 
 import numpy as np
@@ -62,3 +67,36 @@ def test_warp_tiles(stride, rows, V, mode):
             compare_scan(g, o, lay, mode, lam)
     finally:
         stride.stride_force_batch_kernel("auto")
+
+
+@pytest.mark.parametrize("off_s, off_t", [(0, 0), (1, 1), (3, 0), (0, 7), (5, 2)])
+@pytest.mark.parametrize("f32", [False, True])
+def test_unaligned_rows(stride, f32, off_s, off_t):
+    import torch
+
+    stage = 8192 if f32 else 16_384
+    rng = np.random.default_rng(100 + 10 * off_s + off_t + f32)
+    for V in (1, 3, 7, 8, 9, 15, 16, 17, 31, 33, 1001, stage - 1, stage, stage + 1, stage + 7, stage + 8, 2 * stage + 9):
+        rows = 70 if V < 2000 else 9
+        lay = synth.layout_from_turn_lengths([[3, 2], [rows - 5]])
+        # (unit logits, as above; V = 1 has log-prob 0, an exact 0 on both sides)
+        S32 = rng.standard_normal((rows, V), dtype=np.float32)
+        T32 = S32 + rng.standard_normal((rows, V), dtype=np.float32) * np.float32(0.3)
+        S, T = (S32, T32) if f32 else (synth.bf16_bits_from_f32(S32), synth.bf16_bits_from_f32(T32))
+        tok = (S32 * -1.0).argmax(1).astype(np.int32)  # an unlikely token: log-probs well away from 0
+        o = oracle_batch(S, T, tok, lay, 0, np.float32(-1e6))
+        for ld in (V, V + 3):
+            dev = []
+            for a, off in ((S, off_s), (T, off_t)):
+                flat = np.full(16 + rows * ld, np.nan, np.float32) if f32 else np.full(16 + rows * ld, 0x7FC0, np.uint16)
+                np.lib.stride_tricks.as_strided(flat[off:], (rows, V), (ld * flat.itemsize, flat.itemsize))[:] = a
+                t = torch.from_numpy(flat if f32 else flat.view(np.int16)).cuda()
+                dev.append((t if f32 else t.view(torch.bfloat16)).as_strided((rows, V), (ld, 1), off))
+            stride.stride_force_batch_kernel("stream")
+            try:
+                g = run_batch(stride, *dev, tok, lay, 0, np.float32(-1e6), V=V)
+            finally:
+                stride.stride_force_batch_kernel("auto")
+            assert g["status"] == 0, V
+            compare_rows(g, o)
+            compare_scan(g, o, lay, 0, np.float32(-1e6))
