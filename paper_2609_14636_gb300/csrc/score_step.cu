@@ -24,11 +24,18 @@
 // 4-CTA clusters of 128 threads (1,024 CTAs), a 64-row step takes 12, a
 // step of 32 rows or fewer 8-CTA clusters of 512 threads.
 //
-// Steps are launched with programmatic dependent launch: a step's CTAs may be
-// scheduled while the previous kernel on the stream finishes, and each waits
-// (griddepcontrol.wait) for that kernel's completion before its first global
-// read, so the caller's inputs and the carried state are always complete
-// when read.
+// Steps are launched with programmatic dependent launch.  A CTA lets the next
+// kernel be scheduled once its own stream is done, so the next step's CTAs
+// come in as this step's leave; each asks for the start of its slice in L2
+// (a hint, which reads nothing) and then waits (griddepcontrol.wait) for this
+// kernel's completion before its first global read, so the caller's inputs
+// and the carried state are always complete when read.  The loads' ramp thus
+// overlaps the previous step's merges and state updates.  GB300, steps of a
+// 32-step graph (151,936 bf16 logits), before -> now: 61 rows 11.0 -> 9.8 us,
+// 96 rows 13.6 -> 12.6, 128 rows 16.2 -> 14.9, 256 rows 27.0 -> 25.8, 256
+// masked rows 22.7 -> 21.8, 8 rows (in L2 already) 4.95 -> 4.83.  Letting the
+// next step in at the start instead makes its hints compete with this step's
+// loads: 61 rows 9.9, 256 rows 26.1 us at 16 KB per slice.
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -48,6 +55,11 @@ namespace stride {
 
 constexpr int kStepUnroll = STRIDE_STEP_UNROLL;
 constexpr int kStepMaxCluster = 16;
+// Bytes of a step that the hints ahead of the wait ask for, over all its
+// CTAs.  12 / 20 / 32 / 40 / 64 MB: 128 rows 478.6 / 478.2 / 482 / 490 / 508
+// us per 32 steps, 256 rows 823 / 825 / 830 / 832 / 844, 61 rows 315.4 /
+// 313.3 / 314.2 / 312.6 / 312.7: more than the wait lasts only evicts.
+constexpr int64_t kStepPrefetch = 20 << 20;
 // Two CTA shapes, both at most 64 registers per thread: 128 threads, 8 CTAs
 // per SM (the shape of steps with many rows), and 512 threads, 2 per SM (more
 // threads per row when a step has too few rows to fill the GPU with
@@ -108,34 +120,9 @@ __global__ void __launch_bounds__(THREADS, StepShape<THREADS>::kMinBlocks) score
   // store guarantees every CTA of the cluster has started (its shared memory
   // exists); the wait comes after the stream, so it costs nothing
   cluster_arrive_relaxed();
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  if (!COMPACT) {
-    // A stopped rollout's whole cluster leaves before reading a logit (every
-    // CTA reads the flag, which only this step's rank 0 writes, after the
-    // cluster's last remote store).
-    if (__ldcg(&p.state[b].stopped)) {
-      if (rank == 0 && tid == 0) write_row_nan(p, b);
-      return;
-    }
-  }
 
   const LT* srow = reinterpret_cast<const LT*>(p.S) + (int64_t)b * p.ld;
   const LT* trow = reinterpret_cast<const LT*>(p.T) + (int64_t)b * p.ld;
-
-  // The token id (and, compacted, the rollout id) is loaded now, the token's
-  // logits and the rollout's state after the stream, so rank 0 streams as
-  // early as the other ranks (a gather before the stream held rank 0 back by
-  // about 0.7 us on average, GB300 timeline) and the state's latency hides
-  // behind the merge and the cluster barrier.  A compacted row streams
-  // without first reading its rollout's state: the caller passes live
-  // rollouts, and a row whose state turns out stopped is discarded.
-  int32_t y = 0, r = b;
-  if (rank == 0 && tid == 0) {
-    y = __ldg(p.tokens + b);
-    if (COMPACT) r = __ldg(p.rollout_idx + b);
-  }
 
   // vocabulary slice of this rank (whole 16-byte vectors on the vector path;
   // the last rank also takes the ragged tail)
@@ -151,8 +138,42 @@ __global__ void __launch_bounds__(THREADS, StepShape<THREADS>::kMinBlocks) score
     c0 = min(p.V, rank * per);
     c1 = min(p.V, (rank + 1) * per);
   }
+
+  // The start of the slice on its way to L2 while the previous kernel ends
+  // (the stopped flag may be about to change: it only saves a useless hint).
+  if (tid == 0 || tid == 32) {
+    const bool skip = !COMPACT && *reinterpret_cast<const volatile int32_t*>(&p.state[b].stopped) != 0;
+    const int64_t most = kStepPrefetch / (2 * (int64_t)gridDim.x);
+    if (!skip) prefetch_l2((tid == 0 ? srow : trow) + c0, min((int64_t)(c1 - c0) * (int64_t)sizeof(LT), most));
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  if (!COMPACT) {
+    // A stopped rollout's whole cluster leaves before reading a logit (every
+    // CTA reads the flag, which only this step's rank 0 writes, after the
+    // cluster's last remote store).
+    if (__ldcg(&p.state[b].stopped)) {
+      if (rank == 0 && tid == 0) write_row_nan(p, b);
+      return;
+    }
+  }
+
+  // The token id (and, compacted, the rollout id) is loaded now, the token's
+  // logits and the rollout's state after the stream, so rank 0 streams as
+  // early as the other ranks (a gather before the stream held rank 0 back by
+  // about 0.7 us on average, GB300 timeline) and the state's latency hides
+  // behind the merge and the cluster barrier.  A compacted row streams
+  // without first reading its rollout's state: the caller passes live
+  // rollouts, and a row whose state turns out stopped is discarded.
+  int32_t y = 0, r = b;
+  if (rank == 0 && tid == 0) {
+    y = __ldg(p.tokens + b);
+    if (COMPACT) r = __ldg(p.rollout_idx + b);
+  }
+
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
   stream_pair<LT, VEC, kStepUnroll>(srow, trow, c0, c1, tid, THREADS, mS, sS, mT, sT);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   float xs = __int_as_float(0x7fc00000), xt = xs, lam = 0.f;
   bool valid = false, closes = false;

@@ -29,6 +29,18 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   return v;
 }
 
+// Asks for the whole 16-byte vectors of [p, p + bytes) in L2.  A hint: it
+// delivers no value, so it may run before the grid that writes the bytes has
+// completed (L2 is where that grid's stores land).  At most 1 MB.
+__device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
+  const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15);
+  const uintptr_t e = (reinterpret_cast<uintptr_t>(p) + (uintptr_t)bytes) & ~uintptr_t(15);
+  if (e > a) {
+    const uint32_t n = (uint32_t)(e - a < (1u << 20) ? e - a : (1u << 20));
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(n) : "memory");
+  }
+}
+
 // 2^x on the SFU (PTX ex2.approx.ftz.f32: relative error ~2^-22, subnormal
 // results flush to 0, 2^-inf = 0).
 __device__ __forceinline__ float ex2(float x) {
