@@ -132,6 +132,12 @@ constexpr int kSplitMaxCluster = 8;
 constexpr int kSplitThreads = 128;
 constexpr int kSplitWarps = kSplitThreads / 32;
 constexpr int kSplitBlocksPerSm = 8;  // 128 threads at <= 64 registers
+// Bytes of a window that the hints ahead of the wait ask for, over all CTAs.
+// 0 / 12 / 20 / 32 / 48 MB, windows of 512 and 1,024 rows of 151,936 bf16
+// logits: 57.3 / 55.6 / 55.6 / 55.8 / 56.7 and 100.6 / 99.7 / 100.1 / 100.5 /
+// 100.7 us (58.4 and 100.9 us before the state's initialisation was a
+// programmatic dependent too).
+constexpr int64_t kSplitPrefetch = 12 << 20;
 
 template <typename LT, bool VEC>
 __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
@@ -141,6 +147,31 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
   // first cluster-barrier phase: waited on before the first remote store
   // (every CTA of the cluster has started by then)
   cluster_arrive_relaxed();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int n_ranks = (int)cluster.num_blocks();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t tile = blockIdx.x / n_ranks;  // window row
+  const LT* srow = reinterpret_cast<const LT*>(p.S) + tile * p.ld;
+  int c0, c1;
+  if (VEC) {
+    constexpr int P = LogitTraits<LT>::kPerVec;
+    const int nv = p.V / P;
+    const int per = (nv + n_ranks - 1) / n_ranks;
+    c0 = min(nv, rank * per) * P;
+    c1 = (rank == n_ranks - 1) ? p.V : min(nv, (rank + 1) * per) * P;
+  } else {
+    const int per = (p.V + n_ranks - 1) / n_ranks;
+    c0 = min(p.V, rank * per);
+    c1 = min(p.V, (rank + 1) * per);
+  }
+  // The start of the slice on its way to L2 while the previous kernel ends
+  // (the multi-teacher row table is not there yet).
+  if (tid == 0 || (tid == 32 && !p.T_rows)) {
+    const int64_t most = kSplitPrefetch / (2 * (int64_t)gridDim.x);
+    const LT* row = tid == 0 ? srow : reinterpret_cast<const LT*>(p.T) + tile * p.ld;
+    prefetch_l2(row + c0, min((int64_t)(c1 - c0) * (int64_t)sizeof(LT), most));
+  }
   // Launched as a programmatic dependent of the previous kernel on the
   // stream: the CTAs may be scheduled while it finishes, and each waits for
   // its completion before the first global access.  Only then may the
@@ -157,12 +188,6 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
     for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x) p.flags[t * kFlagStride] = 0u;
     if (threadIdx.x == 0) p.ticket[1] = 0u;
   }
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int n_ranks = (int)cluster.num_blocks();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t tile = blockIdx.x / n_ranks;  // window row
-  const LT* srow = reinterpret_cast<const LT*>(p.S) + tile * p.ld;
   const LT* trow = teacher_row<LT>(p, tile);
 
   // The token id is loaded now; its logits are gathered, and this row's
@@ -171,18 +196,6 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
   int32_t y = 0;
   float xs = __int_as_float(0x7fc00000), xt = xs;
   if (rank == 0 && tid == 0) y = __ldg(p.tokens + tile);
-  int c0, c1;
-  if (VEC) {
-    constexpr int P = LogitTraits<LT>::kPerVec;
-    const int nv = p.V / P;
-    const int per = (nv + n_ranks - 1) / n_ranks;
-    c0 = min(nv, rank * per) * P;
-    c1 = (rank == n_ranks - 1) ? p.V : min(nv, (rank + 1) * per) * P;
-  } else {
-    const int per = (p.V + n_ranks - 1) / n_ranks;
-    c0 = min(p.V, rank * per);
-    c1 = min(p.V, (rank + 1) * per);
-  }
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
   stream_pair<LT, VEC, 4>(srow, trow, c0, c1, tid, kSplitThreads, mS, sS, mT, sT);
   if (rank == 0 && tid == 0 && y >= 0 && y < p.V) {
@@ -254,8 +267,8 @@ __global__ void teacher_rows_kernel(const BatchParams p, const TeacherTable tt,
   // previous window's scoring kernel still reading this workspace's table:
   // wait for it before the first store; the clearing and scoring kernels
   // that follow may be scheduled at once (they wait for this grid in turn).
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.n_rows) return;
   const int64_t r = p.row_begin + t;
@@ -391,14 +404,14 @@ static cudaError_t launch_split(const BatchParams& p, int C, cudaStream_t stream
 // kernel on the stream: its CTAs wait for that kernel (which may be the
 // previous window's scoring kernel, still using the same workspace) before
 // the first store.  It lets its own dependent, the scoring kernel, be
-// scheduled at once: that kernel's CTAs set up their shared memory and
+// scheduled even before that: that kernel's CTAs set up their shared memory and
 // barriers while the previous window drains, then wait for this grid to
 // complete.  (It replaces a memset node, which ended the programmatic chain:
 // 7.5 us between one 16,384-row window's last CTA and the next one's first
 // on GB300.)
 __global__ void clear_workspace_kernel(uint4* __restrict__ p, int64_t n16) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = z;
@@ -426,9 +439,9 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
   // take the persistent bulk-copy kernel (score_batch_stream.cu), aligned
   // rows or not, and only rows past its 32-bit byte count one CTA per row.
   // (6,000 packed rows of 151,933 bf16 logits, GB300: 504 us, 7,230 GB/s,
-  // against 631 us with one CTA per row; when S and T also differ in their
-  // misalignment, which the latter reads logit by logit, 286 against 470 us
-  // on one such workload.)
+  // against 631 us with one CTA per row; 4,000 rows against two domains'
+  // buffers, so that S and T differ in misalignment, which the latter reads
+  // logit by logit: 342 against 596 us.)
   int dev = 0;
   cudaError_t qe = cudaSuccess;
   const int sms = current_device_sms(&dev, &qe);

@@ -78,6 +78,12 @@ constexpr int kFirstConsumerWarp = 2 + kRowWarps;
 constexpr int kStreamThreads = 32 * kFirstConsumerWarp + kConsumers;
 constexpr int kInfoEnd = -1;
 constexpr int kInfoLast = 1 << 16;
+// Bytes per tensor and CTA that the hints ahead of the wait ask for.  GB300,
+// 3,001 rows of 151,936 bf16 logits, and 20,000 in windows of 4,096: none
+// 262.3 and 1,689 us, 64 KB 261.5 and 1,686, 128 KB 262.6 and 1,684, 256 KB
+// 264.3 and 1,683 (267.0 and 1,713 us before the 32-row tiles and before the
+// state's initialisation was in the programmatic chain).
+constexpr int64_t kStreamPrefetch = 64 << 10;
 static_assert(kChunk % 16 == 0, "bulk copies move multiples of 16 bytes");
 constexpr int kQueue = 8;  // published tiles waiting for the scan warp
 static_assert(kSlots % kRowWarps == 0, "a row warp keeps its own slots");
@@ -189,9 +195,15 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
   }
   __syncthreads();
   // Launched as a programmatic dependent of the workspace clear: the set-up
-  // above may overlap the previous kernel's end; nothing global is touched
+  // above, and the start of one of the first rows on its way to L2 (not the
+  // teacher's from the multi-teacher row table, which is not there yet), may
+  // overlap the previous kernels' end; nothing global is read or written
   // before the clear (and everything before it) has completed.  Dependents
   // may be scheduled at once: they wait for this grid in turn.
+  if (tid == 32 || (tid == 64 && !p.T_rows)) {
+    const LT* row = reinterpret_cast<const LT*>(tid == 32 ? p.S : p.T) + (int64_t)blockIdx.x * p.ld;
+    prefetch_l2(row, min((int64_t)p.V * (int64_t)sizeof(LT), kStreamPrefetch));
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 

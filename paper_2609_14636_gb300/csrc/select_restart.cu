@@ -88,9 +88,12 @@ __global__ void __launch_bounds__(kSelectThreads) buffer_record_kernel(
 }
 
 __global__ void state_init_kernel(stride_scan_state* s, int32_t n) {
-  // a programmatic dependent (the small-window and decode kernels) may be
-  // scheduled now; each of those waits for this grid before its first read
+  // A programmatic dependent of the previous kernel on the stream, which may
+  // still use the states: waits for it before the store.  Its own dependents
+  // (the scoring kernels) may be scheduled at once; each of those waits for
+  // this grid before its first read.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   stride_scan_state z;
@@ -128,7 +131,17 @@ cudaError_t launch_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32_t 
 }
 
 cudaError_t launch_state_init(stride_scan_state* state, int32_t n, cudaStream_t stream) {
-  state_init_kernel<<<(n + 255) / 256, 256, 0, stream>>>(state, n);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, state_init_kernel, state, n);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

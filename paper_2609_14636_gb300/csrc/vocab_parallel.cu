@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
   // taken in ticket order (a tile's lookback waits only on tiles taken
   // before it, which are running or done) unless the grid is small enough
   // to be resident at once, when the block index is the tile.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
   if (by_ticket) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
