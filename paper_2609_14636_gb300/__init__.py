@@ -1,12 +1,14 @@
 """STRIDE scoring path on one GB300 (arXiv 2609.14636): Python binding.
 
-A thin ctypes layer over ``libstride.so`` (include/stride.h).  The functions
-keep the C names and argument order; they take torch CUDA tensors, check
-their dtype/device/shape, pass raw device pointers and the current CUDA
-stream, and raise :class:`StrideError` on a non-zero status.  Every step of
-the scoring path runs in the library's CUDA kernels: there is no Python or
-CPU fallback, and importing this package fails if the library is missing
-and cannot be built.
+A thin layer over ``libstride.so`` (include/stride.h).  The functions keep
+the C names and argument order; they take torch CUDA tensors, check their
+dtype/device/shape, pass raw device pointers and the current CUDA stream,
+and raise :class:`StrideError` on a non-zero status.  A call whose arguments
+are plain (tensors, ints, floats) is checked and passed on in native code
+(csrc/binding.cpp); any other is taken, or refused, by the ctypes code here.
+Every step of the scoring path runs in the library's CUDA kernels: there is
+no Python or CPU fallback, and importing this package fails if the library
+is missing and cannot be built.
 
 Per-trajectory state and per-turn statistics are opaque byte tensors
 (``[n, 80]`` and ``[n, 40]`` uint8) laid out as ``stride_scan_state`` and
@@ -113,6 +115,30 @@ def lib() -> ctypes.CDLL:
             getattr(L, fn).restype = ctypes.c_int
         _LIB = L
     return _LIB
+
+
+_NATIVE = None
+
+
+def _native():
+    """The native marshalling module (csrc/binding.cpp), calling the library
+    that :func:`lib` loaded.  Each of its functions answers None for a call
+    that it leaves to the general code below."""
+    global _NATIVE
+    if _NATIVE is None:
+        import torch  # noqa: F401  (its libraries are the module's)
+
+        L = lib()
+        from . import _binding
+
+        _binding.bind(*[ctypes.cast(getattr(L, f"stride_{fn}"), ctypes.c_void_p).value for fn in _NATIVE_ENTRIES])
+        _NATIVE = _binding
+    return _NATIVE
+
+
+_NATIVE_ENTRIES = ("state_init", "score_batch", "score_batch_noalloc", "score_batch_multi_teacher", "score_step",
+                   "score_step_compact", "select_restart", "buffer_record", "partial_lse", "combine_partials",
+                   "scan_logprobs")
 
 
 def stride_status_string(code: int) -> str:
@@ -232,6 +258,9 @@ def turn_stats_to_numpy(ts) -> np.ndarray:
 # the C ABI, one function each
 # ---------------------------------------------------------------------------
 def stride_state_init(state, n: int, stream=None) -> None:
+    rc = (_NATIVE or _native()).state_init(state, n, stream)
+    if rc is not None:
+        return _check("stride_state_init", rc)
     torch = _torch()
     p = _dev(state, "state", torch.uint8, n * STATE_DTYPE.itemsize)
     _check("stride_state_init", lib().stride_state_init(p, int(n), _stream(stream)))
@@ -255,6 +284,11 @@ def stride_score_batch(S, T, tokens, traj_row_off, turn_row_off, traj_turn_off, 
     tensor of at least stride_score_batch_workspace_size(rows) bytes (256-byte
     aligned; torch's allocator returns such blocks); profile a float64
     [10, 3] tensor from :func:`new_profile`, added to."""
+    rc = (_NATIVE or _native()).score_batch(S, T, tokens, traj_row_off, turn_row_off, traj_turn_off, row_begin,
+                                            row_end, stop_mode, lam, state, out, turn_stats, dev_status, workspace, V,
+                                            stream, profile)
+    if rc is not None:
+        return _check("stride_score_batch", rc)
     torch = _torch()
     dt, ld = _logits(S, T)
     rows = int(row_end) - int(row_begin)
@@ -280,6 +314,10 @@ def stride_score_step(S, T, tokens, turn_end, stop_mode: int, lam, state, out: d
                       stopped_now=None, turn_out=None, dev_status=None, V: int | None = None,
                       stream=None) -> None:
     """One decode step over B = S.shape[0] rollouts (see include/stride.h)."""
+    rc = (_NATIVE or _native()).score_step(S, T, tokens, turn_end, stop_mode, lam, state, out, stopped_now, turn_out,
+                                           dev_status, V, stream)
+    if rc is not None:
+        return _check("stride_score_step", rc)
     torch = _torch()
     dt, ld = _logits(S, T)
     B = S.shape[0]
@@ -302,6 +340,10 @@ def stride_score_step_compact(S, T, tokens, turn_end, rollout_idx, stop_mode: in
     S, T, tokens, turn_end and the outputs is rollout rollout_idx[b] (int32
     CUDA tensor of n_rows = len(rollout_idx) entries unless given) of the
     state tensor's rollouts (see include/stride.h)."""
+    rc = (_NATIVE or _native()).score_step_compact(S, T, tokens, turn_end, rollout_idx, stop_mode, lam, state, out,
+                                                   stopped_now, turn_out, dev_status, V, n_rows, stream)
+    if rc is not None:
+        return _check("stride_score_step_compact", rc)
     torch = _torch()
     dt, ld = _logits(S, T)
     n = int(rollout_idx.shape[0]) if n_rows is None else int(n_rows)
@@ -334,6 +376,9 @@ def stride_force_step_shape(cta_threads: int, cluster_size: int) -> None:
 def stride_select_restart(turn_mean, n_turns, correct, alpha: float, k_star, k_max, stream=None) -> None:
     """Restart choice (Eq. 6) over N records: turn_mean float32 [N, T_max],
     n_turns int32 [N], correct uint8 [N, T_max] or None; outputs int32 [N]."""
+    rc = (_NATIVE or _native()).select_restart(turn_mean, n_turns, correct, alpha, k_star, k_max, stream)
+    if rc is not None:
+        return _check("stride_select_restart", rc)
     torch = _torch()
     if turn_mean.dim() != 2:
         raise ValueError("turn_mean must be [N, T_max]")
@@ -358,6 +403,12 @@ def stride_score_batch_multi_teacher(S, T_domains, traj_domain, traj_T_row0, tok
     CUDA tensors of S's dtype and a common row stride), a per-trajectory
     domain id (uint8) and the trajectory's first row in its domain buffer
     (int64).  See include/stride.h."""
+    rc = (_NATIVE or _native()).score_batch_multi_teacher(S, T_domains, traj_domain, traj_T_row0, tokens, traj_row_off,
+                                                          turn_row_off, traj_turn_off, row_begin, row_end, stop_mode,
+                                                          lam, state, out, turn_stats, dev_status, workspace, V,
+                                                          stream, profile)
+    if rc is not None:
+        return _check("stride_score_batch_multi_teacher", rc)
     torch = _torch()
     if not isinstance(S, torch.Tensor) or not S.is_cuda or S.dim() != 2 or S.stride(1) != 1:
         raise TypeError("S must be a 2-D CUDA tensor with unit column stride")
@@ -400,6 +451,9 @@ def stride_partial_lse(S, T, tokens, col0: int, partials, dev_status=None, V_sha
                        stream=None) -> None:
     """Partial log-sum-exp of one vocabulary shard (columns col0 .. col0+V_shard-1
     held in S, T [rows, ld]); partials: float32 [rows, 6]."""
+    rc = (_NATIVE or _native()).partial_lse(S, T, tokens, col0, partials, dev_status, V_shard, stream)
+    if rc is not None:
+        return _check("stride_partial_lse", rc)
     torch = _torch()
     dt, ld = _logits(S, T)
     rows = S.shape[0]
@@ -414,6 +468,9 @@ def stride_partial_lse(S, T, tokens, col0: int, partials, dev_status=None, V_sha
 def stride_combine_partials(partials, logp_s=None, logp_t=None, lse_s=None, lse_t=None, dev_status=None,
                             stream=None) -> None:
     """Merge float32 [n_shards, rows, 6] partials into log-probs."""
+    rc = (_NATIVE or _native()).combine_partials(partials, logp_s, logp_t, lse_s, lse_t, dev_status, stream)
+    if rc is not None:
+        return _check("stride_combine_partials", rc)
     torch = _torch()
     if partials.dim() != 3 or partials.shape[2] != 6:
         raise ValueError("partials must be [n_shards, rows, 6]")
@@ -431,6 +488,11 @@ def stride_scan_logprobs(logp_s, logp_t, traj_row_off, turn_row_off, traj_turn_o
                          stream=None, profile=None) -> None:
     """The scan of stride_score_batch on given log-probs (float32, indexed by
     row - row_begin)."""
+    rc = (_NATIVE or _native()).scan_logprobs(logp_s, logp_t, traj_row_off, turn_row_off, traj_turn_off, row_begin,
+                                              row_end, stop_mode, lam, state, opd, turn_stats, dev_status, workspace,
+                                              stream, profile)
+    if rc is not None:
+        return _check("stride_scan_logprobs", rc)
     torch = _torch()
     rows = int(row_end) - int(row_begin)
     n_traj = traj_row_off.numel() - 1
@@ -455,6 +517,10 @@ def stride_buffer_record(buf_mean, buf_n_turns, task_of_traj, k0_of_traj, turn_s
     """Record trajectories' turn means in the prefix buffer H(x) (float32
     [n_tasks, T_max] and int32 [n_tasks], updated in place): each keeps the
     first k0 stored turns of its task, then its own turns (Algorithm 1)."""
+    rc = (_NATIVE or _native()).buffer_record(buf_mean, buf_n_turns, task_of_traj, k0_of_traj, turn_stats,
+                                              traj_turn_off, dev_status, stream)
+    if rc is not None:
+        return _check("stride_buffer_record", rc)
     torch = _torch()
     if buf_mean.dim() != 2:
         raise ValueError("buf_mean must be [n_tasks, T_max]")
@@ -503,6 +569,11 @@ def stride_score_batch_noalloc(S, T, tokens, traj_row_off, turn_row_off, traj_tu
     cannot allocate device memory: the library's built-in scratch (at most
     NOALLOC_MAX_ROWS rows per call) is used instead.  Calls that overlap on
     the GPU race on that scratch; order them on one stream."""
+    rc = (_NATIVE or _native()).score_batch_noalloc(S, T, tokens, traj_row_off, turn_row_off, traj_turn_off, row_begin,
+                                                    row_end, stop_mode, lam, state, out, turn_stats, dev_status, V,
+                                                    stream, profile)
+    if rc is not None:
+        return _check("stride_score_batch_noalloc", rc)
     torch = _torch()
     dt, ld = _logits(S, T)
     rows = int(row_end) - int(row_begin)

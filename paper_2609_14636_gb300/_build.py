@@ -1,8 +1,9 @@
-"""In-tree build of libstride.so for sm_103a (nvcc, no cmake).
+"""In-tree build of libstride.so for sm_103a (nvcc, no cmake) and of the
+Python module's native marshalling, _binding.so (g++, torch's headers).
 
 Each .cu under csrc/ compiles to an object in parallel; the objects link into
 paper_2609_14636_gb300/libstride.so against the shared CUDA runtime.  The
-build is skipped when the library is newer than every source and header.
+build is skipped when both are newer than every source and header.
 """
 from __future__ import annotations
 
@@ -18,6 +19,7 @@ CSRC = PKG / "csrc"
 INCLUDE = ROOT / "include"
 BUILD = PKG / "_build"
 LIB = PKG / "libstride.so"
+BINDING = PKG / "_binding.so"
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-Xptxas", "-v",
@@ -34,20 +36,41 @@ def sources() -> list[Path]:
 
 
 def _deps() -> list[Path]:
-    return sources() + sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted(INCLUDE.glob("*.h"))
+    return sources() + [CSRC / "binding.cpp"] + sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted(INCLUDE.glob("*.h"))
 
 
 def up_to_date() -> bool:
-    if not LIB.exists():
+    if not LIB.exists() or not BINDING.exists():
         return False
-    t = LIB.stat().st_mtime
+    t = min(LIB.stat().st_mtime, BINDING.stat().st_mtime)
     return all(p.stat().st_mtime <= t for p in _deps())
+
+
+def _build_binding() -> None:
+    """_binding.so against the installed torch (its headers and libraries)."""
+    import sysconfig
+
+    import torch
+
+    t = Path(torch.__file__).parent
+    cuda = Path(nvcc()).resolve().parent.parent
+    tmp = BINDING.with_name(BINDING.name + f".tmp{os.getpid()}")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", str(INCLUDE), "-isystem",
+           str(t / "include"), "-isystem", str(t / "include/torch/csrc/api/include"), "-isystem", str(cuda / "include"),
+           "-isystem", sysconfig.get_paths()["include"], str(CSRC / "binding.cpp"), "-o", str(tmp), "-L", str(t / "lib"),
+           "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for binding.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
 
 
 def build(force: bool = False, verbose: bool = False, defines: tuple = (), lib: Path | None = None,
           build_dir: Path | None = None) -> Path:
     """Compile and link.  `defines` adds -D flags (tuning knobs of the
-    kernels); `lib`/`build_dir` redirect the output (default: in-tree)."""
+    kernels); `lib`/`build_dir` redirect the output (default: in-tree, with
+    the Python module's marshalling beside it)."""
     out_lib = LIB if lib is None else Path(lib)
     bdir = BUILD if build_dir is None else Path(build_dir)
     if not force and lib is None and not defines and up_to_date():
@@ -63,8 +86,11 @@ def build(force: bool = False, verbose: bool = False, defines: tuple = (), lib: 
             raise RuntimeError(f"nvcc failed for {src.name}:\n{r.stdout}\n{r.stderr}")
         return obj, r.stderr
 
-    with ThreadPoolExecutor(max_workers=min(8, len(sources()))) as ex:
+    with ThreadPoolExecutor(max_workers=min(8, len(sources())) + 1) as ex:
+        binding = ex.submit(_build_binding) if lib is None else None
         results = list(ex.map(compile_one, sources()))
+        if binding:
+            binding.result()
     log = []
     for obj, err in results:
         objs.append(obj)
