@@ -180,14 +180,6 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
   // it before its own wait.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (blockIdx.x == 0) {
-    // What the scan needs at zero: its tile ticket (the header's second
-    // word) and one flag per tile of kScanTileRowsDependent rows.  The scan
-    // reads them only after this grid has completed.
-    const int64_t n_tiles = (p.n_rows + kScanTileRowsDependent - 1) / kScanTileRowsDependent;
-    for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x) p.flags[t * kFlagStride] = 0u;
-    if (threadIdx.x == 0) p.ticket[1] = 0u;
-  }
   const LT* trow = teacher_row<LT>(p, tile);
 
   // The token id is loaded now; its logits are gathered, and this row's
@@ -458,18 +450,14 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
   }
   if (C > 0 && p.V < 32 * (int64_t)C) C = f_split ? 1 : 0;  // a few logits per rank at least
   if (C > 0) {
-    // no memset: the split kernel clears the scan's ticket and tile flags
+    // (neither kernel needs anything cleared)
     cudaError_t e;
     if (dtype == STRIDE_DTYPE_BF16)
       e = vec ? launch_split<__nv_bfloat16, true>(p, C, stream) : launch_split<__nv_bfloat16, false>(p, C, stream);
     else
       e = vec ? launch_split<float, true>(p, C, stream) : launch_split<float, false>(p, C, stream);
     if (e != cudaSuccess) return e;
-    // the scan on the rows' log-probs; its tile tickets use the header's
-    // second word (cleared with the first)
-    BatchParams q = p;
-    q.ticket = p.ticket + 1;
-    return launch_scan_logprobs(q, p.ws_logp_s, p.ws_logp_t, stream, true);
+    return launch_scan_logprobs(p, p.ws_logp_s, p.ws_logp_t, stream, true);  // the scan on the rows' log-probs
   }
   // (the persistent kernel counts a row's bytes in 32 bits: rows of up to
   // 2 GB, far beyond any vocabulary, take it)

@@ -8,12 +8,11 @@
 // (partial_lse_kernel).  After the ranks exchange those, the pairs merge
 // into the row's log-sum-exp (combine_kernel), which gives the same
 // log-probs as the full row.  The rest of the path (turn statistics, stop
-// rule, OPD loss, profile, carried state) then runs on the log-probs
-// (scan_logprobs_tile_kernel): a segmented scan per tile of 256 rows, and
-// the fused kernels' decoupled lookback (row_scan.cuh) between tiles -- or,
-// for a small window after the small-window kernel, tiles of 128 rows in
-// one thread-block cluster that exchange their aggregates through
-// distributed shared memory.
+// rule, OPD loss, profile, carried state) then runs on the log-probs: in two
+// passes over tiles of rows (scan_aggregate_kernel, scan_complete_kernel), or,
+// for a small window after the small-window kernel, as one thread-block
+// cluster whose tiles exchange their aggregates through distributed shared
+// memory (scan_cluster_kernel).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -23,6 +22,7 @@
 #include "stride.h"
 #include "stride_device.cuh"
 #include "stride_internal.h"
+#include "warp_tile_scan.cuh"
 
 namespace stride {
 
@@ -136,29 +136,19 @@ __global__ void combine_kernel(const float* __restrict__ parts, int32_t n_shards
   if (lse_t) lse_t[r] = lt;
 }
 
-// The scan on given log-probs, one tile of TILE consecutive rows per CTA (one
-// row per thread; kScanTileRows on its own, kScanTileRowsDependent after the
-// small-window kernel), tiles taken in ticket order (by block index in a
-// small dependent grid, below).  Without a logit pass to hide it, a lookback
-// per row is what the time goes to (each row waits on its predecessors'
-// prefixes), so the rows of a tile are scanned together in the CTA and only
-// the tile takes part in the decoupled lookback:
-//   1. warps 0 and 1 find the tile's first turn and trajectory; the CTA
-//      stages the offsets of the next kScanTileRows + 1 turns and
-//      trajectories in shared memory and every thread finds its row's turn
-//      and trajectory there;
+// A small window's scan after the small-window kernel, one tile of TILE
+// consecutive rows per CTA (one row per thread) and all tiles one
+// thread-block cluster:
+//   1. the CTA stages the offsets of the tile's turns and trajectories in
+//      shared memory and every thread finds its row's there;
 //   2. each row's element: the stop-sum term, log pi_T, d, logp_S * d, and
 //      two restart marks -- the open-turn sums restart at a turn's first row,
 //      the running sum at a seeded row (a trajectory's first row, or the
 //      window's), whose element already holds the carried state;
 //   3. a segmented inclusive scan of the tile's elements (warp shuffles, then
 //      the warps' totals);
-//   4. the tile's aggregate is published (as an INCLUSIVE prefix at once if
-//      the tile holds a seeded row, since nothing before it matters then;
-//      tile 0 always does), warp 0 folds its predecessors' (row_scan.cuh
-//      lookback) and publishes the tile's inclusive prefix (the cluster
-//      form, below: the aggregates go to the later tiles' shared memory,
-//      and warp 0 folds its predecessors' there);
+//   4. the tile's aggregate goes to the later tiles' shared memory, and after
+//      one cluster barrier warp 0 folds its predecessors';
 //   5. every row completes with its inclusive and exclusive prefixes: turn
 //      statistics and carried state (row_tail), the within-turn profile into
 //      the CTA's shared bins;
@@ -171,24 +161,16 @@ constexpr int kRestartSum = 2;   // c restarts (a seeded row)
 
 // A row's element inside a tile.  The running stop sum c is fp64 (the stop
 // rule compares it with lambda); the open-turn sums of log pi_T, d and the
-// loss term are fp32 inside the tile (at most kScanTileRows terms each,
-// summed in a tree: relative error a few 1e-7 of the summed magnitudes), in
-// the cluster form's fold of at most 16 tile aggregates, and where the
-// tile's prefix meets a row; the lookback's prefix over tiles and every
-// stored sum are fp64.  GB300 runs FP64 at 1/64 of the FP32 rate, and the
-// tile scans' fp64 adds were what a small window's scan waited on (a
-// 512-row window in one CTA: 6.6 us for the block scan).
+// loss term are fp32 inside the tile (summed in a tree: relative error a few
+// 1e-7 of the summed magnitudes), in the cluster's fold of at most 16 tile
+// aggregates, and where the tile's prefix meets a row; every stored sum is
+// fp64.  GB300 runs FP64 at 1/64 of the FP32 rate, and the tile scans' fp64
+// adds were what a small window's scan waited on (a 512-row window in one
+// CTA: 6.6 us for the block scan).
 struct TileElem {
   double c;
   float st, sd, sl;
   int flags;
-};
-
-// A prefix over tiles as the lookback folds it: fp64 throughout.  (A row's
-// inclusive and exclusive values, and the cluster form's fold, use TileElem:
-// the stop sum fp64, the open-turn sums fp32.)
-struct PreElem {
-  double c, st, sd, sl;
 };
 
 __device__ __forceinline__ TileElem tile_combine(const TileElem& a, const TileElem& b) {
@@ -198,16 +180,6 @@ __device__ __forceinline__ TileElem tile_combine(const TileElem& a, const TileEl
   r.sd = (b.flags & kRestartTurn) ? b.sd : a.sd + b.sd;
   r.sl = (b.flags & kRestartTurn) ? b.sl : a.sl + b.sl;
   r.flags = a.flags | b.flags;
-  return r;
-}
-
-// A tile's prefix followed by an in-tile prefix.
-__device__ __forceinline__ PreElem pre_combine(const PreElem& a, const TileElem& b) {
-  PreElem r;
-  r.c = (b.flags & kRestartSum) ? b.c : a.c + b.c;
-  r.st = (b.flags & kRestartTurn) ? (double)b.st : a.st + (double)b.st;
-  r.sd = (b.flags & kRestartTurn) ? (double)b.sd : a.sd + (double)b.sd;
-  r.sl = (b.flags & kRestartTurn) ? (double)b.sl : a.sl + (double)b.sl;
   return r;
 }
 
@@ -292,24 +264,28 @@ __device__ __forceinline__ int smem_upper_le(const int64_t* a, int n, int64_t r)
   return lo;
 }
 
-// The cluster form (CLUSTER; a small window of at most kClusterMaxTiles
-// tiles, launched as ONE thread-block cluster of one CTA per tile, so that
-// the tiles run at once): in place of the lookback through global memory,
-// each tile stores its aggregate into the shared memory of every later
-// tile of the cluster, and after one cluster barrier folds its
-// predecessors' aggregates itself.  A second role of the barrier: the
-// carried state is read before the dependency wait and written at a
-// trajectory's last row, possibly by a later tile, so every CTA arrives
-// once its reads are done and waits before any write.  (In the lookback
-// form that order comes from the chain of published prefixes.)
+// The tiles of a window of at most kClusterMaxTiles tiles run at once, as
+// ONE thread-block cluster of one CTA per tile: each stores its aggregate
+// into the shared memory of every later tile, and after one cluster barrier
+// folds its predecessors' aggregates itself.  A second role of the barrier:
+// the carried state is read before the dependency wait and written at a
+// trajectory's last row, possibly by a later tile, so every CTA arrives once
+// its reads are done and waits before any write.
 constexpr int kClusterMaxTiles = 16;
+// Rows per tile of the cluster scan (a build define, for sweeps).  A sweep of
+// the lookback form that preceded it on GB300: the 512-row tiny step took 36.6
+// / 36.7 / 37.4 / 39.0 us with tiles of 64 / 128 / 256 / 512 rows.
+#ifndef STRIDE_CLUSTER_TILE_ROWS
+#define STRIDE_CLUSTER_TILE_ROWS 128
+#endif
+constexpr int kClusterTileRows = STRIDE_CLUSTER_TILE_ROWS;
+static_assert(kClusterTileRows % 32 == 0 && kClusterTileRows >= 64 && kClusterTileRows <= 1024,
+              "whole warps, 2 to 32 of them");
 
-template <int TILE, bool CLUSTER>
-__global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchParams p,
-                                                                          const float* __restrict__ logp_s,
-                                                                          const float* __restrict__ logp_t,
-                                                                          int64_t n_tiles, bool validate,
-                                                                          bool by_ticket) {
+
+template <int TILE>
+__global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p, const float* __restrict__ logp_s,
+                                                            const float* __restrict__ logp_t, int64_t n_tiles) {
   constexpr int kWarps = TILE / 32;
   __shared__ int64_t s_turn_off[TILE + 1];
   __shared__ int64_t s_traj_row[TILE + 1];   // traj_row_off
@@ -321,42 +297,22 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
   __shared__ TrajElem s_tpre[kWarps];
   __shared__ TileElem s_excl;  // the tile's exclusive prefix (flags unused)
   __shared__ TileElem s_agg;
-  __shared__ int s_flags;  // bit 0: lookback timed out
   __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
-  __shared__ int64_t s_tile;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // Launched as a programmatic dependent of the kernel that wrote the
-  // log-probs (griddepcontrol.wait is a no-op otherwise).  That kernel
-  // waited for its own predecessors before letting this grid be scheduled,
-  // so the layout and the carried state may be read before the wait; the
-  // log-probs, the tile flags and the ticket only after it.  Tiles are
-  // taken in ticket order (a tile's lookback waits only on tiles taken
-  // before it, which are running or done) unless the grid is small enough
-  // to be resident at once, when the block index is the tile.
+  // log-probs.  That kernel waited for its own predecessors before letting
+  // this grid be scheduled, so the layout and the carried state may be read
+  // before the wait; the log-probs only after it.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
-  if (by_ticket) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid == 0) s_tile = (int64_t)atomicAdd(p.ticket, 1u);
-  } else if (tid == 0) {
-    s_tile = (int64_t)blockIdx.x;
-  }
-  __syncthreads();
-  const int64_t tile = s_tile;
-  if (tile >= n_tiles) return;
+  const int64_t tile = (int64_t)blockIdx.x;
   const int64_t t0 = tile * TILE;           // first window row of the tile
   const int64_t n_here = min((int64_t)TILE, p.n_rows - t0);
   const int64_t r0 = p.row_begin + t0;
   const int64_t w = t0 + tid;  // this thread's window row
   const int64_t r = p.row_begin + w;
   const bool live = tid < n_here;
-  // the row's log-probs, in flight while the layout is looked up (after
-  // the layout, below, when this grid has not waited yet)
   float lps = 0.f, lpt = 0.f;
-  if (live && by_ticket) {
-    lps = __ldcg(logp_s + w);
-    lpt = __ldcg(logp_t + w);
-  }
 
   // 1. the tile's first turn (warp 0) and first trajectory (warp 1), then
   //    the offsets of the next TILE + 1 of each in shared memory (a layout
@@ -387,7 +343,7 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
   }
   __syncthreads();
 
-  __shared__ TileElem s_caggs[CLUSTER ? kClusterMaxTiles : 1];  // (CLUSTER) predecessors' aggregates
+  __shared__ TileElem s_caggs[kClusterMaxTiles];  // predecessors' aggregates
 
   // 2. this thread's row: its turn and trajectory, and its element
   RowMeta meta;
@@ -440,13 +396,11 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
     sl0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_l);
   }
   const float lam = (live && !meta.bad) ? (p.lambda ? __ldg(p.lambda + meta.traj) : p.lambda_all) : 0.f;
-  if (CLUSTER) cluster_arrive_release();  // this CTA's reads of the carried state are done
-  if (!by_ticket) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (live) {
-      lps = __ldcg(logp_s + w);
-      lpt = __ldcg(logp_t + w);
-    }
+  cluster_arrive_release();  // this CTA's reads of the carried state are done
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (live) {
+    lps = __ldcg(logp_s + w);
+    lpt = __ldcg(logp_t + w);
   }
   TileElem x = {0.0, 0.0, 0.0, 0.0, 0};
   double c_before = 0.0, st_before = 0.0, ri_c = 0.0;
@@ -497,70 +451,32 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
   TileElem tile_incl, tile_excl;
   block_scan<kWarps>(x, tile_id, lane, warp, s_wtot, s_wpre, tile_incl, tile_excl);
 
-  // 4. the tile's exclusive prefix: from the cluster's other tiles (CLUSTER),
-  //    else publish the tile's aggregate, fold predecessors, publish its prefix
-  if (CLUSTER) {
-    namespace cg = cooperative_groups;
-    if (tid == (int)(n_here - 1)) s_agg = tile_incl;
-    __syncthreads();
-    cluster_wait_acquire();  // every tile has started and read its carried state
-    if (warp == 0) {
-      const cg::cluster_group cl = cg::this_cluster();
-      const TileElem agg = s_agg;
-      for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) cl.map_shared_rank(s_caggs, (unsigned)j)[tile] = agg;
-    }
-    cluster_arrive_release();
-    cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
-    if (warp == 0) {
-      // the predecessors' aggregates folded in tile order (a warp scan: the
-      // stop sum fp64, the open-turn sums fp32 as inside a tile)
-      TileElem v = {0.0, 0.f, 0.f, 0.f, 0};
-      if (lane < tile) v = s_caggs[lane];
-#pragma unroll
-      for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
-        const TileElem o = tile_shfl_up(v, d);
-        if (lane >= d) v = tile_combine(o, v);
-      }
-      if (lane == (tile > 0 ? (int)tile - 1 : 0)) {
-        s_excl = tile > 0 ? TileElem{v.c, v.st, v.sd, v.sl, 0} : TileElem{0.0, 0.f, 0.f, 0.f, 0};
-        s_flags = 0;
-      }
-    }
-    __syncthreads();
-  } else {
-    if (tid == (int)(n_here - 1)) {
-      ScanElem agg{tile_incl.c, tile_incl.st, tile_incl.sd, tile_incl.sl, tile_incl.flags & kRestartTurn};
-      if (tile_incl.flags & kRestartSum) {
-        publish(p.incl + tile, p.flags + tile * kFlagStride, agg, kStIncl);
-      } else {
-        publish(p.agg + tile, p.flags + tile * kFlagStride, agg,
-                kStAgg | ((tile_incl.flags & kRestartTurn) ? kFlagTurnStart : 0u));
-      }
-      s_agg = tile_incl;  // the aggregate, for warp 0 below
-    }
-    __syncthreads();
-    if (warp == 0) {
-      const TileElem agg = s_agg;
-      PreElem pre = {0.0, 0.0, 0.0, 0.0};
-      bool timed_out = false;
-      // The rows before the tile's first seeded row need the predecessors' sum
-      // (a tile whose first row is seeded needs nothing).
-      if (!(__shfl_sync(0xffffffffu, x.flags, 0) & kRestartSum)) {
-        const ScanElem e = lookback(p, tile, lane, timed_out);
-        pre = PreElem{e.c, e.st, e.sd, e.sl};
-        if (lane == 0 && !(agg.flags & kRestartSum)) {
-          const PreElem inc = pre_combine(pre, agg);
-          ScanElem ie{inc.c, inc.st, inc.sd, inc.sl, 1};
-          publish(p.incl + tile, p.flags + tile * kFlagStride, ie, kStIncl);
-        }
-      }
-      if (lane == 0) {
-        s_excl = TileElem{pre.c, (float)pre.st, (float)pre.sd, (float)pre.sl, 0};
-        s_flags = timed_out ? 1 : 0;
-      }
-    }
-    __syncthreads();
+  // 4. the tile's exclusive prefix, from the cluster's other tiles
+  namespace cg = cooperative_groups;
+  if (tid == (int)(n_here - 1)) s_agg = tile_incl;
+  __syncthreads();
+  cluster_wait_acquire();  // every tile has started and read its carried state
+  if (warp == 0) {
+    const cg::cluster_group cl = cg::this_cluster();
+    const TileElem agg = s_agg;
+    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) cl.map_shared_rank(s_caggs, (unsigned)j)[tile] = agg;
   }
+  cluster_arrive_release();
+  cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
+  if (warp == 0) {
+    // the predecessors' aggregates folded in tile order (a warp scan: the
+    // stop sum fp64, the open-turn sums fp32 as inside a tile)
+    TileElem v = {0.0, 0.f, 0.f, 0.f, 0};
+    if (lane < tile) v = s_caggs[lane];
+#pragma unroll
+    for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
+      const TileElem o = tile_shfl_up(v, d);
+      if (lane >= d) v = tile_combine(o, v);
+    }
+    if (lane == (tile > 0 ? (int)tile - 1 : 0))
+      s_excl = tile > 0 ? TileElem{v.c, v.st, v.sd, v.sl, 0} : TileElem{0.0, 0.f, 0.f, 0.f, 0};
+  }
+  __syncthreads();
 
   // 5. complete every row
   if (live) {
@@ -577,7 +493,7 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
     RowCarry rc;
     rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, fturn};
     const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 1};
-    row_tail(p, r, meta, rc, si, c_before, st_before, (s_flags & 1) != 0, true);
+    row_tail(p, r, meta, rc, si, c_before, st_before, false, true);
     ri_c = ri.c;
   }
 
@@ -620,16 +536,766 @@ __global__ void __launch_bounds__(TILE) scan_logprobs_tile_kernel(const BatchPar
     __syncthreads();
     if (tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
   }
+}
 
-  // Layout checks, spread over every thread of the launch (off the path of
-  // the scan: nothing above waits for them), unless the kernel that wrote
-  // the log-probs made them.
+// The scan on given log-probs, in two passes over tiles of R x kPassThreads
+// consecutive rows, R rows per thread:
+//   scan_aggregate_kernel  each tile's aggregate: the sums after its last
+//                          seeded row and after its last turn start, and the
+//                          carried state of every seeded row set aside
+//                          (before anything writes the states);
+//   scan_complete_kernel   the same rows again: prefixes inside the tile, the
+//                          profile, and, once the first pass is complete, the
+//                          predecessors' aggregates folded back to the
+//                          nearest seeded tile and every row completed.
+// The second pass is the first one's programmatic dependent, and what it does
+// before its wait needs nothing of it, so the passes overlap: the time is one
+// tile's lookups and scan, then one fold.  No flag, ticket or lookback:
+// nothing waits on another CTA, nothing has to be cleared.
+//
+// What bounds it: latency, and FP64 issue (1/64 of the FP32 rate).  So a
+// thread takes R rows one after the other (one fp64 add each), and only the
+// threads' totals are scanned across the CTA; the open-turn sums are pairs
+// of fp32 numbers inside a tile and meet the fp64 prefix where a turn ends.  The profile's
+// sums are formed per thread and per run of equal deciles, in registers: a
+// shared-memory fp64 atomicAdd per row is a compare-and-swap loop that a
+// warp's rows, nearly all in one decile, went through in turn.
+//
+// GB300, 148,909 rows in 64 trajectories of 8 turns with the profile: a tile
+// of 256 rows with a row per thread, shared-memory atomics per row and a
+// lookback took 68.8 us (and its 19 MB clear 3.8 us); the passes take about
+// 21.  The whole chain of a training step on given log-probs (state, profile
+// cleared, scan, record, restart choice): 87.8 -> 33.0 us.
+constexpr int kPassThreads = 256;
+constexpr int kPassWarps = kPassThreads / 32;
+// Up to this many tiles a tile folds its predecessors' aggregates itself
+// (kPassThreads per round, back to the nearest seeded tile); above it one CTA
+// turns them into prefixes first, so that one long trajectory's scan stays
+// linear in its rows.
+constexpr int64_t kDirectTiles = 4096;
+constexpr int kFromSeed = 8;  // the open turn's sums start at a seeded row
+
+// A tile's part of the layout: the offsets of its first turn and of the
+// ROWS turns after it (every turn has a row at least), and of as many
+// trajectories.
+template <int ROWS>
+struct TileLayout {
+  int64_t turn_off[ROWS + 1];
+  int64_t traj_row[ROWS + 1];
+  int64_t traj_turn[ROWS + 1];
+  int64_t first[2];  // first turn and first trajectory, -1 if the layout does not reach the tile's first row
+  int begun[2];      // of the staged turns and trajectories, those that begin at or before the tile's last row
+};
+
+template <int ROWS>
+__device__ __forceinline__ void stage_layout(const BatchParams& p, int64_t r0, int n_here, int tid,
+                                             TileLayout<ROWS>& L) {
+  const int lane = tid & 31, warp = tid >> 5;
+  if (tid < 2) L.begun[tid] = 0;
+  if (p.n_turns <= ROWS && p.n_traj <= ROWS) {  // all of it: no search
+    if (tid == 0) {
+      L.first[0] = p.n_turns > 0 ? 0 : -1;
+      L.first[1] = 0;
+    }
+  } else if (warp == 0) {
+    const bool ok = p.n_turns > 0 && __ldg(p.turn_row_off) <= r0;
+    const int64_t k0 = ok ? warp_upper_le(p.turn_row_off, 0, p.n_turns - 1, r0, lane) : 0;
+    if (lane == 0) L.first[0] = ok ? k0 : -1;
+  } else if (warp == 1) {
+    const bool ok = __ldg(p.traj_row_off) <= r0;
+    const int64_t i0 = ok ? warp_upper_le(p.traj_row_off, 0, p.n_traj - 1, r0, lane) : 0;
+    if (lane == 0) L.first[1] = ok ? i0 : -1;
+  }
+  __syncthreads();
+  const int64_t k0 = L.first[0], i0 = L.first[1];
+  if (k0 >= 0 && i0 >= 0) {
+// (whole warps take part: ROWS is a multiple of the CTA's threads, the
+    // offset after the last is one thread's)
+#pragma unroll
+    for (int i = 0; i <= ROWS; i += kPassThreads) {
+      const int j = i + tid;
+      if (i == ROWS && warp != 0) break;
+      bool turn = false, traj = false;
+      if (j <= ROWS) {
+        if (k0 + j <= p.n_turns) {
+          const int64_t o = __ldg(p.turn_row_off + k0 + j);
+          L.turn_off[j] = o;
+          turn = j < ROWS && k0 + j < p.n_turns && o < r0 + n_here;
+        }
+        if (i0 + j <= p.n_traj) {
+          const int64_t o = __ldg(p.traj_row_off + i0 + j);
+          L.traj_row[j] = o;
+          L.traj_turn[j] = __ldg(p.traj_turn_off + i0 + j);
+          traj = j < ROWS && i0 + j < p.n_traj && o < r0 + n_here;
+        }
+      }
+      const int n_turn = __popc(__ballot_sync(0xffffffffu, turn)), n_traj = __popc(__ballot_sync(0xffffffffu, traj));
+      if (lane == 0 && n_turn) atomicAdd(&L.begun[0], n_turn);
+      if (lane == 0 && n_traj) atomicAdd(&L.begun[1], n_traj);
+    }
+  }
+  __syncthreads();
+}
+
+// Row r's turn and trajectory.  `m` may hold an earlier row's: most rows
+// share its.
+template <int ROWS>
+__device__ __forceinline__ void seek_row(const BatchParams& p, const TileLayout<ROWS>& L, int64_t r, RowMeta& m) {
+  if (!m.bad && r < m.turn_end && r < m.traj_end) return;  // (rows are sought in ascending order)
+  m.bad = true;
+  m.traj = m.turn = m.local_turn = 0;
+  m.traj_start = m.traj_end = m.turn_start = m.turn_end = 0;
+  const int64_t k0 = L.first[0], i0 = L.first[1];
+  if (k0 < 0 || i0 < 0) return;
+  const int j = smem_upper_le(L.turn_off, max(L.begun[0], 1), r);
+  const int ni = max(L.begun[1], 1);
+  const int q = smem_upper_le(L.traj_row, ni, r);
+  int64_t traj = i0 + q, tr_start = L.traj_row[q], tr_end = L.traj_row[q + 1];
+  int64_t tu0 = L.traj_turn[q], tu1 = L.traj_turn[q + 1];
+  if (r >= tr_end && q == ni - 1 && i0 + ni < p.n_traj) {
+    // past the staged trajectories (more than ROWS empty ones in the tile's
+    // rows): search the rest in global memory
+    int64_t lo = i0 + ni, hi = p.n_traj - 1;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(p.traj_row_off + mid) <= r) lo = mid; else hi = mid - 1;
+    }
+    traj = lo;
+    tr_start = __ldg(p.traj_row_off + traj);
+    tr_end = __ldg(p.traj_row_off + traj + 1);
+    tu0 = __ldg(p.traj_turn_off + traj);
+    tu1 = __ldg(p.traj_turn_off + traj + 1);
+  }
+  const int64_t turn = k0 + j;
+  m.turn = (int32_t)turn;
+  m.traj = (int32_t)traj;
+  m.turn_start = L.turn_off[j];
+  m.turn_end = L.turn_off[j + 1];
+  m.local_turn = (int32_t)(turn - tu0);
+  m.traj_start = tr_start;
+  m.traj_end = tr_end;
+  m.bad = !(m.turn_start <= r && r < m.turn_end) || !(tr_start <= r && r < tr_end) || !(tu0 <= turn && turn < tu1);
+}
+
+__device__ __forceinline__ RowMeta no_row() {
+  RowMeta m;
+  m.bad = true;
+  m.traj = m.turn = m.local_turn = 0;
+  m.traj_start = m.traj_end = m.turn_start = m.turn_end = 0;
+  return m;
+}
+
+// A row's stop-sum term: a turn mean's share lpt / n_k is rounded once to
+// fp32 (an fp64 divide is a sequence of fp64 operations; the rounding is 6e-8
+// of the term).
+__device__ __forceinline__ double stop_term(const BatchParams& p, const RowMeta& m, float lpt) {
+  if (p.mode != STRIDE_STOP_TURN_MEAN) return (double)lpt;
+  const int64_t n_k = m.turn_end - m.turn_start;
+  return (double)(lpt / (float)(n_k > 0 ? n_k : 1));
+}
+
+// The log-probs of the tile's rows, coalesced into shared memory.
+template <int R>
+__device__ __forceinline__ void load_logps(const float* __restrict__ logp_s, const float* __restrict__ logp_t,
+                                           int64_t t0, int n_here, int tid, float* s_ls, float* s_lt) {
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int j = i * kPassThreads + tid;
+    s_ls[j] = j < n_here ? __ldcg(logp_s + t0 + j) : 0.f;
+    s_lt[j] = j < n_here ? __ldcg(logp_t + t0 + j) : 0.f;
+  }
+}
+
+// A sum of fp32 terms as the fp32 sum and the sum of its rounding errors
+// (Knuth's TwoSum): hi + lo is good to about 2^-45 of the summed magnitudes
+// over a tile, at seven FP32 operations where an fp64 add costs as much as 64.
+// An infinite or NaN hi is the answer (lo is NaN then).
+struct Sum2 {
+  float hi, lo;
+};
+
+__device__ __forceinline__ void sum_add(Sum2& a, float hi, float lo) {
+  const float s = __fadd_rn(a.hi, hi), b = s - a.hi;
+  const float e = (a.hi - (s - b)) + (hi - b);
+  a.hi = s;
+  a.lo += lo + e;
+}
+
+__device__ __forceinline__ double sum_value(const Sum2& a) {
+  return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi;
+}
+
+__device__ __forceinline__ Sum2 sum_shfl_up(const Sum2& a, int d) {
+  return Sum2{__shfl_up_sync(0xffffffffu, a.hi, d), __shfl_up_sync(0xffffffffu, a.lo, d)};
+}
+
+__device__ __forceinline__ Sum2 warp_sum(Sum2 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    sum_add(v, __shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+  return v;
+}
+
+// Inclusive sum over the lanes from `head` (<= lane) to this one.
+__device__ __forceinline__ Sum2 seg_sum(Sum2 v, int head, int lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const Sum2 o = sum_shfl_up(v, d);
+    if (lane - d >= head) sum_add(v, o.hi, o.lo);
+  }
+  return v;
+}
+
+// A thread's or tile's element without the carried state: sums since the last
+// seeded row (c) and since the last turn start (st, sd, sl).
+struct PassElem {
+  double c;
+  Sum2 st, sd, sl;
+  int flags;
+  int seed;  // the last seeded row, from the tile's first; -1: none
+};
+
+__device__ __forceinline__ void open_rows(Sum2& v, const Sum2& before, bool turn) {
+  if (!turn) sum_add(v, before.hi, before.lo);
+}
+
+__device__ __forceinline__ PassElem elem_combine(const PassElem& a, const PassElem& b) {
+  PassElem r;
+  r.c = (b.flags & kRestartSum) ? b.c : a.c + b.c;
+  const bool turn = (b.flags & kRestartTurn) != 0;
+  r.st = b.st;
+  r.sd = b.sd;
+  r.sl = b.sl;
+  open_rows(r.st, a.st, turn);
+  open_rows(r.sd, a.sd, turn);
+  open_rows(r.sl, a.sl, turn);
+  r.flags = ((a.flags | b.flags) & (kRestartSum | kRestartTurn)) | ((turn ? b.flags : a.flags) & kFromSeed);
+  r.seed = max(a.seed, b.seed);
+  return r;
+}
+
+__device__ __forceinline__ PassElem elem_shfl_up(const PassElem& v, int d) {
+  PassElem o;
+  o.c = __shfl_up_sync(0xffffffffu, v.c, d);
+  o.st = sum_shfl_up(v.st, d);
+  o.sd = sum_shfl_up(v.sd, d);
+  o.sl = sum_shfl_up(v.sl, d);
+  o.flags = __shfl_up_sync(0xffffffffu, v.flags, d);
+  o.seed = __shfl_up_sync(0xffffffffu, v.seed, d);
+  return o;
+}
+
+// Index of the largest thread of the CTA with `has`, -1 if none (two words of
+// s_any per warp; the caller synchronises before s_any is used again).
+__device__ __forceinline__ int last_thread(unsigned ballot, int lane, int warp, int* s_any) {
+  if (lane == 0) s_any[warp] = ballot ? warp * 32 + 31 - __clz(ballot) : -1;
+  __syncthreads();
+  int n = -1;
+#pragma unroll
+  for (int w = 0; w < kPassWarps; ++w) n = max(n, s_any[w]);
+  return n;
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// A slot that the first pass wrote, past this SM's L1.
+__device__ __forceinline__ ScanSlot load_slot(const ScanSlot* s) {
+  const double2 a = __ldcg(reinterpret_cast<const double2*>(s));
+  const double2 b = __ldcg(reinterpret_cast<const double2*>(s) + 1);
+  return ScanSlot{a.x, a.y, b.x, b.y};
+}
+
+// First pass: tile t's aggregate in agg[t], its kRestart marks in flags[t],
+// and in incl[w] the carried state of every seeded row w.
+template <int R>
+__global__ void __launch_bounds__(kPassThreads) scan_aggregate_kernel(const BatchParams p,
+                                                                     const float* __restrict__ logp_s,
+                                                                     const float* __restrict__ logp_t) {
+  constexpr int kRows = R * kPassThreads;
+  __shared__ TileLayout<kRows> L;
+  __shared__ float s_ls[kRows], s_lt[kRows];
+  __shared__ int s_any[2][kPassWarps];
+  __shared__ double s_c[kPassWarps], s_base[4];
+  __shared__ Sum2 s_open[3][kPassWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // Everything before this kernel is complete past the wait, and only then
+  // may the second pass come in: what it reads before its own wait (the
+  // layout, the log-probs, lambda) is complete too.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int64_t tile = blockIdx.x;
+  const int64_t t0 = tile * kRows;
+  const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
+  load_logps<R>(logp_s, logp_t, t0, n_here, tid, s_ls, s_lt);
+  if (tid < 4) s_base[tid] = 0.0;
+  stage_layout(p, p.row_begin + t0, n_here, tid, L);
+
+  RowMeta m = no_row();
+  double c = 0.0, seed_c = 0.0, seed_st = 0.0, seed_sd = 0.0, seed_sl = 0.0;
+  Sum2 st = {0.f, 0.f}, sd = st, sl = st;
+  bool has_sum = false, has_turn = false, from_seed = false;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int j = tid * R + i;
+    if (j >= n_here) break;
+    const int64_t r = p.row_begin + t0 + j;
+    seek_row(p, L, r, m);
+    float lps = s_ls[j], lpt = s_lt[j];
+    if (m.bad) lps = lpt = __int_as_float(0x7fc00000);
+    const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
+    const bool fturn = r == m.turn_start;
+    if (seeded) {
+      ScanSlot z = {0.0, 0.0, 0.0, 0.0};
+      if (!m.bad) {
+        const stride_scan_state* sp = p.state + m.traj;
+        z.c = __ldcg(&sp->cum);
+        if (!fturn) {
+          z.st = __ldcg(&sp->turn_sum_t);
+          z.sd = __ldcg(&sp->turn_sum_d);
+          z.sl = __ldcg(&sp->turn_sum_l);
+        }
+      }
+      p.incl[t0 + j] = z;
+      seed_c = z.c;
+      seed_st = z.st;
+      seed_sd = z.sd;
+      seed_sl = z.sl;
+      c = 0.0;
+      has_sum = true;
+    }
+    if (seeded || fturn) {
+      st = sd = sl = Sum2{0.f, 0.f};
+      has_turn = true;
+      from_seed = seeded;
+    }
+    const float dd = lps - lpt;
+    c += stop_term(p, m, lpt);
+    sum_add(st, lpt, 0.f);
+    sum_add(sd, dd, 0.f);
+    sum_add(sl, lps * dd, 0.f);
+  }
+  // only what follows the last restart counts
+  const int own_c = last_thread(__ballot_sync(0xffffffffu, has_sum), lane, warp, s_any[0]);
+  const int own_t = last_thread(__ballot_sync(0xffffffffu, has_turn), lane, warp, s_any[1]);
+  if (tid == own_c) s_base[0] = seed_c;
+  if (tid == own_t && from_seed) {
+    s_base[1] = seed_st;
+    s_base[2] = seed_sd;
+    s_base[3] = seed_sl;
+  }
+  c = warp * 32 + 31 < own_c ? 0.0 : warp_sum(tid >= own_c ? c : 0.0);
+  if (tid < own_t) st = sd = sl = Sum2{0.f, 0.f};
+  if (warp * 32 + 31 >= own_t) {
+    st = warp_sum(st);
+    sd = warp_sum(sd);
+    sl = warp_sum(sl);
+  }
+  if (lane == 0) {
+    s_c[warp] = c;
+    s_open[0][warp] = st;
+    s_open[1][warp] = sd;
+    s_open[2][warp] = sl;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const Sum2 zero = {0.f, 0.f};
+    c = warp_sum(lane < kPassWarps ? s_c[lane] : 0.0);
+    st = warp_sum(lane < kPassWarps ? s_open[0][lane] : zero);
+    sd = warp_sum(lane < kPassWarps ? s_open[1][lane] : zero);
+    sl = warp_sum(lane < kPassWarps ? s_open[2][lane] : zero);
+    if (lane == 0) {
+      p.agg[tile] =
+          ScanSlot{s_base[0] + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl)};
+      p.flags[tile] = (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0);
+    }
+  }
+}
+
+// Between the passes of a window of many tiles: the aggregates replaced by
+// the prefixes before each tile.  One CTA, in rounds of a tile per thread.
+constexpr int kPrefixThreads = 1024;
+
+struct PrefixElem {
+  double c, st, sd, sl;
+  int flags;
+};
+
+__device__ __forceinline__ PrefixElem elem_combine(const PrefixElem& a, const PrefixElem& b) {
+  PrefixElem r;
+  const bool turn = (b.flags & kRestartTurn) != 0;
+  r.c = (b.flags & kRestartSum) ? b.c : a.c + b.c;
+  r.st = turn ? b.st : a.st + b.st;
+  r.sd = turn ? b.sd : a.sd + b.sd;
+  r.sl = turn ? b.sl : a.sl + b.sl;
+  r.flags = a.flags | b.flags;
+  return r;
+}
+
+__device__ __forceinline__ PrefixElem elem_shfl_up(const PrefixElem& v, int d) {
+  PrefixElem o;
+  o.c = __shfl_up_sync(0xffffffffu, v.c, d);
+  o.st = __shfl_up_sync(0xffffffffu, v.st, d);
+  o.sd = __shfl_up_sync(0xffffffffu, v.sd, d);
+  o.sl = __shfl_up_sync(0xffffffffu, v.sl, d);
+  o.flags = __shfl_up_sync(0xffffffffu, v.flags, d);
+  return o;
+}
+
+__global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(ScanSlot* agg, const uint32_t* flags,
+                                                                     int64_t n_tiles) {
+  constexpr int kWarps = kPrefixThreads / 32;
+  __shared__ PrefixElem s_tot[kWarps], s_pre[kWarps], s_carry;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const PrefixElem id = {0.0, 0.0, 0.0, 0.0, 0};
+  PrefixElem carry = id;
+  for (int64_t t = 0; t < n_tiles; t += kPrefixThreads) {
+    const int64_t j = t + tid;
+    PrefixElem v = id;
+    if (j < n_tiles) {
+      const ScanSlot a = load_slot(agg + j);
+      v = PrefixElem{a.c, a.st, a.sd, a.sl, (int)__ldcg(flags + j)};
+    }
+    PrefixElem incl, excl;
+    block_scan<kWarps>(v, id, lane, warp, s_tot, s_pre, incl, excl);
+    const PrefixElem before = elem_combine(carry, excl);
+    if (j < n_tiles) agg[j] = ScanSlot{before.c, before.st, before.sd, before.sl};
+    if (tid == kPrefixThreads - 1) s_carry = elem_combine(carry, incl);
+    __syncthreads();
+    carry = s_carry;
+    __syncthreads();
+  }
+}
+
+// A trajectory's share of a thread's rows: the loss of its retained rows and
+// its first crossing of lambda here.
+struct TrajPart {
+  int32_t traj, count, cross_turn;  // traj -1: none
+  float loss;
+  int64_t cross_row;  // from the trajectory's first row; -1: none
+};
+
+__device__ __forceinline__ void record_cross(stride_scan_state* sp, const TrajPart& t) {
+  atomicMin(reinterpret_cast<unsigned long long*>(&sp->stop_row), (unsigned long long)t.cross_row);
+  atomicMin(reinterpret_cast<unsigned int*>(&sp->stop_turn), (unsigned int)t.cross_turn);
+  sp->stopped = 1;
+}
+
+__device__ __forceinline__ void record_loss(stride_scan_state* sp, float loss, int count) {
+  atomicAdd(&sp->loss, (double)loss);
+  atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), (unsigned long long)count);
+}
+
+// Second pass.
+template <int R>
+__global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const BatchParams p,
+                                                                    const float* __restrict__ logp_s,
+                                                                    const float* __restrict__ logp_t, int64_t n_tiles,
+                                                                    bool prefixed, bool validate) {
+  constexpr int kRows = R * kPassThreads;
+  __shared__ TileLayout<kRows> L;
+  __shared__ float s_ls[kRows], s_lt[kRows];
+  __shared__ PassElem s_tot[kPassWarps], s_wpre[kPassWarps];
+  __shared__ int s_near[2][kPassWarps];
+  __shared__ double s_fold[4][kPassWarps];
+  __shared__ double s_pre[4];
+  __shared__ int s_needs;
+  __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int64_t tile = blockIdx.x;
+  const int64_t t0 = tile * kRows;
+  const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
+  const float nan = __int_as_float(0x7fc00000);
+  load_logps<R>(logp_s, logp_t, t0, n_here, tid, s_ls, s_lt);
+  if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
+  if (tid < 4) s_pre[tid] = 0.0;
+  stage_layout(p, p.row_begin + t0, n_here, tid, L);
+
+  // ---- this thread's rows: their element, and the profile
+  RowMeta m = no_row();
+  const Sum2 zero = {0.f, 0.f};
+  const PassElem id = {0.0, zero, zero, zero, 0, -1};
+  PassElem x = id;
+  RowMeta first = m;
+  float lam = 0.f;
+  int bin = -1, bin_n = 0;  // the open run of equal deciles
+  Sum2 bin_d = zero, bin_t = zero;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int j = tid * R + i;
+    if (j >= n_here) break;
+    const int64_t r = p.row_begin + t0 + j;
+    seek_row(p, L, r, m);
+    if (i == 0) {
+      first = m;
+      if (!m.bad) lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
+    }
+    const float lps = m.bad ? nan : s_ls[j], lpt = m.bad ? nan : s_lt[j];
+    const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
+    const bool fturn = r == m.turn_start;
+    if (j == 0) s_needs = seeded ? 0 : 1;
+    if (seeded) {
+      x.c = 0.0;
+      x.seed = j;
+      x.flags |= kRestartSum;
+    }
+    if (seeded || fturn) {
+      x.st = x.sd = x.sl = zero;
+      x.flags = (x.flags & kRestartSum) | kRestartTurn | (seeded ? kFromSeed : 0);
+    }
+    const float dd = lps - lpt;
+    x.c += stop_term(p, m, lpt);
+    sum_add(x.st, lpt, 0.f);
+    sum_add(x.sd, dd, 0.f);
+    sum_add(x.sl, lps * dd, 0.f);
+    if (p.profile && !m.bad) {
+      const int64_t pos = r - m.turn_start, n_k = m.turn_end - m.turn_start;
+      const int b = n_k < (1 << 28) ? (int)(10u * (unsigned)pos / (unsigned)n_k) : (int)((10 * pos) / n_k);  // Observation 1 decile
+      if (b != bin) {
+        if (bin >= 0) {
+          atomicAdd(s_prof + 3 * bin + 0, sum_value(bin_d));
+          atomicAdd(s_prof + 3 * bin + 1, sum_value(bin_t));
+          atomicAdd(s_prof + 3 * bin + 2, (double)bin_n);
+        }
+        bin = b;
+        bin_n = 0;
+        bin_d = bin_t = zero;
+      }
+      sum_add(bin_d, dd, 0.f);
+      sum_add(bin_t, lpt, 0.f);
+      ++bin_n;
+    }
+  }
+  if (p.profile) {
+    // the threads' open runs, neighbours of one decile together
+    const int prev = __shfl_up_sync(0xffffffffu, bin, 1);
+    const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || bin != prev);
+    const int h = head_of(m_run, lane);
+    const Sum2 sum_d = seg_sum(bin_d, h, lane), sum_t = seg_sum(bin_t, h, lane);
+    int n = bin_n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, n, d);
+      if (lane - d >= h) n += o;
+    }
+    if (bin >= 0 && (lane == 31 || ((m_run >> lane) & 2u))) {
+      atomicAdd(s_prof + 3 * bin + 0, sum_value(sum_d));
+      atomicAdd(s_prof + 3 * bin + 1, sum_value(sum_t));
+      atomicAdd(s_prof + 3 * bin + 2, (double)n);
+    }
+  }
+  PassElem incl, excl;
+  block_scan<kPassWarps>(x, id, lane, warp, s_tot, s_wpre, incl, excl);
+
+  // ---- the first pass's results
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int32_t seed0 = excl.seed;  // the last seeded row before this thread's
+  ScanSlot seed = {0.0, 0.0, 0.0, 0.0};
+  if (seed0 >= 0 && tid * R < n_here) seed = load_slot(p.incl + t0 + seed0);
+  if (s_needs && prefixed) {
+    if (tid == 0) {
+      const ScanSlot a = load_slot(p.agg + tile);
+      s_pre[0] = a.c;
+      s_pre[1] = a.st;
+      s_pre[2] = a.sd;
+      s_pre[3] = a.sl;
+    }
+  } else if (s_needs) {
+    // Sums of the predecessors' aggregates back to the nearest one with a
+    // seeded row (c), and to the nearest one with a turn start (the others).
+    double f[4] = {0.0, 0.0, 0.0, 0.0};
+    bool turn_open = true, any = false;
+    for (int64_t hi = tile; hi > 0; hi -= kPassThreads) {
+      const int64_t j = hi - 1 - tid;
+      unsigned fl = 0;
+      ScanSlot a = {0.0, 0.0, 0.0, 0.0};
+      if (j >= 0) {
+        fl = __ldcg(p.flags + j);
+        a = load_slot(p.agg + j);
+      }
+      const unsigned b_sum = __ballot_sync(0xffffffffu, (fl & kRestartSum) != 0);
+      const unsigned b_turn = __ballot_sync(0xffffffffu, (fl & kRestartTurn) != 0);
+      if (lane == 0) {
+        s_near[0][warp] = b_sum ? warp * 32 + __ffs(b_sum) - 1 : kPassThreads;
+        s_near[1][warp] = b_turn ? warp * 32 + __ffs(b_turn) - 1 : kPassThreads;
+      }
+      __syncthreads();
+      int n_sum = kPassThreads, n_turn = kPassThreads;
+#pragma unroll
+      for (int w = 0; w < kPassWarps; ++w) {
+        n_sum = min(n_sum, s_near[0][w]);
+        n_turn = min(n_turn, s_near[1][w]);
+      }
+      if (warp * 32 <= n_sum && hi > warp * 32) {
+        any = true;
+        if (tid <= n_sum) f[0] += a.c;
+        if (turn_open && tid <= n_turn) {
+          f[1] += a.st;
+          f[2] += a.sd;
+          f[3] += a.sl;
+        }
+      }
+      turn_open = turn_open && n_turn == kPassThreads;
+      if (n_sum < kPassThreads) break;
+      __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double v = any ? warp_sum(f[k]) : 0.0;
+      if (lane == 0) s_fold[k][warp] = v;
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        double v = lane < kPassWarps ? s_fold[k][lane] : 0.0;
+#pragma unroll
+        for (int o = kPassWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) s_pre[k] = v;
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- complete the rows
+  double c = (seed0 >= 0 ? seed.c : s_pre[0]) + excl.c;
+  double b_st = s_pre[1], b_sd = s_pre[2], b_sl = s_pre[3];  // what the open turn brought into the tile
+  if (excl.flags & kRestartTurn) {
+    const bool from = (excl.flags & kFromSeed) != 0;
+    b_st = from ? seed.st : 0.0;
+    b_sd = from ? seed.sd : 0.0;
+    b_sl = from ? seed.sl : 0.0;
+  }
+  Sum2 st = excl.st, sd = excl.sd, sl = excl.sl;
+  TrajPart part = {-1, 0, 0, 0.f, -1};
+  bool kept = false;  // in turn mode the same for all of a turn's rows
+  m = first;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int j = tid * R + i;
+    if (j >= n_here) break;
+    const int64_t w = t0 + j, r = p.row_begin + w;
+    if (i > 0) seek_row(p, L, r, m);
+    if (m.bad) {
+      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
+      if (p.out.logp_t) p.out.logp_t[w] = nan;
+      if (p.out.opd) p.out.opd[w] = nan;
+      c = (double)nan;  // nothing after a bad row is meaningful
+      continue;
+    }
+    const float lps = s_ls[j], lpt = s_lt[j], dd = lps - lpt, esl = lps * dd;
+    const bool seeded = w == 0 || r == m.traj_start, fturn = r == m.turn_start;
+    stride_scan_state* sp = p.state + m.traj;
+    if (seeded || fturn) {
+      st = sd = sl = zero;
+      b_st = b_sd = b_sl = 0.0;
+    }
+    if (seeded) {
+      const ScanSlot z = load_slot(p.incl + w);
+      c = z.c;
+      b_st = z.st;
+      b_sd = z.sd;
+      b_sl = z.sl;
+    }
+    if (part.traj != m.traj) {  // a new trajectory: the last one's share is complete
+      if (part.traj >= 0) {
+        if (part.cross_row >= 0) record_cross(p.state + part.traj, part);
+        if (part.count > 0) record_loss(p.state + part.traj, part.loss, part.count);
+        lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
+      } else if (i > 0) {
+        lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
+      }
+      part = TrajPart{m.traj, 0, 0, 0.f, -1};
+    }
+    const bool turn_last = r == m.turn_end - 1;
+    const bool token_sum = p.mode == STRIDE_STOP_TOKEN_SUM;
+    const int64_t n_k = m.turn_end - m.turn_start;
+    // retained unless the rule fired before the row (row_scan.cuh); a
+    // trajectory's first token or turn always is
+    if (token_sum) {
+      kept = r == m.traj_start || !(c < (double)lam);
+    } else if (i == 0 || seeded || fturn) {
+      const double before = c - (double)(((float)b_st + st.hi) / (float)n_k);
+      kept = m.local_turn == 0 || !(before < (double)lam);
+    }
+    c += stop_term(p, m, lpt);
+    sum_add(st, lpt, 0.f);
+    sum_add(sd, dd, 0.f);
+    sum_add(sl, esl, 0.f);
+    if (p.out.opd) p.out.opd[w] = dd;
+    if (kept) {
+      part.loss += esl;
+      ++part.count;
+    }
+    if ((token_sum || turn_last) && part.cross_row < 0 && c < (double)lam) {
+      part.cross_row = r - m.traj_start;
+      part.cross_turn = m.local_turn;
+    }
+    if (turn_last || r == m.traj_end - 1 || r == p.row_end - 1) {
+      const double t_st = b_st + sum_value(st), t_sd = b_sd + sum_value(sd), t_sl = b_sl + sum_value(sl);
+      if (turn_last && p.turn_stats) {
+        stride_turn_stats ts;
+        ts.sum_t = t_st;
+        ts.sum_d = t_sd;
+        ts.sum_l = t_sl;
+        ts.cum = c;
+        ts.mean_t = (float)(t_st / (double)n_k);
+        ts.n = (int32_t)n_k;
+        p.turn_stats[m.turn] = ts;
+      }
+      if (r == m.traj_end - 1 || r == p.row_end - 1) {
+        sp->cum = c;
+        sp->turn_sum_t = turn_last ? 0.0 : t_st;
+        sp->turn_sum_d = turn_last ? 0.0 : t_sd;
+        sp->turn_sum_l = turn_last ? 0.0 : t_sl;
+        sp->rows_seen = r - m.traj_start + 1;
+        sp->turn_idx = turn_last ? m.local_turn + 1 : m.local_turn;
+        sp->turn_tokens = turn_last ? 0 : (int32_t)(r - m.turn_start + 1);
+      }
+    }
+  }
+
+  // ---- the trajectories' records: neighbouring threads of one trajectory
+  //      together (the lowest crossing, the sum of the losses)
+  __syncwarp();
+  const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
+  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
+  const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
+  const int h = head_of(m_run, lane);
+  float loss = part.loss;
+  int count = part.count;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const float o = __shfl_up_sync(0xffffffffu, loss, d);
+    const int n = __shfl_up_sync(0xffffffffu, count, d);
+    if (lane - d >= h) {
+      loss += o;
+      count += n;
+    }
+  }
+  if (part.traj >= 0) {
+    stride_scan_state* sp = p.state + part.traj;
+    const unsigned mine = (0xffffffffu >> (31 - lane)) & (0xffffffffu << h);
+    if (part.cross_row >= 0 && __ffs(m_cross & mine) - 1 == lane) record_cross(sp, part);
+    if (count > 0 && (lane == 31 || ((m_run >> lane) & 2u))) record_loss(sp, loss, count);
+  }
+  if (p.profile && tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
+
+  // Layout checks, spread over every thread of the launch, unless the kernel
+  // that wrote the log-probs made them.
   if (!validate) return;
   bool bad = false;
-  const int64_t stride = n_tiles * TILE;
-  for (int64_t k = t0 + tid; k < p.n_turns; k += stride)
-    bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
-  for (int64_t i = t0 + tid; i < p.n_traj; i += stride) {
+  const int64_t stride = n_tiles * kPassThreads;
+  const int64_t at = tile * kPassThreads + tid;
+  for (int64_t k = at; k < p.n_turns; k += stride) bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
+  for (int64_t i = at; i < p.n_traj; i += stride) {
     const int32_t a = __ldg(p.traj_turn_off + i), b = __ldg(p.traj_turn_off + i + 1);
     if (a < 0 || b < a || b > p.n_turns) {
       bad = true;
@@ -668,7 +1334,7 @@ cudaError_t launch_combine_partials(const float* parts, int32_t n_shards, int64_
   return cudaGetLastError();
 }
 
-// Whether one cluster of n CTAs of the cluster form can be placed on this
+// Whether one cluster of n CTAs of the cluster scan can be placed on this
 // device (looked up once per device and size; sizes above 8 need the
 // non-portable cluster attribute, set here first).
 bool scan_cluster_fits(int dev, int n, cudaStream_t stream) {
@@ -677,13 +1343,13 @@ bool scan_cluster_fits(int dev, int n, cudaStream_t stream) {
   if (dev < 0 || dev >= kMaxDev || n < 1 || n > kClusterMaxTiles) return false;
   const int known = fits[dev][n].load(std::memory_order_acquire);
   if (known) return known == 1;
-  auto kern = scan_logprobs_tile_kernel<kScanTileRowsDependent, true>;
+  auto kern = scan_cluster_kernel<kClusterTileRows>;
   bool ok = true;
   if (n > 8) ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   if (ok) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n);
-    cfg.blockDim = dim3(kScanTileRowsDependent);
+    cfg.blockDim = dim3(kClusterTileRows);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -700,50 +1366,70 @@ bool scan_cluster_fits(int dev, int n, cudaStream_t stream) {
   return ok;
 }
 
-cudaError_t launch_scan_logprobs(const BatchParams& p, const float* logp_s, const float* logp_t,
-                                 cudaStream_t stream, bool dependent) {
-  // (the small-window path's split kernel cleared the flags of its tiles)
-  const int tile_rows = dependent ? kScanTileRowsDependent : kScanTileRows;
-  const int64_t n_tiles = (p.n_rows + tile_rows - 1) / tile_rows;
+namespace {
+
+template <int R>
+cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float* logp_t, bool validate,
+                          cudaStream_t stream) {
+  constexpr int kRows = R * kPassThreads;
+  const int64_t n_tiles = (p.n_rows + kRows - 1) / kRows;
+  const bool prefixed = n_tiles > kDirectTiles;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)n_tiles);
-  cfg.blockDim = dim3((unsigned)tile_rows);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(kPassThreads);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  // the small-window kernel checks the layout itself (dependent launches)
-  const bool validate = !dependent;
-  // A dependent grid of at most one CTA per SM is resident at once (the
-  // kernel it waits on always completes), so its tiles may go by block
-  // index: no ticket, and the layout is read before the wait.
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, scan_aggregate_kernel<R>, p, logp_s, logp_t);
+  if (e == cudaSuccess && prefixed) {
+    cudaLaunchConfig_t one = cfg;
+    one.gridDim = dim3(1);
+    one.blockDim = dim3(kPrefixThreads);
+    e = cudaLaunchKernelEx(&one, scan_prefix_kernel, p.agg, (const uint32_t*)p.flags, n_tiles);
+  }
+  if (e == cudaSuccess)
+    e = cudaLaunchKernelEx(&cfg, scan_complete_kernel<R>, p, logp_s, logp_t, n_tiles, prefixed, validate);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_scan_logprobs(const BatchParams& p, const float* logp_s, const float* logp_t,
+                                 cudaStream_t stream, bool dependent) {
   int dev = 0;
   cudaError_t qe = cudaSuccess;
   const int sms = current_device_sms(&dev, &qe);
   if (sms <= 0) return qe != cudaSuccess ? qe : cudaErrorInvalidDevice;
-  const bool by_ticket = !dependent || n_tiles > sms;
-  // a small dependent window runs as one cluster (the cluster form)
-  const bool cluster = dependent && !by_ticket && n_tiles <= kClusterMaxTiles &&
-                       scan_cluster_fits(dev, (int)n_tiles, stream);
-  if (cluster) {
+  // a small window after the small-window kernel (which checks the layout
+  // itself): one cluster
+  const int64_t cluster_tiles = (p.n_rows + kClusterTileRows - 1) / kClusterTileRows;
+  if (dependent && cluster_tiles <= kClusterMaxTiles && scan_cluster_fits(dev, (int)cluster_tiles, stream)) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster_tiles);
+    cfg.blockDim = dim3(kClusterTileRows);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)n_tiles;
+    attr[1].val.clusterDim.x = (unsigned)cluster_tiles;
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
     cfg.numAttrs = 2;
+    const cudaError_t e =
+        cudaLaunchKernelEx(&cfg, scan_cluster_kernel<kClusterTileRows>, p, logp_s, logp_t, cluster_tiles);
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
-  const cudaError_t e =
-      !dependent ? cudaLaunchKernelEx(&cfg, scan_logprobs_tile_kernel<kScanTileRows, false>, p, logp_s, logp_t,
-                                      n_tiles, validate, by_ticket)
-      : cluster  ? cudaLaunchKernelEx(&cfg, scan_logprobs_tile_kernel<kScanTileRowsDependent, true>, p, logp_s,
-                                      logp_t, n_tiles, validate, by_ticket)
-                 : cudaLaunchKernelEx(&cfg, scan_logprobs_tile_kernel<kScanTileRowsDependent, false>, p, logp_s,
-                                      logp_t, n_tiles, validate, by_ticket);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  // A row per thread while its tiles are one per SM, two from there on.
+  // 148,909 rows as above (init to restart choice), 1 / 2 / 4 rows per
+  // thread: 34.9 / 32.9 / 35.1 us (one token-sum trajectory: 40.3 / 32.4 /
+  // 30.4); 38,000 rows: 24.7 each way.
+  if (p.n_rows <= (int64_t)sms * kPassThreads) return launch_passes<1>(p, logp_s, logp_t, !dependent, stream);
+  return launch_passes<2>(p, logp_s, logp_t, !dependent, stream);
 }
 
 }  // namespace stride
