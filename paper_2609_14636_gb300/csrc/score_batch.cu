@@ -282,18 +282,8 @@ __global__ void teacher_rows_kernel(const BatchParams p, const TeacherTable tt,
 
 cudaError_t launch_teacher_rows(const BatchParams& p, const TeacherTable& tt, const uint8_t* traj_domain,
                                 const int64_t* traj_T_row0, const void** rows_out, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((p.n_rows + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, teacher_rows_kernel, p, tt, traj_domain, traj_T_row0, rows_out);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_dependent(teacher_rows_kernel, (unsigned)((p.n_rows + 255) / 256), 256, stream, p, tt, traj_domain,
+                          traj_T_row0, rows_out);
 }
 
 BatchWorkspaceLayout batch_workspace_layout(int64_t n_rows) {
@@ -414,16 +404,7 @@ cudaError_t launch_clear_workspace(void* ws, size_t bytes, int sms, cudaStream_t
   if (n16 <= 0) return cudaSuccess;
   int64_t blocks = (n16 + 255) / 256;
   if (blocks > 2 * (int64_t)sms) blocks = 2 * (int64_t)sms;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3(256);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, clear_workspace_kernel, reinterpret_cast<uint4*>(ws), n16);
+  return launch_dependent(clear_workspace_kernel, (unsigned)blocks, 256, stream, reinterpret_cast<uint4*>(ws), n16);
 }
 
 cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t clear_bytes, cudaStream_t stream) {

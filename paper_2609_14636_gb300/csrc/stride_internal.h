@@ -114,6 +114,24 @@ cudaError_t launch_teacher_rows(const BatchParams& p, const TeacherTable& tt, co
 // (thread-safe); 0 with the CUDA error in *err if it cannot be queried.
 int current_device_sms(int* dev_out, cudaError_t* err);
 
+// Launches kern as a programmatic dependent of the previous kernel on the
+// stream: its CTAs may be scheduled before that kernel has ended, so kern
+// waits (griddepcontrol.wait) before it touches global memory.
+template <typename... K, typename... A>
+cudaError_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // Launchers return a cudaError_t from the launch.
 // Clears what must start at zero in the workspace (clear_bytes from its
 // start: the clearing kernel, or on the small-window path the split kernel

@@ -57,7 +57,18 @@ struct PartialParams {
   int64_t rows;
   float* partials;  // [rows][6]
   int32_t* dev_status;
+  int64_t first_wave;  // rows whose CTAs are resident from the start
 };
+
+// Bytes per tensor and first-wave CTA that the hints ahead of the wait ask
+// for.  GB300, 6,000 rows in 4 shards of 37,984 bf16 logits, and in 8 of
+// 18,992 (passes, merge and scan): plain launches 531 and 577 us; dependent
+// ones with 0 / 4 / 8 / 16 / 32 KB 520 / 517 / 516 / 518 / 531 and 559 / 552 /
+// 551 / 564 / 585: more than the wait lasts only evicts.
+#ifndef STRIDE_PARTIAL_PREFETCH
+#define STRIDE_PARTIAL_PREFETCH 8192
+#endif
+constexpr int64_t kPartialPrefetch = STRIDE_PARTIAL_PREFETCH;
 
 // One CTA per row: (m, s) of S and T over this shard's columns, and the
 // gathered logits when the token is one of them (NaN otherwise).
@@ -68,6 +79,13 @@ __global__ void __launch_bounds__(kPartialThreads, STRIDE_PARTIAL_MIN_BLOCKS) pa
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const LT* srow = reinterpret_cast<const LT*>(p.S) + r * p.ld;
   const LT* trow = reinterpret_cast<const LT*>(p.T) + r * p.ld;
+  // A programmatic dependent: the first wave's CTAs come in as the previous
+  // kernel's leave, ask for the start of their rows in L2 (a hint, which
+  // reads nothing) and wait for that kernel.
+  if (r < p.first_wave && (tid == 0 || tid == 32))
+    prefetch_l2(tid == 0 ? srow : trow, min((int64_t)p.V_shard * (int64_t)sizeof(LT), kPartialPrefetch));
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
   stream_pair<LT, VEC, STRIDE_PARTIAL_UNROLL>(srow, trow, 0, p.V_shard, tid, kPartialThreads, mS, sS, mT, sT);
   warp_merge2(mS, sS, mT, sT);
@@ -108,6 +126,8 @@ __global__ void __launch_bounds__(kPartialThreads, STRIDE_PARTIAL_MIN_BLOCKS) pa
 __global__ void combine_kernel(const float* __restrict__ parts, int32_t n_shards, int64_t rows,
                                float* logp_s, float* logp_t, float* lse_s, float* lse_t,
                                int32_t* dev_status) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= rows) return;
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
@@ -1310,28 +1330,23 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
 cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec, int64_t ld,
                                int32_t V_shard, int64_t col0, const int32_t* tokens, int64_t rows,
                                float* partials, int32_t* dev_status, cudaStream_t stream) {
-  PartialParams p{S, T, ld, V_shard, col0, 0, tokens, rows, partials, dev_status};
-  const dim3 grid((unsigned)rows), block(kPartialThreads);
-  if (dtype == STRIDE_DTYPE_BF16) {
-    if (vec)
-      partial_lse_kernel<__nv_bfloat16, true><<<grid, block, 0, stream>>>(p);
-    else
-      partial_lse_kernel<__nv_bfloat16, false><<<grid, block, 0, stream>>>(p);
-  } else {
-    if (vec)
-      partial_lse_kernel<float, true><<<grid, block, 0, stream>>>(p);
-    else
-      partial_lse_kernel<float, false><<<grid, block, 0, stream>>>(p);
-  }
-  return cudaGetLastError();
+  int dev = 0;
+  cudaError_t qe = cudaSuccess;
+  const int sms = current_device_sms(&dev, &qe);
+  if (sms <= 0) return qe != cudaSuccess ? qe : cudaErrorInvalidDevice;
+  const PartialParams p{S, T, ld, V_shard, col0, 0, tokens, rows, partials, dev_status,
+                        (int64_t)STRIDE_PARTIAL_MIN_BLOCKS * sms};
+  auto* kern = dtype == STRIDE_DTYPE_BF16
+                   ? (vec ? partial_lse_kernel<__nv_bfloat16, true> : partial_lse_kernel<__nv_bfloat16, false>)
+                   : (vec ? partial_lse_kernel<float, true> : partial_lse_kernel<float, false>);
+  return launch_dependent(kern, (unsigned)rows, kPartialThreads, stream, p);
 }
 
 cudaError_t launch_combine_partials(const float* parts, int32_t n_shards, int64_t rows, float* logp_s,
                                     float* logp_t, float* lse_s, float* lse_t, int32_t* dev_status,
                                     cudaStream_t stream) {
-  combine_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, stream>>>(parts, n_shards, rows, logp_s, logp_t,
-                                                                    lse_s, lse_t, dev_status);
-  return cudaGetLastError();
+  return launch_dependent(combine_kernel, (unsigned)((rows + 255) / 256), 256, stream, parts, n_shards, rows, logp_s, logp_t,
+                          lse_s, lse_t, dev_status);
 }
 
 // Whether one cluster of n CTAs of the cluster scan can be placed on this
@@ -1374,25 +1389,13 @@ cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float
   constexpr int kRows = R * kPassThreads;
   const int64_t n_tiles = (p.n_rows + kRows - 1) / kRows;
   const bool prefixed = n_tiles > kDirectTiles;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)n_tiles);
-  cfg.blockDim = dim3(kPassThreads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, scan_aggregate_kernel<R>, p, logp_s, logp_t);
-  if (e == cudaSuccess && prefixed) {
-    cudaLaunchConfig_t one = cfg;
-    one.gridDim = dim3(1);
-    one.blockDim = dim3(kPrefixThreads);
-    e = cudaLaunchKernelEx(&one, scan_prefix_kernel, p.agg, (const uint32_t*)p.flags, n_tiles);
-  }
+  cudaError_t e = launch_dependent(scan_aggregate_kernel<R>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t);
+  if (e == cudaSuccess && prefixed)
+    e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, p.agg, p.flags, n_tiles);
   if (e == cudaSuccess)
-    e = cudaLaunchKernelEx(&cfg, scan_complete_kernel<R>, p, logp_s, logp_t, n_tiles, prefixed, validate);
-  return e != cudaSuccess ? e : cudaGetLastError();
+    e = launch_dependent(scan_complete_kernel<R>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, n_tiles,
+                         prefixed, validate);
+  return e;
 }
 
 }  // namespace
