@@ -20,9 +20,8 @@
 //
 // Launch shape.  CTAs of 128 threads (8 per SM) or 512 threads (2 per SM),
 // both at most 64 registers per thread; the cluster size C and the CTA size
-// come from the step's row count (choose_shape below): a 256-row step keeps
-// 4-CTA clusters of 128 threads (1,024 CTAs), a 64-row step takes 12, a
-// step of 32 rows or fewer 8-CTA clusters of 512 threads.
+// come from the step's row count (choose_shape below): as many CTAs per row
+// as still run at once.
 //
 // Steps are launched with programmatic dependent launch.  A CTA lets the next
 // kernel be scheduled once its own stream is done, so the next step's CTAs
@@ -31,11 +30,13 @@
 // kernel's completion before its first global read, so the caller's inputs
 // and the carried state are always complete when read.  The loads' ramp thus
 // overlaps the previous step's merges and state updates.  GB300, steps of a
-// 32-step graph (151,936 bf16 logits), before -> now: 61 rows 11.0 -> 9.8 us,
-// 96 rows 13.6 -> 12.6, 128 rows 16.2 -> 14.9, 256 rows 27.0 -> 25.8, 256
-// masked rows 22.7 -> 21.8, 8 rows (in L2 already) 4.95 -> 4.83.  Letting the
-// next step in at the start instead makes its hints compete with this step's
-// loads: 61 rows 9.9, 256 rows 26.1 us at 16 KB per slice.
+// 32-step graph (151,936 bf16 logits), before the overlap -> with it -> with
+// the launch shapes of choose_shape and the loop's last batch in one: 8 rows
+// 5.5 -> 4.8 -> 4.7 us, 61 rows 11.0 -> 9.8 -> 9.2, 128 rows 16.2 -> 14.9 ->
+// 13.9, 256 rows 27.0 -> 25.8 -> 24.9, 256 masked rows (16 plain steps) 25.2 ->
+// 24.3 -> 23.5.  Letting the next step in at the start instead makes its hints
+// compete with this step's loads (61 rows 9.8 -> 10.4), and in mid-stream costs
+// a split of the loop (11.9).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -55,11 +56,12 @@ namespace stride {
 
 constexpr int kStepUnroll = STRIDE_STEP_UNROLL;
 constexpr int kStepMaxCluster = 16;
+constexpr int kStepSmallCluster = 14;  // of 128-thread CTAs: clusters of 16 were slower at every row count
 // Bytes of a step that the hints ahead of the wait ask for, over all its
-// CTAs.  12 / 20 / 32 / 40 / 64 MB: 128 rows 478.6 / 478.2 / 482 / 490 / 508
-// us per 32 steps, 256 rows 823 / 825 / 830 / 832 / 844, 61 rows 315.4 /
-// 313.3 / 314.2 / 312.6 / 312.7: more than the wait lasts only evicts.
-constexpr int64_t kStepPrefetch = 20 << 20;
+// CTAs.  12 / 20 / 28 / 40 MB, us per step: 61 rows 9.4 / 9.3 / 9.2 / 9.4, 76
+// rows 11.2 / 10.6 / 10.3 / 10.4, 128 rows 14.2 / 14.0 / 13.9 / 14.4, 256 rows
+// 25.0 / 24.9 / 24.9 / 25.0: more than the wait lasts only evicts.
+constexpr int64_t kStepPrefetch = 28 << 20;
 // Two CTA shapes, both at most 64 registers per thread: 128 threads, 8 CTAs
 // per SM (the shape of steps with many rows), and 512 threads, 2 per SM (more
 // threads per row when a step has too few rows to fill the GPU with
@@ -307,33 +309,6 @@ std::atomic<int> g_force_cluster{0};
 
 constexpr int kMaxDev = 64;
 
-// Launch shape of a step with `rows` rows.  Sweeps on GB300 (B = 256
-// rollouts, V = 151,936 bf16, row counts 8..256, CTAs of 128 threads in
-// clusters of 4..16 and of 512 threads in clusters of 2..16, 64-step
-// graphs, us per step) found the fastest step
-//  * from 33 rows up: 128-thread CTAs, the step's rows x C filling about 0.85
-//    of one wave (8 CTAs per SM), C at most 12 -- 4 CTAs per row at 256 rows
-//    (26.4 us), 8 at 128 (15.7), 12 at 64 (10.6); filling the whole wave
-//    (1,120-1,216 CTAs) or clusters of 16 cost 2-5 us a step;
-//  * at 32 rows or fewer: 512-thread CTAs in clusters of 8 (8 rows: 5.1 us
-//    against 6.0 for 128-thread CTAs in clusters of 16); larger clusters of
-//    512-thread CTAs were slower (16 rows in clusters of 16: 8.9 us).
-struct Shape {
-  int threads, cluster;
-};
-
-Shape choose_shape(int64_t rows, int sms) {
-  const int ft = g_force_threads.load(std::memory_order_relaxed);
-  const int fc = g_force_cluster.load(std::memory_order_relaxed);
-  if (ft > 0 || fc > 0) return Shape{ft > 0 ? ft : kStepThreadsSmall, fc > 0 ? fc : 1};
-  if (rows <= 4) return Shape{kStepThreadsLarge, 16};
-  if (rows <= 32) return Shape{kStepThreadsLarge, 8};
-  const int64_t fill = (int64_t)sms * 8 * 85 / 100;  // 128-thread CTAs in 0.85 of a wave
-  int64_t c = fill / rows;
-  if (c > 12) c = 12;
-  return Shape{kStepThreadsSmall, (int)(c < 1 ? 1 : c)};
-}
-
 // Cluster sizes above 8 need the non-portable attribute, set once per device
 // for each kernel (one set of statics per template instance).
 template <typename LT, bool VEC, bool COMPACT, int THREADS>
@@ -344,6 +319,77 @@ cudaError_t allow_large_clusters(int dev) {
       cudaFuncSetAttribute(score_step_kernel<LT, VEC, COMPACT, THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) done[dev].store(1, std::memory_order_release);
   return e;
+}
+
+// How many clusters of C CTAs of THREADS threads the device holds at once
+// (GB300's GPCs hold whole clusters: 14 of 16 CTAs of 512 threads, 72 of 4),
+// looked up once per device and size.
+template <int THREADS>
+int resident_clusters(int dev, int C) {
+  static std::atomic<int> known[kMaxDev][kStepMaxCluster + 1];  // count + 1, 0 = not looked up yet
+  int n = known[dev][C].load(std::memory_order_relaxed);
+  if (n > 0) return n - 1;
+  auto kern = score_step_kernel<__nv_bfloat16, true, true, THREADS>;  // (the others have the same bounds)
+  int clusters = 0;
+  if (C <= 8 || allow_large_clusters<__nv_bfloat16, true, true, THREADS>(dev) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3(THREADS);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();  // a refused size is an answer, not an error to carry
+      clusters = 0;
+    }
+  }
+  known[dev][C].store(clusters + 1, std::memory_order_relaxed);
+  return clusters;
+}
+
+// The most CTAs of THREADS threads per row that still run at once, with the
+// share of the device's CTAs (percent) that clusters of their size can use
+// before some row waits for another's to end: what the sweeps below found.
+template <int THREADS>
+int one_wave_cluster(int dev, int sms, int64_t rows) {
+  const bool large = THREADS == kStepThreadsLarge;
+  const int64_t slots = (int64_t)StepShape<THREADS>::kMinBlocks * sms;
+  for (int C = large ? kStepMaxCluster : kStepSmallCluster; C > 1; --C) {
+    const int share = large ? (C >= 7 ? 82 : C >= 5 ? 87 : C == 4 ? 95 : C == 3 ? 83 : 100) : (C > 10 ? 83 : 90);
+    if (rows * C * 100 <= share * slots && rows <= resident_clusters<THREADS>(dev, C)) return C;
+  }
+  return 1;
+}
+
+// Launch shape of a step with `rows` rows: as many CTAs per row as still run
+// at once, of 512 threads or of 128.  One cluster too many makes the step
+// wait for a second wave: 24 rows in clusters of 9 / 10 / 11 CTAs of 512
+// threads 6.3 / 6.8 / 8.1 us, 108 rows in 10 / 11 of 128 threads 12.4 / 15.7.
+// GB300, us per step of graphs over 151,936 bf16 logits, each size in its
+// best cluster:
+//   rows         8   16   22   28   36   44   52   56   60   68   76   92  108  124  144  152  168
+//   512 threads 4.7  5.4  5.8  6.4  7.0  7.7  8.2  9.4  9.4  9.4 10.9 12.9 13.8 14.1 15.1 15.5 23.3
+//   128 threads 5.4  6.0  6.4  6.7  7.2  8.2  8.8  9.1  9.3  9.6 10.5 11.6 12.4 14.0 16.2 16.6 18.0
+// so 512 threads from 5 CTAs a row on, and below that where 4 or 2 CTAs a row
+// all but fill the device -- not in the masked form, whose stopped rows leave
+// their CTAs idle (62 rows 9.4 / 8.7, 136 rows 13.6 / 13.0).
+struct Shape {
+  int threads, cluster;
+};
+
+Shape choose_shape(int64_t rows, bool compact, int dev, int sms) {
+  const int ft = g_force_threads.load(std::memory_order_relaxed);
+  const int fc = g_force_cluster.load(std::memory_order_relaxed);
+  if (ft > 0 || fc > 0) return Shape{ft > 0 ? ft : kStepThreadsSmall, fc > 0 ? fc : 1};
+  const int large = one_wave_cluster<kStepThreadsLarge>(dev, sms, rows);
+  const int64_t fill = rows * large * 100 / (StepShape<kStepThreadsLarge>::kMinBlocks * (int64_t)sms);
+  if (large > 4 || (compact && ((large == 4 && fill >= 83) || (large == 2 && fill >= 90))))
+    return Shape{kStepThreadsLarge, large};
+  return Shape{kStepThreadsSmall, one_wave_cluster<kStepThreadsSmall>(dev, sms, rows)};
 }
 
 template <typename LT, bool VEC, bool COMPACT, int THREADS>
@@ -393,7 +439,7 @@ cudaError_t launch_score_step(const StepParams& p, int dtype, bool vec, cudaStre
   cudaError_t e = cudaSuccess;
   const int sms = current_device_sms(&dev, &e);
   if (sms <= 0) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
-  Shape sh = choose_shape(p.B, sms);
+  Shape sh = choose_shape(p.B, p.rollout_idx != nullptr, dev, sms);
   // a few whole vectors per thread of a rank at least
   while (sh.cluster > 1 && (int64_t)p.V < (int64_t)sh.threads * sh.cluster) sh.cluster >>= 1;
   if (sh.threads == kStepThreadsLarge && (int64_t)p.V < (int64_t)kStepThreadsLarge * 2) sh.threads = kStepThreadsSmall;
