@@ -401,7 +401,7 @@ int stride_scan_logprobs(const float* logp_s, const float* logp_t, const int64_t
   p.incl = reinterpret_cast<stride::ScanSlot*>(ws + L.incl_off);
   p.timeout_ns = 2000000000ull;
   cudaStream_t st = (cudaStream_t)stream;
-  return stride::launch_scan_logprobs(p, logp_s, logp_t, st) == cudaSuccess ? STRIDE_OK : STRIDE_ERR_CUDA;
+  return stride::launch_scan_logprobs(p, logp_s, logp_t, st, stride::ScanAfter{false, false, false}) == cudaSuccess ? STRIDE_OK : STRIDE_ERR_CUDA;
 }
 
 int stride_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32_t n_tasks, int32_t T_max,

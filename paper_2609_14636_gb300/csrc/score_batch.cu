@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
   }
   // The start of the slice on its way to L2 while the previous kernel ends
   // (the multi-teacher row table is not there yet).
-  if (tid == 0 || (tid == 32 && !p.T_rows)) {
-    const int64_t most = kSplitPrefetch / (2 * (int64_t)gridDim.x);
+  if (blockIdx.x < p.first_wave && (tid == 0 || (tid == 32 && !p.T_rows))) {
+    const int64_t most = kSplitPrefetch / (2 * min((int64_t)gridDim.x, (int64_t)p.first_wave));
     const LT* row = tid == 0 ? srow : reinterpret_cast<const LT*>(p.T) + tile * p.ld;
     prefetch_l2(row + c0, min((int64_t)(c1 - c0) * (int64_t)sizeof(LT), most));
   }
@@ -424,6 +424,7 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
   const bool f_stream = force == kForceStream;
   const bool f_rows = force == kForceRows;
   int C = (f_stream || f_rows) ? 0 : split_cluster(p.n_rows, sms);
+  const bool small = C > 0;  // one wave of the split kernel
   if (f_split) {
     const int want = force - kForceSplit;
     if (want > 0) C = want;
@@ -433,22 +434,29 @@ cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t
   if (C > 0) {
     // (neither kernel needs anything cleared)
     cudaError_t e;
+    BatchParams q = p;
+    q.first_wave = (uint32_t)(kSplitBlocksPerSm * sms);
     if (dtype == STRIDE_DTYPE_BF16)
-      e = vec ? launch_split<__nv_bfloat16, true>(p, C, stream) : launch_split<__nv_bfloat16, false>(p, C, stream);
+      e = vec ? launch_split<__nv_bfloat16, true>(q, C, stream) : launch_split<__nv_bfloat16, false>(q, C, stream);
     else
-      e = vec ? launch_split<float, true>(p, C, stream) : launch_split<float, false>(p, C, stream);
+      e = vec ? launch_split<float, true>(q, C, stream) : launch_split<float, false>(q, C, stream);
     if (e != cudaSuccess) return e;
-    return launch_scan_logprobs(p, p.ws_logp_s, p.ws_logp_t, stream, true);  // the scan on the rows' log-probs
+    return launch_scan_logprobs(p, p.ws_logp_s, p.ws_logp_t, stream, ScanAfter{true, true, small});  // the scan on the rows' log-probs
   }
   // (the persistent kernel counts a row's bytes in 32 bits: rows of up to
   // 2 GB, far beyond any vocabulary, take it)
   const int64_t row_bytes = (int64_t)p.V * (dtype == STRIDE_DTYPE_BF16 ? 2 : 4);
   const bool persistent = row_bytes <= ((int64_t)1 << 31) && !f_rows;
-  // the persistent kernel scans 32-row tiles: one flag line per tile
-  const size_t clear = persistent ? stream_clear_bytes(p.n_rows) : clear_bytes;
-  const cudaError_t ce = launch_clear_workspace(p.ticket, clear, sms, stream);
+  const cudaError_t ce =
+      launch_clear_workspace(p.ticket, persistent ? stream_clear_bytes(p.n_rows, p.V) : clear_bytes, sms, stream);
   if (ce != cudaSuccess) return ce;
-  if (persistent) return launch_score_batch_stream(p, dtype, vec, stream);
+  if (persistent) {
+    BatchParams q = p;
+    q.scan_inside = stream_scan_inside(p.V);
+    const cudaError_t e = launch_score_batch_stream(q, dtype, vec, stream);
+    if (e != cudaSuccess || q.scan_inside) return e;
+    return launch_scan_logprobs(p, p.ws_logp_s, p.ws_logp_t, stream, ScanAfter{true, false, false});
+  }
   const dim3 grid((unsigned)p.n_rows), block(kBatchThreads);
   if (dtype == STRIDE_DTYPE_BF16) {
     if (vec)

@@ -26,12 +26,16 @@
 //   warp 5, scan warp  completes the queued tiles: lookback, turn
 //                      statistics, stop test, carried state.
 //
+// With short rows the row warps only leave the log-probs, and the scan follows
+// as two passes over them (vocab_parallel.cu): scan_inside below.
+//
 // Rows of any length should be bound by HBM.  With one row warp, which also
 // searched the row's turn and formed its scan element, a row cost about 4.7
 // us of dependent latency, more than its bytes take below about 100,000 bf16
-// logits.  GB300, before -> now: 30,011 rows of 32,000 bf16 logits 919 -> 544
-// us (4,180 -> 7,060 GB/s); 3,001 rows of 151,936 267.5 -> 263.5 us; 20,000
-// rows of 151,936 in two windows 1,654 -> 1,645 us (7,390 GB/s): with long
+// logits.  GB300, before -> four row warps and a scan warp -> now: 30,011 rows
+// of 32,000 bf16 logits 919 -> 544 -> 522 us (7,360 GB/s), 3,000 rows 107 ->
+// 85.7 -> 70.0; 3,001 rows of 151,936 267.5 -> 263.5 -> 262.0 us; 20,000 rows
+// of 151,936 in two windows 1,654 -> 1,645 -> 1,636 us (7,430 GB/s): with long
 // rows what was left is the shorter tail of a window's scan.
 //
 // Hand-offs inside the CTA use mbarriers only (no named barriers): full/empty
@@ -353,6 +357,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
 
   if (warp == kScanWarp) {
     // ----------------------------------------------------------- scan warp
+    if (!p.scan_inside) return;
     int running = kRowWarps;
     uint32_t seen = 0;
     for (uint32_t n = 0; running > 0;) {
@@ -431,15 +436,16 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       const stride_row_outputs& o = p.out;
       if (o.logp_s) o.logp_s[w] = lps;
       if (o.logp_t) o.logp_t[w] = lpt;
-      if (o.opd) o.opd[w] = lps - lpt;
+      if (o.opd && p.scan_inside) o.opd[w] = lps - lpt;  // (the scan on log-probs writes it otherwise)
       if (o.lse_s) o.lse_s[w] = lse_s;
       if (o.lse_t) o.lse_t[w] = lse_t;
       if (o.x_s) o.x_s[w] = xs;
       if (o.x_t) o.x_t[w] = xt;
       p.ws_logp_s[w] = lps;
       p.ws_logp_t[w] = lpt;
-      counted = count_in(p.flags + t * kFlagStride + kCounterWord) + 1;
+      if (p.scan_inside) counted = count_in(p.flags + t * kFlagStride + kCounterWord) + 1;
     }
+    if (!p.scan_inside) continue;
     counted = __shfl_sync(0xffffffffu, counted, 0);
     if ((int64_t)counted == min((int64_t)kTileRows, p.n_rows - t * kTileRows)) {
       int i = lane == 0 ? queue_claim(sh) : 0;
@@ -456,7 +462,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     if (lane == 0) *reinterpret_cast<volatile uint32_t*>(&sh.rows_done[warp - 1]) = (uint32_t)(seq / kRowWarps) + 1;
   }
   // nothing more from this row warp (its rows are done: it may wait here)
-  if (lane == 0) {
+  if (lane == 0 && p.scan_inside) {
     int i;
     const uint64_t t0 = globaltimer_ns();
     while ((i = queue_claim(sh)) < 0 && !*abort) {
@@ -470,7 +476,19 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
   }
 }
 
-size_t stream_clear_bytes(int64_t n_rows) {
+// Whether the window's scan runs inside the kernel, behind the data, with a
+// tail of its last tiles' lookups and lookback; or after it, 3 us later at the
+// window's end but without the row warps' counting and publishing, which short
+// rows wait for.  GB300, us inside / after: 3,000 rows of 32,000 bf16 logits
+// 85.7 / 70.0, of 48,000 101.8 / 95.2, of 64,000 118.3 / 120.9, of 151,936
+// 257.8 / 261.2; of 32,000 fp32 127.3 / 119.2, of 48,000 168.8 / 169.4; 30,011
+// rows of 32,000 bf16 546 / 522.
+constexpr int kScanInsideLogits = 56 << 10;
+
+bool stream_scan_inside(int V) { return V >= kScanInsideLogits; }
+
+size_t stream_clear_bytes(int64_t n_rows, int V) {
+  if (!stream_scan_inside(V)) return 256;
   return 256 + (size_t)((n_rows + kTileRows - 1) / kTileRows) * kFlagStride * sizeof(uint32_t);
 }
 

@@ -53,6 +53,8 @@ struct BatchParams {
   float* ws_logp_s;  // per window row, written by the small-window kernel for the tiled scan
   float* ws_logp_t;
   uint64_t timeout_ns;
+  uint32_t first_wave;  // CTAs of the split kernel that are resident from the start
+  int32_t scan_inside;  // the persistent kernel completes its window's scan
 };
 
 struct StepParams {
@@ -138,9 +140,10 @@ cudaError_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, 
 // itself) and launches the batch scoring kernels.
 cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t clear_bytes, cudaStream_t stream);
 cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, bool aligned, cudaStream_t stream);
-// What the persistent kernel needs at zero from the workspace's start: the
-// header (ticket) and one flag line per 32-row tile.
-size_t stream_clear_bytes(int64_t n_rows);
+// Whether that kernel scans its window itself, and what it needs at zero from
+// the workspace's start: the header (ticket), and one flag line per tile.
+bool stream_scan_inside(int V);
+size_t stream_clear_bytes(int64_t n_rows, int V);
 // Zeroes `bytes` (a multiple of 16) at ws as a programmatic dependent of the
 // previous kernel on the stream (it waits for that kernel first).
 cudaError_t launch_clear_workspace(void* ws, size_t bytes, int sms, cudaStream_t stream);
@@ -157,8 +160,14 @@ cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec
 cudaError_t launch_combine_partials(const float* parts, int32_t n_shards, int64_t rows, float* logp_s,
                                     float* logp_t, float* lse_s, float* lse_t, int32_t* dev_status,
                                     cudaStream_t stream);
+// What the scan on log-probs follows: a scoring kernel of this library, which
+// lets its dependents in only after its own wait; one that has checked the
+// layout; one wave of the split kernel (whose window may run as one cluster).
+struct ScanAfter {
+  bool scoring, checked, small;
+};
 cudaError_t launch_scan_logprobs(const BatchParams& p, const float* logp_s, const float* logp_t,
-                                 cudaStream_t stream, bool dependent = false);
+                                 cudaStream_t stream, const ScanAfter& after);
 cudaError_t launch_buffer_record(float* buf_mean, int32_t* buf_n_turns, int32_t n_tasks, int32_t T_max,
                                  const int32_t* task, const int32_t* k0, const stride_turn_stats* ts,
                                  const int32_t* traj_turn_off, int32_t n_traj, int32_t* dev_status,

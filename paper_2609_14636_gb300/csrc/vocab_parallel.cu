@@ -22,7 +22,6 @@
 #include "stride.h"
 #include "stride_device.cuh"
 #include "stride_internal.h"
-#include "warp_tile_scan.cuh"
 
 namespace stride {
 
@@ -585,7 +584,7 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
 // of 256 rows with a row per thread, shared-memory atomics per row and a
 // lookback took 68.8 us (and its 19 MB clear 3.8 us); the passes take about
 // 21.  The whole chain of a training step on given log-probs (state, profile
-// cleared, scan, record, restart choice): 87.8 -> 33.0 us.
+// cleared, scan, record, restart choice): 87.8 -> 28.8 us.
 constexpr int kPassThreads = 256;
 constexpr int kPassWarps = kPassThreads / 32;
 // Up to this many tiles a tile folds its predecessors' aggregates itself
@@ -705,24 +704,104 @@ __device__ __forceinline__ RowMeta no_row() {
   return m;
 }
 
-// A row's stop-sum term: a turn mean's share lpt / n_k is rounded once to
-// fp32 (an fp64 divide is a sequence of fp64 operations; the rounding is 6e-8
-// of the term).
-__device__ __forceinline__ double stop_term(const BatchParams& p, const RowMeta& m, float lpt) {
-  if (p.mode != STRIDE_STOP_TURN_MEAN) return (double)lpt;
-  const int64_t n_k = m.turn_end - m.turn_start;
-  return (double)(lpt / (float)(n_k > 0 ? n_k : 1));
+// What a row's log pi_T is weighed by in the running stop sum: 1, or for turn
+// means 1 / n_k.  EXACT (after a scoring kernel, whose own scan is fp64): once
+// per thread and turn in fp64, by Newton's iteration x + x (1 - n x) from the
+// fp32 quotient, whose error squares twice (2^-24 -> 2^-48 -> fp64).  Else
+// (log-probs as given) n_k itself, by which each log-prob is divided with one
+// fp32 rounding, 6e-8 of the term.
+template <bool EXACT>
+struct StopWeight {
+  using type = double;
+};
+template <>
+struct StopWeight<false> {
+  using type = float;
+};
+
+template <bool EXACT>
+__device__ __forceinline__ typename StopWeight<EXACT>::type stop_weight(const BatchParams& p, const RowMeta& m) {
+  if (p.mode != STRIDE_STOP_TURN_MEAN) return 1;
+  const int64_t n_k = max(m.turn_end - m.turn_start, (int64_t)1);
+  const float f = (float)n_k;
+  if (!EXACT) return f;
+  const double n = (double)n_k;
+  double x = (double)(1.0f / f);
+  x = fma(x, fma(-n, x, 1.0), x);
+  return fma(x, fma(-n, x, 1.0), x);
 }
 
-// The log-probs of the tile's rows, coalesced into shared memory.
-template <int R>
-__device__ __forceinline__ void load_logps(const float* __restrict__ logp_s, const float* __restrict__ logp_t,
-                                           int64_t t0, int n_here, int tid, float* s_ls, float* s_lt) {
+__device__ __forceinline__ double stop_term(float lpt, double weight) { return (double)lpt * weight; }
+__device__ __forceinline__ double stop_term(float lpt, float weight) { return (double)(lpt / weight); }
+
+// A thread's R rows, what the layout alone says of them: rows tid * R + i of
+// the tile.
+constexpr int kRowLive = 1, kRowBad = 2, kRowSeeded = 4, kRowTurnStart = 8;
+
+template <int R, bool EXACT>
+struct Rows {
+  RowMeta first;     // the first row's
+  float lam;         // its trajectory's threshold
+  int what[R];       // kRow bits
+  typename StopWeight<EXACT>::type weight[R];
+  int bin[R];        // the profile's decile
+  float lps[R], lpt[R];
+};
+
+// Fills all but the log-probs; seed(j, z) is told the carried state of every
+// seeded row j (zeros for a bad one).
+template <int R, bool EXACT, int ROWS, typename Seed>
+__device__ __forceinline__ void find_rows(const BatchParams& p, const TileLayout<ROWS>& L, int64_t t0, int n_here, int tid,
+                                          Rows<R, EXACT>& x, Seed&& seed) {
+  RowMeta m = no_row();
+  x.first = m;
+  x.lam = 0.f;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
-    const int j = i * kPassThreads + tid;
-    s_ls[j] = j < n_here ? __ldcg(logp_s + t0 + j) : 0.f;
-    s_lt[j] = j < n_here ? __ldcg(logp_t + t0 + j) : 0.f;
+    const int j = tid * R + i;
+    x.what[i] = 0;
+    x.weight[i] = 1;
+    x.bin[i] = 0;
+    if (j >= n_here) continue;
+    const int64_t r = p.row_begin + t0 + j;
+    seek_row(p, L, r, m);
+    const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
+    const bool fturn = r == m.turn_start;
+    x.what[i] = kRowLive | (m.bad ? kRowBad : 0) | (seeded ? kRowSeeded : 0) | (fturn ? kRowTurnStart : 0);
+    x.weight[i] = i == 0 || seeded || fturn ? stop_weight<EXACT>(p, m) : x.weight[i > 0 ? i - 1 : 0];
+    if (i == 0) {
+      x.first = m;
+      if (!m.bad) x.lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
+    }
+    if (seeded) {
+      ScanSlot z = {0.0, 0.0, 0.0, 0.0};
+      if (!m.bad) {
+        const stride_scan_state* sp = p.state + m.traj;
+        z.c = __ldcg(&sp->cum);
+        if (!fturn) {
+          z.st = __ldcg(&sp->turn_sum_t);
+          z.sd = __ldcg(&sp->turn_sum_d);
+          z.sl = __ldcg(&sp->turn_sum_l);
+        }
+      }
+      seed(j, z);
+    }
+    if (p.profile && !m.bad) {
+      const int64_t pos = r - m.turn_start, n_k = m.turn_end - m.turn_start;  // Observation 1 decile
+      x.bin[i] = n_k < (1 << 28) ? (int)(10u * (unsigned)pos / (unsigned)n_k) : (int)((10 * pos) / n_k);
+    }
+  }
+}
+
+template <int R, bool EXACT>
+__device__ __forceinline__ void load_logps(const float* __restrict__ logp_s, const float* __restrict__ logp_t, int64_t t0,
+                                           int tid, Rows<R, EXACT>& x) {
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int64_t w = t0 + tid * R + i;
+    const bool live = (x.what[i] & kRowLive) != 0;
+    x.lps[i] = live ? __ldcg(logp_s + w) : 0.f;
+    x.lpt[i] = live ? __ldcg(logp_t + w) : 0.f;
   }
 }
 
@@ -739,6 +818,13 @@ __device__ __forceinline__ void sum_add(Sum2& a, float hi, float lo) {
   const float e = (a.hi - (s - b)) + (hi - b);
   a.hi = s;
   a.lo += lo + e;
+}
+
+// The product a b as a pair: exact, or rounded to fp32.
+template <bool EXACT>
+__device__ __forceinline__ Sum2 product(float a, float b) {
+  const float hi = __fmul_rn(a, b);
+  return Sum2{hi, EXACT ? fmaf(a, b, -hi) : 0.f};
 }
 
 __device__ __forceinline__ double sum_value(const Sum2& a) {
@@ -764,6 +850,11 @@ __device__ __forceinline__ Sum2 seg_sum(Sum2 v, int head, int lane) {
     if (lane - d >= head) sum_add(v, o.hi, o.lo);
   }
   return v;
+}
+
+// Highest set bit of m at or below `lane`, -1 if none.
+__device__ __forceinline__ int head_of(unsigned m, int lane) {
+  return 31 - __clz(m & (0xffffffffu >> (31 - lane)));
 }
 
 // A thread's or tile's element without the carried state: sums since the last
@@ -816,6 +907,78 @@ __device__ __forceinline__ int last_thread(unsigned ballot, int lane, int warp, 
   return n;
 }
 
+// The thread's rows as one element.
+template <int R, bool EXACT>
+__device__ __forceinline__ PassElem rows_elem(const Rows<R, EXACT>& x, int tid) {
+  const Sum2 zero = {0.f, 0.f};
+  PassElem e = {0.0, zero, zero, zero, 0, -1};
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int what = x.what[i];
+    if (!(what & kRowLive)) continue;
+    const float nan = __int_as_float(0x7fc00000);
+    const float lps = (what & kRowBad) ? nan : x.lps[i], lpt = (what & kRowBad) ? nan : x.lpt[i], dd = lps - lpt;
+    const bool seeded = (what & kRowSeeded) != 0;
+    if (seeded) {
+      e.c = 0.0;
+      e.seed = tid * R + i;
+      e.flags |= kRestartSum;
+    }
+    if (what & (kRowSeeded | kRowTurnStart)) {
+      e.st = e.sd = e.sl = zero;
+      e.flags = (e.flags & kRestartSum) | kRestartTurn | (seeded ? kFromSeed : 0);
+    }
+    const Sum2 l = product<EXACT>(lps, dd);
+    e.c += stop_term(lpt, x.weight[i]);
+    sum_add(e.st, lpt, 0.f);
+    sum_add(e.sd, dd, 0.f);
+    sum_add(e.sl, l.hi, l.lo);
+  }
+  return e;
+}
+
+// The thread's rows into the CTA's profile: runs of equal deciles summed in
+// registers, neighbouring threads' open runs of one decile together.
+template <int R, bool EXACT>
+__device__ __forceinline__ void rows_profile(const Rows<R, EXACT>& x, int lane, double* s_prof) {
+  const Sum2 zero = {0.f, 0.f};
+  int bin = -1, n = 0;
+  Sum2 d = zero, t = zero;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    if ((x.what[i] & (kRowLive | kRowBad)) != kRowLive) continue;
+    if (x.bin[i] != bin) {
+      if (bin >= 0) {
+        atomicAdd(s_prof + 3 * bin + 0, sum_value(d));
+        atomicAdd(s_prof + 3 * bin + 1, sum_value(t));
+        atomicAdd(s_prof + 3 * bin + 2, (double)n);
+      }
+      bin = x.bin[i];
+      n = 0;
+      d = t = zero;
+    }
+    sum_add(d, x.lps[i] - x.lpt[i], 0.f);
+    sum_add(t, x.lpt[i], 0.f);
+    ++n;
+  }
+  __syncwarp();
+  const int prev = __shfl_up_sync(0xffffffffu, bin, 1);
+  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || bin != prev);
+  const int h = head_of(m_run, lane);
+  d = seg_sum(d, h, lane);
+  t = seg_sum(t, h, lane);
+#pragma unroll
+  for (int k = 1; k < 32; k <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, n, k);
+    if (lane - k >= h) n += o;
+  }
+  if (bin >= 0 && (lane == 31 || ((m_run >> lane) & 2u))) {
+    atomicAdd(s_prof + 3 * bin + 0, sum_value(d));
+    atomicAdd(s_prof + 3 * bin + 1, sum_value(t));
+    atomicAdd(s_prof + 3 * bin + 2, (double)n);
+  }
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -831,81 +994,47 @@ __device__ __forceinline__ ScanSlot load_slot(const ScanSlot* s) {
 
 // First pass: tile t's aggregate in agg[t], its kRestart marks in flags[t],
 // and in incl[w] the carried state of every seeded row w.
-template <int R>
-__global__ void __launch_bounds__(kPassThreads) scan_aggregate_kernel(const BatchParams p,
+template <int R, bool EXACT>
+__global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const BatchParams p,
                                                                      const float* __restrict__ logp_s,
-                                                                     const float* __restrict__ logp_t) {
+                                                                     const float* __restrict__ logp_t, bool early) {
   constexpr int kRows = R * kPassThreads;
   __shared__ TileLayout<kRows> L;
-  __shared__ float s_ls[kRows], s_lt[kRows];
   __shared__ int s_any[2][kPassWarps];
   __shared__ double s_c[kPassWarps], s_base[4];
   __shared__ Sum2 s_open[3][kPassWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // Everything before this kernel is complete past the wait, and only then
-  // may the second pass come in: what it reads before its own wait (the
-  // layout, the log-probs, lambda) is complete too.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t tile = blockIdx.x;
   const int64_t t0 = tile * kRows;
   const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
-  load_logps<R>(logp_s, logp_t, t0, n_here, tid, s_ls, s_lt);
+  Rows<R, EXACT> x;
+  ScanSlot z = {0.0, 0.0, 0.0, 0.0};  // of the thread's last seeded row
   if (tid < 4) s_base[tid] = 0.0;
+  // Everything before this kernel is complete past the wait, and only then
+  // may the second pass come in: what it reads before its own wait (the
+  // layout, the log-probs, lambda) is complete too.  After a scoring kernel
+  // (`early`), which lets this one in once its own predecessors are complete,
+  // all but the log-probs is read while that kernel ends.
+  if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
   stage_layout(p, p.row_begin + t0, n_here, tid, L);
-
-  RowMeta m = no_row();
-  double c = 0.0, seed_c = 0.0, seed_st = 0.0, seed_sd = 0.0, seed_sl = 0.0;
-  Sum2 st = {0.f, 0.f}, sd = st, sl = st;
-  bool has_sum = false, has_turn = false, from_seed = false;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int j = tid * R + i;
-    if (j >= n_here) break;
-    const int64_t r = p.row_begin + t0 + j;
-    seek_row(p, L, r, m);
-    float lps = s_ls[j], lpt = s_lt[j];
-    if (m.bad) lps = lpt = __int_as_float(0x7fc00000);
-    const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
-    const bool fturn = r == m.turn_start;
-    if (seeded) {
-      ScanSlot z = {0.0, 0.0, 0.0, 0.0};
-      if (!m.bad) {
-        const stride_scan_state* sp = p.state + m.traj;
-        z.c = __ldcg(&sp->cum);
-        if (!fturn) {
-          z.st = __ldcg(&sp->turn_sum_t);
-          z.sd = __ldcg(&sp->turn_sum_d);
-          z.sl = __ldcg(&sp->turn_sum_l);
-        }
-      }
-      p.incl[t0 + j] = z;
-      seed_c = z.c;
-      seed_st = z.st;
-      seed_sd = z.sd;
-      seed_sl = z.sl;
-      c = 0.0;
-      has_sum = true;
-    }
-    if (seeded || fturn) {
-      st = sd = sl = Sum2{0.f, 0.f};
-      has_turn = true;
-      from_seed = seeded;
-    }
-    const float dd = lps - lpt;
-    c += stop_term(p, m, lpt);
-    sum_add(st, lpt, 0.f);
-    sum_add(sd, dd, 0.f);
-    sum_add(sl, lps * dd, 0.f);
-  }
+  find_rows<R, EXACT>(p, L, t0, n_here, tid, x, [&](int j, const ScanSlot& s) {
+    z = s;
+    p.incl[t0 + j] = s;
+  });
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  load_logps<R>(logp_s, logp_t, t0, tid, x);
+  const PassElem e = rows_elem<R, EXACT>(x, tid);
+  double c = e.c;
+  Sum2 st = e.st, sd = e.sd, sl = e.sl;
   // only what follows the last restart counts
-  const int own_c = last_thread(__ballot_sync(0xffffffffu, has_sum), lane, warp, s_any[0]);
-  const int own_t = last_thread(__ballot_sync(0xffffffffu, has_turn), lane, warp, s_any[1]);
-  if (tid == own_c) s_base[0] = seed_c;
-  if (tid == own_t && from_seed) {
-    s_base[1] = seed_st;
-    s_base[2] = seed_sd;
-    s_base[3] = seed_sl;
+  const int own_c = last_thread(__ballot_sync(0xffffffffu, (e.flags & kRestartSum) != 0), lane, warp, s_any[0]);
+  const int own_t = last_thread(__ballot_sync(0xffffffffu, (e.flags & kRestartTurn) != 0), lane, warp, s_any[1]);
+  if (tid == own_c) s_base[0] = z.c;
+  if (tid == own_t && (e.flags & kFromSeed)) {
+    s_base[1] = z.st;
+    s_base[2] = z.sd;
+    s_base[3] = z.sl;
   }
   c = warp * 32 + 31 < own_c ? 0.0 : warp_sum(tid >= own_c ? c : 0.0);
   if (tid < own_t) st = sd = sl = Sum2{0.f, 0.f};
@@ -996,7 +1125,7 @@ __global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(ScanSlot* a
 // its first crossing of lambda here.
 struct TrajPart {
   int32_t traj, count, cross_turn;  // traj -1: none
-  float loss;
+  Sum2 loss;
   int64_t cross_row;  // from the trajectory's first row; -1: none
 };
 
@@ -1006,20 +1135,171 @@ __device__ __forceinline__ void record_cross(stride_scan_state* sp, const TrajPa
   sp->stopped = 1;
 }
 
-__device__ __forceinline__ void record_loss(stride_scan_state* sp, float loss, int count) {
-  atomicAdd(&sp->loss, (double)loss);
+__device__ __forceinline__ void record_loss(stride_scan_state* sp, const Sum2& loss, int count) {
+  atomicAdd(&sp->loss, sum_value(loss));
   atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), (unsigned long long)count);
 }
 
+// Completes the thread's rows, given the exclusive prefix of its rows inside
+// the tile, the tile's (pre) and the carried state of the tile's seeded rows
+// (seed(j), which covers excl.seed too).
+template <int R, bool EXACT, int ROWS, typename Seed>
+__device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLayout<ROWS>& L, int64_t t0, int tid,
+                                              const Rows<R, EXACT>& x, const PassElem& excl, const double* pre, Seed&& seed) {
+  const int lane = tid & 31;
+  const float nan = __int_as_float(0x7fc00000);
+  const Sum2 zero = {0.f, 0.f};
+  ScanSlot z = {0.0, 0.0, 0.0, 0.0};  // the last seeded row's before this thread
+  if (excl.seed >= 0 && (x.what[0] & kRowLive)) z = seed(excl.seed);
+  double c = (excl.seed >= 0 ? z.c : pre[0]) + excl.c;
+  double b_st = pre[1], b_sd = pre[2], b_sl = pre[3];  // what the open turn brought into the tile
+  if (excl.flags & kRestartTurn) {
+    const bool from = (excl.flags & kFromSeed) != 0;
+    b_st = from ? z.st : 0.0;
+    b_sd = from ? z.sd : 0.0;
+    b_sl = from ? z.sl : 0.0;
+  }
+  Sum2 st = excl.st, sd = excl.sd, sl = excl.sl;
+  TrajPart part = {-1, 0, 0, zero, -1};
+  bool kept = false;  // in turn mode the same for all of a turn's rows
+  float lam = x.lam;
+  RowMeta m = x.first;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int what = x.what[i];
+    if (!(what & kRowLive)) break;
+    const int j = tid * R + i;
+    const int64_t w = t0 + j, r = p.row_begin + w;
+    if (what & kRowBad) {
+      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
+      if (p.out.logp_t) p.out.logp_t[w] = nan;
+      if (p.out.opd) p.out.opd[w] = nan;
+      c = (double)nan;  // nothing after a bad row is meaningful
+      continue;
+    }
+    if (i > 0) seek_row(p, L, r, m);
+    const float lps = x.lps[i], lpt = x.lpt[i], dd = lps - lpt;
+    const Sum2 l = product<EXACT>(lps, dd);
+    const bool seeded = (what & kRowSeeded) != 0, fturn = (what & kRowTurnStart) != 0;
+    stride_scan_state* sp = p.state + m.traj;
+    if (seeded || fturn) {
+      st = sd = sl = zero;
+      b_st = b_sd = b_sl = 0.0;
+    }
+    if (seeded) {
+      const ScanSlot own = seed(j);
+      c = own.c;
+      b_st = own.st;
+      b_sd = own.sd;
+      b_sl = own.sl;
+    }
+    if (part.traj != m.traj) {  // a new trajectory: the last one's share is complete
+      if (part.traj >= 0) {
+        if (part.cross_row >= 0) record_cross(p.state + part.traj, part);
+        if (part.count > 0) record_loss(p.state + part.traj, part.loss, part.count);
+      }
+      if (i > 0) lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
+      part = TrajPart{m.traj, 0, 0, zero, -1};
+    }
+    const bool turn_last = r == m.turn_end - 1;
+    const bool token_sum = p.mode == STRIDE_STOP_TOKEN_SUM;
+    const int64_t n_k = m.turn_end - m.turn_start;
+    // retained unless the rule fired before the row (row_scan.cuh); a
+    // trajectory's first token or turn always is
+    if (token_sum) {
+      kept = r == m.traj_start || !(c < (double)lam);
+    } else if (i == 0 || seeded || fturn) {
+      const double before = EXACT ? c - (b_st + sum_value(st)) * x.weight[i]
+                                  : c - (double)(((float)b_st + st.hi) / x.weight[i]);
+      kept = m.local_turn == 0 || !(before < (double)lam);
+    }
+    c += stop_term(lpt, x.weight[i]);
+    sum_add(st, lpt, 0.f);
+    sum_add(sd, dd, 0.f);
+    sum_add(sl, l.hi, l.lo);
+    if (p.out.opd) p.out.opd[w] = dd;
+    if (kept) {
+      sum_add(part.loss, l.hi, l.lo);
+      ++part.count;
+    }
+    if ((token_sum || turn_last) && part.cross_row < 0 && c < (double)lam) {
+      part.cross_row = r - m.traj_start;
+      part.cross_turn = m.local_turn;
+    }
+    const bool last = r == m.traj_end - 1 || r == p.row_end - 1;
+    if (turn_last || last) {
+      const double t_st = b_st + sum_value(st), t_sd = b_sd + sum_value(sd), t_sl = b_sl + sum_value(sl);
+      if (turn_last && p.turn_stats) {
+        stride_turn_stats ts;
+        ts.sum_t = t_st;
+        ts.sum_d = t_sd;
+        ts.sum_l = t_sl;
+        ts.cum = c;
+        ts.mean_t = (float)(t_st / (double)n_k);
+        ts.n = (int32_t)n_k;
+        p.turn_stats[m.turn] = ts;
+      }
+      if (last) {
+        sp->cum = c;
+        sp->turn_sum_t = turn_last ? 0.0 : t_st;
+        sp->turn_sum_d = turn_last ? 0.0 : t_sd;
+        sp->turn_sum_l = turn_last ? 0.0 : t_sl;
+        sp->rows_seen = r - m.traj_start + 1;
+        sp->turn_idx = turn_last ? m.local_turn + 1 : m.local_turn;
+        sp->turn_tokens = turn_last ? 0 : (int32_t)(r - m.turn_start + 1);
+      }
+    }
+  }
+
+  // the trajectories' records: neighbouring threads of one trajectory together
+  // (the lowest crossing, the sum of the losses)
+  __syncwarp();
+  const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
+  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
+  const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
+  const int h = head_of(m_run, lane);
+  const Sum2 loss = seg_sum(part.loss, h, lane);
+  int count = part.count;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, count, d);
+    if (lane - d >= h) count += n;
+  }
+  if (part.traj >= 0) {
+    stride_scan_state* sp = p.state + part.traj;
+    const unsigned mine = (0xffffffffu >> (31 - lane)) & (0xffffffffu << h);
+    if (part.cross_row >= 0 && __ffs(m_cross & mine) - 1 == lane) record_cross(sp, part);
+    if (count > 0 && (lane == 31 || ((m_run >> lane) & 2u))) record_loss(sp, loss, count);
+  }
+}
+
+// Layout checks, spread over every thread of a grid of n_tiles CTAs.
+__device__ __forceinline__ void check_layout(const BatchParams& p, int64_t tile, int64_t n_tiles, int tid) {
+  bool bad = false;
+  const int64_t stride = n_tiles * kPassThreads;
+  const int64_t at = tile * kPassThreads + tid;
+  for (int64_t k = at; k < p.n_turns; k += stride) bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
+  for (int64_t i = at; i < p.n_traj; i += stride) {
+    const int32_t a = __ldg(p.traj_turn_off + i), b = __ldg(p.traj_turn_off + i + 1);
+    if (a < 0 || b < a || b > p.n_turns) {
+      bad = true;
+    } else {
+      bad |= __ldg(p.turn_row_off + a) != __ldg(p.traj_row_off + i);
+      bad |= __ldg(p.turn_row_off + b) != __ldg(p.traj_row_off + i + 1);
+    }
+  }
+  if (bad) set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+}
+
 // Second pass.
-template <int R>
+template <int R, bool EXACT>
 __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const BatchParams p,
-                                                                    const float* __restrict__ logp_s,
-                                                                    const float* __restrict__ logp_t, int64_t n_tiles,
-                                                                    bool prefixed, bool validate) {
+                                                                       const float* __restrict__ logp_s,
+                                                                       const float* __restrict__ logp_t, int64_t n_tiles,
+                                                                       bool prefixed, bool validate) {
   constexpr int kRows = R * kPassThreads;
   __shared__ TileLayout<kRows> L;
-  __shared__ float s_ls[kRows], s_lt[kRows];
   __shared__ PassElem s_tot[kPassWarps], s_wpre[kPassWarps];
   __shared__ int s_near[2][kPassWarps];
   __shared__ double s_fold[4][kPassWarps];
@@ -1031,93 +1311,21 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
   const int64_t tile = blockIdx.x;
   const int64_t t0 = tile * kRows;
   const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
-  const float nan = __int_as_float(0x7fc00000);
-  load_logps<R>(logp_s, logp_t, t0, n_here, tid, s_ls, s_lt);
   if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
   if (tid < 4) s_pre[tid] = 0.0;
   stage_layout(p, p.row_begin + t0, n_here, tid, L);
-
-  // ---- this thread's rows: their element, and the profile
-  RowMeta m = no_row();
+  Rows<R, EXACT> x;
+  find_rows<R, EXACT>(p, L, t0, n_here, tid, x, [](int, const ScanSlot&) {});  // (the first pass set the states aside)
+  load_logps<R>(logp_s, logp_t, t0, tid, x);
+  if (tid == 0) s_needs = !(x.what[0] & kRowSeeded);
+  if (p.profile) rows_profile<R>(x, lane, s_prof);
   const Sum2 zero = {0.f, 0.f};
   const PassElem id = {0.0, zero, zero, zero, 0, -1};
-  PassElem x = id;
-  RowMeta first = m;
-  float lam = 0.f;
-  int bin = -1, bin_n = 0;  // the open run of equal deciles
-  Sum2 bin_d = zero, bin_t = zero;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int j = tid * R + i;
-    if (j >= n_here) break;
-    const int64_t r = p.row_begin + t0 + j;
-    seek_row(p, L, r, m);
-    if (i == 0) {
-      first = m;
-      if (!m.bad) lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
-    }
-    const float lps = m.bad ? nan : s_ls[j], lpt = m.bad ? nan : s_lt[j];
-    const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
-    const bool fturn = r == m.turn_start;
-    if (j == 0) s_needs = seeded ? 0 : 1;
-    if (seeded) {
-      x.c = 0.0;
-      x.seed = j;
-      x.flags |= kRestartSum;
-    }
-    if (seeded || fturn) {
-      x.st = x.sd = x.sl = zero;
-      x.flags = (x.flags & kRestartSum) | kRestartTurn | (seeded ? kFromSeed : 0);
-    }
-    const float dd = lps - lpt;
-    x.c += stop_term(p, m, lpt);
-    sum_add(x.st, lpt, 0.f);
-    sum_add(x.sd, dd, 0.f);
-    sum_add(x.sl, lps * dd, 0.f);
-    if (p.profile && !m.bad) {
-      const int64_t pos = r - m.turn_start, n_k = m.turn_end - m.turn_start;
-      const int b = n_k < (1 << 28) ? (int)(10u * (unsigned)pos / (unsigned)n_k) : (int)((10 * pos) / n_k);  // Observation 1 decile
-      if (b != bin) {
-        if (bin >= 0) {
-          atomicAdd(s_prof + 3 * bin + 0, sum_value(bin_d));
-          atomicAdd(s_prof + 3 * bin + 1, sum_value(bin_t));
-          atomicAdd(s_prof + 3 * bin + 2, (double)bin_n);
-        }
-        bin = b;
-        bin_n = 0;
-        bin_d = bin_t = zero;
-      }
-      sum_add(bin_d, dd, 0.f);
-      sum_add(bin_t, lpt, 0.f);
-      ++bin_n;
-    }
-  }
-  if (p.profile) {
-    // the threads' open runs, neighbours of one decile together
-    const int prev = __shfl_up_sync(0xffffffffu, bin, 1);
-    const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || bin != prev);
-    const int h = head_of(m_run, lane);
-    const Sum2 sum_d = seg_sum(bin_d, h, lane), sum_t = seg_sum(bin_t, h, lane);
-    int n = bin_n;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int o = __shfl_up_sync(0xffffffffu, n, d);
-      if (lane - d >= h) n += o;
-    }
-    if (bin >= 0 && (lane == 31 || ((m_run >> lane) & 2u))) {
-      atomicAdd(s_prof + 3 * bin + 0, sum_value(sum_d));
-      atomicAdd(s_prof + 3 * bin + 1, sum_value(sum_t));
-      atomicAdd(s_prof + 3 * bin + 2, (double)n);
-    }
-  }
   PassElem incl, excl;
-  block_scan<kPassWarps>(x, id, lane, warp, s_tot, s_wpre, incl, excl);
+  block_scan<kPassWarps>(rows_elem<R, EXACT>(x, tid), id, lane, warp, s_tot, s_wpre, incl, excl);
 
   // ---- the first pass's results
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int32_t seed0 = excl.seed;  // the last seeded row before this thread's
-  ScanSlot seed = {0.0, 0.0, 0.0, 0.0};
-  if (seed0 >= 0 && tid * R < n_here) seed = load_slot(p.incl + t0 + seed0);
   if (s_needs && prefixed) {
     if (tid == 0) {
       const ScanSlot a = load_slot(p.agg + tile);
@@ -1182,149 +1390,9 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
     }
   }
   __syncthreads();
-
-  // ---- complete the rows
-  double c = (seed0 >= 0 ? seed.c : s_pre[0]) + excl.c;
-  double b_st = s_pre[1], b_sd = s_pre[2], b_sl = s_pre[3];  // what the open turn brought into the tile
-  if (excl.flags & kRestartTurn) {
-    const bool from = (excl.flags & kFromSeed) != 0;
-    b_st = from ? seed.st : 0.0;
-    b_sd = from ? seed.sd : 0.0;
-    b_sl = from ? seed.sl : 0.0;
-  }
-  Sum2 st = excl.st, sd = excl.sd, sl = excl.sl;
-  TrajPart part = {-1, 0, 0, 0.f, -1};
-  bool kept = false;  // in turn mode the same for all of a turn's rows
-  m = first;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int j = tid * R + i;
-    if (j >= n_here) break;
-    const int64_t w = t0 + j, r = p.row_begin + w;
-    if (i > 0) seek_row(p, L, r, m);
-    if (m.bad) {
-      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
-      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
-      if (p.out.logp_t) p.out.logp_t[w] = nan;
-      if (p.out.opd) p.out.opd[w] = nan;
-      c = (double)nan;  // nothing after a bad row is meaningful
-      continue;
-    }
-    const float lps = s_ls[j], lpt = s_lt[j], dd = lps - lpt, esl = lps * dd;
-    const bool seeded = w == 0 || r == m.traj_start, fturn = r == m.turn_start;
-    stride_scan_state* sp = p.state + m.traj;
-    if (seeded || fturn) {
-      st = sd = sl = zero;
-      b_st = b_sd = b_sl = 0.0;
-    }
-    if (seeded) {
-      const ScanSlot z = load_slot(p.incl + w);
-      c = z.c;
-      b_st = z.st;
-      b_sd = z.sd;
-      b_sl = z.sl;
-    }
-    if (part.traj != m.traj) {  // a new trajectory: the last one's share is complete
-      if (part.traj >= 0) {
-        if (part.cross_row >= 0) record_cross(p.state + part.traj, part);
-        if (part.count > 0) record_loss(p.state + part.traj, part.loss, part.count);
-        lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
-      } else if (i > 0) {
-        lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
-      }
-      part = TrajPart{m.traj, 0, 0, 0.f, -1};
-    }
-    const bool turn_last = r == m.turn_end - 1;
-    const bool token_sum = p.mode == STRIDE_STOP_TOKEN_SUM;
-    const int64_t n_k = m.turn_end - m.turn_start;
-    // retained unless the rule fired before the row (row_scan.cuh); a
-    // trajectory's first token or turn always is
-    if (token_sum) {
-      kept = r == m.traj_start || !(c < (double)lam);
-    } else if (i == 0 || seeded || fturn) {
-      const double before = c - (double)(((float)b_st + st.hi) / (float)n_k);
-      kept = m.local_turn == 0 || !(before < (double)lam);
-    }
-    c += stop_term(p, m, lpt);
-    sum_add(st, lpt, 0.f);
-    sum_add(sd, dd, 0.f);
-    sum_add(sl, esl, 0.f);
-    if (p.out.opd) p.out.opd[w] = dd;
-    if (kept) {
-      part.loss += esl;
-      ++part.count;
-    }
-    if ((token_sum || turn_last) && part.cross_row < 0 && c < (double)lam) {
-      part.cross_row = r - m.traj_start;
-      part.cross_turn = m.local_turn;
-    }
-    if (turn_last || r == m.traj_end - 1 || r == p.row_end - 1) {
-      const double t_st = b_st + sum_value(st), t_sd = b_sd + sum_value(sd), t_sl = b_sl + sum_value(sl);
-      if (turn_last && p.turn_stats) {
-        stride_turn_stats ts;
-        ts.sum_t = t_st;
-        ts.sum_d = t_sd;
-        ts.sum_l = t_sl;
-        ts.cum = c;
-        ts.mean_t = (float)(t_st / (double)n_k);
-        ts.n = (int32_t)n_k;
-        p.turn_stats[m.turn] = ts;
-      }
-      if (r == m.traj_end - 1 || r == p.row_end - 1) {
-        sp->cum = c;
-        sp->turn_sum_t = turn_last ? 0.0 : t_st;
-        sp->turn_sum_d = turn_last ? 0.0 : t_sd;
-        sp->turn_sum_l = turn_last ? 0.0 : t_sl;
-        sp->rows_seen = r - m.traj_start + 1;
-        sp->turn_idx = turn_last ? m.local_turn + 1 : m.local_turn;
-        sp->turn_tokens = turn_last ? 0 : (int32_t)(r - m.turn_start + 1);
-      }
-    }
-  }
-
-  // ---- the trajectories' records: neighbouring threads of one trajectory
-  //      together (the lowest crossing, the sum of the losses)
-  __syncwarp();
-  const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
-  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
-  const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
-  const int h = head_of(m_run, lane);
-  float loss = part.loss;
-  int count = part.count;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const float o = __shfl_up_sync(0xffffffffu, loss, d);
-    const int n = __shfl_up_sync(0xffffffffu, count, d);
-    if (lane - d >= h) {
-      loss += o;
-      count += n;
-    }
-  }
-  if (part.traj >= 0) {
-    stride_scan_state* sp = p.state + part.traj;
-    const unsigned mine = (0xffffffffu >> (31 - lane)) & (0xffffffffu << h);
-    if (part.cross_row >= 0 && __ffs(m_cross & mine) - 1 == lane) record_cross(sp, part);
-    if (count > 0 && (lane == 31 || ((m_run >> lane) & 2u))) record_loss(sp, loss, count);
-  }
+  complete_rows<R, EXACT>(p, L, t0, tid, x, excl, s_pre, [&](int j) { return load_slot(p.incl + t0 + j); });
   if (p.profile && tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
-
-  // Layout checks, spread over every thread of the launch, unless the kernel
-  // that wrote the log-probs made them.
-  if (!validate) return;
-  bool bad = false;
-  const int64_t stride = n_tiles * kPassThreads;
-  const int64_t at = tile * kPassThreads + tid;
-  for (int64_t k = at; k < p.n_turns; k += stride) bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
-  for (int64_t i = at; i < p.n_traj; i += stride) {
-    const int32_t a = __ldg(p.traj_turn_off + i), b = __ldg(p.traj_turn_off + i + 1);
-    if (a < 0 || b < a || b > p.n_turns) {
-      bad = true;
-    } else {
-      bad |= __ldg(p.turn_row_off + a) != __ldg(p.traj_row_off + i);
-      bad |= __ldg(p.turn_row_off + b) != __ldg(p.traj_row_off + i + 1);
-    }
-  }
-  if (bad) set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+  if (validate) check_layout(p, tile, n_tiles, tid);
 }
 
 cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec, int64_t ld,
@@ -1383,33 +1451,33 @@ bool scan_cluster_fits(int dev, int n, cudaStream_t stream) {
 
 namespace {
 
-template <int R>
-cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float* logp_t, bool validate,
+template <int R, bool EXACT>
+cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float* logp_t, const ScanAfter& after,
                           cudaStream_t stream) {
   constexpr int kRows = R * kPassThreads;
   const int64_t n_tiles = (p.n_rows + kRows - 1) / kRows;
   const bool prefixed = n_tiles > kDirectTiles;
-  cudaError_t e = launch_dependent(scan_aggregate_kernel<R>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t);
+  cudaError_t e =
+      launch_dependent(scan_aggregate_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, after.scoring);
   if (e == cudaSuccess && prefixed)
     e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, p.agg, p.flags, n_tiles);
   if (e == cudaSuccess)
-    e = launch_dependent(scan_complete_kernel<R>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, n_tiles,
-                         prefixed, validate);
+    e = launch_dependent(scan_complete_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, n_tiles,
+                         prefixed, !after.checked);
   return e;
 }
 
 }  // namespace
 
 cudaError_t launch_scan_logprobs(const BatchParams& p, const float* logp_s, const float* logp_t,
-                                 cudaStream_t stream, bool dependent) {
+                                 cudaStream_t stream, const ScanAfter& after) {
   int dev = 0;
   cudaError_t qe = cudaSuccess;
   const int sms = current_device_sms(&dev, &qe);
   if (sms <= 0) return qe != cudaSuccess ? qe : cudaErrorInvalidDevice;
-  // a small window after the small-window kernel (which checks the layout
-  // itself): one cluster
+  // a small window: one cluster
   const int64_t cluster_tiles = (p.n_rows + kClusterTileRows - 1) / kClusterTileRows;
-  if (dependent && cluster_tiles <= kClusterMaxTiles && scan_cluster_fits(dev, (int)cluster_tiles, stream)) {
+  if (after.small && cluster_tiles <= kClusterMaxTiles && scan_cluster_fits(dev, (int)cluster_tiles, stream)) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cluster_tiles);
     cfg.blockDim = dim3(kClusterTileRows);
@@ -1428,11 +1496,15 @@ cudaError_t launch_scan_logprobs(const BatchParams& p, const float* logp_s, cons
     return e != cudaSuccess ? e : cudaGetLastError();
   }
   // A row per thread while its tiles are one per SM, two from there on.
-  // 148,909 rows as above (init to restart choice), 1 / 2 / 4 rows per
-  // thread: 34.9 / 32.9 / 35.1 us (one token-sum trajectory: 40.3 / 32.4 /
-  // 30.4); 38,000 rows: 24.7 each way.
-  if (p.n_rows <= (int64_t)sms * kPassThreads) return launch_passes<1>(p, logp_s, logp_t, !dependent, stream);
-  return launch_passes<2>(p, logp_s, logp_t, !dependent, stream);
+  // 148,909 rows as above (state to restart choice), 1 / 2 / 4 per thread:
+  // 34.9 / 32.9 / 35.1 us (one token-sum trajectory: 40.3 / 32.4 / 30.4);
+  // 38,000 rows: 24.7 each way.
+  const bool one = p.n_rows <= (int64_t)sms * kPassThreads;
+  if (after.scoring)
+    return one ? launch_passes<1, true>(p, logp_s, logp_t, after, stream)
+               : launch_passes<2, true>(p, logp_s, logp_t, after, stream);
+  return one ? launch_passes<1, false>(p, logp_s, logp_t, after, stream)
+             : launch_passes<2, false>(p, logp_s, logp_t, after, stream);
 }
 
 }  // namespace stride

@@ -1,8 +1,8 @@
-"""GPU parity of the persistent kernel's 32-row scan tiles at the sizes where
-they can go wrong: windows that end inside, at and just past a tile, turns of
-one row (a tile full of turns), runs of more empty trajectories than a tile
-stages, and very short rows (tiles complete faster than the scan warp takes
-them, so its queue fills).
+"""GPU parity of the persistent kernel's scan at the sizes where it can go
+wrong: windows that end inside, at and just past a tile, turns of one row (a
+tile full of turns), runs of more empty trajectories than a tile stages, and
+very short rows.  From 57,344 logits on the scan runs inside the kernel, in
+32-row tiles; below that it follows in two passes.
 
 And rows at every alignment through the same kernel: S and T starting on
 different element offsets from a 16-byte boundary, strides that move the
@@ -45,7 +45,8 @@ def _layout(rng, rows):
 
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("rows, V", [(1, 64), (31, 64), (32, 64), (33, 64), (95, 264), (1024, 264), (1057, 64),
-                                     (20_000, 16)])
+                                     (20_000, 16), (1, 57_344), (31, 57_344), (33, 57_343), (33, 57_344),
+                                     (95, 57_344), (1057, 57_344)])
 def test_warp_tiles(stride, rows, V, mode):
     rng = np.random.default_rng(rows * 2 + mode)
     lay = _layout(rng, rows)
