@@ -150,7 +150,7 @@ int prepare_batch(stride::BatchParams& p, stride::BatchWorkspaceLayout& L, const
   p.incl = reinterpret_cast<stride::ScanSlot*>(ws + L.incl_off);
   p.ws_logp_s = reinterpret_cast<float*>(ws + L.logp_s_off);
   p.ws_logp_t = reinterpret_cast<float*>(ws + L.logp_t_off);
-  p.timeout_ns = 2000000000ull;  // 2 s bound on any single device-side wait
+  p.timeout_ns = stride::kWaitTimeoutNs;
   return STRIDE_OK;
 }
 
@@ -399,7 +399,7 @@ int stride_scan_logprobs(const float* logp_s, const float* logp_t, const int64_t
   p.flags = reinterpret_cast<uint32_t*>(ws + L.flags_off);
   p.agg = reinterpret_cast<stride::ScanSlot*>(ws + L.agg_off);
   p.incl = reinterpret_cast<stride::ScanSlot*>(ws + L.incl_off);
-  p.timeout_ns = 2000000000ull;
+  p.timeout_ns = stride::kWaitTimeoutNs;
   cudaStream_t st = (cudaStream_t)stream;
   return stride::launch_scan_logprobs(p, logp_s, logp_t, st, stride::ScanAfter{false, false, false}) == cudaSuccess ? STRIDE_OK : STRIDE_ERR_CUDA;
 }

@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
       uint32_t it = 0;  // stages issued
       int64_t seq = 0;  // rows started by this CTA
       bool ok = true;
-      uint32_t t = atomicAdd(p.ticket, 1u);
+      // (a shard pass has no workspace, hence no ticket: rows in turn)
+      uint32_t t = p.partials ? blockIdx.x : atomicAdd(p.ticket, 1u);
       while ((int64_t)t < p.n_rows) {
         const int q = (int)(seq % kSlots);
         const uint32_t use = (uint32_t)(seq / kSlots);
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
         const unsigned char* src_t = reinterpret_cast<const unsigned char*>(trow + body_t.head);
         for (uint32_t c = 0; c < n_chunks; ++c) {
           // the next row's ticket arrives while the last chunk waits for its stage
-          if (c == n_chunks - 1) t = atomicAdd(p.ticket, 1u);
+          if (c == n_chunks - 1) t = p.partials ? t + gridDim.x : atomicAdd(p.ticket, 1u);
           const int s = (int)(it % kStages);
           const uint32_t k = it / kStages;
           if (k > 0 && !mbar_wait(&sh.empty[s], (k - 1) & 1u, tmo, abort)) {
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     if (w < 0) break;
     const LT* srow = reinterpret_cast<const LT*>(p.S) + w * p.ld;
     const LT* trow = teacher_row<LT>(p, w);
-    const int32_t y = __ldg(p.tokens + w);
+    const int64_t y = (int64_t)__ldg(p.tokens + w) - p.col0;
     const bool y_ok = y >= 0 && y < p.V;
     float xs = nan, xt = nan;
     if (y_ok) {
@@ -427,6 +428,15 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     if (in_s) lse_one(es, mS, sS);
     if (in_t) lse_one(et, mT, sT);
     warp_merge2(mS, sS, mT, sT);
+    if (p.partials) {
+      if (lane == 0) {
+        float2* o = reinterpret_cast<float2*>(p.partials + w * 6);
+        o[0] = make_float2(mS, sS);
+        o[1] = make_float2(mT, sT);
+        o[2] = make_float2(xs, xt);
+      }
+      continue;
+    }
     uint32_t counted = 0;
     const int64_t t = w / kTileRows;
     if (lane == 0) {

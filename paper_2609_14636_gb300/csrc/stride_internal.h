@@ -22,6 +22,8 @@ struct alignas(32) ScanSlot {
 // 1,024 rows scored 3-12 % faster with the flags spread out.
 constexpr int kFlagStride = 32;
 
+constexpr uint64_t kWaitTimeoutNs = 2000000000ull;  // bound on any single device-side wait
+
 struct BatchParams {
   const void* S;
   const void* T;
@@ -55,6 +57,10 @@ struct BatchParams {
   uint64_t timeout_ns;
   uint32_t first_wave;  // CTAs of the split kernel that are resident from the start
   int32_t scan_inside;  // the persistent kernel completes its window's scan
+  // A shard pass through the persistent kernel: per row (m, s) of S and T and
+  // the token's logits, its column counted from col0; nothing else is written.
+  float* partials;
+  int64_t col0;
 };
 
 struct StepParams {

@@ -1395,6 +1395,19 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
   if (validate) check_layout(p, tile, n_tiles, tid);
 }
 
+// Whether a shard pass takes the persistent kernel (score_batch_stream.cu)
+// instead of one CTA per row: rows long enough that its ring pays (its rate is
+// higher, a row's end costs it more), or so few that one CTA each leaves most
+// of the device idle.  GB300, us for the passes, merge and scan, one CTA per
+// row / persistent: shard rows of 152 KB (75,968 bf16) 400 rows 64 / 54, 3,000
+// 286 / 271, 10,000 860 / 843; (37,984 fp32) 6,000 rows 1,046 / 1,012; of 76 KB
+// 400 rows 73 / 63, 800 98 / 102, 6,000 522 / 532; of 38 KB 400 rows 85 / 78,
+// 800 115 / 120; of 16 KB 64 rows 45 / 49, 6,000 275 / 337.
+static bool shard_pass_persistent(int64_t rows, int dtype, int32_t V, int sms) {
+  const int64_t bytes = (int64_t)V * (dtype == STRIDE_DTYPE_BF16 ? 2 : 4);
+  return bytes <= ((int64_t)1 << 31) && (bytes >= (128 << 10) || (bytes >= (32 << 10) && rows <= 3 * (int64_t)sms));
+}
+
 cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec, int64_t ld,
                                int32_t V_shard, int64_t col0, const int32_t* tokens, int64_t rows,
                                float* partials, int32_t* dev_status, cudaStream_t stream) {
@@ -1402,6 +1415,20 @@ cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec
   cudaError_t qe = cudaSuccess;
   const int sms = current_device_sms(&dev, &qe);
   if (sms <= 0) return qe != cudaSuccess ? qe : cudaErrorInvalidDevice;
+  if (shard_pass_persistent(rows, dtype, V_shard, sms) && (reinterpret_cast<uintptr_t>(partials) & 7u) == 0) {
+    BatchParams q = {};
+    q.S = S;
+    q.T = T;
+    q.ld = ld;
+    q.V = V_shard;
+    q.tokens = tokens;
+    q.n_rows = rows;
+    q.dev_status = dev_status;
+    q.partials = partials;
+    q.col0 = col0;
+    q.timeout_ns = kWaitTimeoutNs;
+    return launch_score_batch_stream(q, dtype, vec, stream);
+  }
   const PartialParams p{S, T, ld, V_shard, col0, 0, tokens, rows, partials, dev_status,
                         (int64_t)STRIDE_PARTIAL_MIN_BLOCKS * sms};
   auto* kern = dtype == STRIDE_DTYPE_BF16

@@ -1,8 +1,8 @@
 """The streaming loop's end: rows whose share per thread is any number of
 16-byte vectors around its batches of four, through the three kernels that
-stream with it (decode step, small windows, shard pass), and decode steps of
-row counts at the edges of the launch-shape rule.  Against the log-softmax in
-64 bits."""
+stream with it (decode step, small windows, shard pass), decode steps of row counts
+at the edges of the launch-shape rule, and shard passes on both sides of the
+persistent kernel's.  Against the log-softmax in 64 bits."""
 from __future__ import annotations
 
 import numpy as np
@@ -105,3 +105,29 @@ def test_every_launch_shape(stride, compact, V):
     S, T, tok = _logits(max(rows), V, False, V)
     for n in rows:
         _step(stride, S[:n], T[:n], tok[:n], compact)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("rows", [1, 7, 456, 457, 700])
+@pytest.mark.parametrize("kb", [32, 128])
+def test_shard_pass_routes(stride, rows, kb, f32):
+    """Shard rows around the sizes from which the persistent kernel takes the pass, aligned and not, the second shard
+    with and without the row's token."""
+    import torch
+
+    W = kb * 1024 // (4 if f32 else 2)
+    for w0, w1 in ((W, W), (W + 3, W - 1)):
+        S, T, tok = _logits(rows, w0 + w1, f32, rows + w1)
+        parts = torch.full((2, rows, 6), -7.0, device="cuda")
+        for k, (a, b) in enumerate(((0, w0), (w0, w0 + w1))):
+            stride.stride_partial_lse(S[:, a:b], T[:, a:b], tok, a, parts[k], V_shard=b - a)
+        mine = [(tok < w0).cpu().numpy(), (tok >= w0).cpu().numpy()]
+        for k in range(2):
+            assert np.array_equal(~np.isnan(parts[k, :, 4].cpu().numpy()), mine[k])
+            assert np.array_equal(~np.isnan(parts[k, :, 5].cpu().numpy()), mine[k])
+        o = [torch.empty(rows, device="cuda") for _ in range(2)]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        stride.stride_combine_partials(parts, *o, dev_status=status)
+        assert int(status) == 0
+        _close(o[0], S, tok)
+        _close(o[1], T, tok)
