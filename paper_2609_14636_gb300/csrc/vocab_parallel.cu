@@ -155,26 +155,6 @@ __global__ void combine_kernel(const float* __restrict__ parts, int32_t n_shards
   if (lse_t) lse_t[r] = lt;
 }
 
-// A small window's scan after the small-window kernel, one tile of TILE
-// consecutive rows per CTA (one row per thread) and all tiles one
-// thread-block cluster:
-//   1. the CTA stages the offsets of the tile's turns and trajectories in
-//      shared memory and every thread finds its row's there;
-//   2. each row's element: the stop-sum term, log pi_T, d, logp_S * d, and
-//      two restart marks -- the open-turn sums restart at a turn's first row,
-//      the running sum at a seeded row (a trajectory's first row, or the
-//      window's), whose element already holds the carried state;
-//   3. a segmented inclusive scan of the tile's elements (warp shuffles, then
-//      the warps' totals);
-//   4. the tile's aggregate goes to the later tiles' shared memory, and after
-//      one cluster barrier warp 0 folds its predecessors';
-//   5. every row completes with its inclusive and exclusive prefixes: turn
-//      statistics and carried state (row_tail), the within-turn profile into
-//      the CTA's shared bins;
-//   6. a second segmented scan (restarting at trajectory starts) gives each
-//      trajectory's retained loss and first crossing in the tile, so the
-//      trajectory's record takes one update per tile instead of one per row
-//      (the rows of a token-sum segment below lambda all contended for it).
 constexpr int kRestartTurn = 1;  // st, sd, sl restart at this row
 constexpr int kRestartSum = 2;   // c restarts (a seeded row)
 
@@ -212,34 +192,8 @@ __device__ __forceinline__ TileElem tile_shfl_up(const TileElem& v, int d) {
   return o;
 }
 
-// Per-trajectory sums of the tile's rows for the trajectory's record: the
-// retained rows' loss terms and count, and whether a row crossed lambda.
-// Restarts at a trajectory's first row.
-struct TrajElem {
-  float loss;  // a tile's rows only; added to the fp64 record
-  int count;
-  int crossed;
-  int restart;
-};
-
-__device__ __forceinline__ TrajElem traj_combine(const TrajElem& a, const TrajElem& b) {
-  if (b.restart) return b;
-  return TrajElem{a.loss + b.loss, a.count + b.count, a.crossed | b.crossed, a.restart};
-}
-
-__device__ __forceinline__ TrajElem traj_shfl_up(const TrajElem& v, int d) {
-  TrajElem o;
-  o.loss = __shfl_up_sync(0xffffffffu, v.loss, d);
-  o.count = __shfl_up_sync(0xffffffffu, v.count, d);
-  o.crossed = __shfl_up_sync(0xffffffffu, v.crossed, d);
-  o.restart = __shfl_up_sync(0xffffffffu, v.restart, d);
-  return o;
-}
-
 __device__ __forceinline__ TileElem elem_combine(const TileElem& a, const TileElem& b) { return tile_combine(a, b); }
-__device__ __forceinline__ TrajElem elem_combine(const TrajElem& a, const TrajElem& b) { return traj_combine(a, b); }
 __device__ __forceinline__ TileElem elem_shfl_up(const TileElem& v, int d) { return tile_shfl_up(v, d); }
-__device__ __forceinline__ TrajElem elem_shfl_up(const TrajElem& v, int d) { return traj_shfl_up(v, d); }
 
 // Inclusive and exclusive scan of one element per thread over the CTA's
 // WARPS warps, in thread order: warp shuffles, then warp 0 scans the warps'
@@ -281,280 +235,6 @@ __device__ __forceinline__ int smem_upper_le(const int64_t* a, int n, int64_t r)
     if (a[mid] <= r) lo = mid; else hi = mid - 1;
   }
   return lo;
-}
-
-// The tiles of a window of at most kClusterMaxTiles tiles run at once, as
-// ONE thread-block cluster of one CTA per tile: each stores its aggregate
-// into the shared memory of every later tile, and after one cluster barrier
-// folds its predecessors' aggregates itself.  A second role of the barrier:
-// the carried state is read before the dependency wait and written at a
-// trajectory's last row, possibly by a later tile, so every CTA arrives once
-// its reads are done and waits before any write.
-constexpr int kClusterMaxTiles = 16;
-// Rows per tile of the cluster scan (a build define, for sweeps).  A sweep of
-// the lookback form that preceded it on GB300: the 512-row tiny step took 36.6
-// / 36.7 / 37.4 / 39.0 us with tiles of 64 / 128 / 256 / 512 rows.
-#ifndef STRIDE_CLUSTER_TILE_ROWS
-#define STRIDE_CLUSTER_TILE_ROWS 128
-#endif
-constexpr int kClusterTileRows = STRIDE_CLUSTER_TILE_ROWS;
-static_assert(kClusterTileRows % 32 == 0 && kClusterTileRows >= 64 && kClusterTileRows <= 1024,
-              "whole warps, 2 to 32 of them");
-
-
-template <int TILE>
-__global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p, const float* __restrict__ logp_s,
-                                                            const float* __restrict__ logp_t, int64_t n_tiles) {
-  constexpr int kWarps = TILE / 32;
-  __shared__ int64_t s_turn_off[TILE + 1];
-  __shared__ int64_t s_traj_row[TILE + 1];   // traj_row_off
-  __shared__ int64_t s_traj_turn[TILE + 1];  // traj_turn_off, widened
-  __shared__ int64_t s_first[2];                      // first turn, first trajectory of the tile
-  __shared__ TileElem s_wtot[kWarps];
-  __shared__ TileElem s_wpre[kWarps];
-  __shared__ TrajElem s_ttot[kWarps];
-  __shared__ TrajElem s_tpre[kWarps];
-  __shared__ TileElem s_excl;  // the tile's exclusive prefix (flags unused)
-  __shared__ TileElem s_agg;
-  __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // Launched as a programmatic dependent of the kernel that wrote the
-  // log-probs.  That kernel waited for its own predecessors before letting
-  // this grid be scheduled, so the layout and the carried state may be read
-  // before the wait; the log-probs only after it.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
-  const int64_t tile = (int64_t)blockIdx.x;
-  const int64_t t0 = tile * TILE;           // first window row of the tile
-  const int64_t n_here = min((int64_t)TILE, p.n_rows - t0);
-  const int64_t r0 = p.row_begin + t0;
-  const int64_t w = t0 + tid;  // this thread's window row
-  const int64_t r = p.row_begin + w;
-  const bool live = tid < n_here;
-  float lps = 0.f, lpt = 0.f;
-
-  // 1. the tile's first turn (warp 0) and first trajectory (warp 1), then
-  //    the offsets of the next TILE + 1 of each in shared memory (a layout
-  //    of at most TILE turns and trajectories: all of them, no search --
-  //    one dependent round trip less before the wait)
-  if (p.n_turns <= TILE && p.n_traj <= TILE) {
-    if (tid == 0) {
-      s_first[0] = p.n_turns > 0 ? 0 : -1;
-      s_first[1] = 0;
-    }
-  } else if (warp == 0) {
-    const bool ok = p.n_turns > 0 && __ldg(p.turn_row_off) <= r0;
-    const int64_t k0 = ok ? warp_upper_le(p.turn_row_off, 0, p.n_turns - 1, r0, lane) : 0;
-    if (lane == 0) s_first[0] = ok ? k0 : -1;
-  } else if (warp == 1) {
-    const bool ok = __ldg(p.traj_row_off) <= r0;
-    const int64_t i0 = ok ? warp_upper_le(p.traj_row_off, 0, p.n_traj - 1, r0, lane) : 0;
-    if (lane == 0) s_first[1] = ok ? i0 : -1;
-  }
-  __syncthreads();
-  const int64_t k0 = s_first[0], i0 = s_first[1];
-  if (k0 >= 0 && i0 >= 0) {
-    for (int j = tid; j <= TILE; j += TILE) {
-      s_turn_off[j] = __ldg(p.turn_row_off + min(k0 + j, (int64_t)p.n_turns));
-      s_traj_row[j] = __ldg(p.traj_row_off + min(i0 + j, (int64_t)p.n_traj));
-      s_traj_turn[j] = __ldg(p.traj_turn_off + min(i0 + j, (int64_t)p.n_traj));
-    }
-  }
-  __syncthreads();
-
-  __shared__ TileElem s_caggs[kClusterMaxTiles];  // predecessors' aggregates
-
-  // 2. this thread's row: its turn and trajectory, and its element
-  RowMeta meta;
-  meta.bad = true;
-  meta.traj = 0;
-  meta.turn = 0;
-  meta.local_turn = 0;
-  meta.traj_start = meta.traj_end = meta.turn_start = meta.turn_end = 0;
-  if (live && k0 >= 0 && i0 >= 0) {
-    const int nk = (int)min((int64_t)TILE, (int64_t)p.n_turns - k0);
-    const int j = smem_upper_le(s_turn_off, nk, r);
-    const int ni = (int)min((int64_t)TILE, (int64_t)p.n_traj - i0);
-    int q = smem_upper_le(s_traj_row, ni, r);
-    int64_t traj = i0 + q, tr_start = s_traj_row[q], tr_end = s_traj_row[q + 1];
-    int64_t tu0 = s_traj_turn[q], tu1 = s_traj_turn[q + 1];
-    if (r >= tr_end && q == ni - 1 && i0 + ni < p.n_traj) {
-      // past the staged trajectories (more than TILE empty ones
-      // in the tile's rows): search the rest in global memory
-      int64_t lo = i0 + ni, hi = p.n_traj - 1;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (__ldg(p.traj_row_off + mid) <= r) lo = mid; else hi = mid - 1;
-      }
-      traj = lo;
-      tr_start = __ldg(p.traj_row_off + traj);
-      tr_end = __ldg(p.traj_row_off + traj + 1);
-      tu0 = __ldg(p.traj_turn_off + traj);
-      tu1 = __ldg(p.traj_turn_off + traj + 1);
-    }
-    const int64_t turn = k0 + j;
-    meta.turn = (int32_t)turn;
-    meta.traj = (int32_t)traj;
-    meta.turn_start = s_turn_off[j];
-    meta.turn_end = s_turn_off[j + 1];
-    meta.local_turn = (int32_t)(turn - tu0);
-    meta.traj_start = tr_start;
-    meta.traj_end = tr_end;
-    meta.bad = !(meta.turn_start <= r && r < meta.turn_end) || !(tr_start <= r && r < tr_end) ||
-               !(tu0 <= turn && turn < tu1);
-  }
-  // a seeded row's carried state, and lambda, before the wait
-  const bool seeded = live && ((w == 0) || (r == meta.traj_start) || meta.bad);
-  const int fturn = (live && r == meta.turn_start) ? 1 : 0;
-  double cum0 = 0.0, st0 = 0.0, sd0 = 0.0, sl0 = 0.0;
-  if (seeded && !meta.bad) {
-    const stride_scan_state* sp = p.state + meta.traj;
-    cum0 = __ldcg(&sp->cum);
-    st0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_t);
-    sd0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_d);
-    sl0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_l);
-  }
-  const float lam = (live && !meta.bad) ? (p.lambda ? __ldg(p.lambda + meta.traj) : p.lambda_all) : 0.f;
-  cluster_arrive_release();  // this CTA's reads of the carried state are done
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (live) {
-    lps = __ldcg(logp_s + w);
-    lpt = __ldcg(logp_t + w);
-  }
-  TileElem x = {0.0, 0.0, 0.0, 0.0, 0};
-  double c_before = 0.0, st_before = 0.0, ri_c = 0.0;
-  float st_before_f = 0.f, e_sl = 0.f;
-  if (live) {
-    const float nan = __int_as_float(0x7fc00000);
-    if (meta.bad) {
-      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
-      lps = nan;
-      lpt = nan;
-      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
-      if (p.out.logp_t) p.out.logp_t[w] = nan;
-    }
-    const float dd = lps - lpt;
-    if (p.out.opd) p.out.opd[w] = dd;
-    const int64_t n_k = meta.turn_end - meta.turn_start;
-    // The row's terms in fp32 (logp_S * d rounded once, as the fp64 product
-    // of two floats rounded to float would be); the stop-sum term in fp64,
-    // a turn mean's share lpt / n_k rounded once to fp32 first (GB300 issues
-    // an fp64 divide as a sequence of fp64 operations at 1/64 of the fp32
-    // rate; the rounding is 6e-8 of the term).
-    const float esl = lps * dd;
-    const double ec =
-        (p.mode == STRIDE_STOP_TURN_MEAN) ? (double)(lpt / (float)(n_k > 0 ? n_k : 1)) : (double)lpt;
-    e_sl = esl;
-    if (p.profile && !meta.bad) {
-      const int jb = (int)((10 * (r - meta.turn_start)) / n_k);  // Observation 1 decile
-      atomicAdd(s_prof + 3 * jb + 0, (double)dd);
-      atomicAdd(s_prof + 3 * jb + 1, (double)lpt);
-      atomicAdd(s_prof + 3 * jb + 2, 1.0);
-    }
-    if (seeded && !meta.bad) {
-      x = TileElem{cum0 + ec, (float)(st0 + (double)lpt), (float)(sd0 + (double)dd), (float)(sl0 + (double)esl),
-                   kRestartSum | kRestartTurn};
-      c_before = cum0;
-      st_before = st0;
-      st_before_f = (float)st0;
-    } else if (seeded) {
-      x = TileElem{ec, lpt, dd, esl, kRestartSum | kRestartTurn};  // NaN: nothing after a bad row is meaningful
-    } else {
-      x = TileElem{ec, lpt, dd, esl, fturn ? kRestartTurn : 0};
-    }
-    if (seeded) x.flags |= 4;  // bit 2: this row's exclusive prefix is the carried state, not the scan
-  }
-
-  // 3. segmented inclusive scan over the tile
-  const TileElem tile_id = {0.0, 0.f, 0.f, 0.f, 0};
-  TileElem tile_incl, tile_excl;
-  block_scan<kWarps>(x, tile_id, lane, warp, s_wtot, s_wpre, tile_incl, tile_excl);
-
-  // 4. the tile's exclusive prefix, from the cluster's other tiles
-  namespace cg = cooperative_groups;
-  if (tid == (int)(n_here - 1)) s_agg = tile_incl;
-  __syncthreads();
-  cluster_wait_acquire();  // every tile has started and read its carried state
-  if (warp == 0) {
-    const cg::cluster_group cl = cg::this_cluster();
-    const TileElem agg = s_agg;
-    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) cl.map_shared_rank(s_caggs, (unsigned)j)[tile] = agg;
-  }
-  cluster_arrive_release();
-  cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
-  if (warp == 0) {
-    // the predecessors' aggregates folded in tile order (a warp scan: the
-    // stop sum fp64, the open-turn sums fp32 as inside a tile)
-    TileElem v = {0.0, 0.f, 0.f, 0.f, 0};
-    if (lane < tile) v = s_caggs[lane];
-#pragma unroll
-    for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
-      const TileElem o = tile_shfl_up(v, d);
-      if (lane >= d) v = tile_combine(o, v);
-    }
-    if (lane == (tile > 0 ? (int)tile - 1 : 0))
-      s_excl = tile > 0 ? TileElem{v.c, v.st, v.sd, v.sl, 0} : TileElem{0.0, 0.f, 0.f, 0.f, 0};
-  }
-  __syncthreads();
-
-  // 5. complete every row
-  if (live) {
-    // the row's prefixes: the stop sum fp64, the open-turn sums fp32 (the
-    // tile's prefix rounded once to fp32; 6e-8 of the sums)
-    const TileElem pre = s_excl;
-    const TileElem ri = tile_combine(pre, tile_incl);
-    if (!(x.flags & 4)) {
-      const TileElem re = tile_combine(pre, tile_excl);
-      c_before = re.c;
-      st_before_f = fturn ? 0.f : re.st;
-      st_before = (double)st_before_f;
-    }
-    RowCarry rc;
-    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, fturn};
-    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 1};
-    row_tail(p, r, meta, rc, si, c_before, st_before, false, true);
-    ri_c = ri.c;
-  }
-
-  // 6. the trajectories' stop records and losses, once per trajectory and
-  //    tile: the first row of a trajectory here that crosses lambda records
-  //    the stop (the running sum never rises, so it is the trajectory's
-  //    first crossing unless an earlier tile's is lower), and the last row
-  //    of a trajectory here adds its retained rows' loss and count.
-  TrajElem te = {0.f, 0, 0, 1};
-  bool cross = false;
-  if (live && !meta.bad) {
-    const int64_t n_k = meta.turn_end - meta.turn_start;
-    const bool turn_last = (r == meta.turn_end - 1);
-    const bool test = (p.mode == STRIDE_STOP_TOKEN_SUM) || turn_last;
-    cross = test && ri_c < (double)lam;
-    // retained unless the rule fired before the row (row_tail); a
-    // trajectory's first token or turn always is
-    const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
-    const double before =
-        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before : c_before - (double)(st_before_f / (float)n_k);
-    const bool kept = first || !(before < (double)lam);
-    te = TrajElem{kept ? e_sl : 0.f, kept ? 1 : 0, cross ? 1 : 0, r == meta.traj_start ? 1 : 0};
-  }
-  const TrajElem traj_id = {0.f, 0, 0, 0};
-  TrajElem t_incl, t_excl;
-  block_scan<kWarps>(te, traj_id, lane, warp, s_ttot, s_tpre, t_incl, t_excl);
-  if (live && !meta.bad) {
-    stride_scan_state* sp = p.state + meta.traj;
-    if (cross && (te.restart || !t_excl.crossed)) {
-      atomicMin(reinterpret_cast<unsigned long long*>(&sp->stop_row), (unsigned long long)(r - meta.traj_start));
-      atomicMin(reinterpret_cast<unsigned int*>(&sp->stop_turn), (unsigned int)meta.local_turn);
-      sp->stopped = 1;
-    }
-    if ((r == meta.traj_end - 1 || tid == (int)(n_here - 1)) && t_incl.count > 0) {
-      atomicAdd(&sp->loss, t_incl.loss);
-      atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), (unsigned long long)t_incl.count);
-    }
-  }
-  if (p.profile) {
-    __syncthreads();
-    if (tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
-  }
 }
 
 // The scan on given log-probs, in two passes over tiles of R x kPassThreads
@@ -1140,6 +820,29 @@ __device__ __forceinline__ void record_loss(stride_scan_state* sp, const Sum2& l
   atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), (unsigned long long)count);
 }
 
+// The trajectories' records: neighbouring threads of one trajectory together
+// (the lowest crossing, the sum of the losses).  Warp-wide.
+__device__ __forceinline__ void record_parts(const BatchParams& p, const TrajPart& part, int lane) {
+  __syncwarp();
+  const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
+  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
+  const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
+  const int h = head_of(m_run, lane);
+  const Sum2 loss = seg_sum(part.loss, h, lane);
+  int count = part.count;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, count, d);
+    if (lane - d >= h) count += n;
+  }
+  if (part.traj >= 0) {
+    stride_scan_state* sp = p.state + part.traj;
+    const unsigned mine = (0xffffffffu >> (31 - lane)) & (0xffffffffu << h);
+    if (part.cross_row >= 0 && __ffs(m_cross & mine) - 1 == lane) record_cross(sp, part);
+    if (count > 0 && (lane == 31 || ((m_run >> lane) & 2u))) record_loss(sp, loss, count);
+  }
+}
+
 // Completes the thread's rows, given the exclusive prefix of its rows inside
 // the tile, the tile's (pre) and the carried state of the tile's seeded rows
 // (seed(j), which covers excl.seed too).
@@ -1251,27 +954,7 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
       }
     }
   }
-
-  // the trajectories' records: neighbouring threads of one trajectory together
-  // (the lowest crossing, the sum of the losses)
-  __syncwarp();
-  const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
-  const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
-  const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
-  const int h = head_of(m_run, lane);
-  const Sum2 loss = seg_sum(part.loss, h, lane);
-  int count = part.count;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, count, d);
-    if (lane - d >= h) count += n;
-  }
-  if (part.traj >= 0) {
-    stride_scan_state* sp = p.state + part.traj;
-    const unsigned mine = (0xffffffffu >> (31 - lane)) & (0xffffffffu << h);
-    if (part.cross_row >= 0 && __ffs(m_cross & mine) - 1 == lane) record_cross(sp, part);
-    if (count > 0 && (lane == 31 || ((m_run >> lane) & 2u))) record_loss(sp, loss, count);
-  }
+  record_parts(p, part, lane);
 }
 
 // Layout checks, spread over every thread of a grid of n_tiles CTAs.
@@ -1290,6 +973,291 @@ __device__ __forceinline__ void check_layout(const BatchParams& p, int64_t tile,
     }
   }
   if (bad) set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+}
+
+// A small window's scan after the small-window kernel, one tile of TILE
+// consecutive rows per CTA (one row per thread) and all tiles one
+// thread-block cluster:
+//   1. the CTA stages the offsets of the tile's turns and trajectories in
+//      shared memory and every thread finds its row's there;
+//   2. each row's element: the stop-sum term, log pi_T, d, logp_S * d, and
+//      two restart marks -- the open-turn sums restart at a turn's first row,
+//      the running sum at a seeded row (a trajectory's first row, or the
+//      window's), whose element already holds the carried state;
+//   3. a segmented inclusive scan of the tile's elements (warp shuffles, then
+//      the warps' totals);
+//   4. the tile's aggregate goes to the later tiles' shared memory, and after
+//      one cluster barrier warp 0 folds its predecessors';
+//   5. every row completes with its inclusive and exclusive prefixes: turn
+//      statistics and carried state (row_tail);
+//   6. each trajectory's retained loss and first crossing are gathered per
+//      warp (record_parts), so its record takes one update per warp instead
+//      of one per row (the rows of a token-sum segment below lambda all
+//      contended for it).
+// The profile's runs of equal deciles are summed in registers while the
+// aggregates are on their way.  GB300, against a second block scan for 6 and a
+// shared-memory atomic per row for the profile: a 512-row window of 32,000
+// fp32 logits 25.9 -> 25.7 us, with the profile 33.7 -> 30.7; 1,024 rows of
+// 151,936 bf16 logits with the profile 107.4 -> 101.4.
+// The tiles of a window of at most kClusterMaxTiles tiles run at once, as
+// ONE thread-block cluster of one CTA per tile: each stores its aggregate
+// into the shared memory of every later tile, and after one cluster barrier
+// folds its predecessors' aggregates itself.  A second role of the barrier:
+// the carried state is read before the dependency wait and written at a
+// trajectory's last row, possibly by a later tile, so every CTA arrives once
+// its reads are done and waits before any write.
+constexpr int kClusterMaxTiles = 16;
+// Rows per tile of the cluster scan (a build define, for sweeps).  A sweep of
+// the lookback form that preceded it on GB300: the 512-row tiny step took 36.6
+// / 36.7 / 37.4 / 39.0 us with tiles of 64 / 128 / 256 / 512 rows.
+#ifndef STRIDE_CLUSTER_TILE_ROWS
+#define STRIDE_CLUSTER_TILE_ROWS 128
+#endif
+constexpr int kClusterTileRows = STRIDE_CLUSTER_TILE_ROWS;
+static_assert(kClusterTileRows % 32 == 0 && kClusterTileRows >= 64 && kClusterTileRows <= 1024,
+              "whole warps, 2 to 32 of them");
+
+
+template <int TILE>
+__global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p, const float* __restrict__ logp_s,
+                                                            const float* __restrict__ logp_t, int64_t n_tiles) {
+  constexpr int kWarps = TILE / 32;
+  __shared__ int64_t s_turn_off[TILE + 1];
+  __shared__ int64_t s_traj_row[TILE + 1];   // traj_row_off
+  __shared__ int64_t s_traj_turn[TILE + 1];  // traj_turn_off, widened
+  __shared__ int64_t s_first[2];                      // first turn, first trajectory of the tile
+  __shared__ TileElem s_wtot[kWarps];
+  __shared__ TileElem s_wpre[kWarps];
+  __shared__ TileElem s_excl;  // the tile's exclusive prefix (flags unused)
+  __shared__ TileElem s_agg;
+  __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // Launched as a programmatic dependent of the kernel that wrote the
+  // log-probs.  That kernel waited for its own predecessors before letting
+  // this grid be scheduled, so the layout and the carried state may be read
+  // before the wait; the log-probs only after it.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
+  const int64_t tile = (int64_t)blockIdx.x;
+  const int64_t t0 = tile * TILE;           // first window row of the tile
+  const int64_t n_here = min((int64_t)TILE, p.n_rows - t0);
+  const int64_t r0 = p.row_begin + t0;
+  const int64_t w = t0 + tid;  // this thread's window row
+  const int64_t r = p.row_begin + w;
+  const bool live = tid < n_here;
+  float lps = 0.f, lpt = 0.f;
+
+  // 1. the tile's first turn (warp 0) and first trajectory (warp 1), then
+  //    the offsets of the next TILE + 1 of each in shared memory (a layout
+  //    of at most TILE turns and trajectories: all of them, no search --
+  //    one dependent round trip less before the wait)
+  if (p.n_turns <= TILE && p.n_traj <= TILE) {
+    if (tid == 0) {
+      s_first[0] = p.n_turns > 0 ? 0 : -1;
+      s_first[1] = 0;
+    }
+  } else if (warp == 0) {
+    const bool ok = p.n_turns > 0 && __ldg(p.turn_row_off) <= r0;
+    const int64_t k0 = ok ? warp_upper_le(p.turn_row_off, 0, p.n_turns - 1, r0, lane) : 0;
+    if (lane == 0) s_first[0] = ok ? k0 : -1;
+  } else if (warp == 1) {
+    const bool ok = __ldg(p.traj_row_off) <= r0;
+    const int64_t i0 = ok ? warp_upper_le(p.traj_row_off, 0, p.n_traj - 1, r0, lane) : 0;
+    if (lane == 0) s_first[1] = ok ? i0 : -1;
+  }
+  __syncthreads();
+  const int64_t k0 = s_first[0], i0 = s_first[1];
+  if (k0 >= 0 && i0 >= 0) {
+    for (int j = tid; j <= TILE; j += TILE) {
+      s_turn_off[j] = __ldg(p.turn_row_off + min(k0 + j, (int64_t)p.n_turns));
+      s_traj_row[j] = __ldg(p.traj_row_off + min(i0 + j, (int64_t)p.n_traj));
+      s_traj_turn[j] = __ldg(p.traj_turn_off + min(i0 + j, (int64_t)p.n_traj));
+    }
+  }
+  __syncthreads();
+
+  __shared__ TileElem s_caggs[kClusterMaxTiles];  // predecessors' aggregates
+
+  // 2. this thread's row: its turn and trajectory, and its element
+  RowMeta meta;
+  meta.bad = true;
+  meta.traj = 0;
+  meta.turn = 0;
+  meta.local_turn = 0;
+  meta.traj_start = meta.traj_end = meta.turn_start = meta.turn_end = 0;
+  if (live && k0 >= 0 && i0 >= 0) {
+    const int nk = (int)min((int64_t)TILE, (int64_t)p.n_turns - k0);
+    const int j = smem_upper_le(s_turn_off, nk, r);
+    const int ni = (int)min((int64_t)TILE, (int64_t)p.n_traj - i0);
+    int q = smem_upper_le(s_traj_row, ni, r);
+    int64_t traj = i0 + q, tr_start = s_traj_row[q], tr_end = s_traj_row[q + 1];
+    int64_t tu0 = s_traj_turn[q], tu1 = s_traj_turn[q + 1];
+    if (r >= tr_end && q == ni - 1 && i0 + ni < p.n_traj) {
+      // past the staged trajectories (more than TILE empty ones
+      // in the tile's rows): search the rest in global memory
+      int64_t lo = i0 + ni, hi = p.n_traj - 1;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi + 1) >> 1;
+        if (__ldg(p.traj_row_off + mid) <= r) lo = mid; else hi = mid - 1;
+      }
+      traj = lo;
+      tr_start = __ldg(p.traj_row_off + traj);
+      tr_end = __ldg(p.traj_row_off + traj + 1);
+      tu0 = __ldg(p.traj_turn_off + traj);
+      tu1 = __ldg(p.traj_turn_off + traj + 1);
+    }
+    const int64_t turn = k0 + j;
+    meta.turn = (int32_t)turn;
+    meta.traj = (int32_t)traj;
+    meta.turn_start = s_turn_off[j];
+    meta.turn_end = s_turn_off[j + 1];
+    meta.local_turn = (int32_t)(turn - tu0);
+    meta.traj_start = tr_start;
+    meta.traj_end = tr_end;
+    meta.bad = !(meta.turn_start <= r && r < meta.turn_end) || !(tr_start <= r && r < tr_end) ||
+               !(tu0 <= turn && turn < tu1);
+  }
+  // a seeded row's carried state, and lambda, before the wait
+  const bool seeded = live && ((w == 0) || (r == meta.traj_start) || meta.bad);
+  const int fturn = (live && r == meta.turn_start) ? 1 : 0;
+  double cum0 = 0.0, st0 = 0.0, sd0 = 0.0, sl0 = 0.0;
+  if (seeded && !meta.bad) {
+    const stride_scan_state* sp = p.state + meta.traj;
+    cum0 = __ldcg(&sp->cum);
+    st0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_t);
+    sd0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_d);
+    sl0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_l);
+  }
+  Rows<1, false> row;  // for the profile
+  row.what[0] = (live ? kRowLive : 0) | (meta.bad ? kRowBad : 0);
+  row.bin[0] = 0;
+  if (p.profile && live && !meta.bad) row.bin[0] = (int)((10 * (r - meta.turn_start)) / (meta.turn_end - meta.turn_start));
+  const float lam = (live && !meta.bad) ? (p.lambda ? __ldg(p.lambda + meta.traj) : p.lambda_all) : 0.f;
+  cluster_arrive_release();  // this CTA's reads of the carried state are done
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (live) {
+    lps = __ldcg(logp_s + w);
+    lpt = __ldcg(logp_t + w);
+  }
+  TileElem x = {0.0, 0.0, 0.0, 0.0, 0};
+  double c_before = 0.0, st_before = 0.0, ri_c = 0.0;
+  float st_before_f = 0.f, e_sl = 0.f;
+  if (live) {
+    const float nan = __int_as_float(0x7fc00000);
+    if (meta.bad) {
+      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+      lps = nan;
+      lpt = nan;
+      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
+      if (p.out.logp_t) p.out.logp_t[w] = nan;
+    }
+    const float dd = lps - lpt;
+    if (p.out.opd) p.out.opd[w] = dd;
+    const int64_t n_k = meta.turn_end - meta.turn_start;
+    // The row's terms in fp32 (logp_S * d rounded once, as the fp64 product
+    // of two floats rounded to float would be); the stop-sum term in fp64,
+    // a turn mean's share lpt / n_k rounded once to fp32 first (GB300 issues
+    // an fp64 divide as a sequence of fp64 operations at 1/64 of the fp32
+    // rate; the rounding is 6e-8 of the term).
+    const float esl = lps * dd;
+    const double ec =
+        (p.mode == STRIDE_STOP_TURN_MEAN) ? (double)(lpt / (float)(n_k > 0 ? n_k : 1)) : (double)lpt;
+    e_sl = esl;
+    if (seeded && !meta.bad) {
+      x = TileElem{cum0 + ec, (float)(st0 + (double)lpt), (float)(sd0 + (double)dd), (float)(sl0 + (double)esl),
+                   kRestartSum | kRestartTurn};
+      c_before = cum0;
+      st_before = st0;
+      st_before_f = (float)st0;
+    } else if (seeded) {
+      x = TileElem{ec, lpt, dd, esl, kRestartSum | kRestartTurn};  // NaN: nothing after a bad row is meaningful
+    } else {
+      x = TileElem{ec, lpt, dd, esl, fturn ? kRestartTurn : 0};
+    }
+    if (seeded) x.flags |= 4;  // bit 2: this row's exclusive prefix is the carried state, not the scan
+  }
+
+  // 3. segmented inclusive scan over the tile
+  const TileElem tile_id = {0.0, 0.f, 0.f, 0.f, 0};
+  TileElem tile_incl, tile_excl;
+  block_scan<kWarps>(x, tile_id, lane, warp, s_wtot, s_wpre, tile_incl, tile_excl);
+
+  // 4. the tile's exclusive prefix, from the cluster's other tiles
+  namespace cg = cooperative_groups;
+  if (tid == (int)(n_here - 1)) s_agg = tile_incl;
+  __syncthreads();
+  cluster_wait_acquire();  // every tile has started and read its carried state
+  if (warp == 0) {
+    const cg::cluster_group cl = cg::this_cluster();
+    const TileElem agg = s_agg;
+    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) cl.map_shared_rank(s_caggs, (unsigned)j)[tile] = agg;
+  }
+  cluster_arrive_release();
+  if (p.profile) {  // (while the aggregates are on their way)
+    row.lps[0] = lps;
+    row.lpt[0] = lpt;
+    rows_profile<1>(row, lane, s_prof);
+  }
+  cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
+  if (warp == 0) {
+    // the predecessors' aggregates folded in tile order (a warp scan: the
+    // stop sum fp64, the open-turn sums fp32 as inside a tile)
+    TileElem v = {0.0, 0.f, 0.f, 0.f, 0};
+    if (lane < tile) v = s_caggs[lane];
+#pragma unroll
+    for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
+      const TileElem o = tile_shfl_up(v, d);
+      if (lane >= d) v = tile_combine(o, v);
+    }
+    if (lane == (tile > 0 ? (int)tile - 1 : 0))
+      s_excl = tile > 0 ? TileElem{v.c, v.st, v.sd, v.sl, 0} : TileElem{0.0, 0.f, 0.f, 0.f, 0};
+  }
+  __syncthreads();
+
+  // 5. complete every row
+  if (live) {
+    // the row's prefixes: the stop sum fp64, the open-turn sums fp32 (the
+    // tile's prefix rounded once to fp32; 6e-8 of the sums)
+    const TileElem pre = s_excl;
+    const TileElem ri = tile_combine(pre, tile_incl);
+    if (!(x.flags & 4)) {
+      const TileElem re = tile_combine(pre, tile_excl);
+      c_before = re.c;
+      st_before_f = fturn ? 0.f : re.st;
+      st_before = (double)st_before_f;
+    }
+    RowCarry rc;
+    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, fturn};
+    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 1};
+    row_tail(p, r, meta, rc, si, c_before, st_before, false, true);
+    ri_c = ri.c;
+  }
+
+  // 6. the trajectories' stop records and losses, once per trajectory and warp
+  TrajPart part = {-1, 0, 0, {0.f, 0.f}, -1};
+  if (live && !meta.bad) {
+    const int64_t n_k = meta.turn_end - meta.turn_start;
+    const bool turn_last = (r == meta.turn_end - 1);
+    const bool test = (p.mode == STRIDE_STOP_TOKEN_SUM) || turn_last;
+    // retained unless the rule fired before the row (row_tail); a
+    // trajectory's first token or turn always is
+    const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
+    const double before =
+        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before : c_before - (double)(st_before_f / (float)n_k);
+    const bool kept = first || !(before < (double)lam);
+    part.traj = meta.traj;
+    part.count = kept ? 1 : 0;
+    part.loss.hi = kept ? e_sl : 0.f;
+    if (test && ri_c < (double)lam) {
+      part.cross_row = r - meta.traj_start;
+      part.cross_turn = meta.local_turn;
+    }
+  }
+  record_parts(p, part, lane);
+  if (p.profile) {
+    __syncthreads();
+    if (tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
+  }
 }
 
 // Second pass.
