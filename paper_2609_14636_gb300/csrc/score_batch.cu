@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
     sS = lane < kSplitWarps ? s_red[1][lane] : 0.f;
     mT = lane < kSplitWarps ? s_red[2][lane] : kMaxStart;
     sT = lane < kSplitWarps ? s_red[3][lane] : 0.f;
-    warp_merge2(mS, sS, mT, sT);
+    warp_merge2<kSplitWarps>(mS, sS, mT, sT);
     if (lane == 0) cluster.map_shared_rank(s_part, 0)[rank] = make_float4(mS, sS, mT, sT);
   }
   // second phase: the ranks' pairs are released to rank 0; the other ranks
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
       mT = q.z;
       sT = q.w;
     }
-    warp_merge2(mS, sS, mT, sT);
+    warp_merge2<kSplitMaxCluster>(mS, sS, mT, sT);
     if (lane == 0) {
       const float lse_s = lse_finish(mS, sS), lse_t = lse_finish(mT, sT);
       if (!(y >= 0 && y < p.V)) set_status(p.dev_status, STRIDE_DEV_TOKEN_RANGE);

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(THREADS, StepShape<THREADS>::kMinBlocks) score
     sS = lane < kStepWarps ? s_red[1][lane] : 0.f;
     mT = lane < kStepWarps ? s_red[2][lane] : kMaxStart;
     sT = lane < kStepWarps ? s_red[3][lane] : 0.f;
-    warp_merge2(mS, sS, mT, sT);
+    warp_merge2<kStepWarps>(mS, sS, mT, sT);
     if (lane == 0) {
       float4* dst = cluster.map_shared_rank(s_part, 0);
       dst[rank] = make_float4(mS, sS, mT, sT);
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(THREADS, StepShape<THREADS>::kMinBlocks) score
       mT = q.z;
       sT = q.w;
     }
-    warp_merge2(mS, sS, mT, sT);
+    warp_merge2<kStepMaxCluster>(mS, sS, mT, sT);
     if (lane == 0) {
       if (!valid) {
         set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);

@@ -43,7 +43,8 @@ namespace stride {
 #endif
 constexpr int kPartialThreads = STRIDE_PARTIAL_THREADS;
 constexpr int kPartialWarps = kPartialThreads / 32;
-static_assert(kPartialThreads % 32 == 0 && kPartialWarps <= 32, "whole warps, at most 32");
+static_assert(kPartialThreads % 32 == 0 && kPartialWarps <= 32 && (kPartialWarps & (kPartialWarps - 1)) == 0,
+              "whole warps, a power of two of them, at most 32");
 
 struct PartialParams {
   const void* S;
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kPartialThreads, STRIDE_PARTIAL_MIN_BLOCKS) pa
   sS = lane < kPartialWarps ? s_red[1][lane] : 0.f;
   mT = lane < kPartialWarps ? s_red[2][lane] : kMaxStart;
   sT = lane < kPartialWarps ? s_red[3][lane] : 0.f;
-  warp_merge2(mS, sS, mT, sT);
+  warp_merge2<kPartialWarps>(mS, sS, mT, sT);
   if (lane == 0) {
     const float nan = __int_as_float(0x7fc00000);
     const int32_t y = __ldg(p.tokens + r);
