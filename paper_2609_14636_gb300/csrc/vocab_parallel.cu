@@ -25,26 +25,19 @@
 
 namespace stride {
 
-// Shard-pass launch shape (build defines, for sweeps): threads per CTA,
-// 16-byte loads in flight per thread and tensor, and CTAs per SM promised
-// to the register allocator.  A sweep on GB300 (4 shards of the batch-
-// scoring rows, 37,984 bf16 logits per shard row; ms for the 4 passes):
-// 128 threads x 4 loads at 8 CTAs per SM (58 registers) 12.25; 256 x 3 at
-// 8 per SM 12.26; 128 x 4 unbounded (7 per SM) 12.30; 256 x 4 at 4 per SM
-// 12.48; 256 x 2 12.82; 256 x 4 unbounded (66 registers, 3 per SM) 13.03.
-#ifndef STRIDE_PARTIAL_THREADS
-#define STRIDE_PARTIAL_THREADS 128
-#endif
-#ifndef STRIDE_PARTIAL_UNROLL
-#define STRIDE_PARTIAL_UNROLL 4
-#endif
-#ifndef STRIDE_PARTIAL_MIN_BLOCKS
-#define STRIDE_PARTIAL_MIN_BLOCKS 8
-#endif
-constexpr int kPartialThreads = STRIDE_PARTIAL_THREADS;
+// Shard-pass launch shapes: CTAs of 128 threads with U 16-byte loads in flight
+// per thread and tensor, U = 4 at 8 CTAs per SM or U = 5 at 7 (what the
+// registers allow).  Five loads stream faster; eight CTAs hold more rows at
+// once, which decides where it saves a wave.  GB300, us for passes, merge and
+// scan, 4 at 8 / 5 at 7 (5 at 6 / 7 at 6): 6,000 rows in 4 shards of 37,984
+// bf16 logits 520.6 / 520.2 (520.3 / 521.6), in 8 534.1 / 529.3 (529.5 /
+// 527.3), in 4 of 8,000 138.7 / 132.5 (132.7 / 138.3); 800 rows 99.0 / 95.8,
+// 1,500 168.3 / 159.7, 3,000 282.3 / 274.5; a wave more: 1,100 rows 117.8 /
+// 135.8, 1,216 126.4 / 144.0, 2,400 225.0 / 237.5; 600 rows 84.2 / 87.6.  CTAs
+// of 64 threads (4 at 16) 542, of 256 (4 at 4) 518 but 547 in 8 shards.
+constexpr int kPartialThreads = 128;
+constexpr int kPartialManyCtas = 8, kPartialManyLoads = 7;  // CTAs per SM with U = 4, with U = 5
 constexpr int kPartialWarps = kPartialThreads / 32;
-static_assert(kPartialThreads % 32 == 0 && kPartialWarps <= 32 && (kPartialWarps & (kPartialWarps - 1)) == 0,
-              "whole warps, a power of two of them, at most 32");
 
 struct PartialParams {
   const void* S;
@@ -72,8 +65,9 @@ constexpr int64_t kPartialPrefetch = STRIDE_PARTIAL_PREFETCH;
 
 // One CTA per row: (m, s) of S and T over this shard's columns, and the
 // gathered logits when the token is one of them (NaN otherwise).
-template <typename LT, bool VEC>
-__global__ void __launch_bounds__(kPartialThreads, STRIDE_PARTIAL_MIN_BLOCKS) partial_lse_kernel(const PartialParams p) {
+template <typename LT, bool VEC, int U>
+__global__ void __launch_bounds__(kPartialThreads, U == 5 ? kPartialManyLoads : kPartialManyCtas)
+    partial_lse_kernel(const PartialParams p) {
   __shared__ float s_red[4][kPartialWarps];
   const int64_t r = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -87,7 +81,7 @@ __global__ void __launch_bounds__(kPartialThreads, STRIDE_PARTIAL_MIN_BLOCKS) pa
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
-  stream_pair<LT, VEC, STRIDE_PARTIAL_UNROLL>(srow, trow, 0, p.V_shard, tid, kPartialThreads, mS, sS, mT, sT);
+  stream_pair<LT, VEC, U>(srow, trow, 0, p.V_shard, tid, kPartialThreads, mS, sS, mT, sT);
   warp_merge2(mS, sS, mT, sT);
   if (lane == 0) {
     s_red[0][warp] = mS;
@@ -1398,11 +1392,18 @@ cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec
     q.timeout_ns = kWaitTimeoutNs;
     return launch_score_batch_stream(q, dtype, vec, stream);
   }
+  // five loads, unless eight CTAs per SM save one of a few waves, or the rows
+  // are too few to fill either
+  const int64_t waves_many = (rows + kPartialManyCtas * sms - 1) / (kPartialManyCtas * sms);
+  const int64_t waves_loads = (rows + kPartialManyLoads * sms - 1) / (kPartialManyLoads * sms);
+  const bool loads = rows >= 5 * (int64_t)sms && (waves_loads == waves_many || waves_loads > 5);
   const PartialParams p{S, T, ld, V_shard, col0, 0, tokens, rows, partials, dev_status,
-                        (int64_t)STRIDE_PARTIAL_MIN_BLOCKS * sms};
-  auto* kern = dtype == STRIDE_DTYPE_BF16
-                   ? (vec ? partial_lse_kernel<__nv_bfloat16, true> : partial_lse_kernel<__nv_bfloat16, false>)
-                   : (vec ? partial_lse_kernel<float, true> : partial_lse_kernel<float, false>);
+                        (int64_t)(loads ? kPartialManyLoads : kPartialManyCtas) * sms};
+  const bool bf16 = dtype == STRIDE_DTYPE_BF16;
+  auto* kern = loads ? (bf16 ? (vec ? partial_lse_kernel<__nv_bfloat16, true, 5> : partial_lse_kernel<__nv_bfloat16, false, 5>)
+                             : (vec ? partial_lse_kernel<float, true, 5> : partial_lse_kernel<float, false, 5>))
+                     : (bf16 ? (vec ? partial_lse_kernel<__nv_bfloat16, true, 4> : partial_lse_kernel<__nv_bfloat16, false, 4>)
+                             : (vec ? partial_lse_kernel<float, true, 4> : partial_lse_kernel<float, false, 4>));
   return launch_dependent(kern, (unsigned)rows, kPartialThreads, stream, p);
 }
 

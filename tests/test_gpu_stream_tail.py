@@ -108,11 +108,12 @@ def test_every_launch_shape(stride, compact, V):
 
 
 @pytest.mark.parametrize("f32", [False, True])
-@pytest.mark.parametrize("rows", [1, 7, 456, 457, 700])
-@pytest.mark.parametrize("kb", [32, 128])
+@pytest.mark.parametrize("rows", [1, 7, 456, 457, 700, 760, 1065])
+@pytest.mark.parametrize("kb", [11, 32, 128])
 def test_shard_pass_routes(stride, rows, kb, f32):
-    """Shard rows around the sizes from which the persistent kernel takes the pass, aligned and not, the second shard
-    with and without the row's token."""
+    """Shard rows around the sizes from which the persistent kernel takes the pass, and row counts on both sides of the
+    other's two shapes (five loads from 760 rows on, not at 1,065), aligned and not, the second shard with and without
+    the row's token."""
     import torch
 
     W = kb * 1024 // (4 if f32 else 2)
