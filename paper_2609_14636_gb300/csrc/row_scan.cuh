@@ -1,8 +1,8 @@
 // row_scan.cuh -- the per-row tail of the batch kernel that takes one CTA per
 // row: the row's log-probs and outputs, its element of the decoupled-lookback
 // segmented scan, turn statistics, the stop test and the carried state.  The
-// lookback itself also serves the tiled scans (warp_tile_scan.cuh, and the
-// scan on log-probs in vocab_parallel.cu), whose tiles are many rows.
+// lookback itself also serves the persistent kernel's scan, whose tiles are 32
+// rows (warp_tile_scan.cuh), and row_tail the cluster scan (vocab_parallel.cu).
 //
 // The running stop sum is a plain prefix sum over rows of a per-row term:
 //   TOKEN_SUM (Sec. 5.5):   term = log pi_T(y_t)
@@ -312,8 +312,8 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
 // known: incl (running sum and open-turn sums through the row), c_before
 // and st_before (the running sum and open turn's sum of log pi_T before it);
 // of rc only rc.e.sl (the row's loss term) is read.  With defer_traj the
-// trajectory's stop record and loss are left to the caller (the tiled scan
-// aggregates them per trajectory and tile).
+// trajectory's stop record and loss are left to the caller (the cluster scan
+// gathers them per trajectory and warp).
 __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const RowMeta& meta,
                                          const RowCarry& rc, const ScanElem& incl, double c_before,
                                          double st_before, bool timed_out, bool defer_traj = false);

@@ -120,12 +120,11 @@ __global__ void __launch_bounds__(kBatchThreads, 2) score_batch_kernel(const Bat
 // rank 0 merges the ranks' pairs through distributed shared memory, writes
 // the row's outputs and leaves its two log-probs in the workspace.  The scan
 // (turn statistics, stop rule, loss, profile, carried state) then runs as
-// the tiled scan on those log-probs (vocab_parallel.cu), launched as a
+// one cluster on those log-probs (vocab_parallel.cu), launched as a
 // programmatic dependent of this kernel.  In a window whose rows all finish
 // streaming together, a lookback per row cost a chain of prefixes after the
-// last row (12 us on a 512-row segment); the tiled scan scans 128 rows per
-// CTA, and a window of at most 16 such tiles runs as one cluster whose
-// tiles exchange their aggregates through distributed shared memory (no
+// last row (12 us on a 512-row segment); the cluster's CTAs scan 128 rows
+// each and exchange their aggregates through distributed shared memory (no
 // chain at all).
 namespace cg = cooperative_groups;
 constexpr int kSplitMaxCluster = 8;

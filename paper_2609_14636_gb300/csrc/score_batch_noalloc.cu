@@ -16,8 +16,8 @@
 //   STRIDE_ERR_TOO_LARGE before anything is launched);
 // - every call, on every stream, shares the one array per device, and the
 //   array keeps the previous call's contents: the call clears the part that
-//   must start at zero (tickets and flags) before its scan reads it (with
-//   cudaMemsetAsync, or from the small-window kernel).  Two calls that
+//   must start at zero (ticket and flags) with a kernel before the scoring
+//   kernel, where that needs any of it.  Two calls that
 //   overlap in time on the GPU race on the array and give wrong results:
 //   order them on one stream (or with events);
 // - the array's device address comes from cudaGetSymbolAddress (the first

@@ -52,7 +52,7 @@ struct BatchParams {
   uint32_t* flags;
   ScanSlot* agg;
   ScanSlot* incl;
-  float* ws_logp_s;  // per window row, written by the small-window kernel for the tiled scan
+  float* ws_logp_s;  // per window row, for the scan on log-probs and the persistent kernel's tiles
   float* ws_logp_t;
   uint64_t timeout_ns;
   uint32_t first_wave;  // CTAs of the split kernel that are resident from the start
@@ -141,9 +141,8 @@ cudaError_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, 
 }
 
 // Launchers return a cudaError_t from the launch.
-// Clears what must start at zero in the workspace (clear_bytes from its
-// start: the clearing kernel, or on the small-window path the split kernel
-// itself) and launches the batch scoring kernels.
+// Clears what the chosen kernel needs at zero in the workspace (at most
+// clear_bytes from its start) and launches the batch scoring kernels.
 cudaError_t launch_score_batch(const BatchParams& p, int dtype, bool vec, size_t clear_bytes, cudaStream_t stream);
 cudaError_t launch_score_batch_stream(const BatchParams& p, int dtype, bool aligned, cudaStream_t stream);
 // Whether that kernel scans its window itself, and what it needs at zero from
