@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "row_scan.cuh"
 #include "stride.h"
@@ -193,10 +194,11 @@ __device__ __forceinline__ TileElem elem_shfl_up(const TileElem& v, int d) { ret
 // Inclusive and exclusive scan of one element per thread over the CTA's
 // WARPS warps, in thread order: warp shuffles, then warp 0 scans the warps'
 // totals once (each thread then combines with one prefix).  `id` is the
-// identity; s_tot and s_pre hold WARPS elements.
-template <int WARPS, typename E>
-__device__ __forceinline__ void block_scan(const E& v, const E& id, int lane, int warp, E* s_tot, E* s_pre,
-                                           E& incl_out, E& excl_out) {
+// identity; s_tot and s_pre hold WARPS elements.  With ANY the answer is
+// whether any thread's `flag` is set (if so the scan is left there, in all).
+template <int WARPS, bool ANY = false, typename E>
+__device__ __forceinline__ bool block_scan(const E& v, const E& id, int lane, int warp, E* s_tot, E* s_pre,
+                                           E& incl_out, E& excl_out, bool flag = false) {
   E incl = v;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -205,7 +207,10 @@ __device__ __forceinline__ void block_scan(const E& v, const E& id, int lane, in
   }
   const E up1 = elem_shfl_up(incl, 1);
   if (lane == 31) s_tot[warp] = incl;
-  __syncthreads();
+  if (!ANY)
+    __syncthreads();
+  else if (__syncthreads_or(flag))
+    return true;
   if (warp == 0) {
     E t = lane < WARPS ? s_tot[lane] : id;
 #pragma unroll
@@ -220,6 +225,7 @@ __device__ __forceinline__ void block_scan(const E& v, const E& id, int lane, in
   const E wpre = s_pre[warp];
   incl_out = elem_combine(wpre, incl);
   excl_out = (lane == 0) ? wpre : elem_combine(wpre, up1);
+  return false;
 }
 
 // Largest j in [0, n) with a[j] <= r (a ascending, a[0] <= r).
@@ -379,35 +385,23 @@ __device__ __forceinline__ RowMeta no_row() {
   return m;
 }
 
-// What a row's log pi_T is weighed by in the running stop sum: 1, or for turn
-// means 1 / n_k.  EXACT (after a scoring kernel, whose own scan is fp64): once
-// per thread and turn in fp64, by Newton's iteration x + x (1 - n x) from the
-// fp32 quotient, whose error squares twice (2^-24 -> 2^-48 -> fp64).  Else
-// (log-probs as given) n_k itself, by which each log-prob is divided with one
-// fp32 rounding, 6e-8 of the term.
+// A row's term of the running stop sum: its log pi_T, for turn means divided
+// by the turn's length -- EXACT (after a scoring kernel, whose own scan is
+// fp64) in fp64, else (log-probs as given) with one fp32 rounding, 6e-8 of the
+// term.
 template <bool EXACT>
-struct StopWeight {
-  using type = double;
+struct StopTerm {
+  using Length = double;
 };
 template <>
-struct StopWeight<false> {
-  using type = float;
+struct StopTerm<false> {
+  using Length = float;
 };
 
-template <bool EXACT>
-__device__ __forceinline__ typename StopWeight<EXACT>::type stop_weight(const BatchParams& p, const RowMeta& m) {
-  if (p.mode != STRIDE_STOP_TURN_MEAN) return 1;
-  const int64_t n_k = max(m.turn_end - m.turn_start, (int64_t)1);
-  const float f = (float)n_k;
-  if (!EXACT) return f;
-  const double n = (double)n_k;
-  double x = (double)(1.0f / f);
-  x = fma(x, fma(-n, x, 1.0), x);
-  return fma(x, fma(-n, x, 1.0), x);
+template <typename Length>
+__device__ __forceinline__ double stop_term(const BatchParams& p, float lpt, Length n_k) {
+  return p.mode == STRIDE_STOP_TURN_MEAN ? (double)((Length)lpt / n_k) : (double)lpt;
 }
-
-__device__ __forceinline__ double stop_term(float lpt, double weight) { return (double)lpt * weight; }
-__device__ __forceinline__ double stop_term(float lpt, float weight) { return (double)(lpt / weight); }
 
 // A thread's R rows, what the layout alone says of them: rows tid * R + i of
 // the tile.
@@ -418,7 +412,7 @@ struct Rows {
   RowMeta first;     // the first row's
   float lam;         // its trajectory's threshold
   int what[R];       // kRow bits
-  typename StopWeight<EXACT>::type weight[R];
+  typename StopTerm<EXACT>::Length length[R];  // of the row's turn
   int bin[R];        // the profile's decile
   float lps[R], lpt[R];
 };
@@ -435,7 +429,7 @@ __device__ __forceinline__ void find_rows(const BatchParams& p, const TileLayout
   for (int i = 0; i < R; ++i) {
     const int j = tid * R + i;
     x.what[i] = 0;
-    x.weight[i] = 1;
+    x.length[i] = 1;
     x.bin[i] = 0;
     if (j >= n_here) continue;
     const int64_t r = p.row_begin + t0 + j;
@@ -443,7 +437,7 @@ __device__ __forceinline__ void find_rows(const BatchParams& p, const TileLayout
     const bool seeded = t0 + j == 0 || r == m.traj_start || m.bad;
     const bool fturn = r == m.turn_start;
     x.what[i] = kRowLive | (m.bad ? kRowBad : 0) | (seeded ? kRowSeeded : 0) | (fturn ? kRowTurnStart : 0);
-    x.weight[i] = i == 0 || seeded || fturn ? stop_weight<EXACT>(p, m) : x.weight[i > 0 ? i - 1 : 0];
+    x.length[i] = i == 0 || seeded || fturn ? max(m.turn_end - m.turn_start, (int64_t)1) : x.length[i > 0 ? i - 1 : 0];
     if (i == 0) {
       x.first = m;
       if (!m.bad) x.lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
@@ -483,46 +477,77 @@ __device__ __forceinline__ void load_logps(const float* __restrict__ logp_s, con
 // A sum of fp32 terms as the fp32 sum and the sum of its rounding errors
 // (Knuth's TwoSum): hi + lo is good to about 2^-45 of the summed magnitudes
 // over a tile, at seven FP32 operations where an fp64 add costs as much as 64.
-// An infinite or NaN hi is the answer (lo is NaN then).
+// Its range is fp32's.  So a tile (or, for the profile, a warp) that holds a
+// log-prob of 2^58 or more, an infinity or a NaN (`wide`) takes fp64 sums
+// instead: a sampled token masked with the lowest finite logit has log pi =
+// -3.4e38, and two of them, or its product with another log-prob, are finite
+// in fp64 alone.  Below 2^58 a difference is below 2^59, a product below
+// 2^117 and the sum of a tile's 512 rows below 2^126.  GB300, 30,011 rows of
+// 32,000 bf16 logits: pairs 519.3 us, fp64 in every tile 528.0.  Errors of the
+// turns' sums there, in pairs / fp64, of the summed magnitudes: log pi_T and d
+// none / none (48 bits hold them), logp_S * d 5e-16 / 3e-18.
 struct Sum2 {
   float hi, lo;
 };
 
-__device__ __forceinline__ void sum_add(Sum2& a, float hi, float lo) {
-  const float s = __fadd_rn(a.hi, hi), b = s - a.hi;
-  const float e = (a.hi - (s - b)) + (hi - b);
+__device__ __forceinline__ bool wide(float lps, float lpt) {
+  constexpr float kMost = 288230376151711744.0f;  // 2^58
+  return !(fabsf(lps) < kMost && fabsf(lpt) < kMost);
+}
+
+__device__ __forceinline__ void sum_add(double& a, double b) { a += b; }
+__device__ __forceinline__ void sum_add(Sum2& a, const Sum2& b) {
+  const float s = __fadd_rn(a.hi, b.hi), t = s - a.hi;
+  const float e = (a.hi - (s - t)) + (b.hi - t);
   a.hi = s;
-  a.lo += lo + e;
+  a.lo += b.lo + e;
 }
 
-// The product a b as a pair: exact, or rounded to fp32.
-template <bool EXACT>
-__device__ __forceinline__ Sum2 product(float a, float b) {
-  const float hi = __fmul_rn(a, b);
-  return Sum2{hi, EXACT ? fmaf(a, b, -hi) : 0.f};
+template <typename Sum>
+__device__ __forceinline__ Sum sum_of(float x);
+template <>
+__device__ __forceinline__ double sum_of<double>(float x) { return (double)x; }
+template <>
+__device__ __forceinline__ Sum2 sum_of<Sum2>(float x) { return Sum2{x, 0.f}; }
+
+// The product a b, exact; as a pair, of log-probs as given, rounded to fp32.
+template <typename Sum, bool EXACT>
+__device__ __forceinline__ Sum product(float a, float b) {
+  if constexpr (std::is_same<Sum, double>::value) {
+    return (double)a * (double)b;
+  } else {
+    const float hi = __fmul_rn(a, b);
+    return Sum2{hi, EXACT ? fmaf(a, b, -hi) : 0.f};
+  }
 }
 
-__device__ __forceinline__ double sum_value(const Sum2& a) {
-  return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi;
-}
+__device__ __forceinline__ double sum_value(double a) { return a; }
+__device__ __forceinline__ double sum_value(const Sum2& a) { return (double)a.hi + (double)a.lo; }
 
+__device__ __forceinline__ double sum_shfl_up(double a, int d) { return __shfl_up_sync(0xffffffffu, a, d); }
 __device__ __forceinline__ Sum2 sum_shfl_up(const Sum2& a, int d) {
   return Sum2{__shfl_up_sync(0xffffffffu, a.hi, d), __shfl_up_sync(0xffffffffu, a.lo, d)};
 }
 
-__device__ __forceinline__ Sum2 warp_sum(Sum2 v) {
+__device__ __forceinline__ double sum_shfl_xor(double a, int d) { return __shfl_xor_sync(0xffffffffu, a, d); }
+__device__ __forceinline__ Sum2 sum_shfl_xor(const Sum2& a, int d) {
+  return Sum2{__shfl_xor_sync(0xffffffffu, a.hi, d), __shfl_xor_sync(0xffffffffu, a.lo, d)};
+}
+
+template <typename Sum>
+__device__ __forceinline__ Sum warp_sum(Sum v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    sum_add(v, __shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+  for (int o = 16; o > 0; o >>= 1) sum_add(v, sum_shfl_xor(v, o));
   return v;
 }
 
 // Inclusive sum over the lanes from `head` (<= lane) to this one.
-__device__ __forceinline__ Sum2 seg_sum(Sum2 v, int head, int lane) {
+template <typename Sum>
+__device__ __forceinline__ Sum seg_sum(Sum v, int head, int lane) {
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const Sum2 o = sum_shfl_up(v, d);
-    if (lane - d >= head) sum_add(v, o.hi, o.lo);
+    const Sum o = sum_shfl_up(v, d);
+    if (lane - d >= head) sum_add(v, o);
   }
   return v;
 }
@@ -534,19 +559,22 @@ __device__ __forceinline__ int head_of(unsigned m, int lane) {
 
 // A thread's or tile's element without the carried state: sums since the last
 // seeded row (c) and since the last turn start (st, sd, sl).
+template <typename Sum>
 struct PassElem {
   double c;
-  Sum2 st, sd, sl;
+  Sum st, sd, sl;
   int flags;
   int seed;  // the last seeded row, from the tile's first; -1: none
 };
 
-__device__ __forceinline__ void open_rows(Sum2& v, const Sum2& before, bool turn) {
-  if (!turn) sum_add(v, before.hi, before.lo);
+template <typename Sum>
+__device__ __forceinline__ void open_rows(Sum& v, const Sum& before, bool turn) {
+  if (!turn) sum_add(v, before);
 }
 
-__device__ __forceinline__ PassElem elem_combine(const PassElem& a, const PassElem& b) {
-  PassElem r;
+template <typename Sum>
+__device__ __forceinline__ PassElem<Sum> elem_combine(const PassElem<Sum>& a, const PassElem<Sum>& b) {
+  PassElem<Sum> r;
   r.c = (b.flags & kRestartSum) ? b.c : a.c + b.c;
   const bool turn = (b.flags & kRestartTurn) != 0;
   r.st = b.st;
@@ -560,8 +588,9 @@ __device__ __forceinline__ PassElem elem_combine(const PassElem& a, const PassEl
   return r;
 }
 
-__device__ __forceinline__ PassElem elem_shfl_up(const PassElem& v, int d) {
-  PassElem o;
+template <typename Sum>
+__device__ __forceinline__ PassElem<Sum> elem_shfl_up(const PassElem<Sum>& v, int d) {
+  PassElem<Sum> o;
   o.c = __shfl_up_sync(0xffffffffu, v.c, d);
   o.st = sum_shfl_up(v.st, d);
   o.sd = sum_shfl_up(v.sd, d);
@@ -571,22 +600,20 @@ __device__ __forceinline__ PassElem elem_shfl_up(const PassElem& v, int d) {
   return o;
 }
 
-// Index of the largest thread of the CTA with `has`, -1 if none (two words of
-// s_any per warp; the caller synchronises before s_any is used again).
-__device__ __forceinline__ int last_thread(unsigned ballot, int lane, int warp, int* s_any) {
-  if (lane == 0) s_any[warp] = ballot ? warp * 32 + 31 - __clz(ballot) : -1;
-  __syncthreads();
-  int n = -1;
+// Whether the thread's rows need fp64 sums (bad rows are NaN either way).
+template <int R, bool EXACT>
+__device__ __forceinline__ bool rows_wide(const Rows<R, EXACT>& x) {
+  bool any = false;
 #pragma unroll
-  for (int w = 0; w < kPassWarps; ++w) n = max(n, s_any[w]);
-  return n;
+  for (int i = 0; i < R; ++i) any |= (x.what[i] & (kRowLive | kRowBad)) == kRowLive && wide(x.lps[i], x.lpt[i]);
+  return any;
 }
 
 // The thread's rows as one element.
-template <int R, bool EXACT>
-__device__ __forceinline__ PassElem rows_elem(const Rows<R, EXACT>& x, int tid) {
-  const Sum2 zero = {0.f, 0.f};
-  PassElem e = {0.0, zero, zero, zero, 0, -1};
+template <typename Sum, int R, bool EXACT>
+__device__ __forceinline__ PassElem<Sum> rows_elem(const BatchParams& p, const Rows<R, EXACT>& x, int tid) {
+  const Sum zero = sum_of<Sum>(0.f);
+  PassElem<Sum> e = {0.0, zero, zero, zero, 0, -1};
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int what = x.what[i];
@@ -603,22 +630,21 @@ __device__ __forceinline__ PassElem rows_elem(const Rows<R, EXACT>& x, int tid) 
       e.st = e.sd = e.sl = zero;
       e.flags = (e.flags & kRestartSum) | kRestartTurn | (seeded ? kFromSeed : 0);
     }
-    const Sum2 l = product<EXACT>(lps, dd);
-    e.c += stop_term(lpt, x.weight[i]);
-    sum_add(e.st, lpt, 0.f);
-    sum_add(e.sd, dd, 0.f);
-    sum_add(e.sl, l.hi, l.lo);
+    e.c += stop_term(p, lpt, x.length[i]);
+    sum_add(e.st, sum_of<Sum>(lpt));
+    sum_add(e.sd, sum_of<Sum>(dd));
+    sum_add(e.sl, product<Sum, EXACT>(lps, dd));
   }
   return e;
 }
 
 // The thread's rows into the CTA's profile: runs of equal deciles summed in
 // registers, neighbouring threads' open runs of one decile together.
-template <int R, bool EXACT>
-__device__ __forceinline__ void rows_profile(const Rows<R, EXACT>& x, int lane, double* s_prof) {
-  const Sum2 zero = {0.f, 0.f};
+template <typename Sum, int R, bool EXACT>
+__device__ __forceinline__ void rows_profile_in(const Rows<R, EXACT>& x, int lane, double* s_prof) {
+  const Sum zero = sum_of<Sum>(0.f);
   int bin = -1, n = 0;
-  Sum2 d = zero, t = zero;
+  Sum d = zero, t = zero;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     if ((x.what[i] & (kRowLive | kRowBad)) != kRowLive) continue;
@@ -632,8 +658,8 @@ __device__ __forceinline__ void rows_profile(const Rows<R, EXACT>& x, int lane, 
       n = 0;
       d = t = zero;
     }
-    sum_add(d, x.lps[i] - x.lpt[i], 0.f);
-    sum_add(t, x.lpt[i], 0.f);
+    sum_add(d, sum_of<Sum>(x.lps[i] - x.lpt[i]));
+    sum_add(t, sum_of<Sum>(x.lpt[i]));
     ++n;
   }
   __syncwarp();
@@ -654,10 +680,12 @@ __device__ __forceinline__ void rows_profile(const Rows<R, EXACT>& x, int lane, 
   }
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+template <int R, bool EXACT>
+__device__ __forceinline__ void rows_profile(const Rows<R, EXACT>& x, int lane, double* s_prof) {
+  if (__any_sync(0xffffffffu, rows_wide(x)))
+    rows_profile_in<double>(x, lane, s_prof);
+  else
+    rows_profile_in<Sum2>(x, lane, s_prof);
 }
 
 // A slot that the first pass wrote, past this SM's L1.
@@ -668,23 +696,85 @@ __device__ __forceinline__ ScanSlot load_slot(const ScanSlot* s) {
 }
 
 // First pass: tile t's aggregate in agg[t], its kRestart marks in flags[t],
-// and in incl[w] the carried state of every seeded row w.
+// and in incl[w] the carried state of every seeded row w.  z is the carried
+// state of the thread's last seeded row.  False, with nothing written, if the
+// tile's sums need more than Sum.
+template <typename Sum, int R, bool EXACT>
+__device__ __forceinline__ bool aggregate_tile(const BatchParams& p, int64_t tile, int tid, const Rows<R, EXACT>& x,
+                                               const ScanSlot& z) {
+  __shared__ int s_last[2][kPassWarps];
+  __shared__ double s_c[kPassWarps], s_base[4];
+  __shared__ Sum s_open[3][kPassWarps];
+  const int lane = tid & 31, warp = tid >> 5;
+  if (tid < 4) s_base[tid] = 0.0;
+  const Sum zero = sum_of<Sum>(0.f);
+  const PassElem<Sum> e = rows_elem<Sum>(p, x, tid);
+  double c = e.c;
+  Sum st = e.st, sd = e.sd, sl = e.sl;
+  // only what follows the last restart counts: from thread own_c on in the
+  // running sum, from own_t on in the open turn's (-1: from the first)
+  const unsigned b_sum = __ballot_sync(0xffffffffu, (e.flags & kRestartSum) != 0);
+  const unsigned b_turn = __ballot_sync(0xffffffffu, (e.flags & kRestartTurn) != 0);
+  if (lane == 0) {
+    s_last[0][warp] = b_sum ? warp * 32 + 31 - __clz(b_sum) : -1;
+    s_last[1][warp] = b_turn ? warp * 32 + 31 - __clz(b_turn) : -1;
+  }
+  if (std::is_same<Sum, double>::value)
+    __syncthreads();
+  else if (__syncthreads_or(rows_wide(x)))
+    return false;
+  int own_c = -1, own_t = -1;
+#pragma unroll
+  for (int w = 0; w < kPassWarps; ++w) {
+    own_c = max(own_c, s_last[0][w]);
+    own_t = max(own_t, s_last[1][w]);
+  }
+  if (tid == own_c) s_base[0] = z.c;
+  if (tid == own_t && (e.flags & kFromSeed)) {
+    s_base[1] = z.st;
+    s_base[2] = z.sd;
+    s_base[3] = z.sl;
+  }
+  c = warp * 32 + 31 < own_c ? 0.0 : warp_sum(tid >= own_c ? c : 0.0);
+  if (tid < own_t) st = sd = sl = zero;
+  if (warp * 32 + 31 >= own_t) {
+    st = warp_sum(st);
+    sd = warp_sum(sd);
+    sl = warp_sum(sl);
+  }
+  if (lane == 0) {
+    s_c[warp] = c;
+    s_open[0][warp] = st;
+    s_open[1][warp] = sd;
+    s_open[2][warp] = sl;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    c = warp_sum(lane < kPassWarps ? s_c[lane] : 0.0);
+    st = warp_sum(lane < kPassWarps ? s_open[0][lane] : zero);
+    sd = warp_sum(lane < kPassWarps ? s_open[1][lane] : zero);
+    sl = warp_sum(lane < kPassWarps ? s_open[2][lane] : zero);
+    if (lane == 0) {
+      p.agg[tile] =
+          ScanSlot{s_base[0] + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl)};
+      p.flags[tile] = (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0);
+    }
+  }
+  return true;
+}
+
 template <int R, bool EXACT>
 __global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const BatchParams p,
                                                                      const float* __restrict__ logp_s,
                                                                      const float* __restrict__ logp_t, bool early) {
   constexpr int kRows = R * kPassThreads;
   __shared__ TileLayout<kRows> L;
-  __shared__ int s_any[2][kPassWarps];
-  __shared__ double s_c[kPassWarps], s_base[4];
-  __shared__ Sum2 s_open[3][kPassWarps];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int64_t tile = blockIdx.x;
   const int64_t t0 = tile * kRows;
   const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
   Rows<R, EXACT> x;
-  ScanSlot z = {0.0, 0.0, 0.0, 0.0};  // of the thread's last seeded row
-  if (tid < 4) s_base[tid] = 0.0;
+  ScanSlot z = {0.0, 0.0, 0.0, 0.0};
   // Everything before this kernel is complete past the wait, and only then
   // may the second pass come in: what it reads before its own wait (the
   // layout, the log-probs, lambda) is complete too.  After a scoring kernel
@@ -699,44 +789,7 @@ __global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const B
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   load_logps<R>(logp_s, logp_t, t0, tid, x);
-  const PassElem e = rows_elem<R, EXACT>(x, tid);
-  double c = e.c;
-  Sum2 st = e.st, sd = e.sd, sl = e.sl;
-  // only what follows the last restart counts
-  const int own_c = last_thread(__ballot_sync(0xffffffffu, (e.flags & kRestartSum) != 0), lane, warp, s_any[0]);
-  const int own_t = last_thread(__ballot_sync(0xffffffffu, (e.flags & kRestartTurn) != 0), lane, warp, s_any[1]);
-  if (tid == own_c) s_base[0] = z.c;
-  if (tid == own_t && (e.flags & kFromSeed)) {
-    s_base[1] = z.st;
-    s_base[2] = z.sd;
-    s_base[3] = z.sl;
-  }
-  c = warp * 32 + 31 < own_c ? 0.0 : warp_sum(tid >= own_c ? c : 0.0);
-  if (tid < own_t) st = sd = sl = Sum2{0.f, 0.f};
-  if (warp * 32 + 31 >= own_t) {
-    st = warp_sum(st);
-    sd = warp_sum(sd);
-    sl = warp_sum(sl);
-  }
-  if (lane == 0) {
-    s_c[warp] = c;
-    s_open[0][warp] = st;
-    s_open[1][warp] = sd;
-    s_open[2][warp] = sl;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    const Sum2 zero = {0.f, 0.f};
-    c = warp_sum(lane < kPassWarps ? s_c[lane] : 0.0);
-    st = warp_sum(lane < kPassWarps ? s_open[0][lane] : zero);
-    sd = warp_sum(lane < kPassWarps ? s_open[1][lane] : zero);
-    sl = warp_sum(lane < kPassWarps ? s_open[2][lane] : zero);
-    if (lane == 0) {
-      p.agg[tile] =
-          ScanSlot{s_base[0] + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl)};
-      p.flags[tile] = (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0);
-    }
-  }
+  if (!aggregate_tile<Sum2>(p, tile, tid, x, z)) aggregate_tile<double>(p, tile, tid, x, z);
 }
 
 // Between the passes of a window of many tiles: the aggregates replaced by
@@ -798,32 +851,36 @@ __global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(ScanSlot* a
 
 // A trajectory's share of a thread's rows: the loss of its retained rows and
 // its first crossing of lambda here.
+template <typename Sum>
 struct TrajPart {
   int32_t traj, count, cross_turn;  // traj -1: none
-  Sum2 loss;
+  Sum loss;
   int64_t cross_row;  // from the trajectory's first row; -1: none
 };
 
-__device__ __forceinline__ void record_cross(stride_scan_state* sp, const TrajPart& t) {
+template <typename Sum>
+__device__ __forceinline__ void record_cross(stride_scan_state* sp, const TrajPart<Sum>& t) {
   atomicMin(reinterpret_cast<unsigned long long*>(&sp->stop_row), (unsigned long long)t.cross_row);
   atomicMin(reinterpret_cast<unsigned int*>(&sp->stop_turn), (unsigned int)t.cross_turn);
   sp->stopped = 1;
 }
 
-__device__ __forceinline__ void record_loss(stride_scan_state* sp, const Sum2& loss, int count) {
+template <typename Sum>
+__device__ __forceinline__ void record_loss(stride_scan_state* sp, const Sum& loss, int count) {
   atomicAdd(&sp->loss, sum_value(loss));
   atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), (unsigned long long)count);
 }
 
 // The trajectories' records: neighbouring threads of one trajectory together
 // (the lowest crossing, the sum of the losses).  Warp-wide.
-__device__ __forceinline__ void record_parts(const BatchParams& p, const TrajPart& part, int lane) {
+template <typename Sum>
+__device__ __forceinline__ void record_parts(const BatchParams& p, const TrajPart<Sum>& part, int lane) {
   __syncwarp();
   const int prev = __shfl_up_sync(0xffffffffu, part.traj, 1);
   const unsigned m_run = __ballot_sync(0xffffffffu, lane == 0 || part.traj != prev);
   const unsigned m_cross = __ballot_sync(0xffffffffu, part.cross_row >= 0);
   const int h = head_of(m_run, lane);
-  const Sum2 loss = seg_sum(part.loss, h, lane);
+  const Sum loss = seg_sum(part.loss, h, lane);
   int count = part.count;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -841,12 +898,13 @@ __device__ __forceinline__ void record_parts(const BatchParams& p, const TrajPar
 // Completes the thread's rows, given the exclusive prefix of its rows inside
 // the tile, the tile's (pre) and the carried state of the tile's seeded rows
 // (seed(j), which covers excl.seed too).
-template <int R, bool EXACT, int ROWS, typename Seed>
+template <typename Sum, int R, bool EXACT, int ROWS, typename Seed>
 __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLayout<ROWS>& L, int64_t t0, int tid,
-                                              const Rows<R, EXACT>& x, const PassElem& excl, const double* pre, Seed&& seed) {
+                                              const Rows<R, EXACT>& x, const PassElem<Sum>& excl, const double* pre,
+                                              Seed&& seed) {
   const int lane = tid & 31;
   const float nan = __int_as_float(0x7fc00000);
-  const Sum2 zero = {0.f, 0.f};
+  const Sum zero = sum_of<Sum>(0.f);
   ScanSlot z = {0.0, 0.0, 0.0, 0.0};  // the last seeded row's before this thread
   if (excl.seed >= 0 && (x.what[0] & kRowLive)) z = seed(excl.seed);
   double c = (excl.seed >= 0 ? z.c : pre[0]) + excl.c;
@@ -857,8 +915,8 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     b_sd = from ? z.sd : 0.0;
     b_sl = from ? z.sl : 0.0;
   }
-  Sum2 st = excl.st, sd = excl.sd, sl = excl.sl;
-  TrajPart part = {-1, 0, 0, zero, -1};
+  Sum st = excl.st, sd = excl.sd, sl = excl.sl;
+  TrajPart<Sum> part = {-1, 0, 0, zero, -1};
   bool kept = false;  // in turn mode the same for all of a turn's rows
   float lam = x.lam;
   RowMeta m = x.first;
@@ -878,7 +936,7 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     }
     if (i > 0) seek_row(p, L, r, m);
     const float lps = x.lps[i], lpt = x.lpt[i], dd = lps - lpt;
-    const Sum2 l = product<EXACT>(lps, dd);
+    const Sum l = product<Sum, EXACT>(lps, dd);
     const bool seeded = (what & kRowSeeded) != 0, fturn = (what & kRowTurnStart) != 0;
     stride_scan_state* sp = p.state + m.traj;
     if (seeded || fturn) {
@@ -898,7 +956,7 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
         if (part.count > 0) record_loss(p.state + part.traj, part.loss, part.count);
       }
       if (i > 0) lam = p.lambda ? __ldg(p.lambda + m.traj) : p.lambda_all;
-      part = TrajPart{m.traj, 0, 0, zero, -1};
+      part = TrajPart<Sum>{m.traj, 0, 0, zero, -1};
     }
     const bool turn_last = r == m.turn_end - 1;
     const bool token_sum = p.mode == STRIDE_STOP_TOKEN_SUM;
@@ -908,17 +966,17 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     if (token_sum) {
       kept = r == m.traj_start || !(c < (double)lam);
     } else if (i == 0 || seeded || fturn) {
-      const double before = EXACT ? c - (b_st + sum_value(st)) * x.weight[i]
-                                  : c - (double)(((float)b_st + st.hi) / x.weight[i]);
+      using Length = typename StopTerm<EXACT>::Length;
+      const double before = c - (double)((Length)(b_st + sum_value(st)) / x.length[i]);
       kept = m.local_turn == 0 || !(before < (double)lam);
     }
-    c += stop_term(lpt, x.weight[i]);
-    sum_add(st, lpt, 0.f);
-    sum_add(sd, dd, 0.f);
-    sum_add(sl, l.hi, l.lo);
+    c += stop_term(p, lpt, x.length[i]);
+    sum_add(st, sum_of<Sum>(lpt));
+    sum_add(sd, sum_of<Sum>(dd));
+    sum_add(sl, l);
     if (p.out.opd) p.out.opd[w] = dd;
     if (kept) {
-      sum_add(part.loss, l.hi, l.lo);
+      sum_add(part.loss, l);
       ++part.count;
     }
     if ((token_sum || turn_last) && part.cross_row < 0 && c < (double)lam) {
@@ -1191,7 +1249,7 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   if (p.profile) {  // (while the aggregates are on their way)
     row.lps[0] = lps;
     row.lpt[0] = lpt;
-    rows_profile<1>(row, lane, s_prof);
+    rows_profile(row, lane, s_prof);
   }
   cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
   if (warp == 0) {
@@ -1229,7 +1287,7 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   }
 
   // 6. the trajectories' stop records and losses, once per trajectory and warp
-  TrajPart part = {-1, 0, 0, {0.f, 0.f}, -1};
+  TrajPart<Sum2> part = {-1, 0, 0, {0.f, 0.f}, -1};
   if (live && !meta.bad) {
     const int64_t n_k = meta.turn_end - meta.turn_start;
     const bool turn_last = (r == meta.turn_end - 1);
@@ -1255,37 +1313,27 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   }
 }
 
-// Second pass.
-template <int R, bool EXACT>
-__global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const BatchParams p,
-                                                                       const float* __restrict__ logp_s,
-                                                                       const float* __restrict__ logp_t, int64_t n_tiles,
-                                                                       bool prefixed, bool validate) {
-  constexpr int kRows = R * kPassThreads;
-  __shared__ TileLayout<kRows> L;
-  __shared__ PassElem s_tot[kPassWarps], s_wpre[kPassWarps];
+// Second pass.  False, with nothing written, if the tile's sums need more
+// than Sum.
+template <typename Sum, int R, bool EXACT, int ROWS>
+__device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLayout<ROWS>& L, int64_t tile, int tid,
+                                              const Rows<R, EXACT>& x, bool prefixed) {
+  __shared__ PassElem<Sum> s_tot[kPassWarps], s_wpre[kPassWarps];
   __shared__ int s_near[2][kPassWarps];
   __shared__ double s_fold[4][kPassWarps];
   __shared__ double s_pre[4];
   __shared__ int s_needs;
-  __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int64_t tile = blockIdx.x;
-  const int64_t t0 = tile * kRows;
-  const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
-  if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int64_t t0 = tile * ROWS;
   if (tid < 4) s_pre[tid] = 0.0;
-  stage_layout(p, p.row_begin + t0, n_here, tid, L);
-  Rows<R, EXACT> x;
-  find_rows<R, EXACT>(p, L, t0, n_here, tid, x, [](int, const ScanSlot&) {});  // (the first pass set the states aside)
-  load_logps<R>(logp_s, logp_t, t0, tid, x);
   if (tid == 0) s_needs = !(x.what[0] & kRowSeeded);
-  if (p.profile) rows_profile<R>(x, lane, s_prof);
-  const Sum2 zero = {0.f, 0.f};
-  const PassElem id = {0.0, zero, zero, zero, 0, -1};
-  PassElem incl, excl;
-  block_scan<kPassWarps>(rows_elem<R, EXACT>(x, tid), id, lane, warp, s_tot, s_wpre, incl, excl);
+  const Sum zero = sum_of<Sum>(0.f);
+  const PassElem<Sum> id = {0.0, zero, zero, zero, 0, -1};
+  PassElem<Sum> incl, excl;
+  constexpr bool kNarrow = std::is_same<Sum, Sum2>::value;
+  if (block_scan<kPassWarps, kNarrow>(rows_elem<Sum>(p, x, tid), id, lane, warp, s_tot, s_wpre, incl, excl,
+                                      kNarrow && rows_wide(x)))
+    return false;
 
   // ---- the first pass's results
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1353,7 +1401,30 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
     }
   }
   __syncthreads();
-  complete_rows<R, EXACT>(p, L, t0, tid, x, excl, s_pre, [&](int j) { return load_slot(p.incl + t0 + j); });
+  complete_rows<Sum>(p, L, t0, tid, x, excl, s_pre, [&](int j) { return load_slot(p.incl + t0 + j); });
+  return true;
+}
+
+template <int R, bool EXACT>
+__global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const BatchParams p,
+                                                                       const float* __restrict__ logp_s,
+                                                                       const float* __restrict__ logp_t, int64_t n_tiles,
+                                                                       bool prefixed, bool validate) {
+  constexpr int kRows = R * kPassThreads;
+  __shared__ TileLayout<kRows> L;
+  __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
+  const int tid = threadIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int64_t tile = blockIdx.x;
+  const int64_t t0 = tile * kRows;
+  const int n_here = (int)min((int64_t)kRows, p.n_rows - t0);
+  if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
+  stage_layout(p, p.row_begin + t0, n_here, tid, L);
+  Rows<R, EXACT> x;
+  find_rows<R, EXACT>(p, L, t0, n_here, tid, x, [](int, const ScanSlot&) {});  // (the first pass set the states aside)
+  load_logps<R>(logp_s, logp_t, t0, tid, x);
+  if (p.profile) rows_profile(x, tid & 31, s_prof);
+  if (!complete_tile<Sum2>(p, L, tile, tid, x, prefixed)) complete_tile<double>(p, L, tile, tid, x, prefixed);
   if (p.profile && tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
   if (validate) check_layout(p, tile, n_tiles, tid);
 }
