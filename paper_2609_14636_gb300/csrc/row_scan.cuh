@@ -45,18 +45,20 @@ struct ScanElem {
   double st;  // sum of log pi_T within the open turn
   double sd;  // sum of d within the open turn
   double sl;  // sum of the OPD-loss terms logp_S * d within the open turn
+  double c0;  // the sum c before the open turn (with fturn)
   int fturn;  // the range contains a turn's first row
 };
 
 // a (earlier rows) (+) b (later rows).  c never resets inside a lookback
 // (trajectory starts publish inclusive prefixes); st, sd and sl restart at a
-// turn's first row.
+// turn's first row, where c0 is taken.
 __device__ __forceinline__ ScanElem combine(const ScanElem& a, const ScanElem& b) {
   ScanElem r;
   r.c = a.c + b.c;
   r.st = b.fturn ? b.st : a.st + b.st;
   r.sd = b.fturn ? b.sd : a.sd + b.sd;
   r.sl = b.fturn ? b.sl : a.sl + b.sl;
+  r.c0 = b.fturn ? a.c + b.c0 : a.c0;
   r.fturn = a.fturn | b.fturn;
   return r;
 }
@@ -71,8 +73,15 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// c0 of a row's or tile's published element: in its flag's line, the
+// aggregate's (1) and the inclusive prefix's (2) 8 bytes.
+__device__ __forceinline__ double* slot_c0(uint32_t* flag, bool inclusive) {
+  return reinterpret_cast<double*>(flag) + (inclusive ? 2 : 1);
+}
+
 __device__ __forceinline__ void publish(ScanSlot* slot, uint32_t* flag, const ScanElem& e,
                                         uint32_t status) {
+  *slot_c0(flag, (status & kStMask) == kStIncl) = e.c0;
   slot->c = e.c;
   slot->st = e.st;
   slot->sd = e.sd;
@@ -158,7 +167,7 @@ __device__ __forceinline__ void validate_layout(const BatchParams& p, int64_t t)
 // Folds published predecessors of `tile` back to the nearest inclusive
 // prefix.  Warp-wide; every lane returns the same exclusive prefix.
 static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane, bool& timed_out) {
-  ScanElem excl = {0.0, 0.0, 0.0, 0.0, 0};
+  ScanElem excl = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
   int64_t j = tile - 1;
   const uint64_t t0 = globaltimer_ns();
   while (true) {
@@ -179,7 +188,7 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
     const bool is_incl = (f & kStMask) == kStIncl;
     const unsigned inc = __ballot_sync(0xffffffffu, is_incl);
     const int stop = inc ? __ffs(inc) - 1 : 31;
-    ScanElem v = {0.0, 0.0, 0.0, 0.0, 0};
+    ScanElem v = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
     if (valid && lane <= stop && !(f & kFlagTimedOut)) {
       const ScanSlot* src = is_incl ? (p.incl + idx) : (p.agg + idx);
       const double2 a = __ldcg(reinterpret_cast<const double2*>(src));
@@ -188,6 +197,7 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
       v.st = a.y;
       v.sd = b.x;
       v.sl = b.y;
+      v.c0 = __ldcg(slot_c0(p.flags + idx * kFlagStride, is_incl));
       v.fturn = (is_incl || (f & kFlagTurnStart)) ? 1 : 0;
     }
     if (f & kFlagTimedOut) timed_out = true;
@@ -200,6 +210,7 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
       o.st = __shfl_down_sync(0xffffffffu, v.st, d);
       o.sd = __shfl_down_sync(0xffffffffu, v.sd, d);
       o.sl = __shfl_down_sync(0xffffffffu, v.sl, d);
+      o.c0 = __shfl_down_sync(0xffffffffu, v.c0, d);
       o.fturn = __shfl_down_sync(0xffffffffu, v.fturn, d);
       if (lane + d < 32) v = combine(o, v);
     }
@@ -208,6 +219,7 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
     win.st = __shfl_sync(0xffffffffu, v.st, 0);
     win.sd = __shfl_sync(0xffffffffu, v.sd, 0);
     win.sl = __shfl_sync(0xffffffffu, v.sl, 0);
+    win.c0 = __shfl_sync(0xffffffffu, v.c0, 0);
     win.fturn = __shfl_sync(0xffffffffu, v.fturn, 0);
     excl = combine(win, excl);
     if (inc) break;
@@ -226,9 +238,18 @@ struct RowCarry {
   ScanElem e;
   ScanElem incl;      // valid for seeded tiles
   double c_before;    // running sum before this row (seeded tiles)
-  double st_before;   // open-turn sum of log pi_T before this row (seeded tiles)
   int seeded;
 };
+
+// Whether the rule fired before a row's turn, in turn mode: c0 is the sum
+// before that turn.  Of a turn that was open where the window began the
+// carried state tells: the rule is recorded there if it had fired (what this
+// window records is never below that turn).
+__device__ __forceinline__ bool fired_before_turn(const BatchParams& p, const RowMeta& meta, double c0, float lam) {
+  if (meta.turn_start < p.row_begin)
+    return (uint32_t)__ldcg(&p.state[meta.traj].stop_turn) < (uint32_t)meta.local_turn;
+  return c0 < (double)lam;
+}
 
 __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t tile, int64_t r,
                                                  const RowMeta& meta, bool token_ok, float xs, float xt,
@@ -258,6 +279,7 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
   e.st = (double)lpt;
   e.sd = (double)dd;
   e.sl = (double)lps * (double)dd;  // -log pi_S * r_t (Eq. 2)
+  e.c0 = 0.0;
   e.fturn = (r == meta.turn_start) ? 1 : 0;
   if (p.profile && !meta.bad) {
     const int j = (int)((10 * (r - meta.turn_start)) / n_k);  // Observation 1 decile
@@ -268,7 +290,6 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
   rc.e = e;
   rc.seeded = (tile == 0) || (r == meta.traj_start) || meta.bad;
   rc.c_before = 0.0;
-  rc.st_before = 0.0;
   if (rc.seeded) {
     if (meta.bad) {
       rc.incl = e;  // NaN terms; nothing downstream of a bad row is meaningful
@@ -279,11 +300,11 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
       const double sd0 = __ldcg(&sp->turn_sum_d);
       const double sl0 = __ldcg(&sp->turn_sum_l);
       rc.c_before = cum0;
-      rc.st_before = e.fturn ? 0.0 : st0;
       rc.incl.c = cum0 + e.c;
       rc.incl.st = e.fturn ? e.st : st0 + e.st;
       rc.incl.sd = e.fturn ? e.sd : sd0 + e.sd;
       rc.incl.sl = e.fturn ? e.sl : sl0 + e.sl;
+      rc.incl.c0 = cum0;
       rc.incl.fturn = 1;
     }
     publish(p.incl + tile, p.flags + tile * kFlagStride, rc.incl, kStIncl);
@@ -303,43 +324,43 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
 // is: no test precedes it (with a prefix-buffer offset already below lambda
 // that token or turn triggers the stop and is kept).  After it, in token
 // mode that is "the running sum before the row is >= lambda"; in turn mode
-// "the running sum through the previous turn is >= lambda", which is the
-// running sum before the row minus the row's turn's terms so far
-// (c_before - st_before / n_k).  The sums are monotone, so this selects
-// exactly the rows up to the first crossing (its turn, in turn mode).
-// rc is read in lane 0.
+// "the running sum before the row's turn (c0) is >= lambda": the sum that the
+// previous turn's test saw, carried along rather than formed again as the
+// sum before the row minus the turn's terms so far, which near lambda, or
+// beside a masked token's term, differs from it.  The sums are monotone, so
+// this selects exactly the rows up to the first crossing (its turn, in turn
+// mode).  rc is read in lane 0.
 // row_tail is the single-thread part once the row's inclusive prefix is
-// known: incl (running sum and open-turn sums through the row), c_before
-// and st_before (the running sum and open turn's sum of log pi_T before it);
-// of rc only rc.e.sl (the row's loss term) is read.  With defer_traj the
-// trajectory's stop record and loss are left to the caller (the cluster scan
-// gathers them per trajectory and warp).
+// known: incl (running sum and open-turn sums through the row, and before its
+// turn) and c_before (the running sum before it); of rc only rc.e.sl (the
+// row's loss term) is read.  With defer_traj the trajectory's stop record and
+// loss are left to the caller (the cluster scan gathers them per trajectory
+// and warp).
 __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const RowMeta& meta,
                                          const RowCarry& rc, const ScanElem& incl, double c_before,
-                                         double st_before, bool timed_out, bool defer_traj = false);
+                                         bool timed_out, bool defer_traj = false);
 
 __device__ __forceinline__ void row_resolve(const BatchParams& p, int64_t tile, int64_t r,
                                             const RowMeta& meta, RowCarry rc, int lane) {
   const int seeded = __shfl_sync(0xffffffffu, rc.seeded, 0);
   ScanElem incl = rc.incl;
-  double c_before = rc.c_before, st_before = rc.st_before;
+  double c_before = rc.c_before;
   bool timed_out = false;
   if (!seeded) {
     const ScanElem excl = lookback(p, tile, lane, timed_out);
     if (lane == 0) {
       incl = combine(excl, rc.e);
       c_before = excl.c;
-      st_before = rc.e.fturn ? 0.0 : excl.st;
       publish(p.incl + tile, p.flags + tile * kFlagStride, incl, kStIncl);
     }
   }
   if (lane != 0) return;
-  row_tail(p, r, meta, rc, incl, c_before, st_before, timed_out);
+  row_tail(p, r, meta, rc, incl, c_before, timed_out);
 }
 
 __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const RowMeta& meta,
                                          const RowCarry& rc, const ScanElem& incl, double c_before,
-                                         double st_before, bool timed_out, bool defer_traj) {
+                                         bool timed_out, bool defer_traj) {
   if (timed_out) set_status(p.dev_status, STRIDE_DEV_TIMEOUT);
   if (meta.bad) return;
   const int64_t n_k = meta.turn_end - meta.turn_start;
@@ -367,8 +388,9 @@ __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const 
       sp->stopped = 1;
     }
     const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
-    const double before = (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before : c_before - st_before / (double)n_k;
-    if (first || !(before < (double)lam)) {  // the previous test did not fire (a NaN lambda never does)
+    const bool fired =
+        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before < (double)lam : fired_before_turn(p, meta, incl.c0, lam);
+    if (first || !fired) {  // the previous test did not fire (a NaN lambda never does)
       atomicAdd(&sp->loss, rc.e.sl);
       atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), 1ull);
     }

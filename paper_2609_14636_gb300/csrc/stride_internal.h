@@ -10,16 +10,18 @@
 
 namespace stride {
 
-// One published scan element of the batch kernel's lookback (32 bytes):
-// running-sum terms, and the open turn's sums of log pi_T, d and logp_S * d.
+// One published scan element of a lookback (32 bytes): running-sum terms, and
+// the open turn's sums of log pi_T, d and logp_S * d.  (The running sum before
+// the open turn is published in the flag's line: row_scan.cuh.)
 struct alignas(32) ScanSlot {
   double c, st, sd, sl;
 };
 
-// Row r's scan flag is flags[r * kFlagStride]: one flag per 128-byte line.
-// Every row of a window polls and reads its predecessors' flags; packed 32 to
-// a line, a few lines took all of that traffic, and GB300 windows of 512-
-// 1,024 rows scored 3-12 % faster with the flags spread out.
+// The scan flag of row r (one CTA per row) or of 32-row tile r (persistent
+// kernel) is flags[r * kFlagStride]: one flag per 128-byte line.  Each polls
+// and reads its predecessors' flags; packed 32 to a line, a few lines took all
+// of that traffic, and GB300 windows of 512-1,024 rows scored 3-12 % faster,
+// with a flag per row, with the flags spread out.
 constexpr int kFlagStride = 32;
 
 constexpr uint64_t kWaitTimeoutNs = 2000000000ull;  // bound on any single device-side wait

@@ -178,6 +178,18 @@ __device__ __forceinline__ TileElem tile_combine(const TileElem& a, const TileEl
   return r;
 }
 
+// A tile's aggregate or prefix: with (for turn means) the sum c before the
+// last turn mark, a turn's first row or a seeded one, counted from where c is.
+struct TileAgg {
+  TileElem e;
+  double c0;
+};
+
+// c0 of a (earlier, whose c0 is a_c0) and b together.
+__device__ __forceinline__ double tile_c0(const TileElem& a, double a_c0, const TileAgg& b) {
+  return !(b.e.flags & kRestartTurn) ? a_c0 : (b.e.flags & kRestartSum) ? b.c0 : a.c + b.c0;
+}
+
 __device__ __forceinline__ TileElem tile_shfl_up(const TileElem& v, int d) {
   TileElem o;
   o.c = __shfl_up_sync(0xffffffffu, v.c, d);
@@ -264,8 +276,10 @@ __device__ __forceinline__ int smem_upper_le(const int64_t* a, int n, int64_t r)
 // GB300, 148,909 rows in 64 trajectories of 8 turns with the profile: a tile
 // of 256 rows with a row per thread, shared-memory atomics per row and a
 // lookback took 68.8 us (and its 19 MB clear 3.8 us); the passes take about
-// 21.  The whole chain of a training step on given log-probs (state, profile
-// cleared, scan, record, restart choice): 87.8 -> 28.8 us.
+// 20.  The whole chain of a training step on given log-probs (state, profile
+// cleared, scan, record, restart choice): 87.8 -> 27.5 us (with warp 0 alone
+// finding a seeded tile near by, and the first pass at 48 registers, so that
+// two CTAs of the second fit beside its two; 33.0 without both).
 constexpr int kPassThreads = 256;
 constexpr int kPassWarps = kPassThreads / 32;
 // Up to this many tiles a tile folds its predecessors' aggregates itself
@@ -274,6 +288,25 @@ constexpr int kPassWarps = kPassThreads / 32;
 // linear in its rows.
 constexpr int64_t kDirectTiles = 4096;
 constexpr int kFromSeed = 8;  // the open turn's sums start at a seeded row
+
+// A tile's aggregate, or, after scan_prefix_kernel, the prefix before it: as a
+// ScanSlot, with the sum c before the last turn start, and the kRestart marks.
+// (Two of the workspace's slots per row: a tile has more rows than that, or
+// the slots' 256-byte padding holds them.)
+struct alignas(64) TileSlot {
+  double c, st, sd, sl, c0;  // (c0 counted as c is: from the last seeded row, or the tile's first)
+  int marks;
+};
+static_assert(sizeof(TileSlot) == 2 * sizeof(ScanSlot) && sizeof(TileSlot) <= 256, "a tile's share of the workspace");
+
+// Past this SM's L1.
+__device__ __forceinline__ TileSlot load_tile(const TileSlot* t) {
+  const double2 a = __ldcg(reinterpret_cast<const double2*>(t));
+  const double2 b = __ldcg(reinterpret_cast<const double2*>(t) + 1);
+  TileSlot r = {a.x, a.y, b.x, b.y, __ldcg(&t->c0), 0};
+  r.marks = __ldcg(&t->marks);
+  return r;
+}
 
 // A tile's part of the layout: the offsets of its first turn and of the
 // ROWS turns after it (every turn has a row at least), and of as many
@@ -563,7 +596,7 @@ template <typename Sum>
 struct PassElem {
   double c;
   Sum st, sd, sl;
-  int flags;
+  int flags;  // kRestart marks
   int seed;  // the last seeded row, from the tile's first; -1: none
 };
 
@@ -610,10 +643,14 @@ __device__ __forceinline__ bool rows_wide(const Rows<R, EXACT>& x) {
 }
 
 // The thread's rows as one element.
+// c0 and rest: the sum c before the last turn start of the thread's rows (0 if
+// there is none, or a seeded row starts it), and from there on.
 template <typename Sum, int R, bool EXACT>
-__device__ __forceinline__ PassElem<Sum> rows_elem(const BatchParams& p, const Rows<R, EXACT>& x, int tid) {
+__device__ __forceinline__ PassElem<Sum> rows_elem(const BatchParams& p, const Rows<R, EXACT>& x, int tid, double& c0,
+                                                   double& rest) {
   const Sum zero = sum_of<Sum>(0.f);
   PassElem<Sum> e = {0.0, zero, zero, zero, 0, -1};
+  c0 = rest = 0.0;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int what = x.what[i];
@@ -627,10 +664,14 @@ __device__ __forceinline__ PassElem<Sum> rows_elem(const BatchParams& p, const R
       e.flags |= kRestartSum;
     }
     if (what & (kRowSeeded | kRowTurnStart)) {
+      c0 = e.c;
+      rest = 0.0;
       e.st = e.sd = e.sl = zero;
       e.flags = (e.flags & kRestartSum) | kRestartTurn | (seeded ? kFromSeed : 0);
     }
-    e.c += stop_term(p, lpt, x.length[i]);
+    const double term = stop_term(p, lpt, x.length[i]);
+    e.c += term;
+    rest += term;
     sum_add(e.st, sum_of<Sum>(lpt));
     sum_add(e.sd, sum_of<Sum>(dd));
     sum_add(e.sl, product<Sum, EXACT>(lps, dd));
@@ -695,21 +736,31 @@ __device__ __forceinline__ ScanSlot load_slot(const ScanSlot* s) {
   return ScanSlot{a.x, a.y, b.x, b.y};
 }
 
-// First pass: tile t's aggregate in agg[t], its kRestart marks in flags[t],
-// and in incl[w] the carried state of every seeded row w.  z is the carried
-// state of the thread's last seeded row.  False, with nothing written, if the
+// What the CTA's warps of the first pass exchange.  (A pair is as large as a
+// double: the arrays serve either sum.)
+struct AggregateShared {
+  int last[2][kPassWarps];
+  double c[2][kPassWarps];  // before the last turn start, and from there on
+  double base[4];
+  double open[3][kPassWarps];
+};
+
+// First pass: tile t's aggregate in tiles[t], and in incl[w] the carried state
+// of every seeded row w.  z is the carried state of the thread's last seeded
+// row.  False, with nothing written, if the
 // tile's sums need more than Sum.
 template <typename Sum, int R, bool EXACT>
 __device__ __forceinline__ bool aggregate_tile(const BatchParams& p, int64_t tile, int tid, const Rows<R, EXACT>& x,
-                                               const ScanSlot& z) {
-  __shared__ int s_last[2][kPassWarps];
-  __shared__ double s_c[kPassWarps], s_base[4];
-  __shared__ Sum s_open[3][kPassWarps];
+                                               const ScanSlot& z, AggregateShared& sh) {
+  auto& s_last = sh.last;
+  auto& s_c = sh.c;
+  auto& s_base = sh.base;
+  auto& s_open = reinterpret_cast<Sum(&)[3][kPassWarps]>(sh.open);
   const int lane = tid & 31, warp = tid >> 5;
   if (tid < 4) s_base[tid] = 0.0;
   const Sum zero = sum_of<Sum>(0.f);
-  const PassElem<Sum> e = rows_elem<Sum>(p, x, tid);
-  double c = e.c;
+  double c0, c;
+  const PassElem<Sum> e = rows_elem<Sum>(p, x, tid, c0, c);
   Sum st = e.st, sd = e.sd, sl = e.sl;
   // only what follows the last restart counts: from thread own_c on in the
   // running sum, from own_t on in the open turn's (-1: from the first)
@@ -735,40 +786,48 @@ __device__ __forceinline__ bool aggregate_tile(const BatchParams& p, int64_t til
     s_base[2] = z.sd;
     s_base[3] = z.sl;
   }
-  c = warp * 32 + 31 < own_c ? 0.0 : warp_sum(tid >= own_c ? c : 0.0);
-  if (tid < own_t) st = sd = sl = zero;
+  c0 = warp * 32 + 31 < own_c || warp * 32 > own_t ? 0.0 : warp_sum(tid < own_c || tid > own_t ? 0.0 : tid < own_t ? e.c : c0);
+  if (tid < own_t) {
+    c = 0.0;
+    st = sd = sl = zero;
+  }
   if (warp * 32 + 31 >= own_t) {
+    c = warp_sum(c);
     st = warp_sum(st);
     sd = warp_sum(sd);
     sl = warp_sum(sl);
   }
   if (lane == 0) {
-    s_c[warp] = c;
+    s_c[0][warp] = c0;
+    s_c[1][warp] = c;
     s_open[0][warp] = st;
     s_open[1][warp] = sd;
     s_open[2][warp] = sl;
   }
   __syncthreads();
   if (warp == 0) {
-    c = warp_sum(lane < kPassWarps ? s_c[lane] : 0.0);
+    c0 = warp_sum(lane < kPassWarps ? s_c[0][lane] : 0.0);
+    c = warp_sum(lane < kPassWarps ? s_c[1][lane] : 0.0);
     st = warp_sum(lane < kPassWarps ? s_open[0][lane] : zero);
     sd = warp_sum(lane < kPassWarps ? s_open[1][lane] : zero);
     sl = warp_sum(lane < kPassWarps ? s_open[2][lane] : zero);
     if (lane == 0) {
-      p.agg[tile] =
-          ScanSlot{s_base[0] + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl)};
-      p.flags[tile] = (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0);
+      c0 += s_base[0];
+      reinterpret_cast<TileSlot*>(p.agg)[tile] =
+          TileSlot{c0 + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl), c0,
+                   (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0)};
     }
   }
   return true;
 }
 
 template <int R, bool EXACT>
-__global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const BatchParams p,
+__global__ void __launch_bounds__(kPassThreads, EXACT && R > 1 ? 4 : 5) scan_aggregate_kernel(const BatchParams p,
                                                                      const float* __restrict__ logp_s,
                                                                      const float* __restrict__ logp_t, bool early) {
   constexpr int kRows = R * kPassThreads;
   __shared__ TileLayout<kRows> L;
+  __shared__ AggregateShared sh;
   const int tid = threadIdx.x;
   const int64_t tile = blockIdx.x;
   const int64_t t0 = tile * kRows;
@@ -789,7 +848,7 @@ __global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const B
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   load_logps<R>(logp_s, logp_t, t0, tid, x);
-  if (!aggregate_tile<Sum2>(p, tile, tid, x, z)) aggregate_tile<double>(p, tile, tid, x, z);
+  if (!aggregate_tile<Sum2>(p, tile, tid, x, z, sh)) aggregate_tile<double>(p, tile, tid, x, z, sh);
 }
 
 // Between the passes of a window of many tiles: the aggregates replaced by
@@ -797,7 +856,7 @@ __global__ void __launch_bounds__(kPassThreads, 4) scan_aggregate_kernel(const B
 constexpr int kPrefixThreads = 1024;
 
 struct PrefixElem {
-  double c, st, sd, sl;
+  double c, st, sd, sl, c0;
   int flags;
 };
 
@@ -808,6 +867,7 @@ __device__ __forceinline__ PrefixElem elem_combine(const PrefixElem& a, const Pr
   r.st = turn ? b.st : a.st + b.st;
   r.sd = turn ? b.sd : a.sd + b.sd;
   r.sl = turn ? b.sl : a.sl + b.sl;
+  r.c0 = !turn ? a.c0 : (b.flags & kRestartSum) ? b.c0 : a.c + b.c0;
   r.flags = a.flags | b.flags;
   return r;
 }
@@ -818,30 +878,30 @@ __device__ __forceinline__ PrefixElem elem_shfl_up(const PrefixElem& v, int d) {
   o.st = __shfl_up_sync(0xffffffffu, v.st, d);
   o.sd = __shfl_up_sync(0xffffffffu, v.sd, d);
   o.sl = __shfl_up_sync(0xffffffffu, v.sl, d);
+  o.c0 = __shfl_up_sync(0xffffffffu, v.c0, d);
   o.flags = __shfl_up_sync(0xffffffffu, v.flags, d);
   return o;
 }
 
-__global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(ScanSlot* agg, const uint32_t* flags,
-                                                                     int64_t n_tiles) {
+__global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(TileSlot* tiles, int64_t n_tiles) {
   constexpr int kWarps = kPrefixThreads / 32;
   __shared__ PrefixElem s_tot[kWarps], s_pre[kWarps], s_carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const PrefixElem id = {0.0, 0.0, 0.0, 0.0, 0};
+  const PrefixElem id = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
   PrefixElem carry = id;
   for (int64_t t = 0; t < n_tiles; t += kPrefixThreads) {
     const int64_t j = t + tid;
     PrefixElem v = id;
     if (j < n_tiles) {
-      const ScanSlot a = load_slot(agg + j);
-      v = PrefixElem{a.c, a.st, a.sd, a.sl, (int)__ldcg(flags + j)};
+      const TileSlot a = load_tile(tiles + j);
+      v = PrefixElem{a.c, a.st, a.sd, a.sl, a.c0, a.marks};
     }
     PrefixElem incl, excl;
     block_scan<kWarps>(v, id, lane, warp, s_tot, s_pre, incl, excl);
     const PrefixElem before = elem_combine(carry, excl);
-    if (j < n_tiles) agg[j] = ScanSlot{before.c, before.st, before.sd, before.sl};
+    if (j < n_tiles) tiles[j] = TileSlot{before.c, before.st, before.sd, before.sl, before.c0, before.flags};
     if (tid == kPrefixThreads - 1) s_carry = elem_combine(carry, incl);
     __syncthreads();
     carry = s_carry;
@@ -896,18 +956,20 @@ __device__ __forceinline__ void record_parts(const BatchParams& p, const TrajPar
 }
 
 // Completes the thread's rows, given the exclusive prefix of its rows inside
-// the tile, the tile's (pre) and the carried state of the tile's seeded rows
-// (seed(j), which covers excl.seed too).
+// the tile, the tile's (pre), the carried state of the tile's seeded rows
+// (seed(j), which covers excl.seed too), and by thread the sum c before the
+// last turn start of its rows, counted as excl.c is (turn_c0).
 template <typename Sum, int R, bool EXACT, int ROWS, typename Seed>
 __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLayout<ROWS>& L, int64_t t0, int tid,
                                               const Rows<R, EXACT>& x, const PassElem<Sum>& excl, const double* pre,
-                                              Seed&& seed) {
+                                              const double* turn_c0, Seed&& seed) {
   const int lane = tid & 31;
   const float nan = __int_as_float(0x7fc00000);
   const Sum zero = sum_of<Sum>(0.f);
   ScanSlot z = {0.0, 0.0, 0.0, 0.0};  // the last seeded row's before this thread
   if (excl.seed >= 0 && (x.what[0] & kRowLive)) z = seed(excl.seed);
-  double c = (excl.seed >= 0 ? z.c : pre[0]) + excl.c;
+  const double from = excl.seed >= 0 ? z.c : pre[0];
+  double c = from + excl.c;
   double b_st = pre[1], b_sd = pre[2], b_sl = pre[3];  // what the open turn brought into the tile
   if (excl.flags & kRestartTurn) {
     const bool from = (excl.flags & kFromSeed) != 0;
@@ -966,9 +1028,12 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     if (token_sum) {
       kept = r == m.traj_start || !(c < (double)lam);
     } else if (i == 0 || seeded || fturn) {
-      using Length = typename StopTerm<EXACT>::Length;
-      const double before = c - (double)((Length)(b_st + sum_value(st)) / x.length[i]);
-      kept = m.local_turn == 0 || !(before < (double)lam);
+      double c0 = c;  // the sum before the row's turn
+      if (!fturn) {
+        const int64_t at = m.turn_start - (p.row_begin + t0);  // its first row, from the tile's
+        c0 = at < 0 ? pre[4] : from + turn_c0[at / R];
+      }
+      kept = m.local_turn == 0 || !fired_before_turn(p, m, c0, lam);
     }
     c += stop_term(p, lpt, x.length[i]);
     sum_add(st, sum_of<Sum>(lpt));
@@ -1081,8 +1146,9 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   __shared__ int64_t s_first[2];                      // first turn, first trajectory of the tile
   __shared__ TileElem s_wtot[kWarps];
   __shared__ TileElem s_wpre[kWarps];
-  __shared__ TileElem s_excl;  // the tile's exclusive prefix (flags unused)
-  __shared__ TileElem s_agg;
+  __shared__ double s_c0[TILE];  // by row where a turn begins: the sum c before it (from the row where c restarts)
+  __shared__ TileAgg s_excl;     // the tile's exclusive prefix (flags unused)
+  __shared__ TileAgg s_agg;
   __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // Launched as a programmatic dependent of the kernel that wrote the
@@ -1129,7 +1195,7 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   }
   __syncthreads();
 
-  __shared__ TileElem s_caggs[kClusterMaxTiles];  // predecessors' aggregates
+  __shared__ TileAgg s_caggs[kClusterMaxTiles];  // predecessors' aggregates
 
   // 2. this thread's row: its turn and trajectory, and its element
   RowMeta meta;
@@ -1193,8 +1259,8 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
     lpt = __ldcg(logp_t + w);
   }
   TileElem x = {0.0, 0.0, 0.0, 0.0, 0};
-  double c_before = 0.0, st_before = 0.0, ri_c = 0.0;
-  float st_before_f = 0.f, e_sl = 0.f;
+  double c_before = 0.0, c0 = 0.0, ri_c = 0.0;
+  float e_sl = 0.f;
   if (live) {
     const float nan = __int_as_float(0x7fc00000);
     if (meta.bad) {
@@ -1220,8 +1286,6 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
       x = TileElem{cum0 + ec, (float)(st0 + (double)lpt), (float)(sd0 + (double)dd), (float)(sl0 + (double)esl),
                    kRestartSum | kRestartTurn};
       c_before = cum0;
-      st_before = st0;
-      st_before_f = (float)st0;
     } else if (seeded) {
       x = TileElem{ec, lpt, dd, esl, kRestartSum | kRestartTurn};  // NaN: nothing after a bad row is meaningful
     } else {
@@ -1237,13 +1301,23 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
 
   // 4. the tile's exclusive prefix, from the cluster's other tiles
   namespace cg = cooperative_groups;
-  if (tid == (int)(n_here - 1)) s_agg = tile_incl;
+  const bool turn_mean = p.mode == STRIDE_STOP_TURN_MEAN;
+  if (turn_mean && (seeded || fturn)) {
+    const double c0 = seeded ? cum0 : tile_excl.c;
+    s_c0[tid] = c0;
+    if (meta.turn_end >= r0 + n_here) s_agg.c0 = c0;  // the tile's last turn
+  }
+  if (tid == (int)(n_here - 1)) s_agg.e = tile_incl;
   __syncthreads();
   cluster_wait_acquire();  // every tile has started and read its carried state
   if (warp == 0) {
     const cg::cluster_group cl = cg::this_cluster();
-    const TileElem agg = s_agg;
-    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) cl.map_shared_rank(s_caggs, (unsigned)j)[tile] = agg;
+    const TileAgg agg = s_agg;
+    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) {
+      TileAgg* to = cl.map_shared_rank(s_caggs, (unsigned)j) + tile;
+      to->e = agg.e;
+      if (turn_mean) to->c0 = agg.c0;
+    }
   }
   cluster_arrive_release();
   if (p.profile) {  // (while the aggregates are on their way)
@@ -1255,15 +1329,19 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   if (warp == 0) {
     // the predecessors' aggregates folded in tile order (a warp scan: the
     // stop sum fp64, the open-turn sums fp32 as inside a tile)
-    TileElem v = {0.0, 0.f, 0.f, 0.f, 0};
+    const TileAgg none = {{0.0, 0.f, 0.f, 0.f, 0}, 0.0};
+    TileAgg v = none;
     if (lane < tile) v = s_caggs[lane];
 #pragma unroll
     for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
-      const TileElem o = tile_shfl_up(v, d);
-      if (lane >= d) v = tile_combine(o, v);
+      const TileElem o = tile_shfl_up(v.e, d);
+      if (turn_mean) {
+        const double c0 = __shfl_up_sync(0xffffffffu, v.c0, d);
+        if (lane >= d) v.c0 = tile_c0(o, c0, v);
+      }
+      if (lane >= d) v.e = tile_combine(o, v.e);
     }
-    if (lane == (tile > 0 ? (int)tile - 1 : 0))
-      s_excl = tile > 0 ? TileElem{v.c, v.st, v.sd, v.sl, 0} : TileElem{0.0, 0.f, 0.f, 0.f, 0};
+    if (lane == (tile > 0 ? (int)tile - 1 : 0)) s_excl = tile > 0 ? v : none;
   }
   __syncthreads();
 
@@ -1271,33 +1349,30 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   if (live) {
     // the row's prefixes: the stop sum fp64, the open-turn sums fp32 (the
     // tile's prefix rounded once to fp32; 6e-8 of the sums)
-    const TileElem pre = s_excl;
+    const TileElem pre = s_excl.e;
     const TileElem ri = tile_combine(pre, tile_incl);
-    if (!(x.flags & 4)) {
-      const TileElem re = tile_combine(pre, tile_excl);
-      c_before = re.c;
-      st_before_f = fturn ? 0.f : re.st;
-      st_before = (double)st_before_f;
+    const double from = (tile_excl.flags & kRestartSum) ? 0.0 : pre.c;  // what c counts from, before this row
+    if (!(x.flags & 4)) c_before = from + tile_excl.c;
+    if (turn_mean && !meta.bad) {  // the sum before the row's turn
+      const int64_t j = meta.turn_start - r0;
+      c0 = j < 0 ? s_excl.c0 : seeded ? cum0 : from + s_c0[j];
     }
     RowCarry rc;
-    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, fturn};
-    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 1};
-    row_tail(p, r, meta, rc, si, c_before, st_before, false, true);
+    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, 0.0, fturn};
+    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 0.0, 1};
+    row_tail(p, r, meta, rc, si, c_before, false, true);
     ri_c = ri.c;
   }
 
   // 6. the trajectories' stop records and losses, once per trajectory and warp
   TrajPart<Sum2> part = {-1, 0, 0, {0.f, 0.f}, -1};
   if (live && !meta.bad) {
-    const int64_t n_k = meta.turn_end - meta.turn_start;
     const bool turn_last = (r == meta.turn_end - 1);
     const bool test = (p.mode == STRIDE_STOP_TOKEN_SUM) || turn_last;
     // retained unless the rule fired before the row (row_tail); a
     // trajectory's first token or turn always is
     const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
-    const double before =
-        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before : c_before - (double)(st_before_f / (float)n_k);
-    const bool kept = first || !(before < (double)lam);
+    const bool kept = first || !(turn_mean ? fired_before_turn(p, meta, c0, lam) : c_before < (double)lam);
     part.traj = meta.traj;
     part.count = kept ? 1 : 0;
     part.loss.hi = kept ? e_sl : 0.f;
@@ -1313,53 +1388,81 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   }
 }
 
+// What the CTA's warps of the second pass exchange.
+struct CompleteShared {
+  PassElem<double> tot[kPassWarps], wpre[kPassWarps];
+  int near[2][kPassWarps], needs, folded;
+  double fold[5][kPassWarps], pre[5], turn_c0[kPassThreads];
+};
+static_assert(sizeof(PassElem<Sum2>) == sizeof(PassElem<double>), "the arrays serve either sum");
+
 // Second pass.  False, with nothing written, if the tile's sums need more
 // than Sum.
 template <typename Sum, int R, bool EXACT, int ROWS>
 __device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLayout<ROWS>& L, int64_t tile, int tid,
-                                              const Rows<R, EXACT>& x, bool prefixed) {
-  __shared__ PassElem<Sum> s_tot[kPassWarps], s_wpre[kPassWarps];
-  __shared__ int s_near[2][kPassWarps];
-  __shared__ double s_fold[4][kPassWarps];
-  __shared__ double s_pre[4];
-  __shared__ int s_needs;
+                                              const Rows<R, EXACT>& x, bool prefixed, CompleteShared& sh) {
+  auto* const s_tot = reinterpret_cast<PassElem<Sum>*>(sh.tot);
+  auto* const s_wpre = reinterpret_cast<PassElem<Sum>*>(sh.wpre);
+  auto& s_near = sh.near;
+  auto& s_fold = sh.fold;
+  auto& s_pre = sh.pre;
+  auto& s_turn_c0 = sh.turn_c0;
+  auto& s_needs = sh.needs;
+  auto& s_folded = sh.folded;
   const int lane = tid & 31, warp = tid >> 5;
   const int64_t t0 = tile * ROWS;
-  if (tid < 4) s_pre[tid] = 0.0;
-  if (tid == 0) s_needs = !(x.what[0] & kRowSeeded);
+  if (tid < 5) s_pre[tid] = 0.0;
+  if (tid == 0) {
+    s_needs = !(x.what[0] & kRowSeeded);
+    s_folded = 0;
+  }
   const Sum zero = sum_of<Sum>(0.f);
   const PassElem<Sum> id = {0.0, zero, zero, zero, 0, -1};
   PassElem<Sum> incl, excl;
   constexpr bool kNarrow = std::is_same<Sum, Sum2>::value;
-  if (block_scan<kPassWarps, kNarrow>(rows_elem<Sum>(p, x, tid), id, lane, warp, s_tot, s_wpre, incl, excl,
-                                      kNarrow && rows_wide(x)))
+  double c0, rest;
+  const PassElem<Sum> own = rows_elem<Sum>(p, x, tid, c0, rest);
+  if (block_scan<kPassWarps, kNarrow>(own, id, lane, warp, s_tot, s_wpre, incl, excl, kNarrow && rows_wide(x)))
     return false;
+  if (own.flags & kRestartTurn) s_turn_c0[tid] = (own.flags & kRestartSum) ? c0 : excl.c + c0;
+  const TileSlot* tiles = reinterpret_cast<const TileSlot*>(p.agg);
 
   // ---- the first pass's results
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (s_needs && prefixed) {
-    if (tid == 0) {
-      const ScanSlot a = load_slot(p.agg + tile);
-      s_pre[0] = a.c;
-      s_pre[1] = a.st;
-      s_pre[2] = a.sd;
-      s_pre[3] = a.sl;
+  // Sums of the predecessors' aggregates back to the nearest one with a seeded
+  // row (c), and to the nearest one with a turn start (the open turn's); c0 is
+  // that one's, with the sums c before it back to the seeded row.  A seeded
+  // tile among the 32 before this one is warp 0's to find.
+  if (warp == 0 && s_needs) {
+    TileSlot a = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
+    if (prefixed || lane < tile) a = load_tile(tiles + (prefixed ? tile : tile - 1 - lane));
+    const unsigned b_sum = __ballot_sync(0xffffffffu, (a.marks & kRestartSum) != 0);
+    const unsigned b_turn = __ballot_sync(0xffffffffu, (a.marks & kRestartTurn) != 0);
+    double f[5] = {a.c, a.st, a.sd, a.sl, a.c0};
+    if (!prefixed && b_sum) {
+      const int n_sum = __ffs(b_sum) - 1, n_turn = __ffs(b_turn) - 1;  // (a seeded row is a turn's start: n_turn <= n_sum)
+      f[4] = warp_sum(lane == n_turn ? a.c0 : lane > n_turn && lane <= n_sum ? a.c : 0.0);
+      f[0] = warp_sum(lane <= n_sum ? a.c : 0.0);
+      f[1] = warp_sum(lane <= n_turn ? a.st : 0.0);
+      f[2] = warp_sum(lane <= n_turn ? a.sd : 0.0);
+      f[3] = warp_sum(lane <= n_turn ? a.sl : 0.0);
     }
-  } else if (s_needs) {
-    // Sums of the predecessors' aggregates back to the nearest one with a
-    // seeded row (c), and to the nearest one with a turn start (the others).
-    double f[4] = {0.0, 0.0, 0.0, 0.0};
+    if (lane == 0 && (prefixed || b_sum)) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) s_pre[k] = f[k];
+      s_folded = 1;
+    }
+  }
+  __syncthreads();
+  if (s_needs && !s_folded) {
+    double f[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     bool turn_open = true, any = false;
     for (int64_t hi = tile; hi > 0; hi -= kPassThreads) {
       const int64_t j = hi - 1 - tid;
-      unsigned fl = 0;
-      ScanSlot a = {0.0, 0.0, 0.0, 0.0};
-      if (j >= 0) {
-        fl = __ldcg(p.flags + j);
-        a = load_slot(p.agg + j);
-      }
-      const unsigned b_sum = __ballot_sync(0xffffffffu, (fl & kRestartSum) != 0);
-      const unsigned b_turn = __ballot_sync(0xffffffffu, (fl & kRestartTurn) != 0);
+      TileSlot a = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
+      if (j >= 0) a = load_tile(tiles + j);
+      const unsigned b_sum = __ballot_sync(0xffffffffu, (a.marks & kRestartSum) != 0);
+      const unsigned b_turn = __ballot_sync(0xffffffffu, (a.marks & kRestartTurn) != 0);
       if (lane == 0) {
         s_near[0][warp] = b_sum ? warp * 32 + __ffs(b_sum) - 1 : kPassThreads;
         s_near[1][warp] = b_turn ? warp * 32 + __ffs(b_turn) - 1 : kPassThreads;
@@ -1378,6 +1481,9 @@ __device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLa
           f[1] += a.st;
           f[2] += a.sd;
           f[3] += a.sl;
+          if (tid == n_turn) f[4] = a.c0;
+        } else if (tid <= n_sum) {
+          f[4] += a.c;
         }
       }
       turn_open = turn_open && n_turn == kPassThreads;
@@ -1385,23 +1491,23 @@ __device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLa
       __syncthreads();
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 5; ++k) {
       const double v = any ? warp_sum(f[k]) : 0.0;
       if (lane == 0) s_fold[k][warp] = v;
     }
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < 5; ++k) {
         double v = lane < kPassWarps ? s_fold[k][lane] : 0.0;
 #pragma unroll
         for (int o = kPassWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) s_pre[k] = v;
       }
     }
+    __syncthreads();
   }
-  __syncthreads();
-  complete_rows<Sum>(p, L, t0, tid, x, excl, s_pre, [&](int j) { return load_slot(p.incl + t0 + j); });
+  complete_rows<Sum>(p, L, t0, tid, x, excl, s_pre, s_turn_c0, [&](int j) { return load_slot(p.incl + t0 + j); });
   return true;
 }
 
@@ -1412,6 +1518,7 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
                                                                        bool prefixed, bool validate) {
   constexpr int kRows = R * kPassThreads;
   __shared__ TileLayout<kRows> L;
+  __shared__ CompleteShared sh;
   __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
   const int tid = threadIdx.x;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1424,7 +1531,7 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
   find_rows<R, EXACT>(p, L, t0, n_here, tid, x, [](int, const ScanSlot&) {});  // (the first pass set the states aside)
   load_logps<R>(logp_s, logp_t, t0, tid, x);
   if (p.profile) rows_profile(x, tid & 31, s_prof);
-  if (!complete_tile<Sum2>(p, L, tile, tid, x, prefixed)) complete_tile<double>(p, L, tile, tid, x, prefixed);
+  if (!complete_tile<Sum2>(p, L, tile, tid, x, prefixed, sh)) complete_tile<double>(p, L, tile, tid, x, prefixed, sh);
   if (p.profile && tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
   if (validate) check_layout(p, tile, n_tiles, tid);
 }
@@ -1528,7 +1635,7 @@ cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float
   cudaError_t e =
       launch_dependent(scan_aggregate_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, after.scoring);
   if (e == cudaSuccess && prefixed)
-    e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, p.agg, p.flags, n_tiles);
+    e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, reinterpret_cast<TileSlot*>(p.agg), n_tiles);
   if (e == cudaSuccess)
     e = launch_dependent(scan_complete_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, n_tiles,
                          prefixed, !after.checked);

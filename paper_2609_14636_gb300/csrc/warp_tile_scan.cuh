@@ -94,7 +94,7 @@ __device__ __forceinline__ int head_of(unsigned m, int lane) {
 // A published tile on its way to the scan warp (shared memory, by lane).
 struct TileCarry {
   double c[32], st[32], sd[32], sl[32];  // inclusive within the tile (seeded rows: from the carried state)
-  double c_seed[32], st_seed[32];        // a seeded row's carried running sum and open-turn sum of log pi_T
+  double c_seed[32];                     // a seeded row's carried running sum
   float lps[32], lpt[32];
   int32_t turn[32], traj[32];
   uint32_t m_good, m_seed, m_turn;
@@ -151,14 +151,13 @@ __device__ __forceinline__ void publish_tile(const BatchParams& p, int64_t t, in
   // ---- elements; a seeded row's holds the carried state
   double c = !live ? 0.0 : (p.mode == STRIDE_STOP_TURN_MEAN) ? (double)lpt / (double)n_k : (double)lpt;
   double st = (double)lpt, sd = (double)dd, sl = (double)lps * (double)dd;  // -log pi_S * r_t (Eq. 2)
-  double c_seed = 0.0, st_seed = 0.0;
+  double c_seed = 0.0;
   if (seeded && good) {
     const stride_scan_state* sp = p.state + meta.traj;
     c_seed = __ldcg(&sp->cum);
     c += c_seed;
     if (!fturn) {
-      st_seed = __ldcg(&sp->turn_sum_t);
-      st += st_seed;
+      st += __ldcg(&sp->turn_sum_t);
       sd += __ldcg(&sp->turn_sum_d);
       sl += __ldcg(&sp->turn_sum_l);
     }
@@ -171,10 +170,14 @@ __device__ __forceinline__ void publish_tile(const BatchParams& p, int64_t t, in
   sd = seg_sum(sd, max(h_turn, 0), lane);
   sl = seg_sum(sl, max(h_turn, 0), lane);
 
+  // the sum before each row's turn, where that begins here
+  const double c_prev = __shfl_up_sync(0xffffffffu, c, 1);
+  const double c0 = __shfl_sync(0xffffffffu, seeded ? c_seed : lane > 0 ? c_prev : 0.0, max(h_turn, 0));
+
   // ---- the tile's aggregate out, the earlier tiles' prefix in
   uint32_t* flag = p.flags + t * kFlagStride;
   if (lane == n_here - 1) {
-    const ScanElem agg{c, st, sd, sl, 0};
+    const ScanElem agg{c, st, sd, sl, c0, 0};
     if (m_seed)
       publish(p.incl + t, flag, agg, kStIncl);
     else
@@ -185,7 +188,6 @@ __device__ __forceinline__ void publish_tile(const BatchParams& p, int64_t t, in
   tc.sd[lane] = sd;
   tc.sl[lane] = sl;
   tc.c_seed[lane] = c_seed;
-  tc.st_seed[lane] = st_seed;
   tc.lps[lane] = lps;
   tc.lpt[lane] = lpt;
   tc.turn[lane] = meta.turn;
@@ -229,7 +231,7 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
   const int64_t n_k = good ? meta.turn_end - meta.turn_start : 1;
   const bool fturn = good && r == meta.turn_start;
 
-  ScanElem pre{0.0, 0.0, 0.0, 0.0, 0};
+  ScanElem pre{0.0, 0.0, 0.0, 0.0, 0.0, 0};
   if (!(m_seed & 1u)) {
     bool timed_out = false;
     pre = lookback(p, t, lane, timed_out);
@@ -240,20 +242,15 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
       sd += pre.sd;
       sl += pre.sl;
     }
-    if (!m_seed && lane == n_here - 1)
-      publish(p.incl + t, p.flags + t * kFlagStride, ScanElem{c, st, sd, sl, 0}, kStIncl);
   }
-  // the running sum and the open turn's sum of log pi_T before each row
-  double c_before = __shfl_up_sync(0xffffffffu, c, 1), st_before = __shfl_up_sync(0xffffffffu, st, 1);
-  if (lane == 0) {
-    c_before = pre.c;
-    st_before = pre.st;
-  }
-  if (seeded) {
-    c_before = tc.c_seed[lane];
-    st_before = tc.st_seed[lane];
-  }
-  if (fturn) st_before = 0.0;
+  // the running sum before each row, and before its turn
+  double c_before = __shfl_up_sync(0xffffffffu, c, 1);
+  if (lane == 0) c_before = pre.c;
+  if (seeded) c_before = tc.c_seed[lane];
+  const double c0_here = __shfl_sync(0xffffffffu, c_before, max(h_turn, 0));
+  const double c0 = h_turn < 0 ? pre.c0 : c0_here;
+  if (!m_seed && lane == n_here - 1)
+    publish(p.incl + t, p.flags + t * kFlagStride, ScanElem{c, st, sd, sl, c0, 0}, kStIncl);
 
   // ---- turn statistics, stop test, retention (row_scan.cuh states the rule)
   const bool turn_last = good && r == meta.turn_end - 1;
@@ -270,8 +267,7 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
   }
   const bool cross = good && (token_sum || turn_last) && c < (double)lam;
   const bool first = token_sum ? r == meta.traj_start : meta.local_turn == 0;
-  const double before = token_sum ? c_before : c_before - st_before / (double)n_k;
-  const bool kept = good && (first || !(before < (double)lam));
+  const bool kept = good && (first || !(token_sum ? c_before < (double)lam : fired_before_turn(p, meta, c0, lam)));
 
   // ---- the trajectories' records, once per trajectory and tile
   const unsigned m_traj = __ballot_sync(0xffffffffu, !good || r == meta.traj_start);
