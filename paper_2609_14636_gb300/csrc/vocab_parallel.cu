@@ -159,17 +159,19 @@ constexpr int kRestartSum = 2;   // c restarts (a seeded row)
 // loss term are fp32 inside the tile (summed in a tree: relative error a few
 // 1e-7 of the summed magnitudes), in the cluster's fold of at most 16 tile
 // aggregates, and where the tile's prefix meets a row; every stored sum is
-// fp64.  GB300 runs FP64 at 1/64 of the FP32 rate, and the tile scans' fp64
+// fp64, as are all sums of a window whose might leave fp32 (`wide`).  GB300 runs FP64 at 1/64 of the FP32 rate, and the tile scans' fp64
 // adds were what a small window's scan waited on (a 512-row window in one
 // CTA: 6.6 us for the block scan).
+template <typename F>
 struct TileElem {
   double c;
-  float st, sd, sl;
+  F st, sd, sl;
   int flags;
 };
 
-__device__ __forceinline__ TileElem tile_combine(const TileElem& a, const TileElem& b) {
-  TileElem r;
+template <typename F>
+__device__ __forceinline__ TileElem<F> tile_combine(const TileElem<F>& a, const TileElem<F>& b) {
+  TileElem<F> r;
   r.c = (b.flags & kRestartSum) ? b.c : a.c + b.c;
   r.st = (b.flags & kRestartTurn) ? b.st : a.st + b.st;
   r.sd = (b.flags & kRestartTurn) ? b.sd : a.sd + b.sd;
@@ -180,18 +182,21 @@ __device__ __forceinline__ TileElem tile_combine(const TileElem& a, const TileEl
 
 // A tile's aggregate or prefix: with (for turn means) the sum c before the
 // last turn mark, a turn's first row or a seeded one, counted from where c is.
+template <typename F>
 struct TileAgg {
-  TileElem e;
+  TileElem<F> e;
   double c0;
 };
 
 // c0 of a (earlier, whose c0 is a_c0) and b together.
-__device__ __forceinline__ double tile_c0(const TileElem& a, double a_c0, const TileAgg& b) {
+template <typename F>
+__device__ __forceinline__ double tile_c0(const TileElem<F>& a, double a_c0, const TileAgg<F>& b) {
   return !(b.e.flags & kRestartTurn) ? a_c0 : (b.e.flags & kRestartSum) ? b.c0 : a.c + b.c0;
 }
 
-__device__ __forceinline__ TileElem tile_shfl_up(const TileElem& v, int d) {
-  TileElem o;
+template <typename F>
+__device__ __forceinline__ TileElem<F> tile_shfl_up(const TileElem<F>& v, int d) {
+  TileElem<F> o;
   o.c = __shfl_up_sync(0xffffffffu, v.c, d);
   o.st = __shfl_up_sync(0xffffffffu, v.st, d);
   o.sd = __shfl_up_sync(0xffffffffu, v.sd, d);
@@ -200,8 +205,14 @@ __device__ __forceinline__ TileElem tile_shfl_up(const TileElem& v, int d) {
   return o;
 }
 
-__device__ __forceinline__ TileElem elem_combine(const TileElem& a, const TileElem& b) { return tile_combine(a, b); }
-__device__ __forceinline__ TileElem elem_shfl_up(const TileElem& v, int d) { return tile_shfl_up(v, d); }
+template <typename F>
+__device__ __forceinline__ TileElem<F> elem_combine(const TileElem<F>& a, const TileElem<F>& b) {
+  return tile_combine(a, b);
+}
+template <typename F>
+__device__ __forceinline__ TileElem<F> elem_shfl_up(const TileElem<F>& v, int d) {
+  return tile_shfl_up(v, d);
+}
 
 // Inclusive and exclusive scan of one element per thread over the CTA's
 // WARPS warps, in thread order: warp shuffles, then warp 0 scans the warps'
@@ -511,11 +522,11 @@ __device__ __forceinline__ void load_logps(const float* __restrict__ logp_s, con
 // (Knuth's TwoSum): hi + lo is good to about 2^-45 of the summed magnitudes
 // over a tile, at seven FP32 operations where an fp64 add costs as much as 64.
 // Its range is fp32's.  So a tile (or, for the profile, a warp) that holds a
-// log-prob of 2^58 or more, an infinity or a NaN (`wide`) takes fp64 sums
+// log-prob of 2^50 or more, an infinity or a NaN (`wide`) takes fp64 sums
 // instead: a sampled token masked with the lowest finite logit has log pi =
 // -3.4e38, and two of them, or its product with another log-prob, are finite
-// in fp64 alone.  Below 2^58 a difference is below 2^59, a product below
-// 2^117 and the sum of a tile's 512 rows below 2^126.  GB300, 30,011 rows of
+// in fp64 alone.  Below 2^50 a difference is below 2^51, a product below
+// 2^101 and the sum of a tile's 512 rows below 2^110.  GB300, 30,011 rows of
 // 32,000 bf16 logits: pairs 519.3 us, fp64 in every tile 528.0.  Errors of the
 // turns' sums there, in pairs / fp64, of the summed magnitudes: log pi_T and d
 // none / none (48 bits hold them), logp_S * d 5e-16 / 3e-18.
@@ -524,7 +535,7 @@ struct Sum2 {
 };
 
 __device__ __forceinline__ bool wide(float lps, float lpt) {
-  constexpr float kMost = 288230376151711744.0f;  // 2^58
+  constexpr float kMost = 1125899906842624.0f;  // 2^50
   return !(fabsf(lps) < kMost && fabsf(lpt) < kMost);
 }
 
@@ -1112,6 +1123,8 @@ __device__ __forceinline__ void check_layout(const BatchParams& p, int64_t tile,
 //      warp (record_parts), so its record takes one update per warp instead
 //      of one per row (the rows of a token-sum segment below lambda all
 //      contended for it).
+// A tile that holds a log-prob beyond fp32 sums (`wide`) tells all the others
+// with its aggregate, and the window's steps 2 to 6 are done again in fp64.
 // The profile's runs of equal deciles are summed in registers while the
 // aggregates are on their way.  GB300, against a second block scan for 6 and a
 // shared-memory atomic per row for the profile: a 512-row window of 32,000
@@ -1135,20 +1148,166 @@ constexpr int kClusterTileRows = STRIDE_CLUSTER_TILE_ROWS;
 static_assert(kClusterTileRows % 32 == 0 && kClusterTileRows >= 64 && kClusterTileRows <= 1024,
               "whole warps, 2 to 32 of them");
 
+// What a thread of the cluster scan knows of its row before the scan.
+struct ClusterRow {
+  RowMeta meta;
+  int64_t r;
+  float lps, lpt, lam;
+  double cum0, st0, sd0, sl0;  // a seeded row's carried state
+  bool live, seeded, fturn;
+};
+
+// Whether the window needs fp64 sums for this row: its 2,048 rows at most and
+// a carried sum stay below 2^114 otherwise.
+__device__ __forceinline__ bool row_wide(const ClusterRow& q) {
+  if (!q.live || q.meta.bad) return false;
+  constexpr double kMost = 1.3e33;  // (about 2^110)
+  return wide(q.lps, q.lpt) || (q.seeded && !(fabs(q.st0) < kMost && fabs(q.sd0) < kMost && fabs(q.sl0) < kMost));
+}
+
+__device__ __forceinline__ Sum2 cluster_term(float x) { return Sum2{x, 0.f}; }
+__device__ __forceinline__ double cluster_term(double x) { return x; }
+
+// What the CTAs of the cluster scan exchange, and their warps.
+template <typename F, int TILE>
+struct ClusterShared {
+  TileElem<F> wtot[TILE / 32], wpre[TILE / 32];
+  TileAgg<F> caggs[kClusterMaxTiles];  // predecessors' aggregates
+  TileAgg<F> agg, excl;                // the tile's aggregate and exclusive prefix (its flags unused)
+  double c0[TILE];  // by row where a turn begins: the sum c before it (from the row where c restarts)
+};
+
+// Steps 2 to 6 with open-turn sums in F.  False, with nothing written, if any
+// row of the window needs more than F.
+namespace cg = cooperative_groups;
+template <typename F, int TILE, typename Meanwhile>
+__device__ __forceinline__ bool scan_cluster_rows(const BatchParams& p, const ClusterRow& q, int64_t tile, int64_t n_tiles,
+                                                  int64_t r0, int n_here, ClusterShared<F, TILE>& sh, int* s_wide,
+                                                  Meanwhile&& meanwhile) {
+  constexpr int kWarps = TILE / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const RowMeta& meta = q.meta;
+  const bool live = q.live, seeded = q.seeded, fturn = q.fturn, turn_mean = p.mode == STRIDE_STOP_TURN_MEAN;
+  const int64_t r = q.r;
+
+  // 2. the row's element: its terms in F (logp_S * d in fp32 rounded once); the
+  //    stop-sum term in fp64, a turn mean's share lpt / n_k rounded once to
+  //    fp32 first (GB300 issues an fp64 divide as a sequence of fp64
+  //    operations at 1/64 of the fp32 rate; the rounding is 6e-8 of the term)
+  TileElem<F> x = {0.0, 0, 0, 0, 0};
+  double c_before = q.cum0, c0 = 0.0, ri_c = 0.0;
+  F e_sl = 0;
+  if (live) {
+    const float lpt = q.lpt, dd = q.lps - lpt;
+    const int64_t n_k = meta.turn_end - meta.turn_start;
+    const double ec = turn_mean ? (double)(lpt / (float)(n_k > 0 ? n_k : 1)) : (double)lpt;
+    e_sl = (F)q.lps * (F)dd;
+    if (seeded && !meta.bad)
+      x = TileElem<F>{q.cum0 + ec, (F)(q.st0 + (double)lpt), (F)(q.sd0 + (double)dd), (F)(q.sl0 + (double)e_sl),
+                      kRestartSum | kRestartTurn};
+    else  // (a bad row's are NaN: nothing after it is meaningful)
+      x = TileElem<F>{ec, lpt, dd, e_sl, seeded ? kRestartSum | kRestartTurn : fturn ? kRestartTurn : 0};
+  }
+
+  // 3. segmented inclusive scan over the tile
+  const TileElem<F> tile_id = {0.0, 0, 0, 0, 0};
+  TileElem<F> tile_incl, tile_excl;
+  block_scan<kWarps>(x, tile_id, lane, warp, sh.wtot, sh.wpre, tile_incl, tile_excl);
+
+  // 4. the tile's exclusive prefix, from the cluster's other tiles
+  if (turn_mean && (seeded || fturn)) {
+    const double c0 = seeded ? q.cum0 : tile_excl.c;
+    sh.c0[tid] = c0;
+    if (meta.turn_end >= r0 + n_here) sh.agg.c0 = c0;  // the tile's last turn
+  }
+  if (tid == n_here - 1) sh.agg.e = tile_incl;
+  __syncthreads();
+  const cg::cluster_group cl = cg::this_cluster();
+  constexpr bool kNarrow = std::is_same<F, float>::value;
+  if (kNarrow) cluster_wait_acquire();  // every tile has started and read its carried state
+  if (warp == 0) {
+    const TileAgg<F> agg = sh.agg;
+    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) {
+      TileAgg<F>* to = cl.map_shared_rank(sh.caggs, (unsigned)j) + tile;
+      to->e = agg.e;
+      if (turn_mean) to->c0 = agg.c0;
+    }
+  }
+  if (kNarrow && __any_sync(0xffffffffu, row_wide(q)) && lane < n_tiles) *cl.map_shared_rank(s_wide, (unsigned)lane) = 1;
+  __syncwarp();
+  cluster_arrive_release();
+  meanwhile();             // (while the aggregates are on their way)
+  cluster_wait_acquire();  // every aggregate has arrived; nothing touches these arrays after
+  if (kNarrow && *s_wide) return false;
+  if (warp == 0) {
+    // the predecessors' aggregates folded in tile order (a warp scan: the
+    // stop sum fp64, the open-turn sums as inside a tile)
+    const TileAgg<F> none = {{0.0, 0, 0, 0, 0}, 0.0};
+    TileAgg<F> v = none;
+    if (lane < tile) v = sh.caggs[lane];
+#pragma unroll
+    for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
+      const TileElem<F> o = tile_shfl_up(v.e, d);
+      if (turn_mean) {
+        const double c0 = __shfl_up_sync(0xffffffffu, v.c0, d);
+        if (lane >= d) v.c0 = tile_c0(o, c0, v);
+      }
+      if (lane >= d) v.e = tile_combine(o, v.e);
+    }
+    if (lane == (tile > 0 ? (int)tile - 1 : 0)) sh.excl = tile > 0 ? v : none;
+  }
+  __syncthreads();
+
+  // 5. complete every row
+  if (live) {
+    // the row's prefixes: the stop sum fp64, the open-turn sums in F
+    const TileElem<F> pre = sh.excl.e;
+    const TileElem<F> ri = tile_combine(pre, tile_incl);
+    const double from = (tile_excl.flags & kRestartSum) ? 0.0 : pre.c;  // what c counts from, before this row
+    if (!seeded) c_before = from + tile_excl.c;
+    if (turn_mean && !meta.bad) {  // the sum before the row's turn
+      const int64_t j = meta.turn_start - r0;
+      c0 = j < 0 ? sh.excl.c0 : seeded ? q.cum0 : from + sh.c0[j];
+    }
+    RowCarry rc;
+    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, 0.0, fturn};
+    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 0.0, 1};
+    row_tail(p, r, meta, rc, si, c_before, false, true);
+    ri_c = ri.c;
+  }
+
+  // 6. the trajectories' stop records and losses, once per trajectory and warp
+  using Sum = typename std::conditional<kNarrow, Sum2, double>::type;
+  TrajPart<Sum> part = {-1, 0, 0, sum_of<Sum>(0.f), -1};
+  if (live && !meta.bad) {
+    const bool turn_last = (r == meta.turn_end - 1);
+    const bool test = (p.mode == STRIDE_STOP_TOKEN_SUM) || turn_last;
+    // retained unless the rule fired before the row (row_tail); a
+    // trajectory's first token or turn always is
+    const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
+    const bool kept = first || !(turn_mean ? fired_before_turn(p, meta, c0, q.lam) : c_before < (double)q.lam);
+    part.traj = meta.traj;
+    part.count = kept ? 1 : 0;
+    if (kept) part.loss = cluster_term(e_sl);
+    if (test && ri_c < (double)q.lam) {
+      part.cross_row = r - meta.traj_start;
+      part.cross_turn = meta.local_turn;
+    }
+  }
+  record_parts(p, part, lane);
+  return true;
+}
 
 template <int TILE>
 __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p, const float* __restrict__ logp_s,
                                                             const float* __restrict__ logp_t, int64_t n_tiles) {
-  constexpr int kWarps = TILE / 32;
   __shared__ int64_t s_turn_off[TILE + 1];
   __shared__ int64_t s_traj_row[TILE + 1];   // traj_row_off
   __shared__ int64_t s_traj_turn[TILE + 1];  // traj_turn_off, widened
   __shared__ int64_t s_first[2];                      // first turn, first trajectory of the tile
-  __shared__ TileElem s_wtot[kWarps];
-  __shared__ TileElem s_wpre[kWarps];
-  __shared__ double s_c0[TILE];  // by row where a turn begins: the sum c before it (from the row where c restarts)
-  __shared__ TileAgg s_excl;     // the tile's exclusive prefix (flags unused)
-  __shared__ TileAgg s_agg;
+  __shared__ ClusterShared<float, TILE> s_f32;
+  __shared__ ClusterShared<double, TILE> s_f64;
+  __shared__ int s_wide;  // set by any tile of the window
   __shared__ double s_prof[3 * STRIDE_PROFILE_BINS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // Launched as a programmatic dependent of the kernel that wrote the
@@ -1157,6 +1316,7 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
   // before the wait; the log-probs only after it.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid < 3 * STRIDE_PROFILE_BINS) s_prof[tid] = 0.0;
+  if (tid == 0) s_wide = 0;
   const int64_t tile = (int64_t)blockIdx.x;
   const int64_t t0 = tile * TILE;           // first window row of the tile
   const int64_t n_here = min((int64_t)TILE, p.n_rows - t0);
@@ -1194,8 +1354,6 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
     }
   }
   __syncthreads();
-
-  __shared__ TileAgg s_caggs[kClusterMaxTiles];  // predecessors' aggregates
 
   // 2. this thread's row: its turn and trajectory, and its element
   RowMeta meta;
@@ -1247,10 +1405,8 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
     sd0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_d);
     sl0 = fturn ? 0.0 : __ldcg(&sp->turn_sum_l);
   }
-  Rows<1, false> row;  // for the profile
-  row.what[0] = (live ? kRowLive : 0) | (meta.bad ? kRowBad : 0);
-  row.bin[0] = 0;
-  if (p.profile && live && !meta.bad) row.bin[0] = (int)((10 * (r - meta.turn_start)) / (meta.turn_end - meta.turn_start));
+  int bin = 0;
+  if (p.profile && live && !meta.bad) bin = (int)((10 * (r - meta.turn_start)) / (meta.turn_end - meta.turn_start));
   const float lam = (live && !meta.bad) ? (p.lambda ? __ldg(p.lambda + meta.traj) : p.lambda_all) : 0.f;
   cluster_arrive_release();  // this CTA's reads of the carried state are done
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1258,130 +1414,23 @@ __global__ void __launch_bounds__(TILE) scan_cluster_kernel(const BatchParams p,
     lps = __ldcg(logp_s + w);
     lpt = __ldcg(logp_t + w);
   }
-  TileElem x = {0.0, 0.0, 0.0, 0.0, 0};
-  double c_before = 0.0, c0 = 0.0, ri_c = 0.0;
-  float e_sl = 0.f;
-  if (live) {
-    const float nan = __int_as_float(0x7fc00000);
-    if (meta.bad) {
-      set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
-      lps = nan;
-      lpt = nan;
-      if (p.out.logp_s) p.out.logp_s[w] = nan;  // a bad row's log-probs are NaN
-      if (p.out.logp_t) p.out.logp_t[w] = nan;
-    }
-    const float dd = lps - lpt;
-    if (p.out.opd) p.out.opd[w] = dd;
-    const int64_t n_k = meta.turn_end - meta.turn_start;
-    // The row's terms in fp32 (logp_S * d rounded once, as the fp64 product
-    // of two floats rounded to float would be); the stop-sum term in fp64,
-    // a turn mean's share lpt / n_k rounded once to fp32 first (GB300 issues
-    // an fp64 divide as a sequence of fp64 operations at 1/64 of the fp32
-    // rate; the rounding is 6e-8 of the term).
-    const float esl = lps * dd;
-    const double ec =
-        (p.mode == STRIDE_STOP_TURN_MEAN) ? (double)(lpt / (float)(n_k > 0 ? n_k : 1)) : (double)lpt;
-    e_sl = esl;
-    if (seeded && !meta.bad) {
-      x = TileElem{cum0 + ec, (float)(st0 + (double)lpt), (float)(sd0 + (double)dd), (float)(sl0 + (double)esl),
-                   kRestartSum | kRestartTurn};
-      c_before = cum0;
-    } else if (seeded) {
-      x = TileElem{ec, lpt, dd, esl, kRestartSum | kRestartTurn};  // NaN: nothing after a bad row is meaningful
-    } else {
-      x = TileElem{ec, lpt, dd, esl, fturn ? kRestartTurn : 0};
-    }
-    if (seeded) x.flags |= 4;  // bit 2: this row's exclusive prefix is the carried state, not the scan
+  if (live && meta.bad) {
+    set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
+    lps = lpt = __int_as_float(0x7fc00000);
+    if (p.out.logp_s) p.out.logp_s[w] = lps;  // a bad row's log-probs are NaN
+    if (p.out.logp_t) p.out.logp_t[w] = lps;
   }
-
-  // 3. segmented inclusive scan over the tile
-  const TileElem tile_id = {0.0, 0.f, 0.f, 0.f, 0};
-  TileElem tile_incl, tile_excl;
-  block_scan<kWarps>(x, tile_id, lane, warp, s_wtot, s_wpre, tile_incl, tile_excl);
-
-  // 4. the tile's exclusive prefix, from the cluster's other tiles
-  namespace cg = cooperative_groups;
-  const bool turn_mean = p.mode == STRIDE_STOP_TURN_MEAN;
-  if (turn_mean && (seeded || fturn)) {
-    const double c0 = seeded ? cum0 : tile_excl.c;
-    s_c0[tid] = c0;
-    if (meta.turn_end >= r0 + n_here) s_agg.c0 = c0;  // the tile's last turn
-  }
-  if (tid == (int)(n_here - 1)) s_agg.e = tile_incl;
-  __syncthreads();
-  cluster_wait_acquire();  // every tile has started and read its carried state
-  if (warp == 0) {
-    const cg::cluster_group cl = cg::this_cluster();
-    const TileAgg agg = s_agg;
-    for (int64_t j = tile + 1 + lane; j < n_tiles; j += 32) {
-      TileAgg* to = cl.map_shared_rank(s_caggs, (unsigned)j) + tile;
-      to->e = agg.e;
-      if (turn_mean) to->c0 = agg.c0;
-    }
-  }
-  cluster_arrive_release();
-  if (p.profile) {  // (while the aggregates are on their way)
-    row.lps[0] = lps;
-    row.lpt[0] = lpt;
-    rows_profile(row, lane, s_prof);
-  }
-  cluster_wait_acquire();  // every aggregate has arrived; nothing touches this CTA's memory after
-  if (warp == 0) {
-    // the predecessors' aggregates folded in tile order (a warp scan: the
-    // stop sum fp64, the open-turn sums fp32 as inside a tile)
-    const TileAgg none = {{0.0, 0.f, 0.f, 0.f, 0}, 0.0};
-    TileAgg v = none;
-    if (lane < tile) v = s_caggs[lane];
-#pragma unroll
-    for (int d = 1; d < kClusterMaxTiles; d <<= 1) {
-      const TileElem o = tile_shfl_up(v.e, d);
-      if (turn_mean) {
-        const double c0 = __shfl_up_sync(0xffffffffu, v.c0, d);
-        if (lane >= d) v.c0 = tile_c0(o, c0, v);
-      }
-      if (lane >= d) v.e = tile_combine(o, v.e);
-    }
-    if (lane == (tile > 0 ? (int)tile - 1 : 0)) s_excl = tile > 0 ? v : none;
-  }
-  __syncthreads();
-
-  // 5. complete every row
-  if (live) {
-    // the row's prefixes: the stop sum fp64, the open-turn sums fp32 (the
-    // tile's prefix rounded once to fp32; 6e-8 of the sums)
-    const TileElem pre = s_excl.e;
-    const TileElem ri = tile_combine(pre, tile_incl);
-    const double from = (tile_excl.flags & kRestartSum) ? 0.0 : pre.c;  // what c counts from, before this row
-    if (!(x.flags & 4)) c_before = from + tile_excl.c;
-    if (turn_mean && !meta.bad) {  // the sum before the row's turn
-      const int64_t j = meta.turn_start - r0;
-      c0 = j < 0 ? s_excl.c0 : seeded ? cum0 : from + s_c0[j];
-    }
-    RowCarry rc;
-    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, 0.0, fturn};
-    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 0.0, 1};
-    row_tail(p, r, meta, rc, si, c_before, false, true);
-    ri_c = ri.c;
-  }
-
-  // 6. the trajectories' stop records and losses, once per trajectory and warp
-  TrajPart<Sum2> part = {-1, 0, 0, {0.f, 0.f}, -1};
-  if (live && !meta.bad) {
-    const bool turn_last = (r == meta.turn_end - 1);
-    const bool test = (p.mode == STRIDE_STOP_TOKEN_SUM) || turn_last;
-    // retained unless the rule fired before the row (row_tail); a
-    // trajectory's first token or turn always is
-    const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
-    const bool kept = first || !(turn_mean ? fired_before_turn(p, meta, c0, lam) : c_before < (double)lam);
-    part.traj = meta.traj;
-    part.count = kept ? 1 : 0;
-    part.loss.hi = kept ? e_sl : 0.f;
-    if (test && ri_c < (double)lam) {
-      part.cross_row = r - meta.traj_start;
-      part.cross_turn = meta.local_turn;
-    }
-  }
-  record_parts(p, part, lane);
+  if (live && p.out.opd) p.out.opd[w] = lps - lpt;
+  const ClusterRow x = {meta, r, lps, lpt, lam, cum0, st0, sd0, sl0, live, seeded, fturn != 0};
+  Rows<1, false> row;  // for the profile
+  row.what[0] = (live ? kRowLive : 0) | (meta.bad ? kRowBad : 0);
+  row.bin[0] = bin;
+  row.lps[0] = lps;
+  row.lpt[0] = lpt;
+  const bool done = scan_cluster_rows<float, TILE>(p, x, tile, n_tiles, r0, (int)n_here, s_f32, &s_wide, [&] {
+    if (p.profile) rows_profile(row, lane, s_prof);
+  });
+  if (!done) scan_cluster_rows<double, TILE>(p, x, tile, n_tiles, r0, (int)n_here, s_f64, &s_wide, [] {});
   if (p.profile) {
     __syncthreads();
     if (tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);

@@ -24,11 +24,8 @@ def _masked(rng, rows, V, f32, turns):
     """Trajectories of `turns`; in each, one turn (the third, fourth, ... in
     rotation) with masked sampled tokens: once in T, twice, once in S, once in
     both."""
-    per = sum(turns)
-    n = -(-rows // per)
-    lens = [list(turns) for _ in range(n)]
-    lens[-1][-1] -= n * per - rows
-    lay = synth.layout_from_turn_lengths(lens)
+    assert rows % sum(turns) == 0
+    lay = synth.layout_from_turn_lengths([list(turns)] * (rows // sum(turns)))
     S32 = rng.standard_normal((rows, V), dtype=np.float32)
     T32 = S32 + rng.standard_normal((rows, V), dtype=np.float32) * np.float32(0.3)
     S, T = (S32, T32) if f32 else (synth.bf16_bits_from_f32(S32), synth.bf16_bits_from_f32(T32))
@@ -69,18 +66,19 @@ def _compare(g, o, lay, mode):
         assert np.all(np.abs(g["profile"][:, 1 - k] - o["profile"][:, 1 - k]) <= SUM_RTOL * prof[k]), k
 
 
-# 1,300 rows: more than the small-window kernel takes.  Below 57,344 logits the scan follows the persistent kernel,
-# from there on it runs inside.
+# Up to 1,216 rows a window takes the small-window kernel and the cluster scan (tiles of 128 rows).  From there on, below
+# 57,344 logits the scan follows the persistent kernel, else it runs inside.  Windows of both kinds carry state across.
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("rows, V, f32", [(1300, 32_000, False), (2600, 4_099, True), (1300, 57_343, False),
-                                          (1300, 57_344, False), (80_000, 64, False)])
+                                          (1300, 57_344, False), (80_000, 64, False), (100, 64, True), (700, 32_000, False),
+                                          (1200, 4_099, False)])
 def test_lowest_finite_logit(stride, rows, V, f32, mode):
     rng = np.random.default_rng(rows + V + mode)
     lay, S, T, tok = _masked(rng, rows, V, f32, (7, 20, 33, 4, 36))
     lam = np.float32(-1e6)  # only a masked log-prob crosses it
     o = oracle_batch(S, T, tok, lay, mode, lam)
     half = rows // 2 - 13
-    for windows in (None, [(0, half), (half, rows)]) if rows > 2500 else (None,):
+    for windows in (None, [(0, half), (half, rows)], [(0, half), (half, half + 30), (half + 30, rows)]):
         g = run_batch(stride, S, T, tok, lay, mode, lam, windows=windows)
         assert g["status"] == 0
         _compare(g, o, lay, mode)
