@@ -460,6 +460,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) score_batch_stream_kernel(c
     if ((int64_t)counted == min((int64_t)kTileRows, p.n_rows - t * kTileRows)) {
       int i = lane == 0 ? queue_claim(sh) : 0;
       i = __shfl_sync(0xffffffffu, i, 0);
+      // lane 0 has acquired the tile's other rows (count_in) and the queue's
+      // entry (queue_claim); a shuffle orders no memory, so this passes both on
+      __syncwarp();
       TileCarry& tc = i < 0 ? sh.own[warp - 1] : sh.queue[i];
       publish_tile(p, t, lane, tc);
       __syncwarp();
