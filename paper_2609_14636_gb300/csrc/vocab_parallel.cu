@@ -293,30 +293,41 @@ __device__ __forceinline__ int smem_upper_le(const int64_t* a, int n, int64_t r)
 // two CTAs of the second fit beside its two; 33.0 without both).
 constexpr int kPassThreads = 256;
 constexpr int kPassWarps = kPassThreads / 32;
-// Up to this many tiles a tile folds its predecessors' aggregates itself
-// (kPassThreads per round, back to the nearest seeded tile); above it one CTA
-// turns them into prefixes first, so that one long trajectory's scan stays
-// linear in its rows.
-constexpr int64_t kDirectTiles = 4096;
+// A tile folds its predecessors' aggregates itself (kPassThreads per round,
+// back to the nearest seeded tile), or one CTA turns them into prefixes first,
+// so that long trajectories' scans stay linear in their rows: above kDirectTiles
+// tiles, whatever the trajectories, and above kDirectMean tiles per trajectory.
+// GB300, state and scan in turn mode, us folded / prefixed: one trajectory of
+// 262,144 rows 32.6 / 37.9, 524,288 (1,024 tiles) 56.2 / 56.8, 1,048,576 104.5 /
+// 84.6, 2,097,152 (4,096 tiles) 213.9 / 144.5; in trajectories of 65,536 rows
+// 43.1 / 55.1, 74.2 / 80.3 and 140.1 / 149.0 at the last three, of 2,326 rows
+// 49.4 / 60.8, 79.0 / 94.7 and 148.2 / 172.1.
+constexpr int64_t kDirectTiles = 4096, kDirectMean = 1024;
 constexpr int kFromSeed = 8;  // the open turn's sums start at a seeded row
 
-// A tile's aggregate, or, after scan_prefix_kernel, the prefix before it: as a
-// ScanSlot, with the sum c before the last turn start, and the kRestart marks.
-// (Two of the workspace's slots per row: a tile has more rows than that, or
-// the slots' 256-byte padding holds them.)
-struct alignas(64) TileSlot {
-  double c, st, sd, sl, c0;  // (c0 counted as c is: from the last seeded row, or the tile's first)
+// A tile's aggregate, or, after scan_prefix_kernel, the prefix before it: a
+// ScanSlot in agg[tile], and beside it, in the flags' place, the sum c before
+// its last turn start (counted as c is: from the last seeded row, or the tile's
+// first) and its kRestart marks.
+struct alignas(16) TileMark {
+  double c0;
   int marks;
 };
-static_assert(sizeof(TileSlot) == 2 * sizeof(ScanSlot) && sizeof(TileSlot) <= 256, "a tile's share of the workspace");
+struct TileSlot {
+  ScanSlot sum;
+  TileMark mark;
+};
 
 // Past this SM's L1.
-__device__ __forceinline__ TileSlot load_tile(const TileSlot* t) {
-  const double2 a = __ldcg(reinterpret_cast<const double2*>(t));
-  const double2 b = __ldcg(reinterpret_cast<const double2*>(t) + 1);
-  TileSlot r = {a.x, a.y, b.x, b.y, __ldcg(&t->c0), 0};
-  r.marks = __ldcg(&t->marks);
-  return r;
+__device__ __forceinline__ TileSlot load_tile(const BatchParams& p, int64_t tile) {
+  const double2* s = reinterpret_cast<const double2*>(p.agg + tile);
+  const double2 a = __ldcg(s), b = __ldcg(s + 1), m = __ldcg(reinterpret_cast<const double2*>(p.flags) + tile);
+  return TileSlot{{a.x, a.y, b.x, b.y}, {m.x, (int)__double_as_longlong(m.y)}};
+}
+
+__device__ __forceinline__ void store_tile(const BatchParams& p, int64_t tile, const TileSlot& t) {
+  p.agg[tile] = t.sum;
+  reinterpret_cast<TileMark*>(p.flags)[tile] = t.mark;
 }
 
 // A tile's part of the layout: the offsets of its first turn and of the
@@ -824,9 +835,8 @@ __device__ __forceinline__ bool aggregate_tile(const BatchParams& p, int64_t til
     sl = warp_sum(lane < kPassWarps ? s_open[2][lane] : zero);
     if (lane == 0) {
       c0 += s_base[0];
-      reinterpret_cast<TileSlot*>(p.agg)[tile] =
-          TileSlot{c0 + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl), c0,
-                   (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0)};
+      store_tile(p, tile, TileSlot{{c0 + c, s_base[1] + sum_value(st), s_base[2] + sum_value(sd), s_base[3] + sum_value(sl)},
+                                   {c0, (own_c >= 0 ? kRestartSum : 0) | (own_t >= 0 ? kRestartTurn : 0)}});
     }
   }
   return true;
@@ -863,13 +873,17 @@ __global__ void __launch_bounds__(kPassThreads, EXACT && R > 1 ? 4 : 5) scan_agg
 }
 
 // Between the passes of a window of many tiles: the aggregates replaced by
-// the prefixes before each tile.  One CTA, in rounds of a tile per thread.
+// the prefixes before each tile.  One CTA, a run of tiles per thread.
 constexpr int kPrefixThreads = 1024;
 
 struct PrefixElem {
   double c, st, sd, sl, c0;
   int flags;
 };
+
+__device__ __forceinline__ PrefixElem prefix_elem(const TileSlot& t) {
+  return PrefixElem{t.sum.c, t.sum.st, t.sum.sd, t.sum.sl, t.mark.c0, t.mark.marks};
+}
 
 __device__ __forceinline__ PrefixElem elem_combine(const PrefixElem& a, const PrefixElem& b) {
   PrefixElem r;
@@ -894,29 +908,24 @@ __device__ __forceinline__ PrefixElem elem_shfl_up(const PrefixElem& v, int d) {
   return o;
 }
 
-__global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(TileSlot* tiles, int64_t n_tiles) {
+__global__ void __launch_bounds__(kPrefixThreads) scan_prefix_kernel(const BatchParams p, int64_t n_tiles) {
   constexpr int kWarps = kPrefixThreads / 32;
-  __shared__ PrefixElem s_tot[kWarps], s_pre[kWarps], s_carry;
+  __shared__ PrefixElem s_tot[kWarps], s_pre[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PrefixElem id = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
-  PrefixElem carry = id;
-  for (int64_t t = 0; t < n_tiles; t += kPrefixThreads) {
-    const int64_t j = t + tid;
-    PrefixElem v = id;
-    if (j < n_tiles) {
-      const TileSlot a = load_tile(tiles + j);
-      v = PrefixElem{a.c, a.st, a.sd, a.sl, a.c0, a.marks};
-    }
-    PrefixElem incl, excl;
-    block_scan<kWarps>(v, id, lane, warp, s_tot, s_pre, incl, excl);
-    const PrefixElem before = elem_combine(carry, excl);
-    if (j < n_tiles) tiles[j] = TileSlot{before.c, before.st, before.sd, before.sl, before.c0, before.flags};
-    if (tid == kPrefixThreads - 1) s_carry = elem_combine(carry, incl);
-    __syncthreads();
-    carry = s_carry;
-    __syncthreads();
+  const int64_t per = (n_tiles + kPrefixThreads - 1) / kPrefixThreads;
+  const int64_t j0 = min(tid * per, n_tiles), j1 = min(j0 + per, n_tiles);
+  PrefixElem v = id, incl, before;
+#pragma unroll 4
+  for (int64_t j = j0; j < j1; ++j) v = elem_combine(v, prefix_elem(load_tile(p, j)));
+  block_scan<kWarps>(v, id, lane, warp, s_tot, s_pre, incl, before);
+#pragma unroll 4
+  for (int64_t j = j0; j < j1; ++j) {
+    const PrefixElem e = prefix_elem(load_tile(p, j));
+    store_tile(p, j, TileSlot{{before.c, before.st, before.sd, before.sl}, {before.c0, before.flags}});
+    before = elem_combine(before, e);
   }
 }
 
@@ -1474,49 +1483,45 @@ __device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLa
   if (block_scan<kPassWarps, kNarrow>(own, id, lane, warp, s_tot, s_wpre, incl, excl, kNarrow && rows_wide(x)))
     return false;
   if (own.flags & kRestartTurn) s_turn_c0[tid] = (own.flags & kRestartSum) ? c0 : excl.c + c0;
-  const TileSlot* tiles = reinterpret_cast<const TileSlot*>(p.agg);
 
   // ---- the first pass's results
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // Sums of the predecessors' aggregates back to the nearest one with a seeded
   // row (c), and to the nearest one with a turn start (the open turn's); c0 is
   // that one's, with the sums c before it back to the seeded row.  A seeded
-  // tile among the 32 before this one is warp 0's to find.
-  if (warp == 0 && s_needs) {
-    TileSlot a = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
-    if (prefixed || lane < tile) a = load_tile(tiles + (prefixed ? tile : tile - 1 - lane));
-    const unsigned b_sum = __ballot_sync(0xffffffffu, (a.marks & kRestartSum) != 0);
-    const unsigned b_turn = __ballot_sync(0xffffffffu, (a.marks & kRestartTurn) != 0);
-    double f[5] = {a.c, a.st, a.sd, a.sl, a.c0};
-    if (!prefixed && b_sum) {
-      const int n_sum = __ffs(b_sum) - 1, n_turn = __ffs(b_turn) - 1;  // (a seeded row is a turn's start: n_turn <= n_sum)
-      f[4] = warp_sum(lane == n_turn ? a.c0 : lane > n_turn && lane <= n_sum ? a.c : 0.0);
-      f[0] = warp_sum(lane <= n_sum ? a.c : 0.0);
-      f[1] = warp_sum(lane <= n_turn ? a.st : 0.0);
-      f[2] = warp_sum(lane <= n_turn ? a.sd : 0.0);
-      f[3] = warp_sum(lane <= n_turn ? a.sl : 0.0);
+  // tile among the 32 before this one is warp 0's alone to fold.
+  const bool needs = s_needs;
+  TileSlot a = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0}};
+  if (needs) {
+    if (prefixed || tid < tile) a = load_tile(p, prefixed ? tile : tile - 1 - tid);
+    const unsigned b_sum = __ballot_sync(0xffffffffu, (a.mark.marks & kRestartSum) != 0);
+    const unsigned b_turn = __ballot_sync(0xffffffffu, (a.mark.marks & kRestartTurn) != 0);
+    if (lane == 0) {
+      s_near[0][warp] = b_sum ? warp * 32 + __ffs(b_sum) - 1 : kPassThreads;
+      s_near[1][warp] = b_turn ? warp * 32 + __ffs(b_turn) - 1 : kPassThreads;
     }
-    if (lane == 0 && (prefixed || b_sum)) {
+    if (warp == 0 && (prefixed || b_sum)) {
+      double f[5] = {a.sum.c, a.sum.st, a.sum.sd, a.sum.sl, a.mark.c0};
+      if (!prefixed) {
+        const int n_sum = __ffs(b_sum) - 1, n_turn = __ffs(b_turn) - 1;  // (a seeded row starts a turn: n_turn <= n_sum)
+        if (p.mode == STRIDE_STOP_TURN_MEAN)
+          f[4] = warp_sum(lane == n_turn ? f[4] : lane > n_turn && lane <= n_sum ? f[0] : 0.0);
+        f[0] = warp_sum(lane <= n_sum ? f[0] : 0.0);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) s_pre[k] = f[k];
-      s_folded = 1;
+        for (int k = 1; k < 4; ++k) f[k] = warp_sum(lane <= n_turn ? f[k] : 0.0);
+      }
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) s_pre[k] = f[k];
+        s_folded = 1;
+      }
     }
   }
   __syncthreads();
-  if (s_needs && !s_folded) {
+  if (needs && !s_folded) {
     double f[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     bool turn_open = true, any = false;
-    for (int64_t hi = tile; hi > 0; hi -= kPassThreads) {
-      const int64_t j = hi - 1 - tid;
-      TileSlot a = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
-      if (j >= 0) a = load_tile(tiles + j);
-      const unsigned b_sum = __ballot_sync(0xffffffffu, (a.marks & kRestartSum) != 0);
-      const unsigned b_turn = __ballot_sync(0xffffffffu, (a.marks & kRestartTurn) != 0);
-      if (lane == 0) {
-        s_near[0][warp] = b_sum ? warp * 32 + __ffs(b_sum) - 1 : kPassThreads;
-        s_near[1][warp] = b_turn ? warp * 32 + __ffs(b_turn) - 1 : kPassThreads;
-      }
-      __syncthreads();
+    for (int64_t hi = tile;;) {
       int n_sum = kPassThreads, n_turn = kPassThreads;
 #pragma unroll
       for (int w = 0; w < kPassWarps; ++w) {
@@ -1525,22 +1530,33 @@ __device__ __forceinline__ bool complete_tile(const BatchParams& p, const TileLa
       }
       if (warp * 32 <= n_sum && hi > warp * 32) {
         any = true;
-        if (tid <= n_sum) f[0] += a.c;
+        if (tid <= n_sum) f[0] += a.sum.c;
         if (turn_open && tid <= n_turn) {
-          f[1] += a.st;
-          f[2] += a.sd;
-          f[3] += a.sl;
-          if (tid == n_turn) f[4] = a.c0;
+          f[1] += a.sum.st;
+          f[2] += a.sum.sd;
+          f[3] += a.sum.sl;
+          if (tid == n_turn) f[4] = a.mark.c0;
         } else if (tid <= n_sum) {
-          f[4] += a.c;
+          f[4] += a.sum.c;
         }
       }
       turn_open = turn_open && n_turn == kPassThreads;
-      if (n_sum < kPassThreads) break;
+      hi -= kPassThreads;
+      if (n_sum < kPassThreads || hi <= 0) break;
+      __syncthreads();  // (s_near has been read)
+      a = TileSlot{{0.0, 0.0, 0.0, 0.0}, {0.0, 0}};
+      if (tid < hi) a = load_tile(p, hi - 1 - tid);
+      const unsigned b_sum = __ballot_sync(0xffffffffu, (a.mark.marks & kRestartSum) != 0);
+      const unsigned b_turn = __ballot_sync(0xffffffffu, (a.mark.marks & kRestartTurn) != 0);
+      if (lane == 0) {
+        s_near[0][warp] = b_sum ? warp * 32 + __ffs(b_sum) - 1 : kPassThreads;
+        s_near[1][warp] = b_turn ? warp * 32 + __ffs(b_turn) - 1 : kPassThreads;
+      }
       __syncthreads();
     }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
+      if (k == 4 && p.mode != STRIDE_STOP_TURN_MEAN) break;
       const double v = any ? warp_sum(f[k]) : 0.0;
       if (lane == 0) s_fold[k][warp] = v;
     }
@@ -1680,11 +1696,11 @@ cudaError_t launch_passes(const BatchParams& p, const float* logp_s, const float
                           cudaStream_t stream) {
   constexpr int kRows = R * kPassThreads;
   const int64_t n_tiles = (p.n_rows + kRows - 1) / kRows;
-  const bool prefixed = n_tiles > kDirectTiles;
+  const bool prefixed = n_tiles > kDirectTiles || n_tiles > kDirectMean * p.n_traj;
   cudaError_t e =
       launch_dependent(scan_aggregate_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, after.scoring);
   if (e == cudaSuccess && prefixed)
-    e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, reinterpret_cast<TileSlot*>(p.agg), n_tiles);
+    e = launch_dependent(scan_prefix_kernel, 1, kPrefixThreads, stream, p, n_tiles);
   if (e == cudaSuccess)
     e = launch_dependent(scan_complete_kernel<R, EXACT>, (unsigned)n_tiles, kPassThreads, stream, p, logp_s, logp_t, n_tiles,
                          prefixed, !after.checked);

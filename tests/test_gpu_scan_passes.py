@@ -80,6 +80,7 @@ CASES = [(r, s) for r in (1, 31, 255, 256, 257, 5000) for s in ("one", "mixed")]
 CASES += [(ONE_WAVE + d, s) for d in (-1, 0, 1) for s in ("turns", "mixed")]
 CASES += [(512 * 79 + d, s) for d in (0, 1, 511) for s in ("one", "mixed")]
 CASES += [(4096 * 512 + 1, s) for s in ("turns", "mixed")]
+CASES += [(1024 * 512 + d, "turns") for d in (0, 1)]  # the longest trajectory that each tile folds by itself
 
 
 @pytest.mark.parametrize("mode", [0, 1])
