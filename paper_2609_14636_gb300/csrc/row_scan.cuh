@@ -45,20 +45,18 @@ struct ScanElem {
   double st;  // sum of log pi_T within the open turn
   double sd;  // sum of d within the open turn
   double sl;  // sum of the OPD-loss terms logp_S * d within the open turn
-  double c0;  // the sum c before the open turn (with fturn)
   int fturn;  // the range contains a turn's first row
 };
 
 // a (earlier rows) (+) b (later rows).  c never resets inside a lookback
 // (trajectory starts publish inclusive prefixes); st, sd and sl restart at a
-// turn's first row, where c0 is taken.
+// turn's first row.
 __device__ __forceinline__ ScanElem combine(const ScanElem& a, const ScanElem& b) {
   ScanElem r;
   r.c = a.c + b.c;
   r.st = b.fturn ? b.st : a.st + b.st;
   r.sd = b.fturn ? b.sd : a.sd + b.sd;
   r.sl = b.fturn ? b.sl : a.sl + b.sl;
-  r.c0 = b.fturn ? a.c + b.c0 : a.c0;
   r.fturn = a.fturn | b.fturn;
   return r;
 }
@@ -73,15 +71,16 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// c0 of a row's or tile's published element: in its flag's line, the
-// aggregate's (1) and the inclusive prefix's (2) 8 bytes.
+// Beside a row's or tile's published element, in its flag's line: the sum c
+// before the open turn (with fturn), for the aggregate (1) and the inclusive
+// prefix (2) 8 bytes.
 __device__ __forceinline__ double* slot_c0(uint32_t* flag, bool inclusive) {
   return reinterpret_cast<double*>(flag) + (inclusive ? 2 : 1);
 }
 
-__device__ __forceinline__ void publish(ScanSlot* slot, uint32_t* flag, const ScanElem& e,
+__device__ __forceinline__ void publish(ScanSlot* slot, uint32_t* flag, const ScanElem& e, double c0,
                                         uint32_t status) {
-  *slot_c0(flag, (status & kStMask) == kStIncl) = e.c0;
+  *slot_c0(flag, (status & kStMask) == kStIncl) = c0;
   slot->c = e.c;
   slot->st = e.st;
   slot->sd = e.sd;
@@ -165,9 +164,12 @@ __device__ __forceinline__ void validate_layout(const BatchParams& p, int64_t t)
 }
 
 // Folds published predecessors of `tile` back to the nearest inclusive
-// prefix.  Warp-wide; every lane returns the same exclusive prefix.
-static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane, bool& timed_out) {
-  ScanElem excl = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
+// prefix.  Warp-wide; every lane returns the same exclusive prefix, and (for
+// turn means) in c0 the sum c before the open turn.
+static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane, bool& timed_out, double& c0) {
+  ScanElem excl = {0.0, 0.0, 0.0, 0.0, 0};
+  c0 = 0.0;
+  const bool turn_mean = p.mode == STRIDE_STOP_TURN_MEAN;
   int64_t j = tile - 1;
   const uint64_t t0 = globaltimer_ns();
   while (true) {
@@ -188,7 +190,8 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
     const bool is_incl = (f & kStMask) == kStIncl;
     const unsigned inc = __ballot_sync(0xffffffffu, is_incl);
     const int stop = inc ? __ffs(inc) - 1 : 31;
-    ScanElem v = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
+    ScanElem v = {0.0, 0.0, 0.0, 0.0, 0};
+    double before = 0.0;
     if (valid && lane <= stop && !(f & kFlagTimedOut)) {
       const ScanSlot* src = is_incl ? (p.incl + idx) : (p.agg + idx);
       const double2 a = __ldcg(reinterpret_cast<const double2*>(src));
@@ -197,10 +200,14 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
       v.st = a.y;
       v.sd = b.x;
       v.sl = b.y;
-      v.c0 = __ldcg(slot_c0(p.flags + idx * kFlagStride, is_incl));
+      if (turn_mean) before = __ldcg(slot_c0(p.flags + idx * kFlagStride, is_incl));
       v.fturn = (is_incl || (f & kFlagTurnStart)) ? 1 : 0;
     }
     if (f & kFlagTimedOut) timed_out = true;
+    // c0: the nearest turn start's, with the sums before that (past `stop` v is 0)
+    const unsigned m_turn = __ballot_sync(0xffffffffu, v.fturn);
+    const int near = m_turn ? __ffs(m_turn) - 1 : 32;
+    before = lane == near ? before : lane > near ? v.c : 0.0;
     // Ordered fold of lanes stop..0 (lane l+d holds an earlier row than lane
     // l): a 5-step shuffle tree; lanes past `stop` hold the identity.
 #pragma unroll
@@ -210,17 +217,17 @@ static __device__ ScanElem lookback(const BatchParams& p, int64_t tile, int lane
       o.st = __shfl_down_sync(0xffffffffu, v.st, d);
       o.sd = __shfl_down_sync(0xffffffffu, v.sd, d);
       o.sl = __shfl_down_sync(0xffffffffu, v.sl, d);
-      o.c0 = __shfl_down_sync(0xffffffffu, v.c0, d);
       o.fturn = __shfl_down_sync(0xffffffffu, v.fturn, d);
       if (lane + d < 32) v = combine(o, v);
+      if (turn_mean) before += __shfl_xor_sync(0xffffffffu, before, d);
     }
     ScanElem win;
     win.c = __shfl_sync(0xffffffffu, v.c, 0);
     win.st = __shfl_sync(0xffffffffu, v.st, 0);
     win.sd = __shfl_sync(0xffffffffu, v.sd, 0);
     win.sl = __shfl_sync(0xffffffffu, v.sl, 0);
-    win.c0 = __shfl_sync(0xffffffffu, v.c0, 0);
     win.fturn = __shfl_sync(0xffffffffu, v.fturn, 0);
+    c0 = excl.fturn ? c0 + win.c : before;
     excl = combine(win, excl);
     if (inc) break;
     j -= 32;
@@ -238,6 +245,7 @@ struct RowCarry {
   ScanElem e;
   ScanElem incl;      // valid for seeded tiles
   double c_before;    // running sum before this row (seeded tiles)
+  double c0;          // running sum before this row's turn (seeded tiles)
   int seeded;
 };
 
@@ -279,7 +287,6 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
   e.st = (double)lpt;
   e.sd = (double)dd;
   e.sl = (double)lps * (double)dd;  // -log pi_S * r_t (Eq. 2)
-  e.c0 = 0.0;
   e.fturn = (r == meta.turn_start) ? 1 : 0;
   if (p.profile && !meta.bad) {
     const int j = (int)((10 * (r - meta.turn_start)) / n_k);  // Observation 1 decile
@@ -289,7 +296,7 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
   }
   rc.e = e;
   rc.seeded = (tile == 0) || (r == meta.traj_start) || meta.bad;
-  rc.c_before = 0.0;
+  rc.c_before = rc.c0 = 0.0;
   if (rc.seeded) {
     if (meta.bad) {
       rc.incl = e;  // NaN terms; nothing downstream of a bad row is meaningful
@@ -299,18 +306,17 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
       const double st0 = __ldcg(&sp->turn_sum_t);
       const double sd0 = __ldcg(&sp->turn_sum_d);
       const double sl0 = __ldcg(&sp->turn_sum_l);
-      rc.c_before = cum0;
+      rc.c_before = rc.c0 = cum0;
       rc.incl.c = cum0 + e.c;
       rc.incl.st = e.fturn ? e.st : st0 + e.st;
       rc.incl.sd = e.fturn ? e.sd : sd0 + e.sd;
       rc.incl.sl = e.fturn ? e.sl : sl0 + e.sl;
-      rc.incl.c0 = cum0;
       rc.incl.fturn = 1;
     }
-    publish(p.incl + tile, p.flags + tile * kFlagStride, rc.incl, kStIncl);
+    publish(p.incl + tile, p.flags + tile * kFlagStride, rc.incl, rc.c0, kStIncl);
   } else {
     rc.incl = e;
-    publish(p.agg + tile, p.flags + tile * kFlagStride, e, kStAgg | (e.fturn ? kFlagTurnStart : 0u));
+    publish(p.agg + tile, p.flags + tile * kFlagStride, e, 0.0, kStAgg | (e.fturn ? kFlagTurnStart : 0u));
   }
   return rc;
 }
@@ -331,35 +337,36 @@ __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t t
 // this selects exactly the rows up to the first crossing (its turn, in turn
 // mode).  rc is read in lane 0.
 // row_tail is the single-thread part once the row's inclusive prefix is
-// known: incl (running sum and open-turn sums through the row, and before its
-// turn) and c_before (the running sum before it); of rc only rc.e.sl (the
+// known: incl (running sum and open-turn sums through the row), c_before and c0
+// (the running sum before it, and before its turn); of rc only rc.e.sl (the
 // row's loss term) is read.  With defer_traj the trajectory's stop record and
 // loss are left to the caller (the cluster scan gathers them per trajectory
 // and warp).
 __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const RowMeta& meta,
-                                         const RowCarry& rc, const ScanElem& incl, double c_before,
+                                         const RowCarry& rc, const ScanElem& incl, double c_before, double c0,
                                          bool timed_out, bool defer_traj = false);
 
 __device__ __forceinline__ void row_resolve(const BatchParams& p, int64_t tile, int64_t r,
                                             const RowMeta& meta, RowCarry rc, int lane) {
   const int seeded = __shfl_sync(0xffffffffu, rc.seeded, 0);
   ScanElem incl = rc.incl;
-  double c_before = rc.c_before;
+  double c_before = rc.c_before, c0 = rc.c0;
   bool timed_out = false;
   if (!seeded) {
-    const ScanElem excl = lookback(p, tile, lane, timed_out);
+    const ScanElem excl = lookback(p, tile, lane, timed_out, c0);
     if (lane == 0) {
       incl = combine(excl, rc.e);
       c_before = excl.c;
-      publish(p.incl + tile, p.flags + tile * kFlagStride, incl, kStIncl);
+      if (rc.e.fturn) c0 = c_before;
+      publish(p.incl + tile, p.flags + tile * kFlagStride, incl, c0, kStIncl);
     }
   }
   if (lane != 0) return;
-  row_tail(p, r, meta, rc, incl, c_before, timed_out);
+  row_tail(p, r, meta, rc, incl, c_before, c0, timed_out);
 }
 
 __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const RowMeta& meta,
-                                         const RowCarry& rc, const ScanElem& incl, double c_before,
+                                         const RowCarry& rc, const ScanElem& incl, double c_before, double c0,
                                          bool timed_out, bool defer_traj) {
   if (timed_out) set_status(p.dev_status, STRIDE_DEV_TIMEOUT);
   if (meta.bad) return;
@@ -389,7 +396,7 @@ __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const 
     }
     const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
     const bool fired =
-        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before < (double)lam : fired_before_turn(p, meta, incl.c0, lam);
+        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before < (double)lam : fired_before_turn(p, meta, c0, lam);
     if (first || !fired) {  // the previous test did not fire (a NaN lambda never does)
       atomicAdd(&sp->loss, rc.e.sl);
       atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), 1ull);

@@ -20,7 +20,8 @@ namespace stride {
 __global__ void selftest_lookback_kernel(const BatchParams p) {
   const int lane = threadIdx.x & 31;
   bool timed_out = false;
-  (void)lookback(p, 1, lane, timed_out);
+  double c0;
+  (void)lookback(p, 1, lane, timed_out, c0);
   if (lane == 0 && timed_out) set_status(p.dev_status, STRIDE_DEV_TIMEOUT);
 }
 

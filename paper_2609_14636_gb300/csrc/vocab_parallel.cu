@@ -1279,9 +1279,9 @@ __device__ __forceinline__ bool scan_cluster_rows(const BatchParams& p, const Cl
       c0 = j < 0 ? sh.excl.c0 : seeded ? q.cum0 : from + sh.c0[j];
     }
     RowCarry rc;
-    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, 0.0, fturn};
-    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 0.0, 1};
-    row_tail(p, r, meta, rc, si, c_before, false, true);
+    rc.e = ScanElem{0.0, 0.0, 0.0, (double)e_sl, fturn};
+    const ScanElem si{ri.c, (double)ri.st, (double)ri.sd, (double)ri.sl, 1};
+    row_tail(p, r, meta, rc, si, c_before, c0, false, true);
     ri_c = ri.c;
   }
 

@@ -177,11 +177,11 @@ __device__ __forceinline__ void publish_tile(const BatchParams& p, int64_t t, in
   // ---- the tile's aggregate out, the earlier tiles' prefix in
   uint32_t* flag = p.flags + t * kFlagStride;
   if (lane == n_here - 1) {
-    const ScanElem agg{c, st, sd, sl, c0, 0};
+    const ScanElem agg{c, st, sd, sl, 0};
     if (m_seed)
-      publish(p.incl + t, flag, agg, kStIncl);
+      publish(p.incl + t, flag, agg, c0, kStIncl);
     else
-      publish(p.agg + t, flag, agg, kStAgg | (m_turn ? kFlagTurnStart : 0u));
+      publish(p.agg + t, flag, agg, c0, kStAgg | (m_turn ? kFlagTurnStart : 0u));
   }
   tc.c[lane] = c;
   tc.st[lane] = st;
@@ -231,10 +231,11 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
   const int64_t n_k = good ? meta.turn_end - meta.turn_start : 1;
   const bool fturn = good && r == meta.turn_start;
 
-  ScanElem pre{0.0, 0.0, 0.0, 0.0, 0.0, 0};
+  ScanElem pre{0.0, 0.0, 0.0, 0.0, 0};
+  double pre_c0 = 0.0;
   if (!(m_seed & 1u)) {
     bool timed_out = false;
-    pre = lookback(p, t, lane, timed_out);
+    pre = lookback(p, t, lane, timed_out, pre_c0);
     if (timed_out && lane == 0) set_status(p.dev_status, STRIDE_DEV_TIMEOUT);
     if (h_seed < 0) c += pre.c;
     if (h_turn < 0) {
@@ -248,9 +249,9 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
   if (lane == 0) c_before = pre.c;
   if (seeded) c_before = tc.c_seed[lane];
   const double c0_here = __shfl_sync(0xffffffffu, c_before, max(h_turn, 0));
-  const double c0 = h_turn < 0 ? pre.c0 : c0_here;
+  const double c0 = h_turn < 0 ? pre_c0 : c0_here;
   if (!m_seed && lane == n_here - 1)
-    publish(p.incl + t, p.flags + t * kFlagStride, ScanElem{c, st, sd, sl, c0, 0}, kStIncl);
+    publish(p.incl + t, p.flags + t * kFlagStride, ScanElem{c, st, sd, sl, 0}, c0, kStIncl);
 
   // ---- turn statistics, stop test, retention (row_scan.cuh states the rule)
   const bool turn_last = good && r == meta.turn_end - 1;
