@@ -5,7 +5,8 @@ the C names and argument order; they take torch CUDA tensors, check their
 dtype/device/shape, pass raw device pointers and the current CUDA stream,
 and raise :class:`StrideError` on a non-zero status.  A call whose arguments
 are plain (tensors, ints, floats) is checked and passed on in native code
-(csrc/binding.cpp); any other is taken, or refused, by the ctypes code here.
+(csrc/binding.cpp, where it could be built); any other is taken, or refused,
+by the ctypes code here.
 Every step of the scoring path runs in the library's CUDA kernels: there is
 no Python or CPU fallback, and importing this package fails if the library
 is missing and cannot be built.
@@ -18,6 +19,7 @@ view copies of them as numpy structured arrays.
 from __future__ import annotations
 
 import ctypes
+import warnings
 from pathlib import Path
 
 import numpy as np
@@ -120,19 +122,33 @@ def lib() -> ctypes.CDLL:
 _NATIVE = None
 
 
+class _General:
+    """Stands for the native marshalling where it cannot be had: every call is
+    left to the general code."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _native():
     """The native marshalling module (csrc/binding.cpp), calling the library
     that :func:`lib` loaded.  Each of its functions answers None for a call
-    that it leaves to the general code below."""
+    that it leaves to the general code below.  Where it cannot be built or
+    loaded every call is, after a warning."""
     global _NATIVE
     if _NATIVE is None:
-        import torch  # noqa: F401  (its libraries are the module's)
-
         L = lib()
-        from . import _binding
+        try:
+            import torch  # noqa: F401  (its libraries are the module's)
 
-        _binding.bind(*[ctypes.cast(getattr(L, f"stride_{fn}"), ctypes.c_void_p).value for fn in _NATIVE_ENTRIES])
-        _NATIVE = _binding
+            _build.build_binding()
+            from . import _binding
+
+            _binding.bind(*[ctypes.cast(getattr(L, f"stride_{fn}"), ctypes.c_void_p).value for fn in _NATIVE_ENTRIES])
+            _NATIVE = _binding
+        except Exception as e:
+            warnings.warn(f"native marshalling not available, calls are slower to issue: {e}", RuntimeWarning, stacklevel=3)
+            _NATIVE = _General()
     return _NATIVE
 
 

@@ -2,14 +2,17 @@
 Python module's native marshalling, _binding.so (g++, torch's headers).
 
 Each .cu under csrc/ compiles to an object in parallel; the objects link into
-paper_2609_14636_gb300/libstride.so against the shared CUDA runtime.  The
-build is skipped when both are newer than every source and header.
+paper_2609_14636_gb300/libstride.so against the shared CUDA runtime.  Either
+build is skipped when its result is newer than its sources and headers.  The
+library needs nvcc (and its host compiler) alone: without torch, or where
+binding.cpp does not compile against it, only the marshalling is missing.
 """
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
+import warnings
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -35,19 +38,23 @@ def sources() -> list[Path]:
     return sorted(CSRC.glob("*.cu"))
 
 
-def _deps() -> list[Path]:
-    return sources() + [CSRC / "binding.cpp"] + sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted(INCLUDE.glob("*.h"))
+def _newer(out: Path, deps: list[Path]) -> bool:
+    return out.exists() and all(p.stat().st_mtime <= out.stat().st_mtime for p in deps)
 
 
 def up_to_date() -> bool:
-    if not LIB.exists() or not BINDING.exists():
-        return False
-    t = min(LIB.stat().st_mtime, BINDING.stat().st_mtime)
-    return all(p.stat().st_mtime <= t for p in _deps())
+    """Whether libstride.so is."""
+    return _newer(LIB, sources() + sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted(INCLUDE.glob("*.h")))
 
 
-def _build_binding() -> None:
+def binding_up_to_date() -> bool:
+    return _newer(BINDING, [CSRC / "binding.cpp"] + sorted(INCLUDE.glob("*.h")))
+
+
+def build_binding(force: bool = False) -> Path:
     """_binding.so against the installed torch (its headers and libraries)."""
+    if not force and binding_up_to_date():
+        return BINDING
     import sysconfig
 
     import torch
@@ -64,17 +71,29 @@ def _build_binding() -> None:
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for binding.cpp:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, BINDING)
+    return BINDING
 
 
 def build(force: bool = False, verbose: bool = False, defines: tuple = (), lib: Path | None = None,
           build_dir: Path | None = None) -> Path:
     """Compile and link.  `defines` adds -D flags (tuning knobs of the
     kernels); `lib`/`build_dir` redirect the output (default: in-tree, with
-    the Python module's marshalling beside it)."""
-    out_lib = LIB if lib is None else Path(lib)
-    bdir = BUILD if build_dir is None else Path(build_dir)
-    if not force and lib is None and not defines and up_to_date():
-        return LIB
+    the Python module's marshalling beside it; a warning says why where that
+    cannot be built)."""
+    if lib is not None:
+        return _build_lib(Path(lib), BUILD if build_dir is None else Path(build_dir), defines, verbose)
+    with ThreadPoolExecutor(max_workers=1) as ex:
+        binding = ex.submit(build_binding, force)
+        if force or defines or not up_to_date():
+            _build_lib(LIB, BUILD if build_dir is None else Path(build_dir), defines, verbose)
+        try:
+            binding.result()
+        except Exception as e:  # (no torch, no headers, no compiler: the calls take the general code)
+            warnings.warn(f"native marshalling not built: {e}", RuntimeWarning, stacklevel=2)
+    return LIB
+
+
+def _build_lib(out_lib: Path, bdir: Path, defines: tuple, verbose: bool) -> Path:
     bdir.mkdir(parents=True, exist_ok=True)
     objs = []
 
@@ -86,11 +105,8 @@ def build(force: bool = False, verbose: bool = False, defines: tuple = (), lib: 
             raise RuntimeError(f"nvcc failed for {src.name}:\n{r.stdout}\n{r.stderr}")
         return obj, r.stderr
 
-    with ThreadPoolExecutor(max_workers=min(8, len(sources())) + 1) as ex:
-        binding = ex.submit(_build_binding) if lib is None else None
+    with ThreadPoolExecutor(max_workers=min(8, len(sources()))) as ex:
         results = list(ex.map(compile_one, sources()))
-        if binding:
-            binding.result()
     log = []
     for obj, err in results:
         objs.append(obj)
