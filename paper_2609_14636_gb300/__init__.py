@@ -19,6 +19,8 @@ view copies of them as numpy structured arrays.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import warnings
 from pathlib import Path
 
@@ -141,9 +143,10 @@ def _native():
         try:
             import torch  # noqa: F401  (its libraries are the module's)
 
-            _build.build_binding()
-            from . import _binding
-
+            path = str(_build.build_binding())
+            loader = importlib.machinery.ExtensionFileLoader(f"{__name__}._binding", path)
+            _binding = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader, origin=path))
+            loader.exec_module(_binding)
             _binding.bind(*[ctypes.cast(getattr(L, f"stride_{fn}"), ctypes.c_void_p).value for fn in _NATIVE_ENTRIES])
             _NATIVE = _binding
         except Exception as e:

@@ -1,5 +1,7 @@
 """In-tree build of libstride.so for sm_103a (nvcc, no cmake) and of the
-Python module's native marshalling, _binding.so (g++, torch's headers).
+Python module's native marshalling, _binding.<interpreter>.torch-<version>.so
+(g++, torch's headers: it holds that interpreter's and that torch's layouts, so
+another of either gets a file of its own).
 
 Each .cu under csrc/ compiles to an object in parallel; the objects link into
 paper_2609_14636_gb300/libstride.so against the shared CUDA runtime.  Either
@@ -12,6 +14,7 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import sysconfig
 import warnings
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
@@ -22,7 +25,6 @@ CSRC = PKG / "csrc"
 INCLUDE = ROOT / "include"
 BUILD = PKG / "_build"
 LIB = PKG / "libstride.so"
-BINDING = PKG / "_binding.so"
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-Xptxas", "-v",
@@ -47,21 +49,23 @@ def up_to_date() -> bool:
     return _newer(LIB, sources() + sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted(INCLUDE.glob("*.h")))
 
 
-def binding_up_to_date() -> bool:
-    return _newer(BINDING, [CSRC / "binding.cpp"] + sorted(INCLUDE.glob("*.h")))
+def binding() -> Path:
+    """The marshalling of this interpreter and the installed torch."""
+    import torch
+
+    return PKG / f"_binding.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so"
 
 
 def build_binding(force: bool = False) -> Path:
-    """_binding.so against the installed torch (its headers and libraries)."""
-    if not force and binding_up_to_date():
-        return BINDING
-    import sysconfig
-
+    """binding(), built if need be (against torch's headers and libraries)."""
     import torch
 
+    out = binding()
+    if not force and _newer(out, [CSRC / "binding.cpp"] + sorted(INCLUDE.glob("*.h"))):
+        return out
     t = Path(torch.__file__).parent
     cuda = Path(nvcc()).resolve().parent.parent
-    tmp = BINDING.with_name(BINDING.name + f".tmp{os.getpid()}")
+    tmp = out.with_name(out.name + f".tmp{os.getpid()}")
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", str(INCLUDE), "-isystem",
            str(t / "include"), "-isystem", str(t / "include/torch/csrc/api/include"), "-isystem", str(cuda / "include"),
@@ -70,8 +74,8 @@ def build_binding(force: bool = False) -> Path:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for binding.cpp:\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, BINDING)
-    return BINDING
+    os.replace(tmp, out)
+    return out
 
 
 def build(force: bool = False, verbose: bool = False, defines: tuple = (), lib: Path | None = None,
