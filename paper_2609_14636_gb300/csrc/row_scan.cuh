@@ -145,13 +145,18 @@ __device__ __forceinline__ RowMeta find_row_meta(const BatchParams& p, int64_t r
   return m;
 }
 
-// Checks that the CTA owning ticket t makes on the layout arrays: every turn
-// is non-empty, every trajectory's turns cover exactly its rows.
-__device__ __forceinline__ void validate_layout(const BatchParams& p, int64_t t) {
+// Highest set bit of m at or below `lane`, -1 if none.
+__device__ __forceinline__ int head_of(unsigned m, int lane) {
+  return 31 - __clz(m & (0xffffffffu >> (31 - lane)));
+}
+
+// Share `t` of `shares` of the checks on the layout arrays: every turn is
+// non-empty, every trajectory's turns cover exactly its rows.
+__device__ __forceinline__ void validate_layout(const BatchParams& p, int64_t t, int64_t shares) {
   bool bad = false;
-  for (int64_t k = t; k < p.n_turns; k += p.n_rows)
+  for (int64_t k = t; k < p.n_turns; k += shares)
     bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
-  for (int64_t i = t; i < p.n_traj; i += p.n_rows) {
+  for (int64_t i = t; i < p.n_traj; i += shares) {
     const int32_t a = __ldg(p.traj_turn_off + i), b = __ldg(p.traj_turn_off + i + 1);
     if (a < 0 || b < a || b > p.n_turns) {
       bad = true;

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) score_batch_kernel(const Bat
     }
     meta = find_row_meta(p, r, lane);
   } else if (warp == 1 && lane == 0) {
-    validate_layout(p, tile);
+    validate_layout(p, tile, p.n_rows);
   }
 
   float mS = kMaxStart, sS = 0.f, mT = kMaxStart, sT = 0.f;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocksPerSm)
     xs = to_f32(srow[y]);
     xt = to_f32(trow[y]);
   } else if (rank == 0 && tid == 32) {
-    validate_layout(p, tile);
+    validate_layout(p, tile, p.n_rows);
   }
   warp_merge2(mS, sS, mT, sT);
   if (lane == 0) {

@@ -46,7 +46,6 @@ struct PartialParams {
   int64_t ld;
   int32_t V_shard;
   int64_t col0;
-  int32_t V_total;
   const int32_t* tokens;
   int64_t rows;
   float* partials;  // [rows][6]
@@ -607,11 +606,6 @@ __device__ __forceinline__ Sum seg_sum(Sum v, int head, int lane) {
   return v;
 }
 
-// Highest set bit of m at or below `lane`, -1 if none.
-__device__ __forceinline__ int head_of(unsigned m, int lane) {
-  return 31 - __clz(m & (0xffffffffu >> (31 - lane)));
-}
-
 // A thread's or tile's element without the carried state: sums since the last
 // seeded row (c) and since the last turn start (st, sd, sl).
 template <typename Sum>
@@ -1093,24 +1087,6 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     }
   }
   record_parts(p, part, lane);
-}
-
-// Layout checks, spread over every thread of a grid of n_tiles CTAs.
-__device__ __forceinline__ void check_layout(const BatchParams& p, int64_t tile, int64_t n_tiles, int tid) {
-  bool bad = false;
-  const int64_t stride = n_tiles * kPassThreads;
-  const int64_t at = tile * kPassThreads + tid;
-  for (int64_t k = at; k < p.n_turns; k += stride) bad |= __ldg(p.turn_row_off + k + 1) <= __ldg(p.turn_row_off + k);
-  for (int64_t i = at; i < p.n_traj; i += stride) {
-    const int32_t a = __ldg(p.traj_turn_off + i), b = __ldg(p.traj_turn_off + i + 1);
-    if (a < 0 || b < a || b > p.n_turns) {
-      bad = true;
-    } else {
-      bad |= __ldg(p.turn_row_off + a) != __ldg(p.traj_row_off + i);
-      bad |= __ldg(p.turn_row_off + b) != __ldg(p.traj_row_off + i + 1);
-    }
-  }
-  if (bad) set_status(p.dev_status, STRIDE_DEV_BAD_LAYOUT);
 }
 
 // A small window's scan after the small-window kernel, one tile of TILE
@@ -1598,7 +1574,7 @@ __global__ void __launch_bounds__(kPassThreads, 3) scan_complete_kernel(const Ba
   if (p.profile) rows_profile(x, tid & 31, s_prof);
   if (!complete_tile<Sum2>(p, L, tile, tid, x, prefixed, sh)) complete_tile<double>(p, L, tile, tid, x, prefixed, sh);
   if (p.profile && tid < 3 * STRIDE_PROFILE_BINS && s_prof[tid] != 0.0) atomicAdd(p.profile + tid, s_prof[tid]);
-  if (validate) check_layout(p, tile, n_tiles, tid);
+  if (validate) validate_layout(p, tile * kPassThreads + tid, n_tiles * kPassThreads);
 }
 
 // Whether a shard pass takes the persistent kernel (score_batch_stream.cu)
@@ -1640,7 +1616,7 @@ cudaError_t launch_partial_lse(const void* S, const void* T, int dtype, bool vec
   const int64_t waves_many = (rows + kPartialManyCtas * sms - 1) / (kPartialManyCtas * sms);
   const int64_t waves_loads = (rows + kPartialManyLoads * sms - 1) / (kPartialManyLoads * sms);
   const bool loads = rows >= 5 * (int64_t)sms && (waves_loads == waves_many || waves_loads > 5);
-  const PartialParams p{S, T, ld, V_shard, col0, 0, tokens, rows, partials, dev_status,
+  const PartialParams p{S, T, ld, V_shard, col0, tokens, rows, partials, dev_status,
                         (int64_t)(loads ? kPartialManyLoads : kPartialManyCtas) * sms};
   const bool bf16 = dtype == STRIDE_DTYPE_BF16;
   auto* kern = loads ? (bf16 ? (vec ? partial_lse_kernel<__nv_bfloat16, true, 5> : partial_lse_kernel<__nv_bfloat16, false, 5>)

@@ -86,11 +86,6 @@ __device__ __forceinline__ double seg_sum(double v, int head, int lane) {
   return v;
 }
 
-// Highest set bit of m at or below `lane`, -1 if none.
-__device__ __forceinline__ int head_of(unsigned m, int lane) {
-  return 31 - __clz(m & (0xffffffffu >> (31 - lane)));
-}
-
 // A published tile on its way to the scan warp (shared memory, by lane).
 struct TileCarry {
   double c[32], st[32], sd[32], sl[32];  // inclusive within the tile (seeded rows: from the carried state)
@@ -200,7 +195,7 @@ __device__ __forceinline__ void publish_tile(const BatchParams& p, int64_t t, in
     tc.tile = t;
   }
   // this tile's share of the layout checks
-  if (live) validate_layout(p, w);
+  if (live) validate_layout(p, w, p.n_rows);
 }
 
 // Completes a published tile.  Warp-wide.
