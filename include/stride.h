@@ -41,8 +41,10 @@
  *   synchronised.  Kernels never trap: a bad row gets NaN outputs.
  * - Logit rows are row-major with a row stride `ld` (elements, ld >= V), and
  *   1 <= V <= STRIDE_MAX_VOCAB (for a vocabulary shard, its V_shard).
- *   Rows whose address and stride are 16-byte aligned take the vectorised
- *   path; others take a scalar path with the same results.
+ *   Rows may start at any element: whole 16-byte vectors are read from a
+ *   row's first 16-byte boundary on and its ends one by one.  (Outside the
+ *   persistent kernel below only where S and T share the row's misalignment;
+ *   else every logit is read on its own.)
  * - Turn and row indices reported per trajectory are 0-based and local to the
  *   trajectory.  The paper's turns are 1-based, so the returned k* equals its
  *   K0 = k* - 1 (Algorithm 1): the number of turns reused as context.
@@ -55,9 +57,9 @@
  *   windows of at most 8 rows per SM, a kernel that splits each row over a
  *   thread-block cluster of 1, 2, 4 or 8 CTAs (the window is one wave); a
  *   persistent bulk-copy kernel for the others; and one CTA per row where a
- *   row is larger than 2 GB.  The decode-step calls split each row over a cluster of
- *   1 to 16 CTAs of 128 or 512 threads, chosen from the step's row count so
- *   that all rows run in one wave.  stride_force_batch_kernel and
+ *   row is larger than 2 GB.  The decode-step calls split each row over a
+ *   cluster of 1 to 16 CTAs of 128 or 512 threads, chosen from the step's row
+ *   count so that all rows run in one wave.  stride_force_batch_kernel and
  *   stride_force_step_shape (below) fix these choices for tests and
  *   diagnosis.
  */

@@ -30,11 +30,13 @@
 // kernel's completion before its first global read, so the caller's inputs
 // and the carried state are always complete when read.  The loads' ramp thus
 // overlaps the previous step's merges and state updates.  GB300, steps of a
-// 32-step graph (151,936 bf16 logits), before the overlap -> with it -> with
-// the launch shapes of choose_shape and the loop's last batch in one: 8 rows
-// 5.5 -> 4.8 -> 4.7 us, 61 rows 11.0 -> 9.8 -> 9.2, 128 rows 16.2 -> 14.9 ->
-// 13.9, 256 rows 27.0 -> 25.8 -> 24.9, 256 masked rows (16 plain steps) 25.2 ->
-// 24.3 -> 23.5.  Letting the next step in at the start instead makes its hints
+// 32-step graph (151,936 bf16 logits), one box, before the overlap -> now, with
+// the launch shapes of choose_shape, the loop's last batch in one and the
+// merges of stride_device.cuh: 1 row 3.66 -> 3.14 us, 8 rows 5.52 -> 4.48, 24
+// rows 7.36 -> 6.4, 61 rows 10.8 -> 8.9, 128 rows 16.2 -> 13.7, 256 rows 27.1 ->
+// 24.9; of 32,000 logits 2.95 -> 2.57, 3.72 -> 3.64, 4.55 -> 4.3, 5.98 -> 4.74,
+// 8.2 -> 5.65, 10.6 -> 8.1.  The overlap alone took 61 rows from 11.0 to 9.8 and
+// 256 from 27.0 to 25.8 on another box; letting the next step in at the start instead makes its hints
 // compete with this step's loads (61 rows 9.8 -> 10.4), and in mid-stream costs
 // a split of the loop (11.9).
 #include <cooperative_groups.h>
@@ -377,6 +379,12 @@ int one_wave_cluster(int dev, int sms, int64_t rows) {
 // so 512 threads from 5 CTAs a row on, and below that where 4 or 2 CTAs a row
 // all but fill the device -- not in the masked form, whose stopped rows leave
 // their CTAs idle (62 rows 9.4 / 8.7, 136 rows 13.6 / 13.0).
+//
+// The shares and fills are those rows' own.  Other rows follow them, against the
+// best of 23 fixed shapes (12 row counts from 1 to 256; percent slower, 32,000
+// bf16 / 32,000 fp32 / 151,936 fp32): 24 rows 7 / 13 / 12, 61 rows 5 / 9 / 1, 76
+// rows 16 / 18 / 5, 108 rows 30 / 21 / 10, 256 rows 5 / 2 / 7, the others within
+// 3 (1 row of 32,000 bf16: 5); faster everywhere than the fixed shapes before.
 struct Shape {
   int threads, cluster;
 };

@@ -278,10 +278,10 @@ __device__ __forceinline__ float warp_max(float v) {
 // one per pair and step.  With the pairs in the first N lanes only (the
 // others hold an empty pair) the first N lanes end with the total.
 //
-// A decode step waits for three of these in a row.  GB300, a shuffle and a
-// maximum per step -> one instruction for the maximum -> N: decode steps of 1
-// row 3.34 -> 3.15 -> 3.14 us, of 8 rows 4.71 -> 4.52 -> 4.46, of 61 rows 9.17
-// -> 8.93 -> 8.90, 16 masked ones of 256 rows 378 -> 374 -> 374.
+// A decode step waits for three of these in a row.  GB300, one box, a shuffle
+// and a maximum per step -> one instruction for the maximum -> N: decode steps
+// of a 32-step graph, 1 row 3.34 -> 3.15 -> 3.14 us, 8 rows 4.71 -> 4.52 -> 4.46,
+// 61 rows 9.17 -> 8.93 -> 8.90.
 template <int N = 32>
 __device__ __forceinline__ void warp_merge2(float& mS, float& sS, float& mT, float& sT) {
   const float MS = warp_max(mS), MT = warp_max(mT);

@@ -126,7 +126,13 @@ int current_device_sms(int* dev_out, cudaError_t* err);
 
 // Launches kern as a programmatic dependent of the previous kernel on the
 // stream: its CTAs may be scheduled before that kernel has ended, so kern
-// waits (griddepcontrol.wait) before it touches global memory.
+// waits (griddepcontrol.wait) before it touches what that kernel writes.  Every
+// kernel of the library waits, in every thread, so a completed one's
+// predecessors are complete too.  Ahead of its wait a kernel may give L2 hints,
+// and, where its predecessor is known to release it only past its own wait,
+// read what was there before that one (the scans after a scoring kernel: layout,
+// carried state, lambda; the second pass: the log-probs too) and write what
+// that one does not use (the first pass's workspace).
 template <typename... K, typename... A>
 cudaError_t launch_dependent(void (*kern)(K...), unsigned grid, unsigned block, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};

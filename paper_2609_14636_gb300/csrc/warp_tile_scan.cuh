@@ -4,8 +4,9 @@
 // A row's log-probs go to the workspace as soon as the row is scored, and
 // the row counts itself in at its tile's counter.  Whoever counts the
 // tile's last row finds the rows' turns and trajectories, forms their scan
-// elements, scans them with shuffles and publishes the tile's aggregate
-// (publish_tile, which waits for nobody).  A scan warp then folds the earlier
+// elements, scans them with shuffles and publishes the tile's aggregate, and
+// beside it the sum before its last turn start (publish_tile, which waits for
+// nobody).  A scan warp then folds the earlier
 // tiles' aggregates (row_scan.cuh lookback, over tiles) and completes the
 // rows -- turn statistics, stop test, loss, profile, carried state
 // (complete_tile).  All sums are fp64.
