@@ -254,6 +254,20 @@ struct RowCarry {
   int seeded;
 };
 
+// Whether a running sum is below lambda.  The sum at a test and the sum before
+// the next turn (or token) are formed in different orders, some 64 roundings
+// each at most (2^-47), and have to fall on the same side: so within 2^-43 to
+// 2^-44 of lambda they count as equal to it, which is not below.  (Sums equal
+// to lambda but for the rounding of their quotients are no accident: a mean of
+// log-probs on a common grid is an fp32 number as often as their count divides
+// the sum.)  The bound is lambda's low bits in fp64, which are zero otherwise;
+// an infinite, NaN or zero lambda stays itself (-inf as a NaN: nothing is below).
+__device__ __forceinline__ double stop_bound(float lam) {
+  const long long b = __double_as_longlong((double)lam);
+  return __longlong_as_double(lam == 0.f ? b : lam < 0.f ? b + 512 : b - 512);
+}
+__device__ __forceinline__ bool below(double sum, float lam) { return sum < stop_bound(lam); }
+
 // Whether the rule fired before a row's turn, in turn mode: c0 is the sum
 // before that turn.  Of a turn that was open where the window began the
 // carried state tells: the rule is recorded there if it had fired (what this
@@ -261,7 +275,7 @@ struct RowCarry {
 __device__ __forceinline__ bool fired_before_turn(const BatchParams& p, const RowMeta& meta, double c0, float lam) {
   if (meta.turn_start < p.row_begin)
     return (uint32_t)__ldcg(&p.state[meta.traj].stop_turn) < (uint32_t)meta.local_turn;
-  return c0 < (double)lam;
+  return below(c0, lam);
 }
 
 __device__ __forceinline__ RowCarry row_finalize(const BatchParams& p, int64_t tile, int64_t r,
@@ -393,7 +407,7 @@ __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const 
   const float lam = p.lambda ? __ldg(p.lambda + meta.traj) : p.lambda_all;
   stride_scan_state* sp = p.state + meta.traj;
   if (!defer_traj) {
-    if (test && incl.c < (double)lam) {
+    if (test && below(incl.c, lam)) {
       atomicMin(reinterpret_cast<unsigned long long*>(&sp->stop_row),
                 (unsigned long long)(r - meta.traj_start));
       atomicMin(reinterpret_cast<unsigned int*>(&sp->stop_turn), (unsigned int)meta.local_turn);
@@ -401,7 +415,7 @@ __device__ __forceinline__ void row_tail(const BatchParams& p, int64_t r, const 
     }
     const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
     const bool fired =
-        (p.mode == STRIDE_STOP_TOKEN_SUM) ? c_before < (double)lam : fired_before_turn(p, meta, c0, lam);
+        (p.mode == STRIDE_STOP_TOKEN_SUM) ? below(c_before, lam) : fired_before_turn(p, meta, c0, lam);
     if (first || !fired) {  // the previous test did not fire (a NaN lambda never does)
       atomicAdd(&sp->loss, rc.e.sl);
       atomicAdd(reinterpret_cast<unsigned long long*>(&sp->loss_tokens), 1ull);

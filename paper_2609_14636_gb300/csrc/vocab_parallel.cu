@@ -1040,7 +1040,7 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
     // retained unless the rule fired before the row (row_scan.cuh); a
     // trajectory's first token or turn always is
     if (token_sum) {
-      kept = r == m.traj_start || !(c < (double)lam);
+      kept = r == m.traj_start || !below(c, lam);
     } else if (i == 0 || seeded || fturn) {
       double c0 = c;  // the sum before the row's turn
       if (!fturn) {
@@ -1058,7 +1058,7 @@ __device__ __forceinline__ void complete_rows(const BatchParams& p, const TileLa
       sum_add(part.loss, l);
       ++part.count;
     }
-    if ((token_sum || turn_last) && part.cross_row < 0 && c < (double)lam) {
+    if ((token_sum || turn_last) && part.cross_row < 0 && below(c, lam)) {
       part.cross_row = r - m.traj_start;
       part.cross_turn = m.local_turn;
     }
@@ -1270,11 +1270,11 @@ __device__ __forceinline__ bool scan_cluster_rows(const BatchParams& p, const Cl
     // retained unless the rule fired before the row (row_tail); a
     // trajectory's first token or turn always is
     const bool first = (p.mode == STRIDE_STOP_TOKEN_SUM) ? (r == meta.traj_start) : (meta.local_turn == 0);
-    const bool kept = first || !(turn_mean ? fired_before_turn(p, meta, c0, q.lam) : c_before < (double)q.lam);
+    const bool kept = first || !(turn_mean ? fired_before_turn(p, meta, c0, q.lam) : below(c_before, q.lam));
     part.traj = meta.traj;
     part.count = kept ? 1 : 0;
     if (kept) part.loss = cluster_term(e_sl);
-    if (test && ri_c < (double)q.lam) {
+    if (test && below(ri_c, q.lam)) {
       part.cross_row = r - meta.traj_start;
       part.cross_turn = meta.local_turn;
     }

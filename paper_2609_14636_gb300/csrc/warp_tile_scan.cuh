@@ -262,9 +262,9 @@ __device__ __forceinline__ void complete_tile(const BatchParams& p, const TileCa
     ts.n = (int32_t)n_k;
     p.turn_stats[meta.turn] = ts;
   }
-  const bool cross = good && (token_sum || turn_last) && c < (double)lam;
+  const bool cross = good && (token_sum || turn_last) && below(c, lam);
   const bool first = token_sum ? r == meta.traj_start : meta.local_turn == 0;
-  const bool kept = good && (first || !(token_sum ? c_before < (double)lam : fired_before_turn(p, meta, c0, lam)));
+  const bool kept = good && (first || !(token_sum ? below(c_before, lam) : fired_before_turn(p, meta, c0, lam)));
 
   // ---- the trajectories' records, once per trajectory and tile
   const unsigned m_traj = __ballot_sync(0xffffffffu, !good || r == meta.traj_start);

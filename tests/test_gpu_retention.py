@@ -54,7 +54,8 @@ ROUTES = [("split", 700, 64), ("split", 1900, 64), ("stream", 1500, 64), ("strea
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("route, rows, V", ROUTES)
 def test_threshold_at_a_recorded_sum(stride, route, rows, V, mode):
-    """lambda = the running sum after one of the trajectory's turns, rounded to fp32 (1e-8 to 6e-8 off, either way)."""
+    """lambda = the running sum after one of the trajectory's turns, rounded to fp32 (1e-8 to 6e-8 off, either way), or,
+    where the log-probs' grid and the turn's length allow it, the sum itself but for the rounding of its quotients."""
     import torch
 
     rng = np.random.default_rng(rows + mode)
@@ -66,7 +67,7 @@ def test_threshold_at_a_recorded_sum(stride, route, rows, V, mode):
     if V:
         x = torch.from_numpy(rng.standard_normal((rows, V), dtype=np.float32)).cuda()
         y = x + 0.3 * torch.from_numpy(rng.standard_normal((rows, V), dtype=np.float32)).cuda()
-        tok = torch.randint(0, V, (rows,), dtype=torch.int32, device="cuda")
+        tok = torch.from_numpy(rng.integers(0, V, rows).astype(np.int32)).cuda()
 
     def run(lam, windows):
         st, ts = stride.new_state(lay.n_traj), stride.new_turn_stats(lay.n_turns)
@@ -83,11 +84,38 @@ def test_threshold_at_a_recorded_sum(stride, route, rows, V, mode):
     try:
         for windows in (_cuts(rows, 1), _cuts(rows, 2), _cuts(rows, 5)):
             cum = run(-1e30, windows)[1]["cum"]
-            pick = lay.traj_turn_off[:-1] + (rng.random(lay.n_traj) * np.diff(lay.traj_turn_off)).astype(int)
-            lam = cum[pick].astype(np.float32)
-            st, _ = run(torch.from_numpy(lam).cuda(), windows)
-            assert lay.n_traj < 9 or (st["stopped"] != 0).sum() > lay.n_traj // 4
-            np.testing.assert_array_equal(st["loss_tokens"], _kept_rows(st, lay, mode))
+            for _ in range(3 if rows > 1_000_000 else 12):
+                pick = lay.traj_turn_off[:-1] + (rng.random(lay.n_traj) * np.diff(lay.traj_turn_off)).astype(int)
+                lam = cum[pick].astype(np.float32)
+                st, _ = run(torch.from_numpy(lam).cuda(), windows)
+                assert lay.n_traj < 9 or (st["stopped"] != 0).sum() > lay.n_traj // 4
+                np.testing.assert_array_equal(st["loss_tokens"], _kept_rows(st, lay, mode))
+    finally:
+        stride.stride_force_batch_kernel("auto")
+
+
+@pytest.mark.parametrize("route, rows, V", ROUTES[1:6])
+def test_threshold_equal_to_a_sum(stride, route, rows, V):
+    """Every log pi_T is the same number p, so every turn's mean is p, and the running sum after two turns is the fp32
+    number 2 p but for the rounding of the quotients p / n: equal to lambda, not below it.  The third turn stops.  (The
+    cluster scan rounds the quotients to fp32, so there only the kept tokens agree with the stop.)"""
+    import torch
+
+    rng = np.random.default_rng(rows)
+    lay = _layout(rng, rows)
+    x = torch.from_numpy(rng.standard_normal((rows, V), dtype=np.float32)).cuda()
+    y = torch.zeros((rows, V), device="cuda")
+    tok = np.zeros(rows, np.int32)
+    stride.stride_force_batch_kernel(route)
+    try:
+        p = run_batch(stride, x, y, tok, lay, 0, np.float32(-1e30))["logp_t"]
+        assert np.all(p == p[0])
+        for k in (1, 2, 5):
+            st = run_batch(stride, x, y, tok, lay, 0, np.float32(2 * p[0]), windows=_cuts(rows, k))["state"]
+            if route != "split":
+                third = np.minimum(2, np.diff(lay.traj_turn_off) - 1)
+                np.testing.assert_array_equal(st["stop_turn"], np.where(third == 2, 2, -1))
+            np.testing.assert_array_equal(st["loss_tokens"], _kept_rows(st, lay, 0))
     finally:
         stride.stride_force_batch_kernel("auto")
 
