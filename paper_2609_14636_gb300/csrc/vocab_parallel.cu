@@ -158,9 +158,10 @@ constexpr int kRestartSum = 2;   // c restarts (a seeded row)
 // loss term are fp32 inside the tile (summed in a tree: relative error a few
 // 1e-7 of the summed magnitudes), in the cluster's fold of at most 16 tile
 // aggregates, and where the tile's prefix meets a row; every stored sum is
-// fp64, as are all sums of a window whose might leave fp32 (`wide`).  GB300 runs FP64 at 1/64 of the FP32 rate, and the tile scans' fp64
-// adds were what a small window's scan waited on (a 512-row window in one
-// CTA: 6.6 us for the block scan).
+// fp64, and so are all sums of a window that might leave fp32's range (`wide`).
+// GB300 runs FP64 at 1/64 of the FP32 rate, and the tile scans' fp64 adds were
+// what a small window's scan waited on (a 512-row window in one CTA: 6.6 us for
+// the block scan).
 template <typename F>
 struct TileElem {
   double c;
@@ -761,10 +762,9 @@ struct AggregateShared {
   double open[3][kPassWarps];
 };
 
-// First pass: tile t's aggregate in tiles[t], and in incl[w] the carried state
-// of every seeded row w.  z is the carried state of the thread's last seeded
-// row.  False, with nothing written, if the
-// tile's sums need more than Sum.
+// First pass: tile t's aggregate (TileSlot), and in incl[w] the carried state of
+// every seeded row w.  z is the carried state of the thread's last seeded row.
+// False, with nothing written, if the tile's sums need more than Sum.
 template <typename Sum, int R, bool EXACT>
 __device__ __forceinline__ bool aggregate_tile(const BatchParams& p, int64_t tile, int tid, const Rows<R, EXACT>& x,
                                                const ScanSlot& z, AggregateShared& sh) {
